@@ -227,3 +227,20 @@ def tolerance(case):
     # Against the same product in 64 bits: one vector (multiply-adds, each rounded) 0.9e-7 .. 2.3e-7 over the listed shapes;
     # more vectors (the tensor cores' fp32 accumulators) 2.3e-7 .. 3.8e-6, growing with the columns.  About four times that.
     return {"rel": 2e-6 if case["batch"] == 1 else 1.5e-5}
+
+
+def exact(case, seed):
+    """What run() returns for these inputs, in 64 bits: the weights as they were before compression times the activations."""
+    if case["kind"] in ("decode", "compress"):
+        return None
+    gen = torch.Generator(device="cuda").manual_seed(seed)
+    kind = torch.float16 if case["dtype"] in _FP16 else torch.bfloat16
+    groups = _layer_groups(case) if case["kind"] == "layer" else [[(case["rows"], case["cols"])]]
+    ys = []
+    for shapes in groups:                                            # (drawn from the generator in prepare()'s order)
+        x = _activations(case["batch"], shapes[0][1], case["dtype"], gen).view(kind).double()
+        for rows, cols in shapes:
+            w = _weights(rows, cols, case["dtype"], gen).view(kind).double()
+            ys.append(x @ w.T)
+            del w
+    return ys + [None]                                               # (the error flag has no such value)
