@@ -239,20 +239,32 @@ huffllm_status add_matrix(KernelArgs *k, const huffllm_desc *desc, const void *b
 // Close a launch description: shared-memory budget and grid size.
 huffllm_status finish_args(KernelArgs *k, bool product, const DeviceInfo &dev, uint32_t *grid, uint32_t *warps_at_least = nullptr) {
     // (pieces that warps of a CTA exchange: in shared memory up to 8 vectors, in the workspace above)
-    k->part_bytes = product && k->batch <= kKernelBatch ? 2 * 32 * 16 * k->batch * (uint32_t)sizeof(float) : 0;
+    if (product) k->part_bytes = k->batch <= kKernelBatch ? 2 * 32 * 16 * k->batch * (uint32_t)sizeof(float) : 0;
     if (k->fmt && k->lut_bits <= 8) k->lut_size = fp16_table_bytes(k);
     // Two slots per decoder warp, so that a warp's next record lands while it decodes this one.  Where records are so large
     // that this would leave fewer than 31 warps a slot pair, and single slots serve at least a quarter more warps, every
     // warp gets one slot: more decoders at work outweigh the wait for a copy at every chunk start.
     const uint64_t max_w = 31;                                       // decoder warps of a CTA of 1024 threads
-    uint64_t w2 = planned_warps(k->lut_align, k->lut_size, 2ull * k->slot_bytes, k->dyn_smem_bytes, k->part_bytes, k->guard_bytes);
-    uint64_t w1 = planned_warps(k->lut_align, k->lut_size, k->slot_bytes, k->dyn_smem_bytes, k->part_bytes, k->guard_bytes);
-    if (w2 > max_w) w2 = max_w;
-    if (w1 > max_w) w1 = max_w;
+    // (decode to rows that do not start on 16-byte boundaries: every warp takes room for the rows it works on, as many warps
+    // as find both a slot and that room; one always does: its room is no larger than the guard area)
+    const bool row_bufs = !product && k->m[0].cols % 8;
+    auto warps_with = [&](uint64_t pair_bytes) -> uint64_t {
+        uint64_t best = 0;
+        for (uint64_t n = row_bufs ? max_w : 1; n > best; --n) {
+            if (row_bufs) k->part_bytes = (uint32_t)n * 16 * kRowBuf;
+            const uint64_t w = planned_warps(k->lut_align, k->lut_size, pair_bytes, k->dyn_smem_bytes, k->part_bytes, k->guard_bytes);
+            const uint64_t got = row_bufs ? (w < n ? w : n) : (w < max_w ? w : max_w);
+            if (got > best) best = got;
+            if (!row_bufs) break;
+        }
+        return best;
+    };
+    const uint64_t w2 = warps_with(2ull * k->slot_bytes), w1 = warps_with(k->slot_bytes);
     const bool single_ok = k->fmt || k->lut_bits == 8;                // (the kernels that exist with single slots)
     k->slots = single_ok && w2 < max_w && 4 * w1 >= 5 * w2 ? 1u : 2u;
     if ((k->slots == 2 ? w2 : w1) == 0)
         return fail(HUFFLLM_ERR_UNSUPPORTED, "chunk records too large for shared memory (slot %u bytes)", k->slot_bytes);
+    if (row_bufs) k->part_bytes = (uint32_t)(k->slots == 1 ? w1 : w2) * 16 * kRowBuf;
     if (warps_at_least) *warps_at_least = (uint32_t)(k->slots == 1 ? w1 : w2);
     k->pair_recip = (uint32_t)(0x100000000ull / ((uint64_t)k->slots * k->slot_bytes));
     uint64_t g = k->total_chunks < (uint64_t)dev.sms ? k->total_chunks : (uint64_t)dev.sms;

@@ -33,9 +33,58 @@
 
 namespace huffllm {
 
+// ------------------------------------------------------------------------------ decode to rows that start anywhere
+
+// Where the column count is not a multiple of 8, a row starts anywhere in a 32-byte sector of the output, `row_off` weights
+// behind its start.  What bounds the output is L2's handling of sector writes, so the warp stores whole sectors: each of its
+// 16 rows has 96 bytes of shared memory (the row's last sixteen weights of the block before, then the block's 32); a lane
+// writes its own eight weights there and reads back, moved on by row_off weights, the five words that its 16-byte piece of
+// the output covers (a word offset, then half a word by byte permutation).  A quad's four pieces are two whole sectors.
+// Only the pieces at the two ends of a chunk's columns are stored in parts.
+// Measured (BF16, 11007 x 4099 / 28672 x 8191; 11008 x 4096 takes 38.9 us): every lane storing its eight weights one by
+// one, 320 partial sector writes per block of 512 weights, 178 us / -; pieces on 16-byte boundaries through quad shuffles,
+// 48 sectors per block, 57 / 293 us; through shared memory 56 / 291; on 32-byte boundaries (this) 48 / 227 us.
+__device__ __forceinline__ void sts_row(uint32_t addr, const uint32_t *v) {
+    asm volatile("st.shared.v4.u32 [%0], {%1, %2, %3, %4};" ::"r"(addr), "r"(v[0]), "r"(v[1]), "r"(v[2]), "r"(v[3]) : "memory");
+}
+__device__ __forceinline__ uint4 shifted_piece(uint32_t row_word0, uint32_t sel) {     // row_word0: address of the first of the five words
+    uint32_t u[5];
+#pragma unroll
+    for (int j = 0; j < 5; ++j) u[j] = lds_stream(row_word0 + 4 * j);
+    return make_uint4(prmt(u[0], u[1], sel), prmt(u[1], u[2], sel), prmt(u[2], u[3], sel), prmt(u[3], u[4], sel));
+}
+// The part of a piece that lies in columns [0, lim) of its chunk, the piece starting in column c.  A piece that is cut at
+// one end only (all but those of rows shorter than a piece) takes three stores of 8, 4 and 2 bytes: n weights from its
+// front or up to its end fall into such stores by the bits of n.
+__device__ __forceinline__ void store_piece(uint16_t *dst, const uint4 &p, int32_t c, int32_t lim) {
+    if (c >= 0 && c + 8 <= lim) {
+        *(uint4 *)dst = p;
+        return;
+    }
+    const int32_t lo = max(-c, 0), hi = min(lim - c, 8);        // weights lo .. hi - 1 of the piece
+    if (lo >= hi) return;
+    const uint32_t w[4] = {p.x, p.y, p.z, p.w};
+    if (hi == 8) {
+        const int32_t n = 8 - lo;
+        if (n & 4) *(uint2 *)(dst + 4) = make_uint2(w[2], w[3]);
+        if (n & 2) *(uint32_t *)(dst + ((n & 4) ? 2 : 6)) = (n & 4) ? w[1] : w[3];
+        if (n & 1) dst[lo] = (uint16_t)((n & 4) ? ((n & 2) ? w[0] : w[1]) >> 16 : ((n & 2) ? w[2] : w[3]) >> 16);
+    } else if (lo == 0) {
+        if (hi & 4) *(uint2 *)dst = make_uint2(w[0], w[1]);
+        if (hi & 2) *(uint32_t *)(dst + (hi & 4)) = (hi & 4) ? w[2] : w[0];
+        if (hi & 1) dst[hi - 1] = (uint16_t)((hi & 4) ? ((hi & 2) ? w[3] : w[2]) : ((hi & 2) ? w[1] : w[0]));
+    } else {
+#pragma unroll
+        for (int i = 0; i < 8; ++i)
+            if (i >= lo && i < hi) dst[i] = (uint16_t)(w[i >> 1] >> (16 * (i & 1)));
+    }
+}
+
 // ------------------------------------------------------------------------------ the fused kernel
 
-// MODE 0: write the decoded weights.  MODE 1: y = W x for up to 8 activation vectors.
+// MODE 0: write the decoded weights (rows of a multiple of 8 columns: every lane's eight weights are one aligned store).
+// MODE 2: write the decoded weights of a matrix whose rows start anywhere (see store_piece).  MODE 1: y = W x for up to 8
+// activation vectors.
 // LB = table index bits (the blobs' lut_bits): 8 or 9; LB = 12 stands for every longer limit up to 12 (BF16: 10..12,
 // FP16: 9..12): two-level lookup, the number of bits is A.lut_bits.
 // FMT = 0: BF16 blobs; FMT = 1: FP16 {1,5,5,5} blobs (three lookups per weight, sign bits as the raw part); FMT = 2: the same
@@ -86,7 +135,7 @@ __global__ void __launch_bounds__(THREADS, 1) huff_kernel(const __grid_constant_
     pdl_launch_dependents();   // the next kernel's set-up may overlap this kernel's tail
     const uint32_t smem_base = smem_u32(dyn_smem);
     const uint32_t feeder = nwarps_launched - 1;
-    const SmemPlan plan = plan_smem(smem_base, A, feeder, SLOTS);
+    const SmemPlan plan = plan_smem(smem_base, A, MODE == 2 ? min(feeder, A.part_bytes / (16u * kRowBuf)) : feeder, SLOTS);
     const uint32_t nw = plan.warps;                            // decoder warps
     const uint32_t vals = 16 * A.batch;
     // the pieces of row groups that several warps of the CTA share: [2 * warps][16 * batch], in shared memory (NT = 1)
@@ -439,7 +488,18 @@ __global__ void __launch_bounds__(THREADS, 1) huff_kernel(const __grid_constant_
                 const uint32_t col0 = kc * k.chunk_cols + t * 8u;
                 // (activations: lanes of unused output columns repeat the last vector; cols is a multiple of 32
                 // here, so every block of the chunk lies inside the row and xq ends the chunk where the next begins)
-                uint16_t *out0 = MODE == 0 ? k.out + ((uint64_t)rg * 16 + g) * k.cols + col0 : nullptr;
+                // (MODE 2: the chunk's first column, moved back to the 32-byte boundary in front of it; rows g + 8 h)
+                uint32_t row_off[2] = {0u, 0u};
+                if (MODE == 2)
+#pragma unroll
+                    for (int h = 0; h < 2; ++h)
+                        row_off[h] = ((uint32_t)((uint64_t)rg * 16 + g + 8 * h) * (uint32_t)k.cols + (uint32_t)((uintptr_t)k.out >> 1)) & 15u;
+                const int32_t lim = MODE == 2 ? (int32_t)min(k.chunk_cols, (uint32_t)k.cols - kc * k.chunk_cols) : 0;
+                // (MODE 2: this lane's sixteen bytes of row g in the warp's buffer; rows g + 8 follow 8 rows further on; the piece's
+                // five words start (row_off + 1) / 2 words in front of them, its weights half a word further where row_off is odd)
+                const uint32_t row_buf = MODE == 2 ? smem_base + A.dyn_smem_bytes - A.part_bytes + (warp * 16u + g) * kRowBuf + 32u + t * 16u : 0u;
+                const uint32_t half_sel = (row_off[0] & 1u) ? 0x5432u : 0x3210u;       // (rows g and g + 8 start 8 * cols weights apart)
+                uint16_t *out0 = MODE != 1 ? k.out + ((uint64_t)rg * 16 + g) * k.cols + col0 : nullptr;
                 const uint32_t last = nkb - 1;
 
                 // one block: start the fetch of the next block's raw bytes into `nxt`, decode with `cur`
@@ -509,19 +569,26 @@ __global__ void __launch_bounds__(THREADS, 1) huff_kernel(const __grid_constant_
                                 mma_bf16_16816(acc1, a[2], a[6], a[3], a[7], xw.z, xw.w);
                             }
                         }
-                    } else {
-                        const uint32_t col = col0 + kb * 32u;
+                    } else if (MODE == 2) {
+#pragma unroll
+                        for (int h = 0; h < 2; ++h) sts_row(row_buf + 8 * kRowBuf * h, a + 4 * h);
+                        __syncwarp();
 #pragma unroll
                         for (int h = 0; h < 2; ++h) {
-                            if ((uint64_t)rg * 16 + g + 8 * h >= k.rows || col >= (uint32_t)k.cols) continue;
-                            uint16_t *dst = out0 + (uint64_t)(8 * h) * k.cols + kb * 32u;
-                            if (k.cols % 8 == 0) {
-                                *(uint4 *)dst = make_uint4(a[4 * h], a[4 * h + 1], a[4 * h + 2], a[4 * h + 3]);
-                            } else {
+                            const uint4 piece = shifted_piece(row_buf + 8 * kRowBuf * h - ((row_off[h] + 1u) >> 1) * 4u, half_sel);
+                            if ((uint64_t)rg * 16 + g + 8 * h < k.rows)
+                                store_piece(out0 + (uint64_t)(8 * h) * k.cols + kb * 32u - row_off[h], piece, (int32_t)(kb * 32u + t * 8u - row_off[h]), lim);
+                        }
+                        __syncwarp();
+                        if (t >= 2) {                        // the row's last sixteen weights, for the next block's first pieces
 #pragma unroll
-                                for (int i = 0; i < 8; ++i)
-                                    if (col + i < (uint32_t)k.cols) dst[i] = (uint16_t)(a[4 * h + (i >> 1)] >> (16 * (i & 1)));
-                            }
+                            for (int h = 0; h < 2; ++h) sts_row(row_buf + 8 * kRowBuf * h - 64u, a + 4 * h);
+                        }
+                    } else {
+#pragma unroll
+                        for (int h = 0; h < 2; ++h) {
+                            if ((uint64_t)rg * 16 + g + 8 * h >= k.rows || col0 + kb * 32u >= (uint32_t)k.cols) continue;
+                            *(uint4 *)(out0 + (uint64_t)(8 * h) * k.cols + kb * 32u) = make_uint4(a[4 * h], a[4 * h + 1], a[4 * h + 2], a[4 * h + 3]);
                         }
                     }
                 };
@@ -539,6 +606,16 @@ __global__ void __launch_bounds__(THREADS, 1) huff_kernel(const __grid_constant_
                 for (; kb < nkb; kb += 2) {
                     block(kb, raw_a, raw_b, maybe_last);
                     if (kb + 1 < nkb) block(kb + 1, raw_b, raw_a, maybe_last);
+                }
+                if (MODE == 2) {                 // the chunk's last row_off columns: no lane's piece ends behind them
+                    __syncwarp();
+#pragma unroll
+                    for (int h = 0; h < 2; ++h)
+                        if (t * 8u < row_off[h] && (uint64_t)rg * 16 + g + 8 * h < k.rows)
+                            store_piece(out0 + (uint64_t)(8 * h) * k.cols + nkb * 32u - row_off[h],
+                                        shifted_piece(row_buf + 8 * kRowBuf * h - ((row_off[h] + 1u) >> 1) * 4u, half_sel),
+                                        (int32_t)(nkb * 32u + t * 8u - row_off[h]), min(lim, (int32_t)(nkb * 32u)));
+                    __syncwarp();
                 }
                 if (nkb & 1u) raw_a = raw_b;     // the next chunk's first block always starts in raw_a
                 primed = has_next;
@@ -675,12 +752,19 @@ static cudaError_t launch_slots(const KernelArgs &k, uint32_t grid, cudaStream_t
     return launch_one<MODE, LB, kThreads, FMT, NT, 2>(k, grid, stream);
 }
 
+template <int MODE>
+static cudaError_t launch_decode_mode(const KernelArgs &k, uint32_t grid, cudaStream_t stream) {
+    if (k.fmt && k.lut_bits == 7) return launch_slots<MODE, 7, 1>(k, grid, stream);
+    if (k.fmt && k.lut_bits == 8 && k.fp16_flat) return launch_slots<MODE, 8, 2>(k, grid, stream);
+    if (k.fmt) return k.lut_bits > 8 ? launch_slots<MODE, 12, 1>(k, grid, stream) : launch_slots<MODE, 8, 1>(k, grid, stream);
+    if (k.lut_bits > 9) return launch_one<MODE, 12, kThreads, 0>(k, grid, stream);
+    return k.lut_bits == 8 ? launch_slots<MODE, 8, 0>(k, grid, stream) : launch_one<MODE, 9, kThreads, 0>(k, grid, stream);
+}
+// Rows of a multiple of 8 columns start on 16-byte boundaries (the output does): every lane's eight weights are one store.
+// (Multiples of 8 that are not multiples of 16 stay there although rows then straddle sectors: 11008 x 4104 49.1 us against
+// 50 us with the rows going through shared memory, 28672 x 8184 248 against 227 us.)
 cudaError_t launch_decode(const KernelArgs &k, uint32_t grid, cudaStream_t stream) {
-    if (k.fmt && k.lut_bits == 7) return launch_slots<0, 7, 1>(k, grid, stream);
-    if (k.fmt && k.lut_bits == 8 && k.fp16_flat) return launch_slots<0, 8, 2>(k, grid, stream);
-    if (k.fmt) return k.lut_bits > 8 ? launch_slots<0, 12, 1>(k, grid, stream) : launch_slots<0, 8, 1>(k, grid, stream);
-    if (k.lut_bits > 9) return launch_one<0, 12, kThreads, 0>(k, grid, stream);
-    return k.lut_bits == 8 ? launch_slots<0, 8, 0>(k, grid, stream) : launch_one<0, 9, kThreads, 0>(k, grid, stream);
+    return k.m[0].cols % 8 == 0 ? launch_decode_mode<0>(k, grid, stream) : launch_decode_mode<2>(k, grid, stream);
 }
 
 cudaError_t launch_gemm(const KernelArgs &k, uint32_t grid, cudaStream_t stream) {

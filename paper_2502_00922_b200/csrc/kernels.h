@@ -7,6 +7,10 @@ namespace huffllm {
 
 constexpr uint32_t kMaxMats = 8;   // matrices one launch can work through
 
+// Decode to rows that do not start on 16-byte boundaries: bytes of shared memory for each of the 16 rows that a warp works on
+// (sixteen weights of the block before, the block's 32).
+constexpr uint32_t kRowBuf = 96;
+
 // One matrix of a launch.
 struct MatArgs {
     const uint8_t *blob;       // device

@@ -112,6 +112,17 @@ def test_decode_is_bit_exact(hl, torch, rows, cols, ce, budget, gen):
     assert np.array_equal(got, w)                  # lossless: the oracle's result is the original tensor
 
 
+@pytest.mark.parametrize("rows", [1, 16, 23])
+@pytest.mark.parametrize("cols", [1, 7, 9, 35, 250, 509, 774, 1028])
+@pytest.mark.parametrize("ce,budget,dtype", [(512, 0, 0), (4096, 9, 0), (1024, 0, 1), (1024, 7, 1)])
+def test_decode_to_rows_that_start_off_a_16_byte_boundary(hl, torch, rows, cols, ce, budget, dtype):
+    """Column counts of every remainder modulo 8: shorter than a store, around block (32 columns) and chunk (32 .. 256)
+    ends, rows below and above 8 of a row group; full and partial pieces of every row must not touch their neighbours'."""
+    w = wl.gaussian_weights(rows, cols, 0.02, rows + cols, "fp16") if dtype else make("gauss", rows, cols, rows + cols)
+    up = Uploaded(hl, torch, w, ce, budget, dtype=dtype)
+    assert np.array_equal(gpu_decode(hl, torch, up), w)
+
+
 @pytest.mark.parametrize("rows,cols,ce,budget,gen,batch", [
     (1024, 1024, 4096, 0, "gauss", 1), (37, 300, 1024, 0, "student", 0), (256, 2048, 4096, 0, "patterns", 0),
     (512, 4096, 4096, 9, "student", 5), (272, 2080, 16384, 0, "gauss", 4), (16, 512, 512, 0, "constant", 2),
