@@ -7,7 +7,7 @@
 //   pass 1  code lengths only -> words per sequence of every chunk, coded bits
 //   scan    record offsets (the index section), payload size, largest record
 //   pass 2  raw part and coded part of every record
-//   pass 3  the checksum term of every record
+//   pass 3  the checksum term of every record, a warp each
 #include <cuda_runtime.h>
 
 #include <algorithm>
@@ -245,26 +245,184 @@ __global__ void __launch_bounds__(kEncThreads) encode_write_kernel(const __grid_
     if (A.fp16 && (T.nkb & 1u) && T.q < 32) *(uint16_t *)(raw + T.nkb * 64 + T.q * 2) = 0;   // padding of the sign plane
 }
 
-// Checksum term of every record: the same byte-serial hash the host encoder and the validator use, one thread per
-// record (the records were just written and mostly still sit in L2).
-__global__ void __launch_bounds__(128) encode_checksum_kernel(const __grid_constant__ EncArgs A) {
-    const uint64_t c = (uint64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    unsigned long long term = 0;
-    if (c < A.n_chunks) {
-        const uint32_t r0 = A.index[c], r1 = A.index[c + 1];
-        const uint4 *p = (const uint4 *)(A.payload + (uint64_t)r0 * kRecordUnit);
-        unsigned long long h = 1469598103934665603ull;
-        for (uint64_t i = 0; i < (uint64_t)(r1 - r0) * (kRecordUnit / 16); ++i) {
-            const uint4 q = __ldcg(p + i);
-            const uint32_t x[4] = {q.x, q.y, q.z, q.w};
-#pragma unroll
-            for (int k = 0; k < 16; ++k) h = (h ^ ((x[k >> 2] >> (8 * (k & 3))) & 0xFFu)) * 1099511628211ull;
-        }
-        term = h * (2 * c + 1);
+// ------------------------------------------------------------------------------ checksum of the records
+
+// The format's checksum of a record is byte-serial (h = (h ^ byte) * P mod 2^64, the FNV-1a hash).  Taken as written it
+// leaves the GPU idle: one thread per record spent 193 us on an 11008 x 4096 tensor's 72 MB, most of it waiting for one
+// 16-byte load after the other.  Two facts take it apart:
+//   * The exclusive-or touches only the low byte of h.  With x_i = the low byte before byte b_i, h ^ b_i = h + d_i with
+//     d_i = (x_i ^ b_i) - x_i = b_i - 2 (x_i & b_i), so h_end = h_0 P^n + sum_i d_i P^(n - i): a sum that can be taken in any
+//     order once the x_i are known.
+//   * The x_i form a chain of their own, x' = (x ^ b) * P mod 256, in which bit k of x' is bit k of x ^ b plus something that
+//     depends on the bits below k only.  So if the bits below k are known everywhere, bit k at the end of a stretch of
+//     bytes is bit k at its start, exclusive-or a value that the stretch alone determines: an exclusive-or scan over the
+//     stretches gives bit k at the start of each.  Eight rounds, one per bit, give every stretch its starting x.
+// A warp takes a record; a lane walks four stretches of 4 M bytes at a time, one in each byte of a register (stretch 32 s + l
+// in byte s of lane l).  The rounds for bits 1 to 3 need two instructions per four bytes (P mod 16 = 3: four 4-bit values in
+// the bytes of a word times 3 stay in their bytes); from bit 5 on even and odd bytes are multiplied apart.  The weighted sum
+// goes to the tensor cores as an 8-bit product: the record's bytes (and x & b) times the eight byte limbs of the powers of P,
+// exact in 32-bit integers.  Bound by the integer pipe: some 28 instructions per four bytes.
+constexpr uint64_t kFnvPrime = 1099511628211ull, kFnvStart = 1469598103934665603ull;
+__host__ __device__ constexpr uint64_t fnv_pow(uint64_t base, uint32_t e) {
+    uint64_t r = 1;
+    for (; e; e >>= 1, base *= base)
+        if (e & 1u) r *= base;
+    return r;
+}
+constexpr uint64_t fnv_inverse() {                 // P^-1 mod 2^64 (Newton's iteration doubles the correct bits: 3, 6, ..., 96)
+    uint64_t x = kFnvPrime;
+    for (int i = 0; i < 5; ++i) x *= 2 - kFnvPrime * x;
+    return x;
+}
+constexpr uint64_t kFnvInverse = fnv_inverse();
+static_assert(kFnvInverse * kFnvPrime == 1, "inverse of the hash's multiplier");
+// The sum's weights for stretches of M words: byte j of stretch 32 s + 4 g + t has weight P^(512 M - (32 s + 4 g + t) 4 M - j).
+// The factor of g is taken out (row_factor); limb n of the rest is the B operand: for the product of bytes j = 4 i .. 4 i + 3
+// (A registers in this order), lane 4 n + t holds in byte s of word 0 the limb for j = 4 i, of word 1 for j = 4 i + 2; the odd
+// j, rows g + 8 of A, carry one factor P^-1 more.
+template <int M>
+struct FnvWeights {
+    uint32_t b[M][32][2];
+    uint64_t row_factor[8];
+    constexpr FnvWeights() : b(), row_factor() {
+        for (int i = 0; i < M; ++i)
+            for (int h = 0; h < 2; ++h)
+                for (int t = 0; t < 4; ++t)
+                    for (int s = 0; s < 4; ++s) {
+                        const uint64_t w = fnv_pow(kFnvPrime, 512 * M - (32 * s + t) * 4 * M - (4 * i + 2 * h));
+                        for (int n = 0; n < 8; ++n) b[i][4 * n + t][h] |= (uint32_t)(w >> (8 * n) & 0xFFu) << (8 * s);
+                    }
+        for (int g = 0; g < 8; ++g) row_factor[g] = fnv_pow(kFnvInverse, 16 * M * g);
     }
+};
+__device__ const FnvWeights<7> g_fnv7{};
+__device__ const FnvWeights<3> g_fnv3{};
+
+__device__ __forceinline__ uint32_t xor_and(uint32_t a, uint32_t b, uint32_t m) {       // (a ^ b) & m
+    uint32_t d;
+    asm("lop3.b32 %0, %1, %2, %3, 0x28;" : "=r"(d) : "r"(a), "r"(b), "r"(m));
+    return d;
+}
+__device__ __forceinline__ uint32_t byte_perm(uint32_t a, uint32_t b, uint32_t sel) { return __byte_perm(a, b, sel); }
+__device__ __forceinline__ void mma_u8(int32_t (&d)[4], uint32_t a0, uint32_t a1, uint32_t a2, uint32_t a3, uint32_t b0, uint32_t b1) {
+    asm volatile("mma.sync.aligned.m16n8k32.row.col.s32.u8.u8.s32 {%0,%1,%2,%3}, {%4,%5,%6,%7}, {%8,%9}, {%0,%1,%2,%3};"
+                 : "+r"(d[0]), "+r"(d[1]), "+r"(d[2]), "+r"(d[3])
+                 : "r"(a0), "r"(a1), "r"(a2), "r"(a3), "r"(b0), "r"(b1));
+}
+
+// 512 M bytes of a record (`words`, in shared memory): hash `h` moved on over them.  All lanes hold the same h.
+template <int M>
+__device__ __forceinline__ uint64_t fnv_step(uint64_t h, const uint32_t *words, const FnvWeights<M> &wt, uint32_t lane) {
+    constexpr int N = 4 * M;                       // bytes of a stretch
+    constexpr uint32_t kEven = 0x00FF00FFu, kOdd = 0xFF00FF00u;
+    uint32_t G[N];                                 // G[j]: byte j of the lane's four stretches
+    uint32_t all = 0;
 #pragma unroll
-    for (int o = 16; o; o >>= 1) term += __shfl_xor_sync(0xFFFFFFFFu, term, o);
-    if ((threadIdx.x & 31) == 0 && term) atomicAdd(&A.totals->checksum, term);
+    for (int m = 0; m < M; ++m) {
+        const uint32_t a = words[lane * M + m], b = words[(32 + lane) * M + m], c = words[(64 + lane) * M + m], d = words[(96 + lane) * M + m];
+        const uint32_t t0 = byte_perm(a, b, 0x5140), t1 = byte_perm(c, d, 0x5140), t2 = byte_perm(a, b, 0x7362), t3 = byte_perm(c, d, 0x7362);
+        G[4 * m] = byte_perm(t0, t1, 0x5410);
+        G[4 * m + 1] = byte_perm(t0, t1, 0x7632);
+        G[4 * m + 2] = byte_perm(t2, t3, 0x5410);
+        G[4 * m + 3] = byte_perm(t2, t3, 0x7632);
+        all ^= G[4 * m] ^ G[4 * m + 1] ^ G[4 * m + 2] ^ G[4 * m + 3];
+    }
+    uint32_t X = 0;                                // the stretches' starting low bytes, as far as they are known
+    // e: bit k of each byte = bit k at the end of the stretch if it were 0 at its start; settles bit k of X
+    auto settle = [&](uint32_t e, uint32_t k) {
+        const uint32_t own = e & (0x01010101u << k);
+        uint32_t v = own;
+#pragma unroll
+        for (int o = 1; o < 32; o <<= 1) {
+            const uint32_t up = __shfl_up_sync(0xFFFFFFFFu, v, o);
+            if (lane >= (uint32_t)o) v ^= up;
+        }
+        const uint32_t tot = __shfl_sync(0xFFFFFFFFu, v, 31);
+        const uint32_t in = ((uint32_t)h & (1u << k)) * 0x01010101u;
+        X |= v ^ own ^ in ^ (tot << 8) ^ (tot << 16) ^ (tot << 24);
+    };
+    settle(all, 0);
+#pragma unroll
+    for (uint32_t k = 1; k <= 3; ++k) {
+        uint32_t z = X;
+#pragma unroll
+        for (int j = 0; j < N; ++j) z = xor_and(z, G[j], 0x0F0F0F0Fu) * 3u;
+        settle(z, k);
+    }
+    {   // bit 4 of the product with P mod 32 = 19: bit 4 of 3 times the low four bits, bit 4 and bit 0 of x ^ b
+        uint32_t z = X, acc = all, low = 0;
+#pragma unroll
+        for (int j = 0; j < N; j += 2) {
+            const uint32_t y0 = xor_and(z, G[j], 0x0F0F0F0Fu), z0 = y0 * 3u, y1 = xor_and(z0, G[j + 1], 0x0F0F0F0Fu);
+            z = y1 * 3u;
+            acc ^= z0 ^ z;
+            low ^= y0 ^ y1;
+        }
+        settle(acc ^ (low << 4), 4);
+    }
+#pragma unroll 1
+    for (uint32_t k = 5; k <= 7; ++k) {
+        uint32_t ze = X, zo = X;
+#pragma unroll
+        for (int j = 0; j < N; ++j) {
+            ze = xor_and(ze, G[j], kEven) * 0xB3u;
+            zo = xor_and(zo, G[j], kOdd) * 0xB3u;
+        }
+        settle((ze & kEven) | (zo & kOdd), k);
+    }
+    int32_t sb[4] = {0, 0, 0, 0}, sv[4] = {0, 0, 0, 0};
+    uint32_t ze = X, zo = X;
+#pragma unroll
+    for (int i = 0; i < M; ++i) {
+        uint32_t v[4];
+#pragma unroll
+        for (int j = 0; j < 4; ++j) {
+            const uint32_t g = G[4 * i + j];
+            v[j] = ((ze & kEven) | (zo & kOdd)) & g;
+            ze = xor_and(ze, g, kEven) * 0xB3u;
+            zo = xor_and(zo, g, kOdd) * 0xB3u;
+        }
+        const uint2 w = __ldg((const uint2 *)&wt.b[i][lane][0]);
+        mma_u8(sb, G[4 * i], G[4 * i + 1], G[4 * i + 2], G[4 * i + 3], w.x, w.y);
+        mma_u8(sv, v[0], v[1], v[2], v[3], w.x, w.y);
+    }
+    const uint32_t t = lane & 3u;
+    auto limbs = [&](int32_t lo, int32_t hi) -> uint64_t { return ((uint64_t)(int64_t)lo + ((uint64_t)(int64_t)hi << 8)) << (16u * t); };
+    uint64_t sum = (limbs(sb[0] - 2 * sv[0], sb[1] - 2 * sv[1]) + limbs(sb[2] - 2 * sv[2], sb[3] - 2 * sv[3]) * kFnvInverse) *
+                   __ldg((const unsigned long long *)&wt.row_factor[lane >> 2]);
+#pragma unroll
+    for (int o = 16; o; o >>= 1) sum += __shfl_xor_sync(0xFFFFFFFFu, (unsigned long long)sum, o);
+    constexpr uint64_t kOver = fnv_pow(kFnvPrime, 512 * M);
+    return h * kOver + sum;
+}
+
+constexpr uint32_t kSumWarps = 4;
+
+__global__ void __launch_bounds__(32 * kSumWarps) encode_checksum_kernel(const __grid_constant__ EncArgs A) {
+    __shared__ uint32_t s_words[kSumWarps][7 * 128];
+    const uint32_t lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    const uint64_t c = (uint64_t)blockIdx.x * kSumWarps + warp;
+    if (c >= A.n_chunks) return;
+    const uint32_t r0 = A.index[c], r1 = A.index[c + 1];
+    const uint32_t *src = (const uint32_t *)(A.payload + (uint64_t)r0 * kRecordUnit);
+    uint32_t *buf = s_words[warp];
+    const uint32_t n = (r1 - r0) * (kRecordUnit / 4);       // words of the record; what is read behind them is zero and adds nothing
+    uint64_t h = kFnvStart;
+    uint32_t done = 0;
+    while (done < n) {
+        const uint32_t m = n - done > 3 * 128 ? 7u : 3u;
+        __syncwarp();
+#pragma unroll
+        for (int i = 0; i < 7 * 4; ++i)
+            if (i < (int)m * 4) buf[i * 32 + lane] = done + i * 32 < n ? __ldcg(src + done + i * 32 + lane) : 0u;
+        __syncwarp();
+        h = m == 7u ? fnv_step<7>(h, buf, g_fnv7, lane) : fnv_step<3>(h, buf, g_fnv3, lane);
+        done += m * 128;
+    }
+    // the zero bytes behind the record multiplied h by P each: (done - n) words, a multiple of 32
+    constexpr uint64_t kUnitBack = fnv_pow(kFnvInverse, kRecordUnit);
+    for (uint32_t p = n; p < done; p += kRecordUnit / 4) h *= kUnitBack;
+    if (lane == 0) atomicAdd(&A.totals->checksum, (unsigned long long)h * (2 * c + 1));
 }
 
 }  // namespace huffllm
@@ -340,7 +498,7 @@ extern "C" huffllm_status huffllm_encode_device(const huffllm_codebook *cb, cons
 
     if ((e = cudaMemsetAsync((uint8_t *)blob + d.off_payload + d.payload_bytes, 0, kTailSlack, s)) != cudaSuccess) return cuda_fail("clearing the tail");
     encode_write_kernel<<<grid, kEncThreads, 0, s>>>(A);
-    encode_checksum_kernel<<<(uint32_t)((d.n_chunks + 127) / 128), 128, 0, s>>>(A);
+    encode_checksum_kernel<<<(uint32_t)((d.n_chunks + kSumWarps - 1) / kSumWarps), 32 * kSumWarps, 0, s>>>(A);
     if ((e = cudaGetLastError()) != cudaSuccess) return cuda_fail("encode write pass");
     if ((e = cudaMemcpyAsync(&tot, scr, sizeof(tot), cudaMemcpyDeviceToHost, s)) != cudaSuccess || (e = cudaStreamSynchronize(s)) != cudaSuccess)
         return cuda_fail("encode write pass");
