@@ -6,8 +6,9 @@
 // so neighbouring threads write neighbouring raw bytes and the two halves of a lane sit in one warp.
 //   pass 1  code lengths only -> words per sequence of every chunk, coded bits
 //   scan    record offsets (the index section), payload size, largest record
-//   pass 2  raw part and coded part of every record
-//   pass 3  the checksum term of every record, a warp each
+//   pass 2  raw part and coded part of every record (nothing if the scan found the tensor or the buffer unfit)
+//   pass 3  the checksum term of every record, a warp each; the last warp completes the header
+// The host waits once, behind the last pass.
 #include <cuda_runtime.h>
 
 #include <algorithm>
@@ -21,26 +22,39 @@ namespace huffllm {
 struct EncTotals {
     unsigned long long payload_units, coded_bits, checksum;
     uint32_t max_words, bad;     // bad: 1 = a symbol without codeword, 2 = payload beyond the 32-bit record index
+    uint32_t summed;             // CTAs whose records' checksums are in
 };
+
+constexpr uint32_t kNoCode = 1u << 20;       // length of a symbol without codeword: makes any sum it is part of stand out
 
 struct EncArgs {
     const uint16_t *w;
     uint64_t rows, cols, n_chunks;
     uint32_t Kc, KC, fp16, lag_bits, pad, vec_ok;
+    uint64_t max_units;          // what the blob has room for
     uint32_t *words, *chunk_bits, *index;
-    uint8_t *payload;
+    uint8_t *blob, *payload;
     EncTotals *totals;
-    uint8_t len[256];
-    uint32_t bits[256];
+    uint32_t code[256];          // stream bits of a symbol's codeword | its length << 16
+    huffllm_desc desc;           // the header, but for what the totals say
 };
 
-constexpr uint32_t kEncThreads = 256, kEncChunks = kEncThreads / 64;
+__device__ __forceinline__ bool enc_fits(const EncArgs &A) {
+    return __ldcg(&A.totals->bad) == 0u && __ldcg(&A.totals->payload_units) <= A.max_units;
+}
 
 // byte of a group's 32-bit word that takes weight j's mantissa bits, and the one that takes its sign (the raw-byte layout)
 __host__ __device__ constexpr uint32_t raw_mant_byte(uint32_t j) { return ((j & 1u) << 1) | (j >> 1); }
 __host__ __device__ constexpr uint32_t raw_sign_byte(uint32_t j) { return (raw_mant_byte(j) + 1u) & 3u; }
 static_assert(raw_mant_byte(0) == kRawMantByte[0] && raw_mant_byte(1) == kRawMantByte[1] && raw_mant_byte(2) == kRawMantByte[2] &&
               raw_mant_byte(3) == kRawMantByte[3], "raw-byte layout");
+// the same as byte selectors over two words of two weights each: weight j's low byte is byte 2 j, its high byte byte 2 j + 1
+__host__ __device__ constexpr uint32_t raw_sel(bool sign) {
+    uint32_t sel = 0;
+    for (uint32_t j = 0; j < 4; ++j) sel |= (2 * j + (sign ? 1 : 0)) << (4 * (sign ? raw_sign_byte(j) : raw_mant_byte(j)));
+    return sel;
+}
+constexpr uint32_t kRawMantSel = raw_sel(false), kRawSignSel = raw_sel(true);
 static_assert(raw_sign_byte(0) == kRawSignByte[0] && raw_sign_byte(1) == kRawSignByte[1] && raw_sign_byte(2) == kRawSignByte[2] &&
               raw_sign_byte(3) == kRawSignByte[3], "raw-byte layout");
 
@@ -52,25 +66,41 @@ __device__ __forceinline__ uint32_t enc_raw_bytes(const EncArgs &A, uint32_t nkb
     return A.fp16 ? (nkb * 64u + 127u) & ~127u : nkb * 512u;
 }
 
-// The eight weights of (row r, columns c .. c + 7), pad words outside the tensor.
-__device__ __forceinline__ void enc_load8(const EncArgs &A, uint64_t r, uint64_t c, uint32_t (&v)[8]) {
-    if (r < A.rows && c + 8 <= A.cols && A.vec_ok) {
-        const uint4 q = __ldg((const uint4 *)(A.w + r * A.cols + c));
-        const uint32_t x[4] = {q.x, q.y, q.z, q.w};
-#pragma unroll
-        for (int i = 0; i < 8; ++i) v[i] = (x[i >> 1] >> (16 * (i & 1))) & 0xFFFFu;
-    } else {
-#pragma unroll
-        for (int i = 0; i < 8; ++i) v[i] = (r < A.rows && c + i < A.cols) ? A.w[r * A.cols + c + i] : A.pad;
+// A thread's weights: eight in every block of 32 columns, from `p` on, `left` columns (at most) before the row ends.
+struct EncRow {
+    const uint16_t *p;
+    int32_t left;               // 0 for rows outside the tensor
+};
+// The eight weights of block kb as four words, pad words outside the tensor.  Rows that do not start on 16-byte boundaries
+// are read in the aligned words that the eight weights lie in (every word holds one of them at least).
+__device__ __forceinline__ uint4 enc_load8(const EncArgs &A, const EncRow &R, uint32_t kb) {
+    const uint16_t *p = R.p + kb * 32u;
+    const int32_t left = R.left - (int32_t)(kb * 32u);
+    if (left >= 8) {
+        if (A.vec_ok) return __ldg((const uint4 *)p);
+        const uint32_t odd = (uint32_t)((uintptr_t)p >> 1) & 1u, sel = odd ? 0x5432u : 0x3210u;
+        const uint32_t *q = (const uint32_t *)(p - odd);
+        const uint32_t u0 = __ldg(q), u1 = __ldg(q + 1), u2 = __ldg(q + 2), u3 = __ldg(q + 3), u4 = odd ? __ldg(q + 4) : 0u;
+        return make_uint4(__byte_perm(u0, u1, sel), __byte_perm(u1, u2, sel), __byte_perm(u2, u3, sel), __byte_perm(u3, u4, sel));
     }
+    uint32_t x[4];
+#pragma unroll
+    for (int i = 0; i < 4; ++i) {
+        const uint32_t lo = 2 * i < left ? p[2 * i] : A.pad, hi = 2 * i + 1 < left ? p[2 * i + 1] : A.pad;
+        x[i] = lo | hi << 16;
+    }
+    return make_uint4(x[0], x[1], x[2], x[3]);
 }
 
 struct EncThread {
     uint32_t sub, q, lane, half, seq;
-    uint64_t c, r, col0;
-    uint32_t kc, nkb;
+    uint64_t c;
+    uint32_t nkb;
+    EncRow row;
     bool active;
 };
+// CHUNKS chunks per CTA, 64 threads each
+template <uint32_t CHUNKS>
 __device__ __forceinline__ EncThread enc_thread(const EncArgs &A) {
     EncThread T;
     T.sub = threadIdx.x >> 6;
@@ -78,171 +108,182 @@ __device__ __forceinline__ EncThread enc_thread(const EncArgs &A) {
     T.lane = T.q >> 1;
     T.half = T.q & 1;
     T.seq = T.lane + 32 * T.half;
-    T.c = (uint64_t)blockIdx.x * kEncChunks + T.sub;
+    T.c = (uint64_t)blockIdx.x * CHUNKS + T.sub;
     T.active = T.c < A.n_chunks;
     const uint64_t cc = T.active ? T.c : 0;
-    const uint32_t rg = (uint32_t)(cc / A.KC);
-    T.kc = (uint32_t)(cc % A.KC);
-    T.nkb = enc_blocks_of(A, T.kc);
-    T.r = (uint64_t)rg * 16 + (T.lane >> 2) + 8 * T.half;
-    T.col0 = (uint64_t)T.kc * A.Kc + (T.lane & 3) * 8;
+    const uint32_t rg = (uint32_t)cc / A.KC, kc = (uint32_t)cc - rg * A.KC;       // (fewer than 2^31 chunks)
+    T.nkb = enc_blocks_of(A, kc);
+    const uint64_t r = (uint64_t)rg * 16 + (T.lane >> 2) + 8 * T.half, col0 = (uint64_t)kc * A.Kc + (T.lane & 3) * 8;
+    T.row.p = A.w + r * A.cols + col0;
+    T.row.left = r < A.rows && col0 < A.cols ? (int32_t)min(A.cols - col0, (uint64_t)A.Kc) : 0;
     return T;
 }
 
-__global__ void __launch_bounds__(kEncThreads) encode_size_kernel(const __grid_constant__ EncArgs A) {
-    __shared__ uint32_t s_max[kEncChunks], s_sum[kEncChunks], s_bad;
-    __shared__ uint8_t s_len[256];
-    s_len[threadIdx.x] = A.len[threadIdx.x];
-    if (threadIdx.x < kEncChunks) s_max[threadIdx.x] = s_sum[threadIdx.x] = 0;
-    if (threadIdx.x == 0) s_bad = 0;
+// Pass 1.  Bound by the read of the tensor: four blocks' loads are in flight per thread (one at a time took 30 us on an
+// 11008 x 4096 tensor), and a weight costs a shift, a mask, a table read and an addition.
+constexpr uint32_t kSizeThreads = 256, kSizeChunks = kSizeThreads / 64;
+template <bool FP16>
+__global__ void __launch_bounds__(kSizeThreads) encode_size_kernel(const __grid_constant__ EncArgs A) {
+    __shared__ uint32_t s_max[kSizeChunks], s_sum[kSizeChunks], s_len[256];
+    s_len[threadIdx.x] = A.code[threadIdx.x] >> 16 ? A.code[threadIdx.x] >> 16 : kNoCode;
+    if (threadIdx.x < kSizeChunks) s_max[threadIdx.x] = s_sum[threadIdx.x] = 0;
     __syncthreads();
-    const EncThread T = enc_thread(A);
+    const EncThread T = enc_thread<kSizeChunks>(A);
     if (T.active) {
-        uint32_t bits = 0, bad = 0;
-        for (uint32_t kb = 0; kb < T.nkb; ++kb) {
-            uint32_t v[8];
-            enc_load8(A, T.r, T.col0 + kb * 32, v);
+        uint32_t bits = 0;
+        const char *len = (const char *)s_len;
+        auto at = [&](uint32_t byte_off) -> uint32_t { return *(const uint32_t *)(len + byte_off); };
+        auto add = [&](const uint4 &v) {
+            const uint32_t x[4] = {v.x, v.y, v.z, v.w};
 #pragma unroll
-            for (int i = 0; i < 8; ++i) {
-                if (A.fp16) {
-                    const uint32_t l0 = s_len[(v[i] >> 10) & 31], l1 = s_len[32 + ((v[i] >> 5) & 31)], l2 = s_len[64 + (v[i] & 31)];
-                    bad |= (!l0 || !l1 || !l2) ? 1u : 0u;
-                    bits += l0 + l1 + l2;
+            for (int i = 0; i < 4; ++i) {
+                if (FP16) {
+                    bits += at((x[i] >> 8) & 0x7Cu) + at(128u + ((x[i] >> 3) & 0x7Cu)) + at(256u + ((x[i] << 2) & 0x7Cu));
+                    bits += at((x[i] >> 24) & 0x7Cu) + at(128u + ((x[i] >> 19) & 0x7Cu)) + at(256u + ((x[i] >> 14) & 0x7Cu));
                 } else {
-                    const uint32_t l = s_len[(v[i] >> 7) & 0xFF];
-                    bad |= l ? 0u : 1u;
-                    bits += l;
+                    bits += at((x[i] >> 5) & 0x3FCu) + at((x[i] >> 21) & 0x3FCu);
                 }
             }
+        };
+        uint32_t kb = 0;
+        for (; kb + 4 <= T.nkb; kb += 4) {
+            uint4 v[4];
+#pragma unroll
+            for (int i = 0; i < 4; ++i) v[i] = enc_load8(A, T.row, kb + i);
+#pragma unroll
+            for (int i = 0; i < 4; ++i) add(v[i]);
+        }
+        for (; kb < T.nkb; ++kb) add(enc_load8(A, T.row, kb));
+        if (bits >= kNoCode) {
+            atomicOr(&A.totals->bad, 1u);
+            bits = 0;
         }
         atomicMax(&s_max[T.sub], bits + A.lag_bits);
         atomicAdd(&s_sum[T.sub], bits);
-        if (bad) s_bad = 1;
     }
     __syncthreads();
     if (T.active && T.q == 0) {
         A.words[T.c] = max(1u, (s_max[T.sub] + 31) / 32);
         A.chunk_bits[T.c] = s_sum[T.sub];
     }
-    if (threadIdx.x == 0 && s_bad) atomicOr(&A.totals->bad, 1u);
 }
 
-// Record offsets: an exclusive prefix sum of the record sizes (in 128-byte units), by a single CTA.
-__global__ void __launch_bounds__(1024) encode_scan_kernel(const __grid_constant__ EncArgs A) {
-    __shared__ unsigned long long s_warp[32], s_carry, s_bits[32];
-    __shared__ uint32_t s_maxw[32];
+// Record offsets: an exclusive prefix sum of the record sizes (in 128-byte units).  A CTA takes 1024 chunks and sums the words
+// of every chunk in front of them itself (the raw parts in front are known without a sum), so that no CTA waits for another;
+// a single CTA walking all chunks took 20 us for the 11008 chunks of an 11008 x 4096 tensor, most of it barriers.
+constexpr uint32_t kScanThreads = 1024;
+__global__ void __launch_bounds__(kScanThreads) encode_scan_kernel(const __grid_constant__ EncArgs A) {
+    __shared__ unsigned long long s_warp[32], s_front[32];
     const uint32_t tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-    if (tid == 0) s_carry = 0;
-    unsigned long long bits = 0;
-    uint32_t maxw = 0, over = 0;
-    __syncthreads();
-    for (uint64_t base = 0; base < A.n_chunks; base += 1024) {
-        const uint64_t c = base + tid;
-        unsigned long long units = 0;
-        if (c < A.n_chunks) {
-            const uint32_t W = A.words[c];
-            units = (enc_raw_bytes(A, enc_blocks_of(A, (uint32_t)(c % A.KC))) + (unsigned long long)W * 256ull) / kRecordUnit;
-            bits += A.chunk_bits[c];
-            maxw = max(maxw, W);
-        }
-        unsigned long long incl = units;
+    const uint64_t first = (uint64_t)blockIdx.x * kScanThreads, c = first + tid;
+    const uint32_t raw_full = enc_raw_bytes(A, enc_blocks_of(A, 0)) / kRecordUnit, raw_last = enc_raw_bytes(A, enc_blocks_of(A, A.KC - 1)) / kRecordUnit;
+    unsigned long long front = 0;                           // words of the chunks in front of the CTA's
+#pragma unroll 8
+    for (uint64_t i = tid; i < first; i += kScanThreads) front += __ldcg(A.words + i);
+    const uint32_t W = c < A.n_chunks ? __ldcg(A.words + c) : 0u;
+    unsigned long long bits = c < A.n_chunks ? __ldcg(A.chunk_bits + c) : 0u, incl = W;
+    uint32_t maxw = W;
 #pragma unroll
-        for (int o = 1; o < 32; o <<= 1) {
-            unsigned long long n = __shfl_up_sync(0xFFFFFFFFu, incl, o);
-            if (lane >= (uint32_t)o) incl += n;
-        }
-        if (lane == 31) s_warp[warp] = incl;
-        __syncthreads();
-        unsigned long long before = s_carry;
-        for (uint32_t w2 = 0; w2 < warp; ++w2) before += s_warp[w2];
-        const unsigned long long excl = before + incl - units;
-        if (c < A.n_chunks) {
-            A.index[c] = (uint32_t)excl;
-            if (excl + units > 0xFFFFFFFFull) over = 1;
-        }
-        __syncthreads();
-        if (tid == 1023) s_carry = before + incl;
-        __syncthreads();
+    for (int o = 1; o < 32; o <<= 1) {
+        const unsigned long long n = __shfl_up_sync(0xFFFFFFFFu, incl, o);
+        if (lane >= (uint32_t)o) incl += n;
     }
-    // totals
 #pragma unroll
     for (int o = 16; o; o >>= 1) {
+        front += __shfl_xor_sync(0xFFFFFFFFu, front, o);
         bits += __shfl_xor_sync(0xFFFFFFFFu, bits, o);
         maxw = max(maxw, __shfl_xor_sync(0xFFFFFFFFu, maxw, o));
-        over |= __shfl_xor_sync(0xFFFFFFFFu, over, o);
     }
+    if (lane == 31) s_warp[warp] = incl;
     if (lane == 0) {
-        s_bits[warp] = bits;
-        s_maxw[warp] = maxw;
-        if (over) atomicOr(&A.totals->bad, 2u);
+        s_front[warp] = front;
+        if (bits) atomicAdd(&A.totals->coded_bits, bits);
+        if (maxw) atomicMax(&A.totals->max_words, maxw);
     }
     __syncthreads();
-    if (tid == 0) {
-        unsigned long long b = 0;
-        uint32_t m = 0;
-        for (int i = 0; i < 32; ++i) {
-            b += s_bits[i];
-            m = max(m, s_maxw[i]);
-        }
-        A.index[A.n_chunks] = (uint32_t)s_carry;
-        A.totals->payload_units = s_carry;
-        A.totals->coded_bits = b;
-        A.totals->max_words = m;
+    unsigned long long before = incl - W;
+    for (uint32_t i = 0; i < 32; ++i) before += s_front[i] + (i < warp ? s_warp[i] : 0ull);
+    if (c <= A.n_chunks) {                                  // (one entry more than chunks: the payload's end)
+        const uint64_t row = c / A.KC, kc = c - row * A.KC; // raw parts in front: whole rows of chunks, then full chunks of this one
+        const unsigned long long at = row * ((uint64_t)(A.KC - 1) * raw_full + raw_last) + kc * raw_full + 2ull * before;
+        A.index[c] = (uint32_t)at;
+        if (at > 0xFFFFFFFFull) atomicOr(&A.totals->bad, 2u);
+        if (c == A.n_chunks) A.totals->payload_units = at;
+    } else if (c < ((A.n_chunks + 64) & ~63ull)) {
+        A.index[c] = 0;                                     // the section's padding to 256 bytes
     }
 }
 
-__global__ void __launch_bounds__(kEncThreads) encode_write_kernel(const __grid_constant__ EncArgs A) {
-    __shared__ uint8_t s_len[256];
-    __shared__ uint32_t s_bits[256];
-    s_len[threadIdx.x] = A.len[threadIdx.x];
-    s_bits[threadIdx.x] = A.bits[threadIdx.x];
+// Pass 2.  A CTA of 64 threads takes a chunk and collects the coded part in shared memory, row by row as the record has it:
+// stored straight from the threads, whose streams run apart, the words went to L2 one by one as partial sectors.
+constexpr uint32_t kWriteThreads = 64;
+// coded part of the largest chunk (1024 columns) under the longest codes: FP16, three fields of 12 bits
+constexpr uint32_t kMostCodedBytes = (7 + 32 * 8 * 3 * 12 + 31) / 32 * 256;
+template <bool FP16>
+__global__ void __launch_bounds__(kWriteThreads) encode_write_kernel(const __grid_constant__ EncArgs A) {
+    extern __shared__ __align__(16) uint32_t s_coded[];
+    __shared__ uint32_t s_code[256];
+#pragma unroll
+    for (uint32_t i = 0; i < 256 / kWriteThreads; ++i) s_code[i * kWriteThreads + threadIdx.x] = A.code[i * kWriteThreads + threadIdx.x];
+    if (!enc_fits(A)) return;
     __syncthreads();
-    const EncThread T = enc_thread(A);
-    if (!T.active) return;          // whole 64-thread groups leave together: the shuffles below stay inside a group's warps
+    const EncThread T = enc_thread<1>(A);
     const uint32_t W = A.words[T.c], raw_bytes = enc_raw_bytes(A, T.nkb);
     uint8_t *raw = A.payload + (uint64_t)A.index[T.c] * kRecordUnit;
-    uint32_t *coded = (uint32_t *)(raw + raw_bytes) + T.seq;      // word j of this sequence at coded[64 j]
-    unsigned long long acc = 0;
-    uint32_t nacc = A.lag_bits, j = 0;
-    auto append = [&](uint32_t b, uint32_t len) {                 // len <= 16, nacc < 32
-        acc |= (unsigned long long)b << nacc;
+    uint32_t *out = s_coded + T.seq;                              // word j of this sequence at out[64 j]
+    uint32_t acc = 0, nacc = A.lag_bits;
+    auto append = [&](uint32_t b, uint32_t len) {                 // len <= 24, nacc < 32
+        acc |= b << nacc;
+        const uint32_t over = __funnelshift_rc(b, 0u, 32u - nacc);         // (nacc = 0: a shift by 32, nothing left over)
         nacc += len;
-        if (nacc >= 32) {
-            coded[(size_t)64 * j++] = (uint32_t)acc;
-            acc >>= 32;
-            nacc -= 32;
+        if (nacc >= 32u) {
+            *out = acc;
+            out += 64;
+            acc = over;
+            nacc -= 32u;
         }
     };
+    auto code = [&](uint32_t byte_off) -> uint32_t { return *(const uint32_t *)((const char *)s_code + byte_off); };
+    auto append2 = [&](uint32_t e0, uint32_t e1) { append((e0 & 0xFFFFu) | (e1 & 0xFFFFu) << (e0 >> 16), (e0 >> 16) + (e1 >> 16)); };
+    uint4 next = enc_load8(A, T.row, 0);
     for (uint32_t kb = 0; kb < T.nkb; ++kb) {
-        uint32_t v[8];
-        enc_load8(A, T.r, T.col0 + kb * 32, v);
-        if (A.fp16) {
+        const uint32_t x[4] = {next.x, next.y, next.z, next.w};
+        if (kb + 1 < T.nkb) next = enc_load8(A, T.row, kb + 1);
+        if (FP16) {
             // sign bit of weight i: pair p = i / 2 (+ 4 for the row g + 8 sequence), bit p (+ 8 if i is odd)
             uint32_t sg = 0;
 #pragma unroll
-            for (int i = 0; i < 8; ++i) {
-                sg |= (v[i] >> 15) << ((i >> 1) + 4 * T.half + 8 * (i & 1));
-                append(s_bits[(v[i] >> 10) & 31], s_len[(v[i] >> 10) & 31]);
-                append(s_bits[32 + ((v[i] >> 5) & 31)], s_len[32 + ((v[i] >> 5) & 31)]);
-                append(s_bits[64 + (v[i] & 31)], s_len[64 + (v[i] & 31)]);
+            for (int i = 0; i < 4; ++i) {
+                sg |= (x[i] >> 15 & 1u) << (i + 4 * T.half) | (x[i] >> 31) << (i + 4 * T.half + 8);
+                append2(code((x[i] >> 8) & 0x7Cu), code(128u + ((x[i] >> 3) & 0x7Cu)));
+                append2(code(256u + ((x[i] << 2) & 0x7Cu)), code((x[i] >> 24) & 0x7Cu));
+                append2(code(128u + ((x[i] >> 19) & 0x7Cu)), code(256u + ((x[i] >> 14) & 0x7Cu)));
             }
             sg |= __shfl_xor_sync(0xFFFFFFFFu, sg, 1);
             if (T.half == 0) *(uint16_t *)(raw + kb * 64 + T.lane * 2) = (uint16_t)sg;
         } else {
-            uint32_t word[2] = {0, 0};
+            uint32_t word[2];
 #pragma unroll
-            for (int i = 0; i < 8; ++i) {
-                word[i >> 2] |= (v[i] & 0x7Fu) << (8 * raw_mant_byte(i & 3));
-                word[i >> 2] |= ((v[i] >> 8) & 0x80u) << (8 * raw_sign_byte(i & 3));
-                const uint32_t e = (v[i] >> 7) & 0xFF;
-                append(s_bits[e], s_len[e]);
-            }
+            for (int i = 0; i < 2; ++i)                           // bytes in the raw layout's order: low bytes' mantissas, high bytes' signs
+                word[i] = (__byte_perm(x[2 * i], x[2 * i + 1], kRawMantSel) & 0x7F7F7F7Fu) | (__byte_perm(x[2 * i], x[2 * i + 1], kRawSignSel) & 0x80808080u);
+#pragma unroll
+            for (int i = 0; i < 4; ++i) append2(code((x[i] >> 5) & 0x3FCu), code((x[i] >> 21) & 0x3FCu));
             *(uint2 *)(raw + kb * 512 + T.lane * 16 + T.half * 8) = make_uint2(word[0], word[1]);
         }
     }
-    if (nacc) coded[(size_t)64 * j++] = (uint32_t)acc;
-    for (; j < W; ++j) coded[(size_t)64 * j] = 0;
-    if (A.fp16 && (T.nkb & 1u) && T.q < 32) *(uint16_t *)(raw + T.nkb * 64 + T.q * 2) = 0;   // padding of the sign plane
+    uint32_t *const end = s_coded + T.seq + (size_t)64 * W;
+    if (nacc) {
+        *out = acc;
+        out += 64;
+    }
+    for (; out < end; out += 64) *out = 0;
+    if (FP16 && (T.nkb & 1u) && T.q < 32) *(uint16_t *)(raw + T.nkb * 64 + T.q * 2) = 0;   // padding of the sign plane
+    __syncthreads();
+    for (uint32_t i = T.q; i < W * 16; i += kWriteThreads) ((uint4 *)(raw + raw_bytes))[i] = ((const uint4 *)s_coded)[i];
+    if (T.c + 1 == A.n_chunks) {                                  // the zero bytes behind the payload
+        uint4 *tail = (uint4 *)(A.payload + __ldcg(&A.totals->payload_units) * kRecordUnit);
+        for (uint32_t i = T.q; i < kTailSlack / 16; i += kWriteThreads) tail[i] = make_uint4(0, 0, 0, 0);
+    }
 }
 
 // ------------------------------------------------------------------------------ checksum of the records
@@ -312,7 +353,7 @@ __device__ __forceinline__ void mma_u8(int32_t (&d)[4], uint32_t a0, uint32_t a1
 
 // 512 M bytes of a record (`words`, in shared memory): hash `h` moved on over them.  All lanes hold the same h.
 template <int M>
-__device__ __forceinline__ uint64_t fnv_step(uint64_t h, const uint32_t *words, const FnvWeights<M> &wt, uint32_t lane) {
+__device__ __forceinline__ uint64_t fnv_step(uint64_t h, const uint32_t *words, const FnvWeights<M> &wt, uint32_t lane, uint32_t three) {
     constexpr int N = 4 * M;                       // bytes of a stretch
     constexpr uint32_t kEven = 0x00FF00FFu, kOdd = 0xFF00FF00u;
     uint32_t G[N];                                 // G[j]: byte j of the lane's four stretches
@@ -346,15 +387,15 @@ __device__ __forceinline__ uint64_t fnv_step(uint64_t h, const uint32_t *words, 
     for (uint32_t k = 1; k <= 3; ++k) {
         uint32_t z = X;
 #pragma unroll
-        for (int j = 0; j < N; ++j) z = xor_and(z, G[j], 0x0F0F0F0Fu) * 3u;
+        for (int j = 0; j < N; ++j) z = xor_and(z, G[j], 0x0F0F0F0Fu) * three;
         settle(z, k);
     }
     {   // bit 4 of the product with P mod 32 = 19: bit 4 of 3 times the low four bits, bit 4 and bit 0 of x ^ b
         uint32_t z = X, acc = all, low = 0;
 #pragma unroll
         for (int j = 0; j < N; j += 2) {
-            const uint32_t y0 = xor_and(z, G[j], 0x0F0F0F0Fu), z0 = y0 * 3u, y1 = xor_and(z0, G[j + 1], 0x0F0F0F0Fu);
-            z = y1 * 3u;
+            const uint32_t y0 = xor_and(z, G[j], 0x0F0F0F0Fu), z0 = y0 * three, y1 = xor_and(z0, G[j + 1], 0x0F0F0F0Fu);
+            z = y1 * three;
             acc ^= z0 ^ z;
             low ^= y0 ^ y1;
         }
@@ -396,19 +437,32 @@ __device__ __forceinline__ uint64_t fnv_step(uint64_t h, const uint32_t *words, 
     return h * kOver + sum;
 }
 
-constexpr uint32_t kSumWarps = 4;
+// What the totals add to the header.
+__host__ __device__ inline void enc_fill_totals(huffllm_desc &d, const volatile EncTotals &t) {
+    d.max_words = t.max_words;
+    d.payload_bytes = t.payload_units * kRecordUnit;
+    d.blob_bytes = d.off_payload + d.payload_bytes + kTailSlack;
+    d.coded_bits = t.coded_bits;
+    d.payload_checksum = t.checksum;
+}
+
+constexpr uint32_t kSumWarps = 8;
 
 __global__ void __launch_bounds__(32 * kSumWarps) encode_checksum_kernel(const __grid_constant__ EncArgs A) {
     __shared__ uint32_t s_words[kSumWarps][7 * 128];
+    __shared__ unsigned long long s_term[kSumWarps];
     const uint32_t lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     const uint64_t c = (uint64_t)blockIdx.x * kSumWarps + warp;
-    if (c >= A.n_chunks) return;
-    const uint32_t r0 = A.index[c], r1 = A.index[c + 1];
+    if (!enc_fits(A)) return;
+    const uint32_t r0 = c < A.n_chunks ? A.index[c] : 0u, r1 = c < A.n_chunks ? A.index[c + 1] : 0u;
     const uint32_t *src = (const uint32_t *)(A.payload + (uint64_t)r0 * kRecordUnit);
     uint32_t *buf = s_words[warp];
     const uint32_t n = (r1 - r0) * (kRecordUnit / 4);       // words of the record; what is read behind them is zero and adds nothing
     uint64_t h = kFnvStart;
     uint32_t done = 0;
+    // 3, as a value the compiler does not know: times 3 as a shifted addition would join the logic instructions on the
+    // integer pipe that bounds this kernel, as a multiplication it runs beside them
+    const uint32_t three = 3u + (uint32_t)(A.n_chunks >> 32);
     while (done < n) {
         const uint32_t m = n - done > 3 * 128 ? 7u : 3u;
         __syncwarp();
@@ -416,13 +470,25 @@ __global__ void __launch_bounds__(32 * kSumWarps) encode_checksum_kernel(const _
         for (int i = 0; i < 7 * 4; ++i)
             if (i < (int)m * 4) buf[i * 32 + lane] = done + i * 32 < n ? __ldcg(src + done + i * 32 + lane) : 0u;
         __syncwarp();
-        h = m == 7u ? fnv_step<7>(h, buf, g_fnv7, lane) : fnv_step<3>(h, buf, g_fnv3, lane);
+        h = m == 7u ? fnv_step<7>(h, buf, g_fnv7, lane, three) : fnv_step<3>(h, buf, g_fnv3, lane, three);
         done += m * 128;
     }
     // the zero bytes behind the record multiplied h by P each: (done - n) words, a multiple of 32
     constexpr uint64_t kUnitBack = fnv_pow(kFnvInverse, kRecordUnit);
     for (uint32_t p = n; p < done; p += kRecordUnit / 4) h *= kUnitBack;
-    if (lane == 0) atomicAdd(&A.totals->checksum, (unsigned long long)h * (2 * c + 1));
+    if (lane == 0) s_term[warp] = n ? h * (2 * c + 1) : 0ull;
+    __syncthreads();
+    if (threadIdx.x) return;
+    unsigned long long term = 0;
+    for (uint32_t i = 0; i < kSumWarps; ++i) term += s_term[i];
+    atomicAdd(&A.totals->checksum, term);
+    __threadfence();
+    if (atomicAdd(&A.totals->summed, 1u) != gridDim.x - 1u) return;
+    // every record is in: the header
+    __threadfence();
+    huffllm_desc d = A.desc;
+    enc_fill_totals(d, *(const volatile EncTotals *)A.totals);
+    *(huffllm_desc *)A.blob = d;
 }
 
 }  // namespace huffllm
@@ -454,7 +520,7 @@ extern "C" huffllm_status huffllm_encode_device(const huffllm_codebook *cb, cons
     huffllm_desc d;
     fill_desc_fixed(cb, rows, cols, chunk_elems, Kc, RG, KC, &d);
     if (blob_cap < d.off_payload) return fail(HUFFLLM_ERR_BUFFER_TOO_SMALL, "blob capacity below the fixed sections");
-    if (d.n_chunks > 0x7FFFFFFFull * kEncChunks) return fail(HUFFLLM_ERR_UNSUPPORTED, "too many chunks");
+    if (d.n_chunks > 0x7FFFFFFFull) return fail(HUFFLLM_ERR_UNSUPPORTED, "too many chunks");
 
     cudaStream_t s = (cudaStream_t)stream;
     uint8_t *blob = (uint8_t *)blob_dev, *scr = (uint8_t *)scratch_dev;
@@ -469,46 +535,50 @@ extern "C" huffllm_status huffllm_encode_device(const huffllm_codebook *cb, cons
     A.lag_bits = d.lag_bits;
     A.pad = d.pad_word;
     A.vec_ok = (cols % 8 == 0 && ((uintptr_t)w_dev & 15u) == 0) ? 1u : 0u;
+    A.max_units = blob_cap >= d.off_payload + kTailSlack ? (blob_cap - d.off_payload - kTailSlack) / kRecordUnit : 0;
     A.totals = (EncTotals *)scr;
     A.words = (uint32_t *)(scr + 256);
     A.chunk_bits = A.words + d.n_chunks;
     A.index = (uint32_t *)(blob + d.off_index);
+    A.blob = blob;
     A.payload = blob + d.off_payload;
-    encoder_tables(cb, A.len, A.bits);
+    A.desc = d;
+    uint8_t len[256];
+    uint32_t bits[256], longest = 1;
+    encoder_tables(cb, len, bits);
+    for (int i = 0; i < 256; ++i) {
+        A.code[i] = bits[i] | (uint32_t)len[i] << 16;
+        longest = std::max<uint32_t>(longest, len[i]);
+    }
+    // rows of the largest record this code can give a full chunk (the sizes are known on the device only)
+    const uint32_t most_words = (d.lag_bits + Kc / kBlockCols * 8 * longest * (A.fp16 ? 3 : 1) + 31) / 32;
+    const size_t smem = (size_t)most_words * 256;
 
     cudaError_t e;
     auto cuda_fail = [&](const char *what) { return fail(HUFFLLM_ERR_CUDA, "%s: %s", what, cudaGetErrorString(e)); };
-    if ((e = cudaMemsetAsync(scr, 0, 256, s)) != cudaSuccess) return cuda_fail("cudaMemsetAsync");
-    if ((e = cudaMemsetAsync(blob, 0, d.off_payload, s)) != cudaSuccess) return cuda_fail("cudaMemsetAsync");
-    const uint32_t grid = (uint32_t)((d.n_chunks + kEncChunks - 1) / kEncChunks);
-    encode_size_kernel<<<grid, kEncThreads, 0, s>>>(A);
-    encode_scan_kernel<<<1, 1024, 0, s>>>(A);
-    if ((e = cudaGetLastError()) != cudaSuccess) return cuda_fail("encode size pass");
-    EncTotals tot;
-    if ((e = cudaMemcpyAsync(&tot, scr, sizeof(tot), cudaMemcpyDeviceToHost, s)) != cudaSuccess || (e = cudaStreamSynchronize(s)) != cudaSuccess)
-        return cuda_fail("encode size pass");
-    if (tot.bad & 1u) return fail(HUFFLLM_ERR_INVALID_ARG, "a weight uses a symbol the codebook has no codeword for");
-    if (tot.bad & 2u) return fail(HUFFLLM_ERR_UNSUPPORTED, "payload exceeds the 32-bit record index");
-    d.max_words = tot.max_words;
-    d.payload_bytes = tot.payload_units * kRecordUnit;
-    d.blob_bytes = d.off_payload + d.payload_bytes + kTailSlack;
-    d.coded_bits = tot.coded_bits;
-    if (blob_cap < d.blob_bytes)
-        return fail(HUFFLLM_ERR_BUFFER_TOO_SMALL, "blob needs %llu bytes, capacity is %llu", (unsigned long long)d.blob_bytes, (unsigned long long)blob_cap);
-
-    if ((e = cudaMemsetAsync((uint8_t *)blob + d.off_payload + d.payload_bytes, 0, kTailSlack, s)) != cudaSuccess) return cuda_fail("clearing the tail");
-    encode_write_kernel<<<grid, kEncThreads, 0, s>>>(A);
-    encode_checksum_kernel<<<(uint32_t)((d.n_chunks + kSumWarps - 1) / kSumWarps), 32 * kSumWarps, 0, s>>>(A);
-    if ((e = cudaGetLastError()) != cudaSuccess) return cuda_fail("encode write pass");
-    if ((e = cudaMemcpyAsync(&tot, scr, sizeof(tot), cudaMemcpyDeviceToHost, s)) != cudaSuccess || (e = cudaStreamSynchronize(s)) != cudaSuccess)
-        return cuda_fail("encode write pass");
-    d.payload_checksum = tot.checksum;
-
-    // header, code lengths and table: bytes [0, off_index), assembled on the host
+    const auto size_kernel = A.fp16 ? encode_size_kernel<true> : encode_size_kernel<false>;
+    const auto write_kernel = A.fp16 ? encode_write_kernel<true> : encode_write_kernel<false>;
+    if ((e = cudaFuncSetAttribute(write_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kMostCodedBytes)) != cudaSuccess)
+        return cuda_fail("cudaFuncSetAttribute");
+    // code lengths and table, assembled on the host; the header's bytes stay zero until the last kernel writes them
     std::vector<uint8_t> fixed((size_t)d.off_index, 0);
     write_fixed_sections(cb, d, fixed.data());
-    if ((e = cudaMemcpyAsync(blob, fixed.data(), fixed.size(), cudaMemcpyHostToDevice, s)) != cudaSuccess || (e = cudaStreamSynchronize(s)) != cudaSuccess)
-        return cuda_fail("header copy");
+    memset(fixed.data(), 0, sizeof(d));
+    if ((e = cudaMemcpyAsync(blob, fixed.data(), fixed.size(), cudaMemcpyHostToDevice, s)) != cudaSuccess) return cuda_fail("copy of the fixed sections");
+    if ((e = cudaMemsetAsync(scr, 0, 256, s)) != cudaSuccess) return cuda_fail("cudaMemsetAsync");
+    size_kernel<<<(uint32_t)((d.n_chunks + kSizeChunks - 1) / kSizeChunks), kSizeThreads, 0, s>>>(A);
+    encode_scan_kernel<<<(uint32_t)((d.n_chunks + 64 + kScanThreads - 1) / kScanThreads), kScanThreads, 0, s>>>(A);
+    write_kernel<<<(uint32_t)d.n_chunks, kWriteThreads, smem, s>>>(A);
+    encode_checksum_kernel<<<(uint32_t)((d.n_chunks + kSumWarps - 1) / kSumWarps), 32 * kSumWarps, 0, s>>>(A);
+    if ((e = cudaGetLastError()) != cudaSuccess) return cuda_fail("encoder launches");
+    EncTotals tot;
+    if ((e = cudaMemcpyAsync(&tot, scr, sizeof(tot), cudaMemcpyDeviceToHost, s)) != cudaSuccess || (e = cudaStreamSynchronize(s)) != cudaSuccess)
+        return cuda_fail("encoder");
+    if (tot.bad & 1u) return fail(HUFFLLM_ERR_INVALID_ARG, "a weight uses a symbol the codebook has no codeword for");
+    if (tot.bad & 2u) return fail(HUFFLLM_ERR_UNSUPPORTED, "payload exceeds the 32-bit record index");
+    enc_fill_totals(d, tot);
+    if (tot.payload_units > A.max_units)
+        return fail(HUFFLLM_ERR_BUFFER_TOO_SMALL, "blob needs %llu bytes, capacity is %llu", (unsigned long long)d.blob_bytes, (unsigned long long)blob_cap);
     *desc = d;
     return HUFFLLM_OK;
 }

@@ -105,6 +105,44 @@ def test_device_encoder_writes_the_host_encoders_blob(hl, rows, cols, ce, kind, 
 
 
 @pytest.mark.gpu
+@pytest.mark.parametrize("rows,cols,ce,kind,dtype,budget,offset", [
+    (40, 1023, 1024, "gauss", 0, 0, 1),              # rows on every 2-byte boundary, the tensor itself off 4 bytes
+    (17, 4094, 4096, "gauss", 0, 0, 2),              # rows on 4-byte boundaries
+    (16, 4104, 512, "student", 0, 12, 8),            # 16-byte loads, codewords of up to 12 bits (pairs of 24 bits)
+    (33, 1030, 16384, "fp16", 1, 12, 3),             # the longest records: several stretches per checksum
+    (2, 7, 512, "gauss", 0, 0, 0),                   # one chunk, rows shorter than a thread's eight weights
+    (16, 32 * 1023, 512, "constant", 0, 0, 0),       # 1023 / 1024 / 1025 chunks of one block, records of the least size:
+    (16, 32 * 1024, 512, "constant", 0, 0, 0),       # around the end of a scan CTA
+    (16, 32 * 1025, 512, "constant", 0, 0, 0),
+    (1040, 1024, 512, "fp16", 1, 7, 0),              # 2080 chunks, records of an odd number of 128-byte units
+])
+def test_device_encoder_at_the_edges_of_its_passes(hl, rows, cols, ce, kind, dtype, budget, offset):
+    """Loads that are not aligned, sequences that fill their rows, the scan's and the checksum's borders: host blob, byte for byte."""
+    import torch
+    w = gen(kind, rows, cols, 5)
+    buf = torch.zeros(rows * cols + 16, dtype=torch.int16, device="cuda")
+    w_dev = buf[offset:offset + rows * cols]
+    w_dev.copy_(torch.from_numpy(w.view(np.int16).reshape(-1)))
+    cb = hl.build_codebook(w, dtype, budget)
+    cap = hl.encode_bound(rows, cols, dtype, ce)
+    blob_dev = torch.full((cap + 256,), 0xA5, dtype=torch.uint8, device="cuda")
+    n_scr = hl.encode_device_scratch_bytes(rows, cols, ce)
+    scratch = torch.full((n_scr,), 0x5A, dtype=torch.uint8, device="cuda")
+    desc = hl.encode_device(cb, w_dev, rows, cols, ce, blob_dev, cap, scratch, n_scr)
+    want, desc_host = hl.encode(cb, w, ce)
+    got = blob_dev.cpu().numpy()
+    assert np.all(got[desc.blob_bytes:] == 0xA5)
+    assert bytes(desc) == bytes(desc_host) and np.array_equal(got[:desc.blob_bytes], want)
+    # a buffer one byte short is refused and nothing is written behind what it holds
+    blob_dev.fill_(0xA5)
+    with pytest.raises(hl.HuffllmError) as e:
+        hl.encode_device(cb, w_dev, rows, cols, ce, blob_dev, int(desc.blob_bytes) - 1, scratch, n_scr)
+    assert e.value.status_name == "BUFFER_TOO_SMALL"
+    assert np.all(blob_dev.cpu().numpy()[desc.off_payload:] == 0xA5)
+    cb.free()
+
+
+@pytest.mark.gpu
 def test_full_size_matrix_on_the_device_equals_the_host_blob(hl):
     """A full-size FFN matrix of the benchmark's layer (45 M weights, 11008 chunks)."""
     import torch
