@@ -4,14 +4,19 @@
 // entropies and Huffman code costs.
 //
 // Counting is one streaming pass over the weights (2 bytes per weight from HBM).  Every CTA keeps private counters in
-// shared memory and adds them to the global 64-bit counters at the end.  LLM weights are very skewed (a handful of
-// exponent values cover almost all weights), so a narrow field's counters are replicated 32 times, one copy per
-// lane: the lanes of a warp never touch the same address or the same bank, whatever the data.  Wider fields get
-// fewer copies; a field whose counters do not fit is counted in several launches, each owning a range of values.
+// shared memory and adds them to the global 64-bit counters at the end.  What bounds it is the shared-memory atomic unit,
+// one counter update per weight and counted piece, so neighbouring narrow fields are counted together, as one piece of up
+// to ten bits, and told apart when the CTA adds its counters up.  LLM weights are very skewed (a handful of exponent values
+// cover almost all weights), so a piece's counters are replicated 32 times, one copy per lane: the lanes of a warp never
+// touch the same address or the same bank, whatever the data.  Wider fields get fewer copies; a field whose counters do
+// not fit is counted in several launches, each owning a range of values.
+// (45 M weights, splits 1-8-7 / 1-5-5-5: 40 / 49 us with every field counted on its own, one load in flight per thread and a
+// loop over the fields.)
 #include <cuda_runtime.h>
 
 #include <algorithm>
 #include <cmath>
+#include <cstring>
 #include <vector>
 
 #include "internal.h"
@@ -20,21 +25,27 @@ namespace huffllm {
 
 constexpr uint32_t kHistThreads = 1024;
 constexpr uint32_t kHistBudgetWords = 48u * 1024u;   // shared-memory counters of one launch (192 KB)
-constexpr uint32_t kFieldWords = 8u * 1024u;         // target size of one field's counters, copies included
+constexpr uint32_t kFieldWords = 8u * 1024u;         // target size of a wide field's counters, copies included
+constexpr uint32_t kPieceBits = 10;                  // most bits of a piece of several fields: 1024 counters, 32 copies, 128 KB
 
-struct FieldPlan {
-    uint32_t shift, mask;        // value of the field = (word >> shift) & mask
+struct PiecePlan {
+    uint32_t shift, mask;        // value of the piece = (word >> shift) & mask
     uint32_t bin_lo, bin_n;      // values counted by this launch: bin_lo .. bin_lo + bin_n - 1
     uint32_t smem_off;           // first counter, in 32-bit words
     uint32_t rep_log2;           // log2 of the copies per value
+    uint32_t ranged;             // 1 if the launch covers only a part of the piece's values
+    uint32_t field_first, n_fields;
+};
+struct FieldPlan {
+    uint32_t shift, width;       // inside its piece
     uint32_t out_off;            // index of the field's value 0 in the output counters
-    uint32_t ranged;             // 1 if the launch covers only a part of the field's values
 };
 struct HistArgs {
     const uint16_t *w;
     uint64_t n;
     unsigned long long *counts;
-    uint32_t n_fields, smem_words;
+    uint32_t n_pieces, smem_words;
+    PiecePlan p[HUFFLLM_MAX_FIELDS];
     FieldPlan f[HUFFLLM_MAX_FIELDS];
 };
 
@@ -42,7 +53,9 @@ __device__ __forceinline__ void red_shared_inc(uint32_t addr) {
     asm volatile("red.shared.add.u32 [%0], 1;" ::"r"(addr) : "memory");
 }
 
-__global__ void __launch_bounds__(kHistThreads) split_histogram_kernel(const __grid_constant__ HistArgs A) {
+// PIECES: 2 = two unranged pieces whose counters are 32-fold (the splits of the two formats), 0 = any
+template <int PIECES>
+__global__ void __launch_bounds__(kHistThreads, 2) split_histogram_kernel(const __grid_constant__ HistArgs A) {
     extern __shared__ __align__(16) uint32_t hist[];
     const uint32_t tid = threadIdx.x, lane = tid & 31;
     for (uint32_t i = tid; i < A.smem_words; i += blockDim.x) hist[i] = 0;
@@ -52,56 +65,104 @@ __global__ void __launch_bounds__(kHistThreads) split_histogram_kernel(const __g
     // 16-byte vectors of eight weights, dealt to the grid's threads in turn; the last n % 8 weights go to one thread
     const uint64_t n_vec = A.n / 8, stride = (uint64_t)gridDim.x * blockDim.x;
     const uint4 *src = (const uint4 *)A.w;
-    auto count_word = [&](uint32_t word, uint32_t n_in_word) {     // one or two weights of a 32-bit word
+    // the n_in_word weights of a 32-bit word
+    auto count_word = [&](uint32_t word, uint32_t n_in_word) {
 #pragma unroll 1
-        for (uint32_t fi = 0; fi < A.n_fields; ++fi) {
-            const FieldPlan &f = A.f[fi];
-            const uint32_t lane_off = base + ((f.smem_off + (lane & ((1u << f.rep_log2) - 1u))) << 2);
-            const uint32_t step = 4u << f.rep_log2;
+        for (uint32_t pi = 0; pi < A.n_pieces; ++pi) {
+            const PiecePlan &p = A.p[pi];
+            const uint32_t lane_off = base + ((p.smem_off + (lane & ((1u << p.rep_log2) - 1u))) << 2);
+            const uint32_t step = 4u << p.rep_log2;
 #pragma unroll
             for (uint32_t j = 0; j < 2; ++j) {
                 if (j >= n_in_word) break;
-                uint32_t b = ((word >> (f.shift + 16 * j)) & f.mask) - f.bin_lo;
-                if (!f.ranged || b < f.bin_n) red_shared_inc(lane_off + b * step);
+                uint32_t b = ((word >> (p.shift + 16 * j)) & p.mask) - p.bin_lo;
+                if (!p.ranged || b < p.bin_n) red_shared_inc(lane_off + b * step);
             }
         }
     };
-    for (uint64_t v = (uint64_t)blockIdx.x * blockDim.x + tid; v < n_vec; v += stride) {
-        const uint4 q = __ldg(src + v);
-        const uint32_t word[4] = {q.x, q.y, q.z, q.w};
-#pragma unroll 1
-        for (uint32_t fi = 0; fi < A.n_fields; ++fi) {
-            const FieldPlan &f = A.f[fi];
-            const uint32_t lane_off = base + ((f.smem_off + (lane & ((1u << f.rep_log2) - 1u))) << 2);
-            const uint32_t step = 4u << f.rep_log2, sh = f.shift, mask = f.mask, lo = f.bin_lo, nb = f.bin_n;
-            if (!f.ranged) {
+    uint32_t off[PIECES ? PIECES : 1], mask[PIECES ? PIECES : 1], sh[PIECES ? PIECES : 1];
 #pragma unroll
-                for (int i = 0; i < 4; ++i) {
-                    red_shared_inc(lane_off + ((word[i] >> sh) & mask) * step);
-                    red_shared_inc(lane_off + ((word[i] >> (sh + 16)) & mask) * step);
+    for (int pi = 0; pi < PIECES; ++pi) {
+        off[pi] = A.p[pi].smem_off << 2;
+        mask[pi] = A.p[pi].mask << 7;
+        sh[pi] = A.p[pi].shift;
+    }
+    const uint32_t lane4 = lane << 2;
+    auto inc = [&](uint32_t table, uint32_t byte_off) { atomicAdd((uint32_t *)((char *)hist + table + byte_off), 1u); };
+    auto count = [&](const uint4 &q) {
+        const uint32_t word[4] = {q.x, q.y, q.z, q.w};
+#pragma unroll
+        for (int i = 0; i < 4; ++i) {
+            if (PIECES) {
+                // a counter's 32 copies are 128 bytes: the value, moved to bit 7, is its byte offset.  (The upper weight's
+                // value is moved down by at least 9, 16 + shift - 7; the lower one's up or down: as a 64-bit shift, one instruction.)
+#pragma unroll
+                for (int pi = 0; pi < PIECES; ++pi) {
+                    inc(off[pi], ((uint32_t)(((uint64_t)word[i] << 7) >> sh[pi]) & mask[pi]) | lane4);
+                    inc(off[pi], ((word[i] >> (sh[pi] + 9u)) & mask[pi]) | lane4);
                 }
             } else {
-#pragma unroll
-                for (int i = 0; i < 4; ++i) {
-                    uint32_t b0 = ((word[i] >> sh) & mask) - lo, b1 = ((word[i] >> (sh + 16)) & mask) - lo;
-                    if (b0 < nb) red_shared_inc(lane_off + b0 * step);
-                    if (b1 < nb) red_shared_inc(lane_off + b1 * step);
-                }
+                count_word(word[i], 2);
             }
         }
+    };
+    uint64_t v = (uint64_t)blockIdx.x * blockDim.x + tid;
+    for (; v + 3 * stride < n_vec; v += 4 * stride) {          // four loads in flight per thread
+        uint4 q[4];
+#pragma unroll
+        for (int i = 0; i < 4; ++i) q[i] = __ldg(src + v + i * stride);
+#pragma unroll
+        for (int i = 0; i < 4; ++i) count(q[i]);
     }
+    for (; v < n_vec; v += stride) count(__ldg(src + v));
     if (blockIdx.x == 0 && tid == 0)
         for (uint64_t i = n_vec * 8; i < A.n; ++i) count_word(A.w[i], 1);
     __syncthreads();
 
-    // add the CTA's counters to the global ones (copies of a value summed first; zero sums are skipped)
-    for (uint32_t fi = 0; fi < A.n_fields; ++fi) {
-        const FieldPlan &f = A.f[fi];
-        const uint32_t reps = 1u << f.rep_log2;
-        for (uint32_t b = tid; b < f.bin_n; b += blockDim.x) {
-            unsigned long long s = 0;
-            for (uint32_t r = 0; r < reps; ++r) s += hist[f.smem_off + (b << f.rep_log2) + ((r + tid) & (reps - 1u))];
-            if (s) atomicAdd(A.counts + f.out_off + f.bin_lo + b, s);
+    // the copies of every value summed (into the first one, which no other thread reads)
+    for (uint32_t pi = 0; pi < A.n_pieces; ++pi) {
+        const PiecePlan &p = A.p[pi];
+        const uint32_t reps = 1u << p.rep_log2;
+        for (uint32_t b = tid; b < p.bin_n; b += blockDim.x) {
+            uint32_t s = 0;
+            for (uint32_t r = 0; r < reps; ++r) s += hist[p.smem_off + (b << p.rep_log2) + ((r + tid) & (reps - 1u))];
+            hist[p.smem_off + (b << p.rep_log2)] = s;
+        }
+    }
+    __syncthreads();
+    // add the CTA's counters to the global ones (zero sums are skipped): a piece of one field as it stands, a piece of
+    // several with a thread or a warp per field value, which sums the piece's values that have it
+    for (uint32_t pi = 0; pi < A.n_pieces; ++pi) {
+        const PiecePlan &p = A.p[pi];
+        if (p.n_fields == 1) {
+            for (uint32_t b = tid; b < p.bin_n; b += blockDim.x) {
+                const uint32_t s = hist[p.smem_off + (b << p.rep_log2)];
+                if (s) atomicAdd(A.counts + A.f[p.field_first].out_off + p.bin_lo + b, (unsigned long long)s);
+            }
+            continue;
+        }
+        for (uint32_t fi = p.field_first; fi < p.field_first + p.n_fields; ++fi) {
+            const FieldPlan &f = A.f[fi];
+            const uint32_t others = p.bin_n >> f.width;        // piece values with a given field value
+            auto at = [&](uint32_t val, uint32_t i) -> uint32_t {
+                const uint32_t b = ((i >> f.shift) << (f.shift + f.width)) | (val << f.shift) | (i & ((1u << f.shift) - 1u));
+                return hist[p.smem_off + (b << p.rep_log2)];
+            };
+            if (others <= 8u) {                                // few: a thread per field value
+                for (uint32_t val = tid; val < 1u << f.width; val += kHistThreads) {
+                    uint32_t s = 0;
+                    for (uint32_t i = 0; i < others; ++i) s += at(val, i);
+                    if (s) atomicAdd(A.counts + f.out_off + val, (unsigned long long)s);
+                }
+                continue;
+            }
+            for (uint32_t val = tid >> 5; val < 1u << f.width; val += kHistThreads / 32) {
+                uint32_t s = 0;
+                for (uint32_t i = lane; i < others; i += 32) s += at(val, i);
+#pragma unroll
+                for (int o = 16; o; o >>= 1) s += __shfl_xor_sync(0xFFFFFFFFu, s, o);
+                if (lane == 0 && s) atomicAdd(A.counts + f.out_off + val, (unsigned long long)s);
+            }
         }
     }
 }
@@ -147,25 +208,38 @@ extern "C" huffllm_status huffllm_split_histogram(const uint16_t *w_dev, uint64_
     if ((e = cudaGetDevice(&dev)) != cudaSuccess || (e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev)) != cudaSuccess)
         return fail(HUFFLLM_ERR_CUDA, "device query: %s", cudaGetErrorString(e));
 
-    // the pieces to count: a field, or a range of values of a wide field, each with its counters' size
-    std::vector<FieldPlan> pieces;
+    // the pieces to count: neighbouring fields of up to kPieceBits bits together, a wider field, or a range of a wide
+    // field's values, each with its counters' size.  (A split has 16 bits, so two pieces are the least there can be, and no
+    // split of fields of up to ten bits needs more than three.)
+    std::vector<PiecePlan> pieces;
+    FieldPlan fields[HUFFLLM_MAX_FIELDS] = {};
     uint32_t hi = 16, out_off = 0;
-    for (uint32_t i = 0; i < n_fields; ++i) {
-        const uint32_t wd = widths[i], n_bins = 1u << wd;
-        FieldPlan f = {};
-        f.shift = hi - wd;
-        f.mask = n_bins - 1u;
-        f.out_off = out_off;
-        while (f.rep_log2 < 5u && (n_bins << (f.rep_log2 + 1u)) <= kFieldWords) ++f.rep_log2;
+    for (uint32_t i = 0; i < n_fields;) {
+        uint32_t bits = widths[i], last = i + 1;
+        while (last < n_fields && bits + widths[last] <= kPieceBits) bits += widths[last++];
+        const uint32_t n_bins = 1u << bits;
+        PiecePlan p = {};
+        p.shift = hi - bits;
+        p.mask = n_bins - 1u;
+        p.field_first = i;
+        p.n_fields = last - i;
+        for (uint32_t rel = bits; i < last; ++i) {
+            rel -= widths[i];
+            fields[i].shift = rel;
+            fields[i].width = widths[i];
+            fields[i].out_off = out_off;
+            out_off += 1u << widths[i];
+        }
+        const uint32_t target = bits <= kPieceBits ? n_bins << 5 : kFieldWords;
+        while (p.rep_log2 < 5u && (n_bins << (p.rep_log2 + 1u)) <= target) ++p.rep_log2;
         const uint32_t per_piece = std::min(n_bins, kHistBudgetWords / 2u >= n_bins ? n_bins : 32u * 1024u);
         for (uint32_t lo = 0; lo < n_bins; lo += per_piece) {
-            f.bin_lo = lo;
-            f.bin_n = per_piece;
-            f.ranged = per_piece < n_bins ? 1u : 0u;
-            pieces.push_back(f);
+            p.bin_lo = lo;
+            p.bin_n = per_piece;
+            p.ranged = per_piece < n_bins ? 1u : 0u;
+            pieces.push_back(p);
         }
-        hi -= wd;
-        out_off += n_bins;
+        hi -= bits;
     }
     // launches: pieces in order, as many as fit the shared-memory budget
     size_t p = 0;
@@ -174,24 +248,28 @@ extern "C" huffllm_status huffllm_split_histogram(const uint16_t *w_dev, uint64_
         A.w = w_dev;
         A.n = n_weights;
         A.counts = (unsigned long long *)counts_dev;
+        memcpy(A.f, fields, sizeof(fields));
         uint32_t words = 0;
-        while (p < pieces.size() && A.n_fields < HUFFLLM_MAX_FIELDS) {
-            FieldPlan f = pieces[p];
+        bool plain = true;
+        while (p < pieces.size() && A.n_pieces < HUFFLLM_MAX_FIELDS) {
+            PiecePlan f = pieces[p];
             const uint32_t need = f.bin_n << f.rep_log2;
-            if (A.n_fields && words + need > kHistBudgetWords) break;
+            if (A.n_pieces && words + need > kHistBudgetWords) break;
             f.smem_off = words;
             words += need;
-            A.f[A.n_fields++] = f;
+            plain = plain && !f.ranged && f.rep_log2 == 5u;
+            A.p[A.n_pieces++] = f;
             ++p;
         }
         A.smem_words = words;
         const size_t smem = (size_t)words * 4u;
-        if ((e = cudaFuncSetAttribute(split_histogram_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)(kHistBudgetWords * 4u))) != cudaSuccess)
+        const auto kernel = plain && A.n_pieces == 2 ? split_histogram_kernel<2> : split_histogram_kernel<0>;
+        if ((e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)(kHistBudgetWords * 4u))) != cudaSuccess)
             return fail(HUFFLLM_ERR_CUDA, "cudaFuncSetAttribute: %s", cudaGetErrorString(e));
         const uint64_t n_vec = n_weights / 8;
         uint32_t grid = (uint32_t)sms * (smem <= 100u * 1024u ? 2u : 1u);
         grid = (uint32_t)std::max<uint64_t>(1, std::min<uint64_t>(grid, (n_vec + kHistThreads - 1) / kHistThreads));
-        split_histogram_kernel<<<grid, kHistThreads, smem, s>>>(A);
+        kernel<<<grid, kHistThreads, smem, s>>>(A);
         if ((e = cudaGetLastError()) != cudaSuccess) return fail(HUFFLLM_ERR_CUDA, "split_histogram_kernel: %s", cudaGetErrorString(e));
     }
     return HUFFLLM_OK;
