@@ -144,38 +144,61 @@ bool tc_fits(const huffllm_desc *d, uint32_t npad, uint32_t tiles, bool flat, ui
     const uint32_t n_dec = 8 * tiles < 31 ? 8 * tiles : 31;
     return planned_warps(n.table_align, n.table_bytes, 2ull * n.slot_bytes, dyn_smem, b_stages, n.guard_bytes) >= n_dec;
 }
-// `sms`: the CTAs this matrix can have (all SMs, or its share of a launch over several matrices); `tiles_cap`: the tiles
-// the launch's other matrices leave room for; `max_bytes`: the workspace at hand (column ranges whose pieces would not
-// fit are not considered: a share of the SMs can favour more ranges than the whole GPU, for which workspaces are sized).
-TcPlan tc_plan(const huffllm_desc *d, uint32_t batch, uint32_t sms, uint32_t dyn_smem, bool flat, uint32_t tiles_cap = 4,
-               size_t max_bytes = ~(size_t)0) {
+// As many 8-warp tiles per CTA as the chunk slots leave room for, up to `tiles_cap`.
+uint32_t tc_npad_of(uint32_t batch) { return batch <= 16 ? 16 : (batch <= 32 ? 32 : 64); }
+uint32_t tc_tiles(const huffllm_desc *d, uint32_t npad, bool flat, uint32_t dyn_smem, uint32_t tiles_cap) {
+    uint32_t tiles = tiles_cap;
+    while (tiles > 1 && !tc_fits(d, npad, tiles, flat, dyn_smem)) --tiles;
+    return tiles;
+}
+// The longest any CTA works when `ks` column ranges of `m_tiles` row tiles are dealt to `sms` CTAs: CTA b takes items b,
+// b + grid, ... in turn; an item costs its blocks of 32 columns (ranges of one matrix differ by a chunk when ks does not
+// divide the chunk count) plus `item_blocks` for its start and epilogue.  Item i is of range i mod ks, so what a CTA gets
+// depends on b mod ks and on whether it has an item in the last round: ks times two sums instead of one per CTA.  (Walking
+// every item of every candidate took 15 to 30 us of host time per matrix and launch: the four launches of a 7B-shaped layer
+// at 32 vectors were bound by it, 225 us a layer for 165 us of GPU time.)
+uint64_t tc_span(const huffllm_desc *d, uint32_t m_tiles, uint32_t ks, uint32_t sms, uint64_t item_blocks) {
+    const uint64_t items = (uint64_t)m_tiles * ks;
+    const uint32_t grid = (uint32_t)(items < sms ? items : sms), rounds = (uint32_t)((items + grid - 1) / grid);
+    const uint32_t in_last = (uint32_t)(items - (uint64_t)(rounds - 1) * grid);      // CTAs with an item in the last round: the first ones
+    const uint32_t chunk_blocks = d->chunk_cols / kBlockCols, step = grid % ks;
+    uint32_t cost[16];                                                               // of an item of range r
+    for (uint32_t r = 0, at = 0; r < ks; ++r) {
+        const uint32_t end = (uint32_t)((uint64_t)d->col_chunks * (r + 1) / ks);
+        cost[r] = (end - at) * chunk_blocks + (uint32_t)item_blocks;
+        at = end;
+    }
+    uint64_t span = 0;
+    for (uint32_t rho = 0; rho < ks && rho < grid; ++rho) {
+        const uint32_t n = rho < in_last ? rounds : rounds - 1;                      // CTA rho has the most items of its residue
+        uint64_t sum = 0;
+        for (uint32_t i = 0, r = rho; i < n; ++i) {
+            sum += cost[r];
+            r = r + step >= ks ? r + step - ks : r + step;
+        }
+        if (sum > span) span = sum;
+    }
+    return span;
+}
+// `sms`: the CTAs this matrix can have (all SMs, or its share of a launch over several matrices); `tiles`: its tiles per CTA;
+// `max_bytes`: the workspace at hand (column ranges whose pieces would not fit are not considered: a share of the SMs can
+// favour more ranges than the whole GPU, for which workspaces are sized).
+TcPlan tc_plan(const huffllm_desc *d, uint32_t batch, uint32_t sms, uint32_t tiles, size_t max_bytes = ~(size_t)0) {
     TcPlan p;
-    p.npad = batch <= 16 ? 16 : (batch <= 32 ? 32 : 64);
-    p.tiles = tiles_cap;                            // as many 8-warp tiles as the chunk slots leave room for
-    while (p.tiles > 1 && !tc_fits(d, p.npad, p.tiles, flat, dyn_smem)) --p.tiles;
+    p.npad = tc_npad_of(batch);
+    p.tiles = tiles;
     const uint32_t n_dec = 8 * p.tiles < 31 ? 8 * p.tiles : 31;      // the CTA's last warp issues the MMAs and never decodes
     p.m_tiles = (d->row_groups + n_dec - 1) / n_dec;
-    // Column ranges: the one with the shortest finish time.  A CTA takes items b, b + grid, ... in turn; an item costs its
-    // blocks of 32 columns (ranges of one matrix differ by a chunk when ksplit does not divide the chunk count) plus a start
-    // and an epilogue worth a few blocks.  Counting whole waves alone would pick many short, unequal ranges.
+    // Column ranges: the count with the shortest finish time.  Counting whole waves alone would pick many short, unequal ranges.
     // (measured on the 70B-FFN shapes at 64 vectors: a block of 32 columns takes 1.25 us of an item, the item's start and
     // epilogue together 5 to 8 us)
     constexpr uint64_t kItemBlocks = 5;
     uint32_t best = 1;
     uint64_t best_span = ~0ull;
     for (uint32_t ks = 1; ks <= 16 && ks <= d->col_chunks; ++ks) {
-        const uint64_t items = (uint64_t)p.m_tiles * ks, grid = items < sms ? items : sms;
+        const uint64_t items = (uint64_t)p.m_tiles * ks;
         if (ks > 1 && ws_partial_offset(d) + (size_t)items * 32 * (p.npad / 2) * 32 * sizeof(float) > max_bytes) break;
-        uint64_t span = 0;
-        for (uint64_t b = 0; b < grid; ++b) {
-            uint64_t t = 0;
-            for (uint64_t it = b; it < items; it += grid) {
-                const uint32_t r = (uint32_t)(it % ks);
-                const uint32_t len = (uint32_t)((uint64_t)d->col_chunks * (r + 1) / ks) - (uint32_t)((uint64_t)d->col_chunks * r / ks);
-                t += (uint64_t)len * (d->chunk_cols / kBlockCols) + kItemBlocks;
-            }
-            if (t > span) span = t;
-        }
+        const uint64_t span = tc_span(d, p.m_tiles, ks, sms, kItemBlocks);
         if (span < best_span) { best_span = span; best = ks; }
     }
     p.ksplit = best;
@@ -312,7 +335,8 @@ huffllm_status huffllm_workspace_bytes(const huffllm_desc *desc, uint32_t batch,
         clear_error();
         const int sms = have ? dev.sms : 148;
         const uint32_t dyn = (have ? (uint32_t)dev.smem_optin : 232448u) - kStaticSmem;
-        size_t tc = tc_plan(desc, batch, (uint32_t)sms, dyn, false).bytes;     // (with all three FP16 tables: the larger plan)
+        const uint32_t tiles = tc_tiles(desc, tc_npad_of(batch), false, dyn, 4);     // (with all three FP16 tables: the larger plan)
+        size_t tc = tc_plan(desc, batch, (uint32_t)sms, tiles).bytes;
         if (tc > *bytes) *bytes = tc;
     }
     return HUFFLLM_OK;
@@ -421,10 +445,9 @@ huffllm_status huffllm_decode_gemm_multi(uint32_t n, const huffllm_desc *const *
         const uint32_t npad = batch <= 32 ? 32 : 64;
         uint32_t tiles = 4;                             // what the matrix with the largest records leaves room for
         for (uint32_t i = 0; i < n; ++i) {
-            const TcPlan tp = tc_plan(descs[i], batch, (uint32_t)dev.sms, k.dyn_smem_bytes, k.fp16_flat != 0);
-            if (!tc_fits(descs[i], tp.npad, tp.tiles, k.fp16_flat != 0, k.dyn_smem_bytes))
+            tiles = tc_tiles(descs[i], npad, k.fp16_flat != 0, k.dyn_smem_bytes, tiles);
+            if (tiles == 1 && !tc_fits(descs[i], npad, 1, k.fp16_flat != 0, k.dyn_smem_bytes))
                 return fail(HUFFLLM_ERR_UNSUPPORTED, "chunk records of matrix %u too large for the tensor-core kernel's slots", i);
-            if (tp.tiles < tiles) tiles = tp.tiles;
         }
         k.part_bytes = tc_stages(npad) * npad * 128;
         k.slots = 2;
@@ -433,7 +456,7 @@ huffllm_status huffllm_decode_gemm_multi(uint32_t n, const huffllm_desc *const *
         k.tc_tiles = tiles;
         uint32_t first = 0;
         for (uint32_t i = 0; i < n; ++i) {
-            const TcPlan tp = tc_plan(descs[i], batch, k.m[i].cta_count, k.dyn_smem_bytes, k.fp16_flat != 0, tiles, workspace_bytes_each);
+            const TcPlan tp = tc_plan(descs[i], batch, k.m[i].cta_count, tiles, workspace_bytes_each);
             if (workspace_bytes_each < tp.bytes) return fail(HUFFLLM_ERR_BUFFER_TOO_SMALL, "workspace of matrix %u too small for batch %u", i, batch);
             t.m_tiles[i] = tp.m_tiles;
             t.ksplit[i] = tp.ksplit;
@@ -511,7 +534,8 @@ huffllm_status huffllm_decode_gemm(const huffllm_desc *desc, const void *blob, c
         // vectors through the register-path kernel and its two-level lookup)
         if (!tc_blob(desc)) return HUFFLLM_OK;
         // (column ranges are planned within the workspace at hand)
-        const TcPlan tp = tc_plan(desc, batch, (uint32_t)dev.sms, (uint32_t)dev.smem_optin - kStaticSmem, flat_fp16(desc), 4, workspace_bytes);
+        const uint32_t dyn = (uint32_t)dev.smem_optin - kStaticSmem, tiles = tc_tiles(desc, tc_npad_of(batch), flat_fp16(desc), dyn, 4);
+        const TcPlan tp = tc_plan(desc, batch, (uint32_t)dev.sms, tiles, workspace_bytes);
         TcArgs t;
         memset(&t, 0, sizeof(t));
         KernelArgs &k = t.k;

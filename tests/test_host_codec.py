@@ -376,3 +376,31 @@ def test_code_length_limits_accepted_per_format():
         with pytest.raises(hl.HuffllmError) as e:
             hl.build_codebook(w, dt, b)
         assert e.value.status_name == "UNSUPPORTED"
+
+
+def test_column_ranges_finish_first_among_all_simulated():
+    """The tensor-core path's column ranges (seen through the workspace they need) are those of a walk over every work item."""
+    import random
+    w = wl.gaussian_weights(16, 1024, 0.02, 1)
+    cb = hl.build_codebook(w)
+    _, d = hl.encode(cb, w, 2048)
+    cb.free()
+    rng = random.Random(3)
+    for rows, cols in [(64, 128), (4096, 4096), (28672, 8192), (8192, 28672), (1024, 14336)] + \
+                      [(rng.randrange(1, 30000), 32 * rng.randrange(1, 900)) for _ in range(60)]:
+        d.rows, d.cols, d.row_groups = rows, cols, (rows + 15) // 16
+        d.col_chunks = (cols + d.chunk_cols - 1) // d.chunk_cols
+        d.n_chunks = d.row_groups * d.col_chunks
+        d.off_payload = (d.off_index + 4 * (d.n_chunks + 1) + 255) // 256 * 256
+        d.payload_bytes, d.blob_bytes = 128 * d.n_chunks, d.off_payload + 128 * d.n_chunks + 4096
+        m_tiles, best, best_span = (d.row_groups + 30) // 31, 1, None
+        for ks in range(1, min(16, d.col_chunks) + 1):
+            items = m_tiles * ks
+            grid = min(items, 148)
+            cost = [(d.col_chunks * (r + 1) // ks - d.col_chunks * r // ks) * (d.chunk_cols // 32) + 5 for r in range(ks)]
+            span = max(sum(cost[i % ks] for i in range(b, items, grid)) for b in range(grid))
+            if best_span is None or span < best_span:
+                best, best_span = ks, span
+        tc = 4096 + ((d.row_groups + 7) // 8 * 128 + 255) // 256 * 256 + (m_tiles * best * 32 * 32 * 32 * 4 if best > 1 else 0)
+        two_tiles = 4096 + ((d.row_groups + 7) // 8 * 128 + 255) // 256 * 256 + 512 * (2 + 64) * 16 * 16 * 4
+        assert hl.workspace_bytes(d, 64) == max(tc, two_tiles), (rows, cols)
