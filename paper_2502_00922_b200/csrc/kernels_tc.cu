@@ -157,29 +157,91 @@ __global__ void __launch_bounds__(1024, 1) huff_gemm_tc_kernel(const __grid_cons
     const uint32_t bar0 = smem_u32(&bars[warp * 2]);
     const uint32_t slot0 = slot_addr(plan, warp, 0, A.slot_bytes);    // (this kernel always runs with two slots per warp)
 
-    // ---- set-up: table, barriers, tensor memory
-    {
-        const uint32_t *lut_g = (const uint32_t *)(k.blob + k.off_lut);
-        uint32_t *lut_s = (uint32_t *)(dyn_smem + (plan.lut - smem_base));
-        // (FP16: three tables of 256 entries, sixteen copies each: word j holds entry j / 16)
-        constexpr uint32_t kLutWords = FMT == 2 ? 16u * 256u : FMT ? 3u * 16u * 256u : 32u << LB;   // (flat mantissa codes: the exponent's table alone)
-        for (uint32_t i = tid; i < kLutWords; i += 1024) {
-            const uint32_t v = __ldg(lut_g + (i >> (FMT ? 4 : 5)));
-            lut_s[i] = SKIP ? lut_entry_inplace(v) : SKIP16 ? fp16_entry_inplace(v) : v;
+    // ---- roles
+    const uint32_t tile = warp >> 3, q = warp & 3, h = (warp >> 2) & 1;
+    const uint32_t rgi = tile * 8 + q * 2 + h;                              // row group of the CTA's 32 that this warp decodes
+    const uint32_t a_lane = (32u * q + 16u * h) << 16;
+    const uint32_t KC = k.col_chunks, RG = (uint32_t)((k.rows + 15) / 16);
+    const uint32_t *index = (const uint32_t *)(k.blob + k.off_index);
+    const uint8_t *payload = k.blob + k.off_payload;
+    const uint32_t ksplit = T.ksplit[MULTI ? mi : 0], n_items = T.m_tiles[MULTI ? mi : 0] * ksplit;
+    auto blocks_of = [&](uint32_t kc) -> uint32_t {
+        uint32_t left = (uint32_t)k.cols - kc * k.chunk_cols;
+        return (min(left, k.chunk_cols) + 31u) >> 5;
+    };
+    auto record_ok = [&](uint32_t r0, uint32_t r1, uint32_t nkb) -> bool {
+        return r1 > r0 && r1 <= k.payload_units && (r1 - r0) * 128u > raw_part(nkb) &&
+               (r1 - r0) * 128u - raw_part(nkb) <= A.slot_bytes;
+    };
+    auto issue_record = [&](uint32_t c, uint32_t which, uint32_t r0, uint32_t r1) {
+        uint32_t nkb = blocks_of(c % KC), bar = bar0 + which * 8;
+        if (record_ok(r0, r1, nkb)) {
+            uint32_t bytes = (r1 - r0) * 128u - raw_part(nkb);
+            mbar_expect_tx(bar, bytes);
+            bulk_g2s(slot0 + which * A.slot_bytes, payload + (uint64_t)r0 * 128u + raw_part(nkb), bytes, bar);
+        } else {
+            mbar_expect_tx(bar, 0);
         }
-    }
-    if (lane == 0) {
-        mbar_init(bar0, 1);
-        mbar_init(bar0 + 8, 1);
-    }
-    if (tid < S) {
-        mbar_init(smem_u32(&empty_bar[tid]), 1);
-        mbar_init(smem_u32(&full_bar[tid]), n_dec);
-    }
-    asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
-    if (warp == 0) {
-        tmem_alloc(smem_u32(&s_tmem_base), 512);
-        tmem_relinquish();
+    };
+    auto issue = [&](uint32_t c, uint32_t which) { issue_record(c, which, __ldg(index + c), __ldg(index + c + 1)); };
+    // first and last chunk of this warp's row group in a work item (false: the row group lies outside the matrix)
+    auto item_chunks = [&](uint32_t it, uint32_t &cb, uint32_t &ce) -> bool {
+        const uint32_t mt_i = it / ksplit, ks_i = it % ksplit, rg_i = mt_i * n_dec + rgi;
+        cb = rg_i * KC + (uint32_t)((uint64_t)KC * ks_i / ksplit);
+        ce = rg_i * KC + (uint32_t)((uint64_t)KC * (ks_i + 1) / ksplit);
+        return rg_i < RG;
+    };
+
+    // ---- set-up: table, barriers, tensor memory.  The offsets of the warp's first two records are asked for before anything
+    // else and their copies started between the table's loads and stores (a warp's barriers are its own, so the copies need
+    // nothing that the CTA has to meet for): the records arrive while the table is built.  (With the copies started behind
+    // the set-up a CTA's first block was decoded 7.3 us after its start, 3.6 of them set-up.)
+    bool primed = false;                 // the item's first two record copies are under way
+    {
+        uint32_t cb = 0, ce = 0, o0 = 0, o1 = 0, o2 = 0;
+        primed = warp < n_dec && J < n_items && item_chunks(J, cb, ce);
+        if (primed && lane == 0) {
+            o0 = __ldg(index + cb);
+            o1 = __ldg(index + cb + 1);
+            if (cb + 1 < ce) o2 = __ldg(index + cb + 2);
+            mbar_init(bar0, 1);
+            mbar_init(bar0 + 8, 1);
+        }
+        // the table goes to shared memory in 16-byte pieces: four neighbouring copies of one entry per piece
+        // (FP16: three tables of 256 entries, sixteen copies each; flat mantissa codes: the exponent's table alone)
+        constexpr uint32_t kLutVecs = FMT == 2 ? 4u * 256u : FMT ? 3u * 4u * 256u : 8u << LB;
+        constexpr int kLutLoads = (kLutVecs + 1023) / 1024;
+        const uint32_t *lut_g = (const uint32_t *)(k.blob + k.off_lut);
+        uint32_t lut_v[kLutLoads];
+#pragma unroll
+        for (int i = 0; i < kLutLoads; ++i) {
+            const uint32_t v = tid + i * 1024u;
+            lut_v[i] = v < kLutVecs ? __ldg(lut_g + (v >> (FMT ? 2 : 3))) : 0u;
+        }
+        if (tid < S) {
+            mbar_init(smem_u32(&empty_bar[tid]), 1);
+            mbar_init(smem_u32(&full_bar[tid]), n_dec);
+        }
+        asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+        if (warp == issuer) {
+            tmem_alloc(smem_u32(&s_tmem_base), 512);
+            tmem_relinquish();
+        }
+        if (primed && lane == 0) {
+            asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
+            issue_record(cb, 0, o0, o1);
+            if (cb + 1 < ce) issue_record(cb + 1, 1, o1, o2);
+        } else if (!primed && lane == 0) {                      // (a warp without rows in the first item may have some in a later one)
+            mbar_init(bar0, 1);
+            mbar_init(bar0 + 8, 1);
+            asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+        }
+        uint4 *lut_s = (uint4 *)(dyn_smem + (plan.lut - smem_base));
+#pragma unroll
+        for (int i = 0; i < kLutLoads; ++i) {
+            const uint32_t v = tid + i * 1024u, e = SKIP ? lut_entry_inplace(lut_v[i]) : SKIP16 ? fp16_entry_inplace(lut_v[i]) : lut_v[i];
+            if (v < kLutVecs) lut_s[v] = make_uint4(e, e, e, e);
+        }
     }
     tc_fence_before();
     __syncthreads();
@@ -195,38 +257,11 @@ __global__ void __launch_bounds__(1024, 1) huff_gemm_tc_kernel(const __grid_cons
     // kernel in front of this one in the stream may still be producing
     pdl_wait_prior_grid();
 
-    // ---- roles
-    const uint32_t tile = warp >> 3, q = warp & 3, h = (warp >> 2) & 1;
-    const uint32_t rgi = tile * 8 + q * 2 + h;                              // row group of the CTA's 32 that this warp decodes
-    const uint32_t a_lane = (32u * q + 16u * h) << 16;
-    const uint32_t KC = k.col_chunks, RG = (uint32_t)((k.rows + 15) / 16);
-    const uint32_t *index = (const uint32_t *)(k.blob + k.off_index);
-    const uint8_t *payload = k.blob + k.off_payload;
-    const uint32_t ksplit = T.ksplit[MULTI ? mi : 0], n_items = T.m_tiles[MULTI ? mi : 0] * ksplit;
     float *const tc_partial = T.partial[MULTI ? mi : 0];
     unsigned int *const tc_ticket = T.ticket[MULTI ? mi : 0];
     uint32_t phase = 0, gb = 0;          // coded-copy barrier parities; blocks this CTA has gone through so far
     bool failed = false;                 // a wait ran out: stop waiting, keep moving, report
 
-    auto blocks_of = [&](uint32_t kc) -> uint32_t {
-        uint32_t left = (uint32_t)k.cols - kc * k.chunk_cols;
-        return (min(left, k.chunk_cols) + 31u) >> 5;
-    };
-    auto record_ok = [&](uint32_t r0, uint32_t r1, uint32_t nkb) -> bool {
-        return r1 > r0 && r1 <= k.payload_units && (r1 - r0) * 128u > raw_part(nkb) &&
-               (r1 - r0) * 128u - raw_part(nkb) <= A.slot_bytes;
-    };
-    auto issue = [&](uint32_t c, uint32_t which) {
-        uint32_t nkb = blocks_of(c % KC), r0 = __ldg(index + c), r1 = __ldg(index + c + 1);
-        uint32_t bar = bar0 + which * 8;
-        if (record_ok(r0, r1, nkb)) {
-            uint32_t bytes = (r1 - r0) * 128u - raw_part(nkb);
-            mbar_expect_tx(bar, bytes);
-            bulk_g2s(slot0 + which * A.slot_bytes, payload + (uint64_t)r0 * 128u + raw_part(nkb), bytes, bar);
-        } else {
-            mbar_expect_tx(bar, 0);
-        }
-    };
     auto bounded_wait = [&](uint32_t bar, uint32_t parity) {
         if (failed) return;
         uint32_t spins = 0;
@@ -307,15 +342,6 @@ __global__ void __launch_bounds__(1024, 1) huff_gemm_tc_kernel(const __grid_cons
         __syncwarp();
         ++gb;
     };
-
-    // first and last chunk of this warp's row group in a work item (false: the row group lies outside the matrix)
-    auto item_chunks = [&](uint32_t it, uint32_t &cb, uint32_t &ce) -> bool {
-        const uint32_t mt_i = it / ksplit, ks_i = it % ksplit, rg_i = mt_i * n_dec + rgi;
-        cb = rg_i * KC + (uint32_t)((uint64_t)KC * ks_i / ksplit);
-        ce = rg_i * KC + (uint32_t)((uint64_t)KC * (ks_i + 1) / ksplit);
-        return rg_i < RG;
-    };
-    bool primed = false;                 // the item's first two record copies were started at the end of the item before
 
 #pragma unroll 1
     for (uint32_t item = J; item < n_items; item += n_cta) {
@@ -479,7 +505,7 @@ __global__ void __launch_bounds__(1024, 1) huff_gemm_tc_kernel(const __grid_cons
     // ---- teardown
     tc_fence_before();
     __syncthreads();
-    if (warp == 0) tmem_dealloc(tmem, 512);
+    if (warp == issuer) tmem_dealloc(tmem, 512);
 }
 
 template <int LB, int NPAD, int FMT, bool MULTI>
