@@ -125,47 +125,81 @@ uint32_t planned_warps(uint32_t lut_align, uint32_t lut_size, uint64_t pair_byte
     return (uint32_t)(least > 64 ? 64 : least);
 }
 
-// Geometry of the tensor-core small-batch path (batch 9..64): row tiles of 512 rows, column chunks cut into
-// `ksplit` ranges so that the work items fill the GPU's SMs in whole waves as well as they can.
-struct TcPlan {
-    uint32_t npad, tiles, m_tiles, ksplit, items;
-    size_t ticket_off, partial_off, bytes;
+// ---- the tensor-core small-batch path (batch 9..64)
+// What a CTA of a launch decodes side by side: `na` tiles of 128 rows in each of `slices` column slices, at most four tiles in
+// all (eight warps each), and the stages through which they hand it to the tensor core.
+struct TcShape {
+    uint32_t na, slices, stages, row_groups;
+    uint32_t decoders() const { return row_groups * slices; }
+    uint32_t part_bytes(uint32_t npad) const { return stages * slices * npad * 128; }  // the stages of activations
+    uint32_t piece_columns(uint32_t npad) const { return npad / (2 * slices); }        // columns of a warp's share of the accumulators
 };
-// Shared memory the tensor-core kernel needs with `tiles` 128-row tiles per CTA.
-// Stages of the tensor-core kernel: four, two at the widest batch padding, where shared memory is short.
-uint32_t tc_stages(uint32_t npad) { return npad == 64 ? 2u : 3u; }
+uint32_t tc_npad_of(uint32_t batch) { return batch <= 16 ? 16 : (batch <= 32 ? 32 : 64); }
 // (`flat`: every matrix of the launch has flat FP16 mantissa codes: the exponent's table alone is kept)
 bool flat_fp16(const huffllm_desc *d) { return d->dtype == HUFFLLM_FP16 && d->lut_bits == 8 && (d->flat_fields & 6u) == 6u; }
-// Do the slot pairs of `tiles` tiles' decoder warps fit beside the tables and the stages of activations?
-bool tc_fits(const huffllm_desc *d, uint32_t npad, uint32_t tiles, bool flat, uint32_t dyn_smem) {
-    SmemNeeds n = smem_needs(d);
-    if (d->dtype == HUFFLLM_FP16 && d->lut_bits == 8) n.table_bytes = flat ? 16384u : 49152u;   // (a launch-wide choice)
-    const uint32_t b_stages = tc_stages(npad) * npad * 128;          // the guard area may lie over them
-    const uint32_t n_dec = 8 * tiles < 31 ? 8 * tiles : 31;
-    return planned_warps(n.table_align, n.table_bytes, 2ull * n.slot_bytes, dyn_smem, b_stages, n.guard_bytes) >= n_dec;
+// Do the slot pairs of the shape's decoder warps fit beside the tables and the stages of activations (the guard area may lie
+// over those), for the largest records among the launch's matrices?
+bool tc_fits(const huffllm_desc *const *d, uint32_t n, uint32_t npad, const TcShape &sh, bool flat, uint32_t dyn_smem) {
+    SmemNeeds need = smem_needs(d[0]);
+    if (d[0]->dtype == HUFFLLM_FP16 && d[0]->lut_bits == 8) need.table_bytes = flat ? 16384u : 49152u;   // (a launch-wide choice)
+    for (uint32_t i = 1; i < n; ++i) {
+        const SmemNeeds o = smem_needs(d[i]);
+        if (o.slot_bytes > need.slot_bytes) need.slot_bytes = o.slot_bytes;
+        if (o.guard_bytes > need.guard_bytes) need.guard_bytes = o.guard_bytes;
+    }
+    return planned_warps(need.table_align, need.table_bytes, 2ull * need.slot_bytes, dyn_smem, sh.part_bytes(npad), need.guard_bytes) >= sh.decoders();
 }
-// As many 8-warp tiles per CTA as the chunk slots leave room for, up to `tiles_cap`.
-uint32_t tc_npad_of(uint32_t batch) { return batch <= 16 ? 16 : (batch <= 32 ? 32 : 64); }
-uint32_t tc_tiles(const huffllm_desc *d, uint32_t npad, bool flat, uint32_t dyn_smem, uint32_t tiles_cap) {
-    uint32_t tiles = tiles_cap;
-    while (tiles > 1 && !tc_fits(d, npad, tiles, flat, dyn_smem)) --tiles;
-    return tiles;
+// The shapes a launch chooses from: 0 = one slice, as many tiles of rows as find room; 1 = one slice and a warp of its own for
+// the activations (at the widest batch padding: there the issuer, which carries them otherwise, bounds the CTA, 8192 x 28672
+// at 64 vectors 138 us against 122 with one decoder fewer); 2, 3 = two and four slices.  False: it does not fit or apply.
+constexpr uint32_t kTcShapes = 4;
+bool tc_shape(const huffllm_desc *const *d, uint32_t n, uint32_t npad, uint32_t which, bool flat, uint32_t dyn_smem, TcShape *sh) {
+    const uint32_t slices = which < 2 ? 1 : which == 2 ? 2 : 4;
+    // three stages, two at the widest batch padding, where tensor memory holds no more; the CTA's last warp issues the MMAs
+    *sh = TcShape{4 / slices, slices, npad == 64 ? 2u : 3u, 32 / slices - (which == 1 ? 2 : 1)};
+    if (which == 0) {
+        for (; sh->na; --sh->na) {
+            sh->row_groups = sh->na == 4 ? 31 : 8 * sh->na;
+            if (tc_fits(d, n, npad, *sh, flat, dyn_smem)) return true;
+        }
+        return false;
+    }
+    if (which == 1 && npad != 64) return false;
+    if (slices == 4 && npad == 64) return false;             // (seven row groups' worth of rows do not pay for 64 columns of sums)
+    for (; sh->stages >= 2; --sh->stages)
+        if (tc_fits(d, n, npad, *sh, flat, dyn_smem)) return true;
+    return false;
 }
+
+// The plan of one matrix: its row tiles and the ranges its column chunks are cut into.
+struct TcPlan {
+    uint32_t m_tiles, ksplit, items;
+    uint32_t chunks;          // most column chunks that one accumulator adds up
+    uint64_t span;            // estimated time of the CTA that works longest, and of the last sum
+    size_t ticket_off, partial_off, bytes;
+};
+// Estimated costs, in 1/32 of the time that a CTA of one slice takes for a block of 32 columns (0.93 us, 31 decoders).  Time
+// stamps: with two slices (30 decoders) a block takes 0.99 us, with four (28) 1.14; an item's start and epilogue take 5 to 6 us,
+// with several slices, whose pieces are smaller, 4.5; the last CTA's sum of a row tile's pieces 9 us for 16 ranges of 16 columns
+// per warp, 5.5 for 5 of 16, 6 for 14 of 8.
+constexpr uint32_t kTcUnit = 32;
+uint32_t tc_block_cost(const TcShape &sh) { return sh.slices == 1 ? kTcUnit : sh.slices == 2 ? 34 : 39; }
+constexpr uint32_t kTcItemCost = 5 * kTcUnit;
+uint32_t tc_sum_cost(const TcShape &sh, uint32_t npad, uint32_t ks) { return ks > 1 ? 2 * ks * sh.piece_columns(npad) : 0; }
 // The longest any CTA works when `ks` column ranges of `m_tiles` row tiles are dealt to `sms` CTAs: CTA b takes items b,
-// b + grid, ... in turn; an item costs its blocks of 32 columns (ranges of one matrix differ by a chunk when ks does not
-// divide the chunk count) plus `item_blocks` for its start and epilogue.  Item i is of range i mod ks, so what a CTA gets
-// depends on b mod ks and on whether it has an item in the last round: ks times two sums instead of one per CTA.  (Walking
-// every item of every candidate took 15 to 30 us of host time per matrix and launch: the four launches of a 7B-shaped layer
-// at 32 vectors were bound by it, 225 us a layer for 165 us of GPU time.)
-uint64_t tc_span(const huffllm_desc *d, uint32_t m_tiles, uint32_t ks, uint32_t sms, uint64_t item_blocks) {
+// b + grid, ... in turn.  Item i is of range i mod ks, so what a CTA gets depends on b mod ks and on whether it has an item
+// in the last round: one sum per residue instead of one per CTA.  (Walking every item of every candidate took 15 to 30 us
+// of host time per matrix and launch: the four launches of a 7B-shaped layer at 32 vectors were bound by it, 225 us a layer
+// for 165 us of GPU time.)
+uint64_t tc_span(const huffllm_desc *d, const TcShape &sh, uint32_t m_tiles, uint32_t ks, uint32_t sms) {
     const uint64_t items = (uint64_t)m_tiles * ks;
     const uint32_t grid = (uint32_t)(items < sms ? items : sms), rounds = (uint32_t)((items + grid - 1) / grid);
     const uint32_t in_last = (uint32_t)(items - (uint64_t)(rounds - 1) * grid);      // CTAs with an item in the last round: the first ones
-    const uint32_t chunk_blocks = d->chunk_cols / kBlockCols, step = grid % ks;
-    uint32_t cost[16];                                                               // of an item of range r
+    const uint32_t chunk_cost = d->chunk_cols / kBlockCols * tc_block_cost(sh), step = grid % ks;
+    uint64_t cost[16];                                                               // of an item of range r
     for (uint32_t r = 0, at = 0; r < ks; ++r) {
-        const uint32_t end = (uint32_t)((uint64_t)d->col_chunks * (r + 1) / ks);
-        cost[r] = (end - at) * chunk_blocks + (uint32_t)item_blocks;
+        const uint32_t end = d->col_chunks * (r + 1) / ks;       // (at most 2^26 chunks: the product fits)
+        cost[r] = (uint64_t)((end - at + sh.slices - 1) / sh.slices) * chunk_cost + kTcItemCost;
         at = end;
     }
     uint64_t span = 0;
@@ -180,35 +214,62 @@ uint64_t tc_span(const huffllm_desc *d, uint32_t m_tiles, uint32_t ks, uint32_t 
     }
     return span;
 }
-// `sms`: the CTAs this matrix can have (all SMs, or its share of a launch over several matrices); `tiles`: its tiles per CTA;
-// `max_bytes`: the workspace at hand (column ranges whose pieces would not fit are not considered: a share of the SMs can
-// favour more ranges than the whole GPU, for which workspaces are sized).
-TcPlan tc_plan(const huffllm_desc *d, uint32_t batch, uint32_t sms, uint32_t tiles, size_t max_bytes = ~(size_t)0) {
+// `sms`: the CTAs this matrix can have (all SMs, or its share of a launch over several matrices); `max_bytes`: the workspace
+// at hand (column ranges whose pieces would not fit are not considered: a share of the SMs can favour more ranges than the
+// whole GPU, for which workspaces are sized); `max_chunks`: the most column chunks that one accumulator may add up.
+TcPlan tc_plan(const huffllm_desc *d, uint32_t npad, uint32_t sms, const TcShape &sh, size_t max_bytes, uint32_t max_chunks) {
     TcPlan p;
-    p.npad = tc_npad_of(batch);
-    p.tiles = tiles;
-    const uint32_t n_dec = 8 * p.tiles < 31 ? 8 * p.tiles : 31;      // the CTA's last warp issues the MMAs and never decodes
-    p.m_tiles = (d->row_groups + n_dec - 1) / n_dec;
-    // Column ranges: the count with the shortest finish time.  Counting whole waves alone would pick many short, unequal ranges.
-    // (measured on the 70B-FFN shapes at 64 vectors: a block of 32 columns takes 1.25 us of an item, the item's start and
-    // epilogue together 5 to 8 us)
-    constexpr uint64_t kItemBlocks = 5;
-    uint32_t best = 1;
+    p.m_tiles = (d->row_groups + sh.row_groups - 1) / sh.row_groups;
+    const size_t item_bytes = (size_t)32 * sh.piece_columns(npad) * 32 * sizeof(float);
+    // Column ranges: in shape 0 (no limit on the chunks) the count whose items are done first, their sums not considered (fewer,
+    // longer ranges would be a little faster, but an accumulator's error grows with the columns it adds up: 1e-6 for 1024,
+    // 3.8e-6 for 3584); in the others all costs count, and no accumulator may add up more columns than in shape 0.
+    const bool base = max_chunks == ~0u;
+    uint32_t best = 0;
     uint64_t best_span = ~0ull;
     for (uint32_t ks = 1; ks <= 16 && ks <= d->col_chunks; ++ks) {
-        const uint64_t items = (uint64_t)p.m_tiles * ks;
-        if (ks > 1 && ws_partial_offset(d) + (size_t)items * 32 * (p.npad / 2) * 32 * sizeof(float) > max_bytes) break;
-        const uint64_t span = tc_span(d, p.m_tiles, ks, sms, kItemBlocks);
+        if (ks > 1 && ws_partial_offset(d) + (size_t)p.m_tiles * ks * item_bytes > max_bytes) break;
+        const uint32_t range = (d->col_chunks + ks - 1) / ks;
+        if ((range + sh.slices - 1) / sh.slices > max_chunks) continue;
+        const uint64_t span = tc_span(d, sh, p.m_tiles, ks, sms) + (base ? 0 : tc_sum_cost(sh, npad, ks));
         if (span < best_span) { best_span = span; best = ks; }
     }
-    p.ksplit = best;
+    p.ksplit = best;                                     // (0: no number of ranges is within the limits)
     p.items = p.m_tiles * best;
+    // (at the widest padding an issuer that carries the activations as well makes a block take an eighth longer)
+    p.span = !best ? ~0ull : !base ? best_span : (npad == 64 ? best_span * 9 / 8 : best_span) + tc_sum_cost(sh, npad, best);
+    p.chunks = best ? ((d->col_chunks + best - 1) / best + sh.slices - 1) / sh.slices : 0;
     // the counters' region is sized for the smallest tile (most row tiles), so that plans for different batch sizes
     // sharing one workspace never put partial sums where another plan keeps counters
     p.ticket_off = ws_ctrl_bytes(d);
     p.partial_off = ws_partial_offset(d);
-    p.bytes = p.partial_off + (best > 1 ? (size_t)p.items * 32 * (p.npad / 2) * 32 * sizeof(float) : 0);
+    p.bytes = p.partial_off + (best > 1 ? p.items * item_bytes : 0);
     return p;
+}
+// The shape and plans of a launch over n matrices with cta[i] CTAs each: the shape whose slowest matrix is done first.  False: no
+// shape fits.
+bool tc_best(const huffllm_desc *const *d, uint32_t n, uint32_t npad, const uint32_t *cta, bool flat, uint32_t dyn_smem, size_t max_bytes,
+             TcShape *shape, TcPlan *plans) {
+    uint64_t best_span = ~0ull;
+    uint32_t most[kMaxMats];
+    for (uint32_t i = 0; i < n; ++i) most[i] = ~0u;
+    for (uint32_t which = 0; which < kTcShapes; ++which) {
+        TcShape sh;
+        if (!tc_shape(d, n, npad, which, flat, dyn_smem, &sh)) continue;
+        TcPlan p[kMaxMats];
+        uint64_t span = 0;
+        for (uint32_t i = 0; i < n; ++i) {
+            p[i] = tc_plan(d[i], npad, cta[i], sh, max_bytes, most[i]);
+            if (p[i].span > span) span = p[i].span;
+            if (which == 0) most[i] = p[i].chunks;
+        }
+        if (span < best_span) {
+            best_span = span;
+            *shape = sh;
+            for (uint32_t i = 0; i < n; ++i) plans[i] = p[i];
+        }
+    }
+    return best_span != ~0ull;
 }
 
 // Bytes of the FP16 tables a launch keeps in shared memory: three sixteen-fold tables of 8-bit codes, or the exponent's
@@ -257,6 +318,18 @@ huffllm_status add_matrix(KernelArgs *k, const huffllm_desc *desc, const void *b
     if (need.slot_bytes > k->slot_bytes) k->slot_bytes = need.slot_bytes;
     if (need.guard_bytes > k->guard_bytes) k->guard_bytes = need.guard_bytes;
     return HUFFLLM_OK;
+}
+
+// The tensor-core kernel's part of a launch description.
+void set_tc_shape(KernelArgs *k, uint32_t npad, const TcShape &sh) {
+    k->part_bytes = sh.part_bytes(npad);
+    k->slots = 2;
+    k->pair_recip = (uint32_t)(0x100000000ull / (2ull * k->slot_bytes));
+    k->tc_npad = npad;
+    k->tc_tiles = sh.na;
+    k->tc_slices = sh.slices;
+    k->tc_stages = sh.stages;
+    k->tc_row_groups = sh.row_groups;
 }
 
 // Close a launch description: shared-memory budget and grid size.
@@ -335,9 +408,12 @@ huffllm_status huffllm_workspace_bytes(const huffllm_desc *desc, uint32_t batch,
         clear_error();
         const int sms = have ? dev.sms : 148;
         const uint32_t dyn = (have ? (uint32_t)dev.smem_optin : 232448u) - kStaticSmem;
-        const uint32_t tiles = tc_tiles(desc, tc_npad_of(batch), false, dyn, 4);     // (with all three FP16 tables: the larger plan)
-        size_t tc = tc_plan(desc, batch, (uint32_t)sms, tiles).bytes;
-        if (tc > *bytes) *bytes = tc;
+        for (uint32_t flat = 0; flat < (flat_fp16(desc) ? 2u : 1u); ++flat) {      // (with all three FP16 tables, and with one)
+            const uint32_t cta = (uint32_t)sms;
+            TcShape sh;
+            TcPlan p;
+            if (tc_best(&desc, 1, tc_npad_of(batch), &cta, flat != 0, dyn, ~(size_t)0, &sh, &p) && p.bytes > *bytes) *bytes = p.bytes;
+        }
     }
     return HUFFLLM_OK;
 }
@@ -442,21 +518,17 @@ huffllm_status huffllm_decode_gemm_multi(uint32_t n, const huffllm_desc *const *
             k.m[i].y = ys[i];
         }
         if ((st = finish_args(&k, true, dev, &grid)) != HUFFLLM_OK) return st;      // (deals the CTAs to the matrices by their chunks)
-        const uint32_t npad = batch <= 32 ? 32 : 64;
-        uint32_t tiles = 4;                             // what the matrix with the largest records leaves room for
-        for (uint32_t i = 0; i < n; ++i) {
-            tiles = tc_tiles(descs[i], npad, k.fp16_flat != 0, k.dyn_smem_bytes, tiles);
-            if (tiles == 1 && !tc_fits(descs[i], npad, 1, k.fp16_flat != 0, k.dyn_smem_bytes))
-                return fail(HUFFLLM_ERR_UNSUPPORTED, "chunk records of matrix %u too large for the tensor-core kernel's slots", i);
-        }
-        k.part_bytes = tc_stages(npad) * npad * 128;
-        k.slots = 2;
-        k.pair_recip = (uint32_t)(0x100000000ull / (2ull * k.slot_bytes));
-        k.tc_npad = npad;
-        k.tc_tiles = tiles;
+        const uint32_t npad = tc_npad_of(batch);
+        uint32_t cta[kMaxMats];
+        for (uint32_t i = 0; i < n; ++i) cta[i] = k.m[i].cta_count;
+        TcShape sh;
+        TcPlan plans[kMaxMats];
+        if (!tc_best(descs, n, npad, cta, k.fp16_flat != 0, k.dyn_smem_bytes, workspace_bytes_each, &sh, plans))
+            return fail(HUFFLLM_ERR_UNSUPPORTED, "chunk records too large for the tensor-core kernel's slots");
+        set_tc_shape(&k, npad, sh);
         uint32_t first = 0;
         for (uint32_t i = 0; i < n; ++i) {
-            const TcPlan tp = tc_plan(descs[i], batch, k.m[i].cta_count, tiles, workspace_bytes_each);
+            const TcPlan &tp = plans[i];
             if (workspace_bytes_each < tp.bytes) return fail(HUFFLLM_ERR_BUFFER_TOO_SMALL, "workspace of matrix %u too small for batch %u", i, batch);
             t.m_tiles[i] = tp.m_tiles;
             t.ksplit[i] = tp.ksplit;
@@ -534,26 +606,24 @@ huffllm_status huffllm_decode_gemm(const huffllm_desc *desc, const void *blob, c
         // vectors through the register-path kernel and its two-level lookup)
         if (!tc_blob(desc)) return HUFFLLM_OK;
         // (column ranges are planned within the workspace at hand)
-        const uint32_t dyn = (uint32_t)dev.smem_optin - kStaticSmem, tiles = tc_tiles(desc, tc_npad_of(batch), flat_fp16(desc), dyn, 4);
-        const TcPlan tp = tc_plan(desc, batch, (uint32_t)dev.sms, tiles, workspace_bytes);
+        const uint32_t npad = tc_npad_of(batch), cta = (uint32_t)dev.sms;
+        TcShape sh;
+        TcPlan tp;
+        if (!tc_best(&desc, 1, npad, &cta, flat_fp16(desc), (uint32_t)dev.smem_optin - kStaticSmem, workspace_bytes, &sh, &tp))
+            return HUFFLLM_OK;      // records too large for this kernel's slots
         TcArgs t;
         memset(&t, 0, sizeof(t));
         KernelArgs &k = t.k;
         begin_args(&k, batch, dev);
         huffllm_status s2 = add_matrix(&k, desc, blob);
         if (s2 != HUFFLLM_OK) return s2;
-        k.part_bytes = tc_stages(tp.npad) * tp.npad * 128;      // the stages of activations
-        k.slots = 2;
-        k.pair_recip = (uint32_t)(0x100000000ull / (2ull * k.slot_bytes));
-        if (!tc_fits(desc, tp.npad, tp.tiles, flat_fp16(desc), k.dyn_smem_bytes)) return HUFFLLM_OK;   // records too large for this kernel's slots
+        set_tc_shape(&k, npad, sh);
         if (workspace_bytes < tp.bytes) {
             if (other_path_left) return HUFFLLM_OK;     // (the register path needs less)
             return fail(HUFFLLM_ERR_BUFFER_TOO_SMALL, "workspace too small for batch %u", batch);
         }
         k.m[0].x = x;
         k.m[0].y = y;
-        k.tc_npad = tp.npad;
-        k.tc_tiles = tp.tiles;
         t.m_tiles[0] = tp.m_tiles;
         t.ksplit[0] = tp.ksplit;
         t.ticket[0] = (unsigned int *)((uint8_t *)workspace + tp.ticket_off);

@@ -41,9 +41,13 @@ struct KernelArgs {
     int32_t *err;              // may be null
     // tensor-core small-batch path only
     uint32_t tc_npad;          // batch rounded up to 16, 32 or 64
-    uint32_t tc_tiles;         // 128-row tiles a CTA decodes side by side (8 warps each): 1..4
-    uint32_t tc_reserved[2];   // (the per-matrix values of that path live in TcArgs; these words keep the fields behind
-    void *tc_reserved_p[2];    //  them where the register-path kernels were measured with them)
+    uint32_t tc_tiles;         // 128-row tiles of a CTA's rows: 1..4
+    uint32_t tc_slices;        // column slices in which it decodes them side by side (8 warps per tile and slice, at most 4 in all)
+    uint32_t tc_stages;        // stages of activations and decoded weights: 2 or 3
+    uint32_t tc_row_groups;    // row groups of a CTA (its decoders in each slice)
+    uint32_t tc_reserved;
+    void *tc_reserved_p;       // (the per-matrix values of that path live in TcArgs; these words keep the fields behind
+                               //  them where the register-path kernels were measured with them)
     MatArgs m[kMaxMats];
     // (behind the matrices, so that the fields the hot loops read keep their places)
     uint32_t slots;            // slots per decoder warp: 2 (the next record lands while this one is decoded), or 1 where two would
@@ -58,8 +62,8 @@ struct TcArgs {
     KernelArgs k;
     uint32_t m_tiles[kMaxMats];        // row tiles (of the decoder warps' row groups) of matrix i
     uint32_t ksplit[kMaxMats];         // ranges its column chunks are cut into; work items = m_tiles * ksplit
-    float *partial[kMaxMats];          // [m_tiles * ksplit][32 warps][npad / 2][32]
-    unsigned int *ticket[kMaxMats];    // [m_tiles][32], zero between calls
+    float *partial[kMaxMats];          // [m_tiles * ksplit][32 warps][npad / (2 * slices)][32]
+    unsigned int *ticket[kMaxMats];    // [m_tiles][32] (several slices: [m_tiles]), zero between calls
 };
 
 cudaError_t launch_decode(const KernelArgs &k, uint32_t grid, cudaStream_t stream);

@@ -10,29 +10,44 @@
 //
 // Geometry of a CTA: 4 tiles of 8 warps; a tile is 128 rows (8 row groups of 16), warp (q = warp % 4, h = warp / 4 % 2)
 // of a tile owns tensor-memory lanes 32 q + 16 h .. + 15, which is what the 16x256b store shape of a warp can reach.
-// The CTA's LAST warp does not decode: it issues the MMAs (so a CTA decodes 31 row groups at a time, and the last 16 rows
-// of the fourth tile are never read).  Tensor memory (512 columns): 4 accumulators of N columns, then 4 tiles x S stages
-// x 32 columns of A (a stage = two blocks of 32 weight columns = four K = 16 steps; a chunk's odd last block makes a
-// stage of one block).
-// A work item is (31 row groups) x (a range of column chunks); partial results of the ranges of one row tile are
-// added in a fixed order by whoever finishes last (per-warp arrival counters, nobody waits).
+// The tiles are dealt to `tc_slices` slices of the columns (1, 2 or 4): with one slice the four tiles are four times 128
+// rows; with four they are the same 128 rows in four neighbouring column ranges, whose accumulators the epilogue adds.
+// More slices mean fewer rows per CTA and therefore fewer CTAs per row to add up in global memory: that sum is what a
+// launch over a small matrix would otherwise spend a third of its time on (a 4096 x 4096 matrix at 32 vectors: 16 column
+// ranges of 496 rows, of which the last CTA to finish read 1 MB of pieces for 9 of the launch's 27 us).  The host picks the
+// slices with the column ranges (tc_best).
+// The CTA's LAST warp does not decode: it issues the MMAs.  A CTA's rows are therefore 8 row groups per tile of a slice,
+// less one where all four tiles are in use (31, 15 or 7: the last 16 rows of a slice's last tile are never read).
+// Tensor memory (512 columns): 4 accumulators of N columns, then stages x 4 tiles x 32 columns of A (a stage = two
+// blocks of 32 weight columns = four K = 16 steps; a chunk's odd last block makes a stage of one block).
+// A work item is (the CTA's row groups) x (a range of column chunks); partial results of the ranges of one row tile are
+// added in a fixed order by whoever finishes last (arrival counters, nobody waits).
 //
-// Stage protocol: a decoder warp fills its share of stage s (A rows, a slice of B; each block into its half of the stage
-// as soon as it is decoded), arrives on the stage's "full" mbarrier and goes on decoding; no warp waits for another one except through the depth of the stage ring.  The issuer
-// warp waits for a stage to be full, issues its 16 MMAs and a tcgen05.commit onto the stage's "empty" mbarrier, which the
-// decoders wait on (with a limit) before they reuse the stage.  (With the issue taking turns among the decoder warps and a
-// barrier after every block, each block cost the CTA its decode time plus the 2000 cycles one warp needs to issue the
-// MMAs: that warp had to decode its next block before the next barrier could open.)
+// Stage protocol: a decoder warp fills its rows of stage s of A (each block into its half of the stage as soon as it is
+// decoded), arrives on the stage's "full" mbarrier and goes on decoding; no warp waits for another one except through the
+// depth of the stage ring.  The activations of a slice are brought to shared memory by a warp that does not decode (8-byte
+// cp.async, as the B operand's permuted columns want them); the issuer waits for a stage to be full, issues its MMAs and a
+// tcgen05.commit onto the stage's "empty" mbarrier, which the others wait on (with a limit) before they reuse the stage.
+// (With the issue taking turns among the decoder warps and a barrier after every block, each block cost the CTA its decode
+// time plus the 2000 cycles one warp needs to issue the MMAs: that warp had to decode its next block before the next barrier
+// could open.  With the activations carried through the first decoder warps' registers, every decoder paid for their
+// predicates, pointers and sixteen registers; with cp.async from those warps, all waited for them: a 7B-shaped layer at 32
+// vectors 153 us against 134, 8192 x 28672 at 64 vectors 159 against 142.)
 // BF16 and FP16 {1,5,5,5} blobs share the kernel (template parameter FMT): tables, raw part and operand format differ.
 #include <atomic>
+#include <type_traits>
 
 #include "decode_common.cuh"
 
 namespace huffllm {
 
-constexpr int kTcStages = 3;
+constexpr int kTcStages = 3;      // most stages; A.tc_stages are in use (shared memory is short at wide paddings and many slices)
 constexpr int kTcTiles = 4;
 
+// 8 bytes global -> shared without a register in between; the first `bytes` (0 or 8) are read, the rest is zero.
+__device__ __forceinline__ void cp_async8(uint32_t dst, const void *src, uint32_t bytes) {
+    asm volatile("cp.async.ca.shared.global [%0], [%1], 8, %2;" ::"r"(dst), "l"(src), "r"(bytes) : "memory");
+}
 __device__ __forceinline__ void tmem_alloc(uint32_t smem_dst, uint32_t ncols) {
     asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_dst), "r"(ncols) : "memory");
 }
@@ -67,6 +82,14 @@ __device__ __forceinline__ void tc_commit(uint32_t bar) {
 template <int N>
 __device__ __forceinline__ void tc_ld_32x32b(uint32_t taddr, uint32_t (&v)[N]);
 template <>
+__device__ __forceinline__ void tc_ld_32x32b<2>(uint32_t taddr, uint32_t (&v)[2]) {
+    asm volatile("tcgen05.ld.sync.aligned.32x32b.x2.b32 {%0, %1}, [%2];" : "=r"(v[0]), "=r"(v[1]) : "r"(taddr) : "memory");
+}
+template <>
+__device__ __forceinline__ void tc_ld_32x32b<4>(uint32_t taddr, uint32_t (&v)[4]) {
+    asm volatile("tcgen05.ld.sync.aligned.32x32b.x4.b32 {%0, %1, %2, %3}, [%4];" : "=r"(v[0]), "=r"(v[1]), "=r"(v[2]), "=r"(v[3]) : "r"(taddr) : "memory");
+}
+template <>
 __device__ __forceinline__ void tc_ld_32x32b<8>(uint32_t taddr, uint32_t (&v)[8]) {
     asm volatile("tcgen05.ld.sync.aligned.32x32b.x8.b32 {%0, %1, %2, %3, %4, %5, %6, %7}, [%8];"
                  : "=r"(v[0]), "=r"(v[1]), "=r"(v[2]), "=r"(v[3]), "=r"(v[4]), "=r"(v[5]), "=r"(v[6]), "=r"(v[7])
@@ -96,9 +119,14 @@ __device__ __forceinline__ void tc_ld_32x32b<32>(uint32_t taddr, uint32_t (&v)[3
 }
 
 // Shared-memory matrix descriptor of a K-major operand without swizzle: 8-row x 16-byte core matrices,
-// `lbo` bytes between core matrices along K, `sbo` bytes between 8-row groups.
-__device__ __forceinline__ uint64_t smem_desc_kmajor(uint32_t addr, uint32_t lbo, uint32_t sbo) {
-    return (uint64_t)((addr & 0x3FFFFu) >> 4) | ((uint64_t)(lbo >> 4) << 16) | ((uint64_t)(sbo >> 4) << 32) | (1ull << 46);
+// `lbo` bytes between core matrices along K, `sbo` bytes between 8-row groups.  Low word: address and lbo, in units of 16 bytes.
+__device__ __forceinline__ uint32_t smem_desc_lo(uint32_t addr, uint32_t lbo) { return ((addr & 0x3FFFFu) >> 4) | ((lbo >> 4) << 16); }
+__device__ __forceinline__ uint64_t smem_desc(uint32_t lo, uint32_t sbo) { return (uint64_t)lo | ((uint64_t)(sbo >> 4) << 32) | (1ull << 46); }
+// One thread of the (converged) warp.
+__device__ __forceinline__ bool elect_one() {
+    uint32_t p;
+    asm volatile("{\n\t.reg .pred p;\n\telect.sync _|p, 0xFFFFFFFF;\n\tselp.u32 %0, 1, 0, p;\n\t}" : "=r"(p));
+    return p != 0;
 }
 
 // LB = table index bits; NPAD = batch rounded up to 16, 32 or 64 (the MMA's N); FMT = 0: BF16 blobs, 1: FP16 {1,5,5,5} blobs, 2: FP16 blobs with flat mantissa codes
@@ -120,8 +148,7 @@ __global__ void __launch_bounds__(1024, 1) huff_gemm_tc_kernel(const __grid_cons
     constexpr int SKIP16 = FMT ? (FMT == 2 ? 3 : 1) : 0;
     constexpr int R = SKIP ? 4 : LB == 8 ? 3 : 2;
     constexpr uint32_t kIdxMask = ((1u << LB) - 1u) << 7;
-    constexpr int S = NPAD == 64 ? 2 : kTcStages;          // the host's tc_stages(): shared memory is short at the widest padding
-    constexpr uint32_t kBStage = NPAD * 128;                // bytes of B per stage: NPAD rows x 64 columns (two blocks) of bf16
+    constexpr uint32_t kBStage = NPAD * 128;                // bytes of B per slice and stage: NPAD rows x 64 columns (two blocks) of bf16
     constexpr uint32_t kLbo = 128, kSbo = 1024;             // core matrices: 8 along K side by side, then the next 8 rows
     constexpr uint32_t kACol0 = kTcTiles * NPAD;            // first tensor-memory column of the A stages
     // instruction descriptor: fp32 accumulate, bf16 x bf16, both K-major, N = NPAD, M = 128
@@ -129,9 +156,9 @@ __global__ void __launch_bounds__(1024, 1) huff_gemm_tc_kernel(const __grid_cons
 
     extern __shared__ __align__(128) uint8_t dyn_smem[];
     __shared__ __align__(8) uint64_t bars[kMaxWarps * 2];   // per warp: its two coded-copy barriers
-    __shared__ __align__(8) uint64_t empty_bar[S];          // stage may be refilled (arrived on by tcgen05.commit)
-    __shared__ __align__(8) uint64_t full_bar[S];           // every decoder warp's share of the stage is in place
-    __shared__ uint32_t s_tmem_base;
+    __shared__ __align__(8) uint64_t empty_bar[kTcStages];  // stage may be refilled (arrived on by tcgen05.commit)
+    __shared__ __align__(8) uint64_t full_bar[kTcStages];   // every decoder warp's share of the stage is in place
+    __shared__ uint32_t s_tmem_base, s_last;
 
     const uint32_t tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
     pdl_launch_dependents();   // the next kernel in the stream may be scheduled early; it waits for this one before it reads results
@@ -143,23 +170,16 @@ __global__ void __launch_bounds__(1024, 1) huff_gemm_tc_kernel(const __grid_cons
     const MatArgs &k = A.m[MULTI ? mi : 0];
     const uint32_t J = blockIdx.x - k.cta_first, n_cta = k.cta_count;
     const uint32_t smem_base = smem_u32(dyn_smem);
-    // decoder warps: eight per tile, except that the CTA's last warp never decodes: it issues the MMAs (with four tiles the
-    // last tile has seven row groups; its last 16 rows are never read).  Warps between the decoders and the issuer leave at once.
-    const uint32_t n_tiles = A.tc_tiles, n_dec = min(n_tiles * 8u, 31u), issuer = 31u;
-    const SmemPlan plan = plan_smem(smem_base, A, n_dec);
-    if (plan.warps < n_dec) {                                   // the entry point sizes shared memory so that this cannot happen
-        if (tid == 0 && A.err) atomicExch(A.err, -3);
-        return;
-    }
-    const uint32_t b_base = smem_base + A.dyn_smem_bytes - A.part_bytes;   // S stages of B behind everything else
-    uint32_t lut_lane = plan.lut | ((FMT ? lane & 15u : lane) << 2);
-    asm volatile("mov.u32 %0, %0;" : "+r"(lut_lane));
-    const uint32_t bar0 = smem_u32(&bars[warp * 2]);
-    const uint32_t slot0 = slot_addr(plan, warp, 0, A.slot_bytes);    // (this kernel always runs with two slots per warp)
-
-    // ---- roles
-    const uint32_t tile = warp >> 3, q = warp & 3, h = (warp >> 2) & 1;
-    const uint32_t rgi = tile * 8 + q * 2 + h;                              // row group of the CTA's 32 that this warp decodes
+    // `na` row tiles of `n_rg` row groups, in each of `slices` column slices.  Warp w belongs to slice w / (8 na), has row group
+    // `rgi` there and decodes if the CTA has that many.  Where all 32 warps belong to slices (four tiles) a slice's warp that does
+    // not decode carries its activations, the very last one, the issuer, only where its slice has no other; with fewer tiles
+    // (one slice) the issuer carries them and the warps between the tiles and the issuer leave at once.
+    const uint32_t S = A.tc_stages, slices = A.tc_slices, na = A.tc_tiles, tiles = na * slices, issuer = 31u;
+    const uint32_t n_rg = A.tc_row_groups, n_dec = n_rg * slices;
+    const uint32_t slice = warp == issuer ? slices - 1u : warp / (8u * na), li = warp - warp / (8u * na) * 8u * na;
+    const uint32_t tile = warp >> 3, q = warp & 3, h = (warp >> 2) & 1, rgi = (li & ~7u) + q * 2 + h;
+    const bool decodes = warp < tiles * 8u && rgi < n_rg, serves = warp != issuer && warp < tiles * 8u && rgi >= n_rg;
+    const bool issuer_carries = tiles < 4u || n_rg == na * 8u - 1u;
     const uint32_t a_lane = (32u * q + 16u * h) << 16;
     const uint32_t KC = k.col_chunks, RG = (uint32_t)((k.rows + 15) / 16);
     const uint32_t *index = (const uint32_t *)(k.blob + k.off_index);
@@ -169,12 +189,50 @@ __global__ void __launch_bounds__(1024, 1) huff_gemm_tc_kernel(const __grid_cons
         uint32_t left = (uint32_t)k.cols - kc * k.chunk_cols;
         return (min(left, k.chunk_cols) + 31u) >> 5;
     };
+    // column chunks [k0, k1) of work item `it`, and of them those of slice sl: the first slices take what does not divide
+    auto item_range = [&](uint32_t it, uint32_t &k0, uint32_t &k1) {
+        const uint32_t ks_i = it % ksplit;
+        k0 = KC * ks_i / ksplit;                            // (at most 2^26 column chunks and 16 ranges)
+        k1 = KC * (ks_i + 1) / ksplit;
+    };
+    auto slice_beg = [&](uint32_t k0, uint32_t k1, uint32_t sl) -> uint32_t { return k0 + (((k1 - k0) * sl + slices - 1) >> (slices >> 1)); };   // (1, 2, 4 slices)
+    // first and last chunk of this warp's row group in a work item (false: nothing to decode there)
+    auto item_chunks = [&](uint32_t it, uint32_t &cb, uint32_t &ce) -> bool {
+        uint32_t k0, k1;
+        item_range(it, k0, k1);
+        const uint32_t rg_i = it / ksplit * n_rg + rgi;
+        cb = rg_i * KC + slice_beg(k0, k1, slice);
+        ce = rg_i * KC + slice_beg(k0, k1, slice + 1);
+        return rg_i < RG && cb < ce;
+    };
+
+    // ---- set-up: table, barriers, tensor memory.  The offsets of the warp's first two records are asked for before anything
+    // else and their copies started between the table's loads and stores (a warp's barriers are its own, so the copies need
+    // nothing that the CTA has to meet for): the records arrive while the table is built.  (With the copies started behind
+    // the set-up a CTA's first block was decoded 7.3 us after its start; now 4.4.)
+    uint32_t cb = 0, ce = 0, o0 = 0, o1 = 0, o2 = 0;
+    bool primed = decodes && J < n_items && item_chunks(J, cb, ce);      // the item's first two record copies are under way
+    if (primed && lane == 0) {
+        o0 = __ldg(index + cb);
+        o1 = __ldg(index + cb + 1);
+        if (cb + 1 < ce) o2 = __ldg(index + cb + 2);
+    }
+    const SmemPlan plan = plan_smem(smem_base, A, n_dec);
+    if (plan.warps < n_dec) {                                   // the entry point sizes shared memory so that this cannot happen
+        if (tid == 0 && A.err) atomicExch(A.err, -3);
+        return;
+    }
+    const uint32_t b_base = smem_base + A.dyn_smem_bytes - A.part_bytes;   // the stages of B behind everything else
+    uint32_t lut_lane = plan.lut | ((FMT ? lane & 15u : lane) << 2);
+    asm volatile("mov.u32 %0, %0;" : "+r"(lut_lane));
+    const uint32_t bar0 = smem_u32(&bars[warp * 2]);
+    const uint32_t slot0 = slot_addr(plan, decodes ? slice * n_rg + rgi : 0u, 0, A.slot_bytes);    // (this kernel always runs with two slots per warp)
     auto record_ok = [&](uint32_t r0, uint32_t r1, uint32_t nkb) -> bool {
         return r1 > r0 && r1 <= k.payload_units && (r1 - r0) * 128u > raw_part(nkb) &&
                (r1 - r0) * 128u - raw_part(nkb) <= A.slot_bytes;
     };
-    auto issue_record = [&](uint32_t c, uint32_t which, uint32_t r0, uint32_t r1) {
-        uint32_t nkb = blocks_of(c % KC), bar = bar0 + which * 8;
+    auto issue_record = [&](uint32_t kc, uint32_t which, uint32_t r0, uint32_t r1) {       // kc: the chunk's column chunk
+        uint32_t nkb = blocks_of(kc), bar = bar0 + which * 8;
         if (record_ok(r0, r1, nkb)) {
             uint32_t bytes = (r1 - r0) * 128u - raw_part(nkb);
             mbar_expect_tx(bar, bytes);
@@ -183,27 +241,9 @@ __global__ void __launch_bounds__(1024, 1) huff_gemm_tc_kernel(const __grid_cons
             mbar_expect_tx(bar, 0);
         }
     };
-    auto issue = [&](uint32_t c, uint32_t which) { issue_record(c, which, __ldg(index + c), __ldg(index + c + 1)); };
-    // first and last chunk of this warp's row group in a work item (false: the row group lies outside the matrix)
-    auto item_chunks = [&](uint32_t it, uint32_t &cb, uint32_t &ce) -> bool {
-        const uint32_t mt_i = it / ksplit, ks_i = it % ksplit, rg_i = mt_i * n_dec + rgi;
-        cb = rg_i * KC + (uint32_t)((uint64_t)KC * ks_i / ksplit);
-        ce = rg_i * KC + (uint32_t)((uint64_t)KC * (ks_i + 1) / ksplit);
-        return rg_i < RG;
-    };
-
-    // ---- set-up: table, barriers, tensor memory.  The offsets of the warp's first two records are asked for before anything
-    // else and their copies started between the table's loads and stores (a warp's barriers are its own, so the copies need
-    // nothing that the CTA has to meet for): the records arrive while the table is built.  (With the copies started behind
-    // the set-up a CTA's first block was decoded 7.3 us after its start, 3.6 of them set-up.)
-    bool primed = false;                 // the item's first two record copies are under way
+    auto issue = [&](uint32_t c, uint32_t which) { issue_record(c % KC, which, __ldg(index + c), __ldg(index + c + 1)); };
     {
-        uint32_t cb = 0, ce = 0, o0 = 0, o1 = 0, o2 = 0;
-        primed = warp < n_dec && J < n_items && item_chunks(J, cb, ce);
-        if (primed && lane == 0) {
-            o0 = __ldg(index + cb);
-            o1 = __ldg(index + cb + 1);
-            if (cb + 1 < ce) o2 = __ldg(index + cb + 2);
+        if (lane == 0) {
             mbar_init(bar0, 1);
             mbar_init(bar0 + 8, 1);
         }
@@ -220,7 +260,7 @@ __global__ void __launch_bounds__(1024, 1) huff_gemm_tc_kernel(const __grid_cons
         }
         if (tid < S) {
             mbar_init(smem_u32(&empty_bar[tid]), 1);
-            mbar_init(smem_u32(&full_bar[tid]), n_dec);
+            mbar_init(smem_u32(&full_bar[tid]), n_dec + (issuer_carries ? slices - 1u : slices));
         }
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
         if (warp == issuer) {
@@ -229,12 +269,9 @@ __global__ void __launch_bounds__(1024, 1) huff_gemm_tc_kernel(const __grid_cons
         }
         if (primed && lane == 0) {
             asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
-            issue_record(cb, 0, o0, o1);
-            if (cb + 1 < ce) issue_record(cb + 1, 1, o1, o2);
-        } else if (!primed && lane == 0) {                      // (a warp without rows in the first item may have some in a later one)
-            mbar_init(bar0, 1);
-            mbar_init(bar0 + 8, 1);
-            asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+            const uint32_t kc_b = cb % KC;
+            issue_record(kc_b, 0, o0, o1);
+            if (cb + 1 < ce) issue_record(kc_b + 1, 1, o1, o2);
         }
         uint4 *lut_s = (uint4 *)(dyn_smem + (plan.lut - smem_base));
 #pragma unroll
@@ -247,7 +284,7 @@ __global__ void __launch_bounds__(1024, 1) huff_gemm_tc_kernel(const __grid_cons
     __syncthreads();
     tc_fence_after();
     const uint32_t tmem = s_tmem_base;
-    if (warp >= n_dec && warp != issuer) {   // neither decoder nor issuer in this configuration: only the teardown barrier is left
+    if (warp >= tiles * 8u && warp != issuer) {   // in no tile: only the teardown barrier is left
         tc_fence_before();
         __syncthreads();
         return;
@@ -259,7 +296,14 @@ __global__ void __launch_bounds__(1024, 1) huff_gemm_tc_kernel(const __grid_cons
 
     float *const tc_partial = T.partial[MULTI ? mi : 0];
     unsigned int *const tc_ticket = T.ticket[MULTI ? mi : 0];
-    uint32_t phase = 0, gb = 0;          // coded-copy barrier parities; blocks this CTA has gone through so far
+    uint32_t phase = 0;                  // coded-copy barrier parities
+    uint32_t st_s = 0, st_use = 0;       // the stage ring: the next stage and how often the ring has gone round
+    auto next_stage = [&]() {
+        if (++st_s == S) {
+            st_s = 0;
+            ++st_use;
+        }
+    };
     bool failed = false;                 // a wait ran out: stop waiting, keep moving, report
 
     auto bounded_wait = [&](uint32_t bar, uint32_t parity) {
@@ -275,92 +319,250 @@ __global__ void __launch_bounds__(1024, 1) huff_gemm_tc_kernel(const __grid_cons
             done = mbar_try_wait(bar, parity);
         }
     };
+    auto stage_free = [&]() {            // the stage's last MMAs are done
+        if (st_use > 0) bounded_wait(smem_u32(&empty_bar[st_s]), (st_use - 1) & 1u);
+    };
 
-    // The activations of a block are NPAD * 4 pieces of 16 bytes, 32 per warp, carried by the first warps.  A warp's
-    // piece u = 32 warp + lane belongs to vector n = u / 4 and K positions 8 kap .. 8 kap + 7 (kap = u % 4) of the
-    // tile, which hold columns base .. base + 3 and base + 8 .. base + 11 of the block, base = 16 (kap & 1) + 4 (kap >> 1).
-    const bool x_carrier = warp * 32 + lane < NPAD * 4;
-    const bool x_carrier_warp = warp * 32 < NPAD * 4;            // (NPAD * 4 is a multiple of 32: whole warps carry)
-    const uint32_t x_n = (warp * 32 + lane) >> 2, x_kap = lane & 3;
-    const uint16_t *x_src = k.x + (uint64_t)x_n * k.cols + (x_kap & 1) * 16 + (x_kap >> 1) * 4;
-    const bool x_loads = x_carrier && x_n < A.batch;         // carriers of padding vectors stage zeros
-    auto load_x = [&](uint4 &v, const uint16_t *p) {         // fetched one block ahead of its use
-        if (x_loads) {
-            uint2 lo = __ldg((const uint2 *)p), hi = __ldg((const uint2 *)(p + 8));
-            v = make_uint4(lo.x, lo.y, hi.x, hi.y);
+    // The activations of a block: vector n's K positions 8 kap .. 8 kap + 7 (kap = 0 .. 3) of the tile hold its columns
+    // base .. base + 3 and base + 8 .. base + 11 of the block, base = 16 (kap & 1) + 4 (kap >> 1), each four a copy of 8 bytes.
+    // Eight lanes take a vector's 64 bytes, a warp instruction four vectors (whole sectors are read, and four lines at a
+    // time: with four lanes to a vector it was eight).  `nblk` blocks (1 or 2) from column `col` on go to stage st_s; vectors
+    // of the padding are filled with zeros.
+    auto carry_x = [&](uint32_t col, uint32_t nblk) {
+        const uint32_t kap = (lane >> 1) & 3u, half = lane & 1u;
+        uint32_t n = lane >> 3;
+        const uint32_t dst = b_base + (st_s * slices + slice) * kBStage + kap * kLbo + n * 16u + half * 8u;
+        const uint16_t *src = k.x + (uint64_t)min(n, A.batch - 1) * k.cols + col + (kap & 1) * 16 + (kap >> 1) * 4 + half * 8;
+#pragma unroll
+        for (int i = 0; i < NPAD / 4; ++i, n += 4) {
+            const uint32_t bytes = n < A.batch ? 8u : 0u, to = dst + (i >> 1) * kSbo + (i & 1) * 64u;    // (nothing is read for 0)
+            cp_async8(to, src, bytes);
+            if (nblk > 1) cp_async8(to + 4 * kLbo, src + 32, bytes);
+            if (n + 4 < A.batch) src += 4 * k.cols;
         }
     };
-    // addresses that change only with the stage: this warp's rows of the A operand, its piece of the B slice
-    const uint32_t a_dst0 = tmem + a_lane + kACol0 + tile * S * 32;
-    const uint32_t x_dst0 = b_base + (x_n >> 3) * kSbo + x_kap * kLbo + (x_n & 7) * 16;
+    auto x_landed = [&]() {                                  // the B slice must be visible to the tensor core's reads
+        asm volatile("cp.async.wait_all;" ::: "memory");
+        asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
+        __syncwarp();
+    };
+    // this warp's rows of the A operand
+    const uint32_t a_dst0 = tmem + a_lane + kACol0 + tile * 32;
 
-    // One block of the stage protocol, decoder side.  `a` = this warp's decoded 16 rows x 32 columns (null if the warp has
-    // no rows).  The warp stores its share, says so on the stage's "full" barrier and goes on decoding: nobody waits for
+    // One block of the stage protocol, decoder side.  `a` = this warp's decoded 16 rows x 32 columns, block `half` of the
+    // stage's `nblk`.  The warp stores its share, says so on the stage's "full" barrier and goes on decoding: nobody waits for
     // the other warps here.  A warp can run ahead of the slowest one by the depth of the stage ring and no further (it
     // needs the stage back, which the issuer's tcgen05.commit announces on the "empty" barrier).
-    auto stage_block = [&](const uint32_t *a, const uint4 &xv, uint32_t half, bool publish) {
-        const uint32_t s = gb % S, use = gb / S;
+    auto stage_block = [&](const uint32_t *a, uint32_t half, uint32_t nblk) {
         if (half == 0) {
-            if (use > 0) bounded_wait(smem_u32(&empty_bar[s]), (use - 1) & 1u);
+            stage_free();
             tc_fence_after();
         }
-        if (a) {
-            // lane (g, t): row g's weights 0..3 -> 32-bit columns 2t, 2t+1; weights 4..7 -> columns 8 + 2t, 8 + 2t + 1
-            const uint32_t r[8] = {a[0], a[1], a[4], a[5], a[2], a[3], a[6], a[7]};
-            tc_st_16x256b_x2(a_dst0 + s * 32 + half * 16, r);
-        }
-        if (x_carrier)
-            asm volatile("st.shared.v4.u32 [%0], {%1, %2, %3, %4};" ::"r"(x_dst0 + s * kBStage + half * 4 * kLbo), "r"(xv.x), "r"(xv.y), "r"(xv.z), "r"(xv.w) : "memory");
-        if (!publish) return;
+        // lane (g, t): row g's weights 0..3 -> 32-bit columns 2t, 2t+1; weights 4..7 -> columns 8 + 2t, 8 + 2t + 1
+        const uint32_t r[8] = {a[0], a[1], a[4], a[5], a[2], a[3], a[6], a[7]};
+        tc_st_16x256b_x2(a_dst0 + st_s * 128 + half * 16, r);
+        if (half + 1 < nblk) return;
         tc_wait_st();
-        if (x_carrier_warp) asm volatile("fence.proxy.async.shared::cta;" ::: "memory");   // the B slice must be visible to the tensor core's reads
         tc_fence_before();
         __syncwarp();
-        if (lane == 0) mbar_arrive(smem_u32(&full_bar[s]));
-        ++gb;
+        if (lane == 0) mbar_arrive(smem_u32(&full_bar[st_s]));
+        next_stage();
     };
-    // The same block, issuer side: when every decoder warp has arrived, one lane issues the block's MMAs for every tile
-    // and commits them onto the stage's "empty" barrier.  (After a wait that ran out the commit still goes out: the
-    // stage ring keeps moving and the kernel ends with its error flag set.)
-    auto issue_block = [&](bool first_of_item, uint32_t halves) {
-        const uint32_t s = gb % S, use = gb / S;
-        bounded_wait(smem_u32(&full_bar[s]), use & 1u);
-        if (lane == 0) {
-            tc_fence_after();
-            const uint32_t bst = b_base + s * kBStage;
-            if (!failed) {
-                for (uint32_t tl = 0; tl < n_tiles; ++tl) {
+    // A stage to which this warp has nothing to add (rows outside the matrix, a slice that is done).
+    auto stage_nothing = [&]() {
+        stage_free();
+        if (lane == 0) mbar_arrive(smem_u32(&full_bar[st_s]));
+        next_stage();
+    };
+    // The same stage, issuer side: when every warp has arrived, one lane issues the stage's MMAs for every tile and commits
+    // them onto the stage's "empty" barrier.  halves(sl): blocks of slice sl in the stage.  (After a wait that ran out the
+    // commit still goes out: the stage ring keeps moving and the kernel ends with its error flag set.)
+    // What bounds this warp is the number of instructions per MMA (its scheduler has seven decoding warps to serve, so each
+    // costs some eight cycles): the thread is elected, not chosen by its number, and every operand is a base and a constant,
+    // so that addresses and descriptors are worked out on the uniform datapath, where the MMA wants them.  (28672 x 8192 at
+    // 32 vectors: 154 us with a loop over runtime strides in lane 0, 125 so; a stage's 16 MMAs take 500 to 600 cycles.)
+    auto issue_tiles = [&](auto n_slices, bool first_of_item) {                    // a stage whose slices all have two blocks
+        constexpr uint32_t SL = decltype(n_slices)::value, NA = 4u / SL;
+        const uint32_t ac = tmem + kACol0 + st_s * 128u;
+        const uint32_t bd = smem_desc_lo(b_base + st_s * SL * kBStage, kLbo);
 #pragma unroll
-                    for (uint32_t j = 0; j < 4; ++j)      // four K = 16 steps per full stage, two for the odd last block of a chunk
-                        if (j < 2 * halves)
-                            tc_mma_f16_tmem_a(tmem + tl * NPAD, tmem + kACol0 + (tl * S + s) * 32 + j * 8,
-                                              smem_desc_kmajor(bst + j * 2 * kLbo, kLbo, kSbo), kIdesc, (first_of_item && j == 0) ? 0u : 1u);
+        for (uint32_t t = 0; t < 4; ++t)
+#pragma unroll
+            for (uint32_t j = 0; j < 4; ++j)
+                tc_mma_f16_tmem_a(tmem + t * NPAD, ac + t * 32u + j * 8u, smem_desc(bd + ((t / NA * kBStage + j * 2u * kLbo) >> 4), kSbo), kIdesc,
+                                  j == 0 ? (first_of_item ? 0u : 1u) : 1u);
+    };
+    auto issue_stage = [&](bool first_of_item, bool full, auto halves) {           // full: four tiles, two blocks of every slice
+        bounded_wait(smem_u32(&full_bar[st_s]), st_use & 1u);
+        if (elect_one()) {
+            tc_fence_after();
+            if (failed) {
+            } else if (full && slices == 1u) {
+                issue_tiles(std::integral_constant<uint32_t, 1>{}, first_of_item);
+            } else if (full && slices == 2u) {
+                issue_tiles(std::integral_constant<uint32_t, 2>{}, first_of_item);
+            } else if (full) {
+                issue_tiles(std::integral_constant<uint32_t, 4>{}, first_of_item);
+            } else {
+                uint32_t ac = tmem + kACol0 + st_s * 128u;
+                for (uint32_t sl = 0; sl < slices; ++sl) {
+                    const uint32_t steps = 2 * halves(sl);                // K = 16 steps: four per full stage, two for an odd last block
+                    const uint32_t bd = smem_desc_lo(b_base + (st_s * slices + sl) * kBStage, kLbo);
+                    for (uint32_t tl = 0; tl < na; ++tl, ac += 32u)
+                        for (uint32_t j = 0; j < steps; ++j)
+                            tc_mma_f16_tmem_a(tmem + (sl * na + tl) * NPAD, ac + j * 8u, smem_desc(bd + (j * 2u * kLbo >> 4), kSbo), kIdesc,
+                                              (first_of_item && j == 0) ? 0u : 1u);
                 }
             }
-            tc_commit(smem_u32(&empty_bar[s]));
+            tc_commit(smem_u32(&empty_bar[st_s]));
         }
         __syncwarp();
-        ++gb;
+        next_stage();
+    };
+
+    // The end of a work item: the warps of a quarter of the lanes share the columns of the row tiles' accumulators; a warp adds
+    // its columns of the slices' accumulators up, in slice order, and either writes them or leaves them as the piece of its
+    // range, which the last range to arrive adds up in range order.
+    auto epilogue = [&](auto n_slices, uint32_t item, uint32_t mt, uint32_t k0, uint32_t k1) {
+        constexpr uint32_t SL = decltype(n_slices)::value;
+        constexpr int CW = NPAD / (2 * SL);
+        const uint32_t col0 = (warp >> 2) * CW, acc_tile = col0 / NPAD, n0 = col0 % NPAD;
+        float v[CW];
+#pragma unroll
+        for (uint32_t sl = 0; sl < SL; ++sl) {
+            if (sl && slice_beg(k0, k1, sl) == slice_beg(k0, k1, sl + 1)) continue;      // (no chunk: nothing was accumulated)
+            uint32_t t[CW];
+            tc_ld_32x32b<CW>(tmem + ((32u * q) << 16) + sl * (4 / SL) * NPAD + col0, t);
+            tc_wait_ld();
+#pragma unroll
+            for (int i = 0; i < CW; ++i) v[i] = sl ? v[i] + __uint_as_float(t[i]) : __uint_as_float(t[i]);
+        }
+        tc_fence_before();
+        // thread `lane` holds row 32 q + lane of the tile, columns n = n0 + i
+        const uint64_t row = (uint64_t)(mt * n_rg + acc_tile * 8) * 16 + 32u * q + lane;
+        const bool row_ok = row < k.rows && acc_tile * 8 + 2 * q + (lane >> 4) < n_rg;   // (row groups behind the CTA's belong to the next item)
+        auto write = [&](const float (&out)[CW]) {
+#pragma unroll
+            for (int i = 0; i < CW; ++i)
+                if (n0 + i < A.batch && row_ok) k.y[(uint64_t)(n0 + i) * k.rows + row] = out[i];
+        };
+        if (ksplit == 1) {
+            write(v);
+            return;
+        }
+        // piece of (item, warp): [CW][32] floats, 32 piece slots per item
+        float *piece = tc_partial + ((size_t)item * 32 + warp) * CW * 32;
+#pragma unroll
+        for (int i = 0; i < CW; ++i) piece[i * 32 + lane] = v[i];
+        __syncwarp();
+        uint32_t last = 0;
+        if (SL == 1) {                                       // every warp finds its own pieces: a counter per row tile and warp
+            if (lane == 0) {
+                unsigned int *ctr = tc_ticket + mt * 32 + warp;
+                last = arrive_acq_rel(ctr) == ksplit - 1 ? 1u : 0u;
+                if (last) *ctr = 0;
+            }
+            last = __shfl_sync(0xFFFFFFFFu, last, 0);
+        } else {                                             // small pieces: one counter per row tile (all 32 warps are here)
+            __syncthreads();
+            if (tid == 0) {
+                unsigned int *ctr = tc_ticket + mt;
+                s_last = arrive_acq_rel(ctr) == ksplit - 1 ? 1u : 0u;
+                if (s_last) *ctr = 0;
+            }
+            __syncthreads();
+            last = s_last;
+        }
+        if (!last) return;
+        // 32 independent loads in flight: every column of as many ranges as make 32; every output adds its pieces in range order
+        constexpr int U = CW >= 32 ? 1 : 32 / CW;
+        constexpr size_t kRange = (size_t)32 * CW * 32;
+        const float *pc = tc_partial + ((size_t)mt * ksplit * 32 + warp) * CW * 32 + lane;
+#pragma unroll
+        for (int i = 0; i < CW; ++i) v[i] = 0.f;
+        uint32_t r = 0;
+#pragma unroll 1
+        for (; r + U <= ksplit; r += U, pc += U * kRange) {
+            float p[U][CW];
+#pragma unroll
+            for (int u = 0; u < U; ++u)
+#pragma unroll
+                for (int i = 0; i < CW; ++i) p[u][i] = __ldcg(pc + u * kRange + i * 32);
+#pragma unroll
+            for (int u = 0; u < U; ++u)
+#pragma unroll
+                for (int i = 0; i < CW; ++i) v[i] += p[u][i];
+        }
+#pragma unroll 1
+        for (; r < ksplit; ++r, pc += kRange)
+#pragma unroll
+            for (int i = 0; i < CW; ++i) v[i] += __ldcg(pc + i * 32);
+        write(v);
     };
 
 #pragma unroll 1
     for (uint32_t item = J; item < n_items; item += n_cta) {
-        const uint32_t mt = item / ksplit, ks = item % ksplit;
-        const uint32_t rg = mt * n_dec + rgi;
-        const bool active = rg < RG;
-        const uint32_t kc0 = (uint32_t)((uint64_t)KC * ks / ksplit), kc1 = (uint32_t)((uint64_t)KC * (ks + 1) / ksplit);
-        const uint32_t gb_item = gb;
-        // the item's blocks are consecutive 32-column blocks of the matrix, from col_lo up to col_hi
-        const uint32_t col_lo = kc0 * k.chunk_cols, col_hi = min(kc1 * k.chunk_cols, (uint32_t)k.cols);
-        // activations: x_a holds the current block's piece at the top of every chunk; the pointer names the block after it
-        const uint16_t *x_p = x_src + col_lo + 32, *const x_end = x_src + col_hi;
-        uint4 x_a = make_uint4(0, 0, 0, 0), x_b = make_uint4(0, 0, 0, 0);
-        load_x(x_a, x_src + col_lo);
+        const uint32_t mt = item / ksplit;
+        uint32_t k0, k1;
+        item_range(item, k0, k1);
+        const uint32_t kc0 = slice_beg(k0, k1, slice), kc1 = slice_beg(k0, k1, slice + 1);
+        const uint32_t rg = mt * n_rg + rgi;
+        const bool active = decodes && rg < RG && kc0 < kc1;
+        // The slices go through their chunks side by side: a chunk's stages (pairs of blocks), `steps` times.  (One slice: the
+        // stages of the chunk at hand; several: those of a full chunk, some of which the row's last chunk leaves empty.)
+        const uint32_t steps = slice_beg(k0, k1, 1) - k0, full_stages = (k.chunk_cols / 32u + 1u) >> 1;
+        const uint32_t col_lo = kc0 * k.chunk_cols;         // the slice's first column
+        // blocks of the chunk that slice sl has in step j, and of those in the stage that holds its pair p
+        auto step_blocks = [&](uint32_t sl, uint32_t j) -> uint32_t {
+            const uint32_t kc = slice_beg(k0, k1, sl) + j;
+            return kc < slice_beg(k0, k1, sl + 1) ? blocks_of(kc) : 0u;
+        };
+        auto halves = [](uint32_t nkb, uint32_t p) -> uint32_t { return nkb > 2 * p ? min(nkb - 2 * p, 2u) : 0u; };
+        auto stages_of = [&](uint32_t j) -> uint32_t { return slices == 1u ? (blocks_of(k0 + j) + 1u) >> 1 : full_stages; };
 
         if (warp == issuer) {
-            for (uint32_t kc = kc0; kc < kc1; ++kc) {       // stages are cut like the decoders': pairs of blocks inside a chunk
-                const uint32_t nkb = blocks_of(kc);
-                for (uint32_t kb = 0; kb < nkb; kb += 2) issue_block(gb == gb_item, min(nkb - kb, 2u));
+            // the activations of the stage behind the one at hand are always under way
+            uint32_t own = step_blocks(slice, 0);           // blocks of the carried slice in the step at hand
+            if (issuer_carries) {
+                stage_free();
+                if (own) carry_x(col_lo, min(own, 2u));
+            }
+            for (uint32_t j = 0; j < steps; ++j) {          // stages are cut like the decoders': pairs of blocks inside a chunk
+                const uint32_t n_st = stages_of(j);
+                uint32_t nkb[4], least = ~0u;               // blocks of every slice in this step, and the fewest
+#pragma unroll
+                for (uint32_t sl = 0; sl < 4; ++sl) {
+                    nkb[sl] = sl < slices ? step_blocks(sl, j) : 0u;
+                    if (sl < slices) least = min(least, nkb[sl]);
+                }
+                for (uint32_t p = 0; p < n_st; ++p) {
+                    if (issuer_carries) x_landed();
+                    issue_stage(j == 0 && p == 0, tiles == 4u && least >= 2 * p + 2, [&](uint32_t sl) -> uint32_t {
+                        return halves(sl == 0 ? nkb[0] : sl == 1 ? nkb[1] : sl == 2 ? nkb[2] : nkb[3], p);
+                    });
+                    if (!issuer_carries) continue;
+                    uint32_t p2 = p + 1;
+                    if (p2 == n_st) {
+                        if (j + 1 == steps) break;
+                        own = step_blocks(slice, j + 1);
+                        p2 = 0;
+                    }
+                    stage_free();
+                    const uint32_t n2 = halves(own, p2);
+                    if (n2) carry_x(col_lo + (p2 ? j : j + 1) * k.chunk_cols + p2 * 64u, n2);
+                }
+            }
+        } else if (serves) {
+            for (uint32_t j = 0; j < steps; ++j) {
+                const uint32_t own = step_blocks(slice, j), n_st = stages_of(j);
+                for (uint32_t p = 0; p < n_st; ++p) {
+                    stage_free();
+                    const uint32_t n2 = halves(own, p);
+                    if (n2) carry_x(col_lo + j * k.chunk_cols + p * 64u, n2);
+                    x_landed();
+                    if (lane == 0) mbar_arrive(smem_u32(&full_bar[st_s]));
+                    next_stage();
+                }
             }
         } else if (active) {
             const uint32_t c_beg = rg * KC + kc0, c_end = rg * KC + kc1;
@@ -369,81 +571,76 @@ __global__ void __launch_bounds__(1024, 1) huff_gemm_tc_kernel(const __grid_cons
                 if (c_beg + 1 < c_end) issue(c_beg + 1, 1);
             }
             uint32_t kc = kc0;
-            uint32_t r0 = __ldg(index + c_beg), r1 = __ldg(index + c_beg + 1);
+            // record offsets are known two chunks ahead, the first raw block of a record is asked for in the last block of the
+            // one before: a chunk's start waits for neither
+            uint32_t r0 = __ldg(index + c_beg), r1 = __ldg(index + c_beg + 1), r2 = c_beg + 1 < c_end ? __ldg(index + c_beg + 2) : r1;
+            bool raw_there = false;
+            const uint8_t *raw_p = payload;
+            uint4 raw_cur = make_uint4(0, 0, 0, 0), raw_b = make_uint4(0, 0, 0, 0);
 #pragma unroll 1
             for (uint32_t c = c_beg; c < c_end; ++c, ++kc) {
                 const uint32_t which = (c - c_beg) & 1u;
                 const uint32_t nkb = blocks_of(kc);
-                const bool ok = record_ok(r0, r1, nkb);
-                const uint32_t r2 = c + 1 < c_end ? __ldg(index + c + 2) : r1;
-                const uint8_t *raw_p = payload + (uint64_t)r0 * 128u + lane * kRawLane;
-                uint4 raw_cur = make_uint4(0, 0, 0, 0);
-                if (ok) raw_cur = load_raw(raw_p);
+                const bool ok = record_ok(r0, r1, nkb), has_next = c + 1 < c_end;
+                const uint32_t r3 = c + 2 < c_end ? __ldg(index + c + 3) : r2;
+                if (ok && !raw_there) {
+                    raw_p = payload + (uint64_t)r0 * 128u + lane * kRawLane;
+                    raw_cur = load_raw(raw_p);
+                }
                 bounded_wait(bar0 + which * 8, (phase >> which) & 1u);
                 phase ^= 1u << which;
                 if (!ok && A.err && lane == 0) atomicExch(A.err, (int32_t)min(c + 1, 0x7FFFFFFFu));
                 if (!ok) {
                     // record offsets out of range (reported above): nothing of the record is touched, zeros go to the stages
                     const uint32_t zero[8] = {0u, 0u, 0u, 0u, 0u, 0u, 0u, 0u};
-                    for (uint32_t kb = 0; kb < nkb; ++kb) {
-                        if (x_p < x_end) load_x(x_b, x_p);
-                        x_p += 32;
-                        stage_block(zero, x_a, kb & 1u, (kb & 1u) || kb + 1 == nkb);
-                        x_a = x_b;
-                    }
-                    __syncwarp();
-                    if (lane == 0 && c + 2 < c_end) issue(c + 2, which);
-                    r0 = r1;
-                    r1 = r2;
-                    continue;
-                }
-                LaneStream sa, sb;
-                stream_open(sa, slot0 + which * A.slot_bytes + (lane << 2), SKIP ? 7u : SKIP16 ? 6u : 0u);
-                stream_open(sb, slot0 + which * A.slot_bytes + 128u + (lane << 2), SKIP ? 7u : SKIP16 ? 6u : 0u);
-                // one block: fetch the next block's raw bytes and activations into the other register set, decode
-                // this one, hand it to the tensor core
-                auto block = [&](const uint4 &raw_c, uint4 &raw_n, const uint4 &x_c, uint4 &x_n2, bool more, uint32_t half, bool publish) {
-                    raw_p += kRawBlock;
-                    if (more) raw_n = load_raw(raw_p);
-                    if (x_p < x_end) load_x(x_n2, x_p);
-                    x_p += 32;
-                    uint32_t a[8];
-                    if (FMT) decode_block_fp16<false, SKIP16>(sa, sb, lut_lane, raw_c.x, a);
-                    else decode_block<R, SKIP>(sa, sb, kIdxMask, lut_lane, raw_c, a);
-                    stage_block(a, x_c, half, publish);
-                };
-                uint4 raw_b = make_uint4(0, 0, 0, 0);
-                uint32_t kb = 0;
+                    for (uint32_t kb = 0; kb < nkb; ++kb) stage_block(zero, kb & 1u, (kb & 1u) || kb + 1 < nkb ? 2u : 1u);
+                    raw_there = false;
+                } else {
+                    LaneStream sa, sb;
+                    stream_open(sa, slot0 + which * A.slot_bytes + (lane << 2), SKIP ? 7u : SKIP16 ? 6u : 0u);
+                    stream_open(sb, slot0 + which * A.slot_bytes + 128u + (lane << 2), SKIP ? 7u : SKIP16 ? 6u : 0u);
+                    // one block: fetch the next block's raw bytes into the other register set (behind the record's last one: the
+                    // next record's first, an address inside the blob whatever its offsets turn out to be), decode this one, hand
+                    // it to the tensor core
+                    auto block = [&](const uint4 &raw_c, uint4 &raw_n, bool last, uint32_t half, uint32_t nblk) {
+                        raw_p += kRawBlock;
+                        if (last) raw_p = payload + (uint64_t)r1 * 128u + lane * kRawLane;
+                        if (!last || has_next) raw_n = load_raw(raw_p);
+                        uint32_t a[8];
+                        if (FMT) decode_block_fp16<false, SKIP16>(sa, sb, lut_lane, raw_c.x, a);
+                        else decode_block<R, SKIP>(sa, sb, kIdxMask, lut_lane, raw_c, a);
+                        stage_block(a, half, nblk);
+                    };
+                    uint32_t kb = 0;
 #pragma unroll 1
-                for (; kb + 2 <= nkb; kb += 2) {                  // the usual case: pairs of blocks, two register sets in turn
-                    block(raw_cur, raw_b, x_a, x_b, true, 0, false);
-                    block(raw_b, raw_cur, x_b, x_a, kb + 2 < nkb, 1, true);
+                    for (; kb + 2 <= nkb; kb += 2) {                  // the usual case: pairs of blocks, two register sets in turn
+                        block(raw_cur, raw_b, false, 0, 2);
+                        block(raw_b, raw_cur, kb + 2 == nkb, 1, 2);
+                    }
+                    if (kb < nkb) {                                   // odd block count (a ragged last chunk): a stage of one block
+                        block(raw_cur, raw_b, true, 0, 1);
+                        raw_cur = raw_b;
+                    }
+                    raw_there = has_next;
                 }
-                if (kb < nkb) {                                   // odd block count (a ragged last chunk): a stage of one block
-                    block(raw_cur, raw_b, x_a, x_b, false, 0, true);
-                    x_a = x_b;
-                }
+                if (slices > 1u)
+                    for (uint32_t p = (nkb + 1u) >> 1; p < full_stages; ++p) stage_nothing();
                 __syncwarp();
-                if (lane == 0 && c + 2 < c_end) issue(c + 2, which);
+                if (lane == 0 && c + 2 < c_end) issue_record(kc + 2, which, r2, r3);
                 r0 = r1;
                 r1 = r2;
+                r2 = r3;
             }
+            for (uint32_t j = kc1 - kc0; j < steps; ++j)    // steps in which only other slices have a chunk
+                for (uint32_t p = 0; p < full_stages; ++p) stage_nothing();
         } else {
-            // no rows of the matrix for this warp: it still carries its slice of the activations and its arrivals
-            for (uint32_t kc = kc0; kc < kc1; ++kc) {
-                const uint32_t nkb = blocks_of(kc);
-                for (uint32_t kb = 0; kb < nkb; ++kb) {
-                    if (x_p < x_end) load_x(x_b, x_p);
-                    x_p += 32;
-                    stage_block(nullptr, x_a, kb & 1u, (kb & 1u) || kb + 1 == nkb);
-                    x_a = x_b;
-                }
-            }
+            for (uint32_t j = 0; j < steps; ++j)            // nothing to decode for this warp: its arrivals are still waited for
+                for (uint32_t p = stages_of(j); p; --p) stage_nothing();
         }
 
         // both slots are free again: the next item's first records are asked for now, so that they arrive behind the epilogue
         primed = false;
-        if (warp < n_dec && item + n_cta < n_items) {
+        if (decodes && item + n_cta < n_items) {
             uint32_t nb, ne;
             if (item_chunks(item + n_cta, nb, ne)) {
                 if (lane == 0) {
@@ -454,51 +651,15 @@ __global__ void __launch_bounds__(1024, 1) huff_gemm_tc_kernel(const __grid_cons
             }
         }
 
-        // ---- epilogue of the item: wait for the last stage's MMAs, read this warp's 32 rows x NPAD/2 columns
-        // (the issuer has a share like every warp of a tile; with fewer than four tiles its tile does not exist)
-        if (tile < n_tiles) {
-            const uint32_t gl = gb - 1;
-            bounded_wait(smem_u32(&empty_bar[gl % S]), (gl / S) & 1u);
+        // wait for the last stage's MMAs.  (The issuer has a share in the epilogue like every warp; with fewer than four tiles
+        // only the tiles' warps have one.)
+        if (warp < tiles * 8u) {
+            const uint32_t ls = st_s == 0 ? S - 1u : st_s - 1u, lu = st_s == 0 ? st_use - 1u : st_use;
+            bounded_wait(smem_u32(&empty_bar[ls]), lu & 1u);
             tc_fence_after();
-            uint32_t v[NPAD / 2];
-            tc_ld_32x32b<NPAD / 2>(tmem + ((32u * q) << 16) + tile * NPAD + h * (NPAD / 2), v);
-            tc_wait_ld();
-            tc_fence_before();
-            // thread `lane` holds row 32 q + lane of the tile, columns n = h * NPAD/2 + i
-            const uint64_t row = (uint64_t)(mt * n_dec + tile * 8) * 16 + 32u * q + lane;
-            const bool row_ok = row < k.rows && tile * 8 + 2 * q + (lane >> 4) < n_dec;   // (the last tile's last row group belongs to the next item)
-            const uint32_t n0 = h * (NPAD / 2);
-            if (ksplit == 1) {
-#pragma unroll
-                for (int i = 0; i < NPAD / 2; ++i)
-                    if (n0 + i < A.batch && row_ok) k.y[(uint64_t)(n0 + i) * k.rows + row] = __uint_as_float(v[i]);
-            } else {
-                // piece of (item, warp): [NPAD/2][32] floats; the last range to arrive adds the pieces in range order
-                float *piece = tc_partial + ((size_t)item * 32 + warp) * (NPAD / 2) * 32;   // 32 piece slots per item, n_dec used
-#pragma unroll
-                for (int i = 0; i < NPAD / 2; ++i) piece[i * 32 + lane] = __uint_as_float(v[i]);
-                __syncwarp();
-                uint32_t last = 0;
-                if (lane == 0) {
-                    unsigned int *ctr = tc_ticket + mt * 32 + warp;
-                    last = arrive_acq_rel(ctr) == ksplit - 1 ? 1u : 0u;
-                    if (last) *ctr = 0;
-                }
-                if (__shfl_sync(0xFFFFFFFFu, last, 0)) {
-                    // range after range, NPAD/2 independent loads in flight each time; every output adds its pieces in range order
-                    float sum[NPAD / 2];
-#pragma unroll
-                    for (int i = 0; i < NPAD / 2; ++i) sum[i] = 0.f;
-                    for (uint32_t s2 = 0; s2 < ksplit; ++s2) {
-                        const float *pc = tc_partial + ((size_t)(mt * ksplit + s2) * 32 + warp) * (NPAD / 2) * 32 + lane;
-#pragma unroll
-                        for (int i = 0; i < NPAD / 2; ++i) sum[i] += __ldcg(pc + i * 32);
-                    }
-#pragma unroll
-                    for (int i = 0; i < NPAD / 2; ++i)
-                        if (n0 + i < A.batch && row_ok) k.y[(uint64_t)(n0 + i) * k.rows + row] = sum[i];
-                }
-            }
+            if (slices == 1u) epilogue(std::integral_constant<uint32_t, 1>{}, item, mt, k0, k1);
+            else if (slices == 2u) epilogue(std::integral_constant<uint32_t, 2>{}, item, mt, k0, k1);
+            else epilogue(std::integral_constant<uint32_t, 4>{}, item, mt, k0, k1);
         }
     }
 

@@ -378,29 +378,49 @@ def test_code_length_limits_accepted_per_format():
         assert e.value.status_name == "UNSUPPORTED"
 
 
-def test_column_ranges_finish_first_among_all_simulated():
-    """The tensor-core path's column ranges (seen through the workspace they need) are those of a walk over every work item."""
+@pytest.mark.parametrize("batch,npad", [(64, 64), (20, 32), (9, 16)])
+def test_column_ranges_finish_first_among_all_simulated(batch, npad):
+    """The tensor-core path's shape and column ranges (seen through the workspace they need) are those of a walk over every work item."""
     import random
     w = wl.gaussian_weights(16, 1024, 0.02, 1)
     cb = hl.build_codebook(w)
-    _, d = hl.encode(cb, w, 2048)
+    _, d = hl.encode(cb, w, 2048)                               # (records small enough for every shape)
     cb.free()
     rng = random.Random(3)
-    for rows, cols in [(64, 128), (4096, 4096), (28672, 8192), (8192, 28672), (1024, 14336)] + \
+    seen = set()
+    for rows, cols in [(64, 128), (4096, 4096), (28672, 8192), (8192, 28672), (1024, 14336), (300, 28672)] + \
                       [(rng.randrange(1, 30000), 32 * rng.randrange(1, 900)) for _ in range(60)]:
         d.rows, d.cols, d.row_groups = rows, cols, (rows + 15) // 16
         d.col_chunks = (cols + d.chunk_cols - 1) // d.chunk_cols
         d.n_chunks = d.row_groups * d.col_chunks
         d.off_payload = (d.off_index + 4 * (d.n_chunks + 1) + 255) // 256 * 256
         d.payload_bytes, d.blob_bytes = 128 * d.n_chunks, d.off_payload + 128 * d.n_chunks + 4096
-        m_tiles, best, best_span = (d.row_groups + 30) // 31, 1, None
-        for ks in range(1, min(16, d.col_chunks) + 1):
-            items = m_tiles * ks
-            grid = min(items, 148)
-            cost = [(d.col_chunks * (r + 1) // ks - d.col_chunks * r // ks) * (d.chunk_cols // 32) + 5 for r in range(ks)]
-            span = max(sum(cost[i % ks] for i in range(b, items, grid)) for b in range(grid))
-            if best_span is None or span < best_span:
-                best, best_span = ks, span
-        tc = 4096 + ((d.row_groups + 7) // 8 * 128 + 255) // 256 * 256 + (m_tiles * best * 32 * 32 * 32 * 4 if best > 1 else 0)
-        two_tiles = 4096 + ((d.row_groups + 7) // 8 * 128 + 255) // 256 * 256 + 512 * (2 + 64) * 16 * 16 * 4
-        assert hl.workspace_bytes(d, 64) == max(tc, two_tiles), (rows, cols)
+        best, most = None, None
+        for which, slices, groups, block in ((0, 1, 31, 32), (1, 1, 30, 32), (2, 2, 15, 34), (3, 4, 7, 39)):
+            if (which == 1 and npad != 64) or (which == 3 and npad == 64):
+                continue
+            m_tiles, cw, plan = (d.row_groups + groups - 1) // groups, npad // (2 * slices), None
+            for ks in range(1, min(16, d.col_chunks) + 1):
+                items = m_tiles * ks
+                grid = min(items, 148)
+                parts = [d.col_chunks * (r + 1) // ks - d.col_chunks * r // ks for r in range(ks)]
+                if which and -(-max(parts) // slices) > most:
+                    continue
+                cost = [-(-n // slices) * (d.chunk_cols // 32) * block + 160 for n in parts]
+                sums = 2 * ks * cw if ks > 1 else 0
+                span = max(sum(cost[i % ks] for i in range(b, items, grid)) for b in range(grid)) + (sums if which else 0)
+                if plan is None or span < plan[0]:
+                    plan = (span, ks, sums, max(parts))
+            if plan is None:
+                continue
+            if which == 0:
+                most = plan[3]
+                plan = ((plan[0] * 9 // 8 if npad == 64 else plan[0]) + plan[2],) + plan[1:]
+            if best is None or plan[0] < best[0]:
+                best = (plan[0], which, m_tiles * plan[1], plan[1], cw)
+        seen.add(best[1])
+        ctrl = 4096 + ((d.row_groups + 7) // 8 * 128 + 255) // 256 * 256
+        tc = ctrl + (best[2] * 32 * best[4] * 32 * 4 if best[3] > 1 else 0)
+        two_tiles = ctrl + 512 * (2 + 64) * 16 * min(batch, 16) * 4
+        assert hl.workspace_bytes(d, batch) == max(tc, two_tiles), (rows, cols, best)
+    assert seen >= ({0, 1, 2} if npad == 64 else {0, 2, 3})
