@@ -220,7 +220,7 @@ huffllm_status huffllm_validate_blob(const void *blob_host, size_t bytes, huffll
 /* --------------------------------------------------------- device: decode, and decode fused with products */
 
 /*
- * Scratch bytes the fused products need for this matrix and `batch` activation vectors.  The workspace must be
+ * Scratch bytes the fused products need for this matrix and `batch` activation vectors, or fewer.  The workspace must be
  * zero-filled once after allocation.  Its first huffllm_workspace_control_bytes(desc) bytes are arrival counters:
  * every call that completes leaves them zero again; the rest holds partial sums and is overwritten freely.
  * After a call that set the error flag, clear those leading bytes before the workspace is used again.
@@ -262,6 +262,18 @@ huffllm_status huffllm_decode_smem_plan(const huffllm_desc *desc, uint32_t *tabl
  */
 huffllm_status huffllm_decode_launch_plan(const huffllm_desc *desc, uint32_t batch, uint32_t smem_bytes_per_cta,
                                           uint32_t *slots_per_warp, uint32_t *decoder_warps);
+
+/*
+ * How the tensor-core kernel would work through a product of `batch` (9..64) vectors with these n matrices in one launch (host
+ * call, no device needed; the B200's figures without one; any output may be null).  `workspace_bytes_each` as in the product
+ * calls, 0 = no limit.  column_slices: column ranges a CTA decodes side by side; row_groups: groups of 16 rows a CTA works on;
+ * per matrix (arrays of n): ranges its column chunks are cut into, work items (row tiles times ranges), and the most column
+ * chunks one fp32 accumulator adds up (one matrix: the same in every workspace of at least huffllm_workspace_bytes).
+ * (Blobs of 9..16 vectors may take the register path instead.)  HUFFLLM_ERR_UNSUPPORTED if the kernel does not take these blobs.
+ */
+huffllm_status huffllm_gemm_launch_plan(uint32_t n, const huffllm_desc *const *descs, uint32_t batch, size_t workspace_bytes_each,
+                                        uint32_t *column_slices, uint32_t *row_groups, uint32_t *ranges, uint32_t *work_items,
+                                        uint32_t *chunks_per_sum);
 
 /*
  * y = W x with W taken straight from the compressed blob: weights are decoded in registers and

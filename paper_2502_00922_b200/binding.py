@@ -49,6 +49,7 @@ _SIGNATURES = {
     "huffllm_workspace_control_bytes": [C.POINTER(Desc), C.POINTER(C.c_size_t)],
     "huffllm_decode_smem_plan": [C.POINTER(Desc), C.POINTER(C.c_uint32), C.POINTER(C.c_uint32), C.POINTER(C.c_uint32), C.POINTER(C.c_uint32)],
     "huffllm_decode_launch_plan": [C.POINTER(Desc), C.c_uint32, C.c_uint32, C.POINTER(C.c_uint32), C.POINTER(C.c_uint32)],
+    "huffllm_gemm_launch_plan": [C.c_uint32, C.c_void_p, C.c_uint32, C.c_size_t, C.c_void_p, C.c_void_p, C.c_void_p, C.c_void_p, C.c_void_p],
     "huffllm_decode": [C.POINTER(Desc), C.c_void_p, C.c_void_p, C.c_void_p, C.c_void_p],
     "huffllm_decode_gemv": [C.POINTER(Desc), C.c_void_p, C.c_void_p, C.c_void_p, C.c_void_p, C.c_size_t, C.c_void_p, C.c_void_p],
     "huffllm_decode_gemm": [C.POINTER(Desc), C.c_void_p, C.c_void_p, C.c_uint32, C.c_void_p, C.c_void_p, C.c_size_t, C.c_void_p, C.c_void_p],
@@ -219,6 +220,16 @@ def decode_launch_plan(desc: Desc, batch: int = 1, smem_bytes_per_cta: int = 0) 
     s, w = C.c_uint32(), C.c_uint32()
     _check(lib().huffllm_decode_launch_plan(C.byref(desc), batch, smem_bytes_per_cta, C.byref(s), C.byref(w)))
     return {"slots_per_warp": s.value, "decoder_warps": w.value}
+
+
+def gemm_launch_plan(descs, batch: int, workspace_bytes_each: int = 0) -> dict:
+    """huffllm_gemm_launch_plan: the tensor-core kernel's shape, and per matrix its column ranges, work items and chunks per sum."""
+    n = len(descs)
+    desc_arr = (C.POINTER(Desc) * n)(*[C.pointer(d) for d in descs])
+    sl, rg = C.c_uint32(), C.c_uint32()
+    ranges, items, chunks = (C.c_uint32 * n)(), (C.c_uint32 * n)(), (C.c_uint32 * n)()
+    _check(lib().huffllm_gemm_launch_plan(n, desc_arr, batch, workspace_bytes_each, C.byref(sl), C.byref(rg), ranges, items, chunks))
+    return {"column_slices": sl.value, "row_groups": rg.value, "ranges": list(ranges), "work_items": list(items), "chunks_per_sum": list(chunks)}
 
 
 def decode(desc: Desc, blob_dev, out_dev, err_flag_dev=None, stream=None):

@@ -246,30 +246,39 @@ TcPlan tc_plan(const huffllm_desc *d, uint32_t npad, uint32_t sms, const TcShape
     p.bytes = p.partial_off + (best > 1 ? p.items * item_bytes : 0);
     return p;
 }
-// The shape and plans of a launch over n matrices with cta[i] CTAs each: the shape whose slowest matrix is done first.  False: no
-// shape fits.
+// The shape and plans of a launch over n matrices with cta[i] CTAs each: the shape whose slowest matrix is done first among those
+// whose plans fit `max_bytes` of workspace.  No accumulator may add up more columns than in shape 0 without a limit on the
+// workspace: what a caller hands over as workspace decides about time, not about rounding.  (With the limit taken from a shape-0
+// plan that the workspace had already cut, 28672 x 4096 at 64 vectors in a workspace of exactly the size asked for added up 2048
+// columns instead of 1024.)  Only where no plan of any shape is within both, the cut shape-0 plan is the measure.
+// False: no shape fits.
 bool tc_best(const huffllm_desc *const *d, uint32_t n, uint32_t npad, const uint32_t *cta, bool flat, uint32_t dyn_smem, size_t max_bytes,
              TcShape *shape, TcPlan *plans) {
-    uint64_t best_span = ~0ull;
-    uint32_t most[kMaxMats];
-    for (uint32_t i = 0; i < n; ++i) most[i] = ~0u;
-    for (uint32_t which = 0; which < kTcShapes; ++which) {
-        TcShape sh;
-        if (!tc_shape(d, n, npad, which, flat, dyn_smem, &sh)) continue;
-        TcPlan p[kMaxMats];
-        uint64_t span = 0;
-        for (uint32_t i = 0; i < n; ++i) {
-            p[i] = tc_plan(d[i], npad, cta[i], sh, max_bytes, most[i]);
-            if (p[i].span > span) span = p[i].span;
-            if (which == 0) most[i] = p[i].chunks;
+    TcShape base;
+    if (!tc_shape(d, n, npad, 0, flat, dyn_smem, &base)) return false;
+    for (size_t base_bytes = ~(size_t)0;; base_bytes = max_bytes) {
+        uint64_t best_span = ~0ull;
+        uint32_t most[kMaxMats];
+        for (uint32_t which = 0; which < kTcShapes; ++which) {
+            TcShape sh = base;
+            if (which && !tc_shape(d, n, npad, which, flat, dyn_smem, &sh)) continue;
+            TcPlan p[kMaxMats];
+            uint64_t span = 0;
+            for (uint32_t i = 0; i < n; ++i) {
+                p[i] = tc_plan(d[i], npad, cta[i], sh, which ? max_bytes : base_bytes, which ? most[i] : ~0u);
+                const uint64_t t = p[i].bytes > max_bytes ? ~0ull : p[i].span;
+                if (t > span) span = t;
+                if (which == 0) most[i] = p[i].chunks;
+            }
+            if (span < best_span) {
+                best_span = span;
+                *shape = sh;
+                for (uint32_t i = 0; i < n; ++i) plans[i] = p[i];
+            }
         }
-        if (span < best_span) {
-            best_span = span;
-            *shape = sh;
-            for (uint32_t i = 0; i < n; ++i) plans[i] = p[i];
-        }
+        if (best_span != ~0ull) return true;
+        if (base_bytes == max_bytes) return false;
     }
-    return best_span != ~0ull;
 }
 
 // Bytes of the FP16 tables a launch keeps in shared memory: three sixteen-fold tables of 8-bit codes, or the exponent's
@@ -408,12 +417,19 @@ huffllm_status huffllm_workspace_bytes(const huffllm_desc *desc, uint32_t batch,
         clear_error();
         const int sms = have ? dev.sms : 148;
         const uint32_t dyn = (have ? (uint32_t)dev.smem_optin : 232448u) - kStaticSmem;
-        for (uint32_t flat = 0; flat < (flat_fp16(desc) ? 2u : 1u); ++flat) {      // (with all three FP16 tables, and with one)
-            const uint32_t cta = (uint32_t)sms;
-            TcShape sh;
-            TcPlan p;
-            if (tc_best(&desc, 1, tc_npad_of(batch), &cta, flat != 0, dyn, ~(size_t)0, &sh, &p) && p.bytes > *bytes) *bytes = p.bytes;
-        }
+        const uint32_t cta = (uint32_t)sms;
+        // The plan that will run for this and for every smaller batch, and the shape-0 plan, which a launch over several matrices
+        // may fall back on; with all three FP16 tables, and with one.
+        for (uint32_t npad = 16; npad <= tc_npad_of(batch); npad *= 2)
+            for (uint32_t flat = 0; flat < (flat_fp16(desc) ? 2u : 1u); ++flat) {
+                TcShape sh;
+                TcPlan p;
+                if (!tc_best(&desc, 1, npad, &cta, flat != 0, dyn, ~(size_t)0, &sh, &p)) continue;
+                if (p.bytes > *bytes) *bytes = p.bytes;
+                if (!tc_shape(&desc, 1, npad, 0, flat != 0, dyn, &sh)) continue;
+                p = tc_plan(desc, npad, cta, sh, ~(size_t)0, ~0u);
+                if (p.bytes > *bytes) *bytes = p.bytes;
+            }
     }
     return HUFFLLM_OK;
 }
@@ -456,6 +472,43 @@ huffllm_status huffllm_decode_launch_plan(const huffllm_desc *desc, uint32_t bat
     if ((st = finish_args(&k, batch != 0, dev, &grid, &warps)) != HUFFLLM_OK) return st;
     if (slots_per_warp) *slots_per_warp = k.slots;
     if (decoder_warps) *decoder_warps = warps;
+    return HUFFLLM_OK;
+}
+
+huffllm_status huffllm_gemm_launch_plan(uint32_t n, const huffllm_desc *const *descs, uint32_t batch, size_t workspace_bytes_each,
+                                        uint32_t *column_slices, uint32_t *row_groups, uint32_t *ranges, uint32_t *work_items,
+                                        uint32_t *chunks_per_sum) {
+    clear_error();
+    if (!descs) return fail(HUFFLLM_ERR_INVALID_ARG, "null pointer");
+    if (n == 0 || n > kMaxMats) return fail(HUFFLLM_ERR_INVALID_ARG, "between 1 and %u matrices per call", kMaxMats);
+    if (batch <= kKernelBatch || batch > 64) return fail(HUFFLLM_ERR_INVALID_ARG, "the plan is that of the tensor-core path: batch %u to 64", kKernelBatch + 1);
+    DeviceInfo dev;
+    if (device_info(&dev) != HUFFLLM_OK) {
+        clear_error();
+        dev.sms = 148;
+        dev.smem_optin = 232448;
+    }
+    KernelArgs k;
+    uint32_t grid = 0, cta[kMaxMats];
+    begin_args(&k, batch, dev);
+    huffllm_status st;
+    for (uint32_t i = 0; i < n; ++i) {
+        if ((st = add_matrix(&k, descs[i], (const void *)256)) != HUFFLLM_OK) return st;     // (the pointer is only checked for alignment)
+        if (!tc_blob(descs[i])) return fail(HUFFLLM_ERR_UNSUPPORTED, "the tensor-core path takes tables of up to 9 bits (FP16: 8)");
+    }
+    if (n > 1 && (st = finish_args(&k, true, dev, &grid)) != HUFFLLM_OK) return st;
+    for (uint32_t i = 0; i < n; ++i) cta[i] = n > 1 ? k.m[i].cta_count : (uint32_t)dev.sms;
+    TcShape sh;
+    TcPlan plans[kMaxMats];
+    if (!tc_best(descs, n, tc_npad_of(batch), cta, k.fp16_flat != 0, k.dyn_smem_bytes, workspace_bytes_each ? workspace_bytes_each : ~(size_t)0, &sh, plans))
+        return fail(HUFFLLM_ERR_UNSUPPORTED, "chunk records too large for the tensor-core kernel's slots");
+    if (column_slices) *column_slices = sh.slices;
+    if (row_groups) *row_groups = sh.row_groups;
+    for (uint32_t i = 0; i < n; ++i) {
+        if (ranges) ranges[i] = plans[i].ksplit;
+        if (work_items) work_items[i] = plans[i].items;
+        if (chunks_per_sum) chunks_per_sum[i] = plans[i].chunks;
+    }
     return HUFFLLM_OK;
 }
 

@@ -378,23 +378,32 @@ def test_code_length_limits_accepted_per_format():
         assert e.value.status_name == "UNSUPPORTED"
 
 
+def planned_desc(rows, cols, chunk_elems, budget=0, dtype=0, _made={}):
+    """The descriptor of a rows x cols matrix of Gaussian weights, without the matrix: record sizes are those of a small one."""
+    key = (chunk_elems, budget, dtype)
+    if key not in _made:
+        w = wl.gaussian_weights(64, 2048, 0.02, 1, "fp16") if dtype else wl.gaussian_weights(64, 2048, 0.02, 1)
+        cb = hl.build_codebook(w, dtype, budget)
+        _made[key] = bytes(hl.encode(cb, w, chunk_elems)[1])
+        cb.free()
+    d = hl.Desc.from_buffer_copy(_made[key])
+    d.rows, d.cols, d.row_groups = rows, cols, (rows + 15) // 16
+    d.col_chunks = (cols + d.chunk_cols - 1) // d.chunk_cols
+    d.n_chunks = d.row_groups * d.col_chunks
+    d.off_payload = (d.off_index + 4 * (d.n_chunks + 1) + 255) // 256 * 256
+    d.payload_bytes, d.blob_bytes = 128 * d.n_chunks, d.off_payload + 128 * d.n_chunks + 4096
+    return d
+
+
 @pytest.mark.parametrize("batch,npad", [(64, 64), (20, 32), (9, 16)])
 def test_column_ranges_finish_first_among_all_simulated(batch, npad):
-    """The tensor-core path's shape and column ranges (seen through the workspace they need) are those of a walk over every work item."""
+    """The tensor-core path's shape, column ranges and work items are those of a walk over every work item of every candidate."""
     import random
-    w = wl.gaussian_weights(16, 1024, 0.02, 1)
-    cb = hl.build_codebook(w)
-    _, d = hl.encode(cb, w, 2048)                               # (records small enough for every shape)
-    cb.free()
     rng = random.Random(3)
     seen = set()
     for rows, cols in [(64, 128), (4096, 4096), (28672, 8192), (8192, 28672), (1024, 14336), (300, 28672)] + \
                       [(rng.randrange(1, 30000), 32 * rng.randrange(1, 900)) for _ in range(60)]:
-        d.rows, d.cols, d.row_groups = rows, cols, (rows + 15) // 16
-        d.col_chunks = (cols + d.chunk_cols - 1) // d.chunk_cols
-        d.n_chunks = d.row_groups * d.col_chunks
-        d.off_payload = (d.off_index + 4 * (d.n_chunks + 1) + 255) // 256 * 256
-        d.payload_bytes, d.blob_bytes = 128 * d.n_chunks, d.off_payload + 128 * d.n_chunks + 4096
+        d = planned_desc(rows, cols, 2048)                      # (records small enough for every shape)
         best, most = None, None
         for which, slices, groups, block in ((0, 1, 31, 32), (1, 1, 30, 32), (2, 2, 15, 34), (3, 4, 7, 39)):
             if (which == 1 and npad != 64) or (which == 3 and npad == 64):
@@ -410,17 +419,34 @@ def test_column_ranges_finish_first_among_all_simulated(batch, npad):
                 sums = 2 * ks * cw if ks > 1 else 0
                 span = max(sum(cost[i % ks] for i in range(b, items, grid)) for b in range(grid)) + (sums if which else 0)
                 if plan is None or span < plan[0]:
-                    plan = (span, ks, sums, max(parts))
+                    plan = (span, ks, sums, -(-max(parts) // slices))
             if plan is None:
                 continue
             if which == 0:
                 most = plan[3]
                 plan = ((plan[0] * 9 // 8 if npad == 64 else plan[0]) + plan[2],) + plan[1:]
             if best is None or plan[0] < best[0]:
-                best = (plan[0], which, m_tiles * plan[1], plan[1], cw)
-        seen.add(best[1])
-        ctrl = 4096 + ((d.row_groups + 7) // 8 * 128 + 255) // 256 * 256
-        tc = ctrl + (best[2] * 32 * best[4] * 32 * 4 if best[3] > 1 else 0)
-        two_tiles = ctrl + 512 * (2 + 64) * 16 * min(batch, 16) * 4
-        assert hl.workspace_bytes(d, batch) == max(tc, two_tiles), (rows, cols, best)
-    assert seen >= ({0, 1, 2} if npad == 64 else {0, 2, 3})
+                best = (plan[0], slices, groups, plan[1], m_tiles * plan[1], plan[3])
+        got = hl.gemm_launch_plan([d], batch)
+        assert (got["column_slices"], got["row_groups"], got["ranges"], got["work_items"], got["chunks_per_sum"]) == \
+               (best[1], best[2], [best[3]], [best[4]], [best[5]]), (rows, cols, best)
+        seen.add((best[1], best[2]))
+    assert seen == ({(1, 31), (1, 30), (2, 15)} if npad == 64 else {(1, 31), (2, 15), (4, 7)})       # every shape is chosen for some
+
+
+@pytest.mark.parametrize("rows,cols,ce,batch,most", [
+    # columns per fp32 accumulator of the one-slice plan
+    (28672, 4096, 4096, 48, 1024), (28672, 4096, 4096, 64, 1024), (12288, 12288, 2048, 48, 1152), (12288, 12288, 2048, 64, 1152),
+    (20480, 5120, 4096, 64, 768), (25088, 7168, 4096, 32, 512), (16384, 44032, 4096, 64, 3584), (15289, 7584, 4096, 64, None),
+    (4096, 14336, 4096, 16, None), (28672, 8192, 4096, 33, None)])
+def test_sums_are_no_longer_in_the_workspace_asked_for_than_in_any(rows, cols, ce, batch, most):
+    """Rounding must not depend on how large a workspace happens to be: the plan that sized it is the plan that runs, also
+    for a smaller batch, and no fp32 accumulator adds up more columns than in the plan of one slice."""
+    d = planned_desc(rows, cols, ce)
+    for b in sorted({9, 16, 17, 24, 32, 33, 48, 64, batch}):
+        free = hl.gemm_launch_plan([d], b)
+        for sized_for in sorted({b, 16, 32, 64, batch}):
+            if sized_for >= b:
+                assert hl.gemm_launch_plan([d], b, hl.workspace_bytes(d, sized_for)) == free, (b, sized_for)
+        if most and b == batch:
+            assert free["chunks_per_sum"][0] * d.chunk_cols <= most
