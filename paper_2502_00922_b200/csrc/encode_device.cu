@@ -72,16 +72,18 @@ struct EncRow {
     int32_t left;               // 0 for rows outside the tensor
 };
 // The eight weights of block kb as four words, pad words outside the tensor.  Rows that do not start on 16-byte boundaries
-// are read in the aligned words that the eight weights lie in (every word holds one of them at least).
+// are read in words; where those straddle the weights, the first and the last weight are read alone: nothing outside the
+// eight is touched (the word's other half may lie in front of the tensor or behind it).
 __device__ __forceinline__ uint4 enc_load8(const EncArgs &A, const EncRow &R, uint32_t kb) {
     const uint16_t *p = R.p + kb * 32u;
     const int32_t left = R.left - (int32_t)(kb * 32u);
     if (left >= 8) {
         if (A.vec_ok) return __ldg((const uint4 *)p);
-        const uint32_t odd = (uint32_t)((uintptr_t)p >> 1) & 1u, sel = odd ? 0x5432u : 0x3210u;
-        const uint32_t *q = (const uint32_t *)(p - odd);
-        const uint32_t u0 = __ldg(q), u1 = __ldg(q + 1), u2 = __ldg(q + 2), u3 = __ldg(q + 3), u4 = odd ? __ldg(q + 4) : 0u;
-        return make_uint4(__byte_perm(u0, u1, sel), __byte_perm(u1, u2, sel), __byte_perm(u2, u3, sel), __byte_perm(u3, u4, sel));
+        const bool odd = ((uintptr_t)p & 2u) != 0;
+        const uint32_t *q = (const uint32_t *)(p + (odd ? 1 : 0)), sel = odd ? 0x5432u : 0x7654u;
+        const uint32_t u0 = __ldg(q), u1 = __ldg(q + 1), u2 = __ldg(q + 2);
+        const uint32_t first = odd ? __ldg(p) : 0u, u3 = odd ? __ldg(p + 7) : __ldg(q + 3);
+        return make_uint4(__byte_perm(first, u0, odd ? 0x5410u : 0x7654u), __byte_perm(u0, u1, sel), __byte_perm(u1, u2, sel), __byte_perm(u2, u3, sel));
     }
     uint32_t x[4];
 #pragma unroll
