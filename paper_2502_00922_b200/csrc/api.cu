@@ -236,8 +236,8 @@ TcPlan tc_plan(const huffllm_desc *d, uint32_t npad, uint32_t sms, const TcShape
     }
     p.ksplit = best;                                     // (0: no number of ranges is within the limits)
     p.items = p.m_tiles * best;
-    // (at the widest padding an issuer that carries the activations as well makes a block take an eighth longer)
-    p.span = !best ? ~0ull : !base ? best_span : (npad == 64 ? best_span * 9 / 8 : best_span) + tc_sum_cost(sh, npad, best);
+    // (at the widest padding an issuer that carries the activations of four tiles as well makes a block take an eighth longer)
+    p.span = !best ? ~0ull : !base ? best_span : (npad == 64 && sh.na == 4 ? best_span * 9 / 8 : best_span) + tc_sum_cost(sh, npad, best);
     p.chunks = best ? ((d->col_chunks + best - 1) / best + sh.slices - 1) / sh.slices : 0;
     // the counters' region is sized for the smallest tile (most row tiles), so that plans for different batch sizes
     // sharing one workspace never put partial sums where another plan keeps counters

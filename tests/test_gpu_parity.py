@@ -709,3 +709,26 @@ def test_results_straight_to_pinned_host_memory_and_kernel_copy(hl, torch):
     assert np.array_equal(gpu_gemm(hl, torch, up, x), y[:3 * rows].reshape(3, rows))
     with pytest.raises(hl.HuffllmError):
         hl.stage_copy(x_dev, x_host, 24)                      # not a multiple of 16
+
+
+# ------------------------------------------------------------------ the tensor-core kernel's shapes
+
+def tc_case(hl, torch, shapes, ce, batch, budget=0, dtype=0, seed=2100):
+    ups, xs = [], []
+    for i, (rows, cols) in enumerate(shapes):
+        w = wl.gaussian_weights(rows, cols, 0.02, seed + i, "fp16") if dtype else make("gauss", rows, cols, seed + i)
+        ups.append(Uploaded(hl, torch, w, ce, budget, batch, dtype=dtype))
+        xs.append(wl.activations(batch, cols, seed + 50 + i, "fp16") if dtype else wl.activations(batch, cols, seed + 50 + i))
+    return ups, xs
+
+
+@pytest.mark.parametrize("rows,cols,ce,dtype", [(5000, 2080, 8192, 0), (9000, 544, 4096, 1), (300, 4128, 8192, 0)])
+@pytest.mark.parametrize("batch", [17, 64])
+def test_fewer_tiles_than_four(hl, torch, rows, cols, ce, dtype, batch):
+    """Records so large that a CTA has room for one, two or three tiles: the activations have a warp of their own behind the tiles."""
+    ups, xs = tc_case(hl, torch, [(rows, cols)], ce, batch, dtype=dtype)
+    plan = hl.gemm_launch_plan([ups[0].desc], batch, ups[0].ws_bytes)
+    assert plan["column_slices"] == 1 and plan["row_groups"] in (8, 16, 24)
+    y = gpu_gemm(hl, torch, ups[0], xs[0])
+    check_product(y, ups[0].w, xs[0], dtype)
+    assert np.array_equal(y, gpu_gemm(hl, torch, ups[0], xs[0])), "results must be bitwise reproducible"
