@@ -585,10 +585,21 @@ __global__ void __launch_bounds__(THREADS, 1) huff_kernel(const __grid_constant_
                             for (int h = 0; h < 2; ++h) sts_row(row_buf + 8 * kRowBuf * h - 64u, a + 4 * h);
                         }
                     } else {
+                        // (With the one-by-one stores left out of this kernel, which one branch skips, the compiler ordered the
+                        // block's instructions differently and an aligned decode took 5 to 10 % longer: BF16 11008 x 4096
+                        // in chunks of 4096 / 16384 elements 46.9 / 71.6 us against 42.9 / 64.6, FP16 28672 x 8192 211 against 196.)
+                        const uint32_t col = col0 + kb * 32u;
 #pragma unroll
                         for (int h = 0; h < 2; ++h) {
-                            if ((uint64_t)rg * 16 + g + 8 * h >= k.rows || col0 + kb * 32u >= (uint32_t)k.cols) continue;
-                            *(uint4 *)(out0 + (uint64_t)(8 * h) * k.cols + kb * 32u) = make_uint4(a[4 * h], a[4 * h + 1], a[4 * h + 2], a[4 * h + 3]);
+                            if ((uint64_t)rg * 16 + g + 8 * h >= k.rows || col >= (uint32_t)k.cols) continue;
+                            uint16_t *dst = out0 + (uint64_t)(8 * h) * k.cols + kb * 32u;
+                            if (k.cols % 8 == 0) {
+                                *(uint4 *)dst = make_uint4(a[4 * h], a[4 * h + 1], a[4 * h + 2], a[4 * h + 3]);
+                            } else {
+#pragma unroll
+                                for (int i = 0; i < 8; ++i)
+                                    if (col + i < (uint32_t)k.cols) dst[i] = (uint16_t)(a[4 * h + (i >> 1)] >> (16 * (i & 1)));
+                            }
                         }
                     }
                 };
