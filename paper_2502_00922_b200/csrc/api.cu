@@ -341,6 +341,16 @@ void set_tc_shape(KernelArgs *k, uint32_t npad, const TcShape &sh) {
     k->tc_row_groups = sh.row_groups;
 }
 
+// Does a decode send its rows through shared memory?  Rows of a multiple of 8 columns start on 16-byte boundaries (the output
+// does) and are stored directly, also where multiples of 8 that are not multiples of 16 make rows straddle sectors: the detour
+// reads a word behind a piece whose row starts on a 32-byte boundary, for which a tile's last row has no room (it never does
+// off 16 bytes), and has little to give there (28672 x 8184 stored directly takes 250 us, 28672 x 8188 through shared memory 245).
+// Other rows pay for the detour from 64 columns and 3/4 2^20 weights on: below that a launch is bound by its set-up and a warp's
+// few blocks, and direct stores, many as they are, take less (BF16, chunks of 4096, direct / through shared memory:
+// 100000 x 7 12.2 / 15.7 us, 100000 x 33 19.2 / 19.6, 1000 x 515 13.6 / 13.3; 4096 x 257 14.2 / 14.2, 30000 x 65 15.5 / 14.3,
+// 1000 x 1027 15.6 / 14.4, 11007 x 4099 186 / 59).
+bool rows_through_smem(const MatArgs &m) { return m.cols % 8 && m.cols >= 64 && m.rows * m.cols >= 3ull << 18; }
+
 // Close a launch description: shared-memory budget and grid size.
 huffllm_status finish_args(KernelArgs *k, bool product, const DeviceInfo &dev, uint32_t *grid, uint32_t *warps_at_least = nullptr) {
     // (pieces that warps of a CTA exchange: in shared memory up to 8 vectors, in the workspace above)
@@ -350,9 +360,9 @@ huffllm_status finish_args(KernelArgs *k, bool product, const DeviceInfo &dev, u
     // that this would leave fewer than 31 warps a slot pair, and single slots serve at least a quarter more warps, every
     // warp gets one slot: more decoders at work outweigh the wait for a copy at every chunk start.
     const uint64_t max_w = 31;                                       // decoder warps of a CTA of 1024 threads
-    // (decode to rows that do not start on 16-byte boundaries: every warp takes room for the rows it works on, as many warps
-    // as find both a slot and that room; one always does: its room is no larger than the guard area)
-    const bool row_bufs = !product && k->m[0].cols % 8;
+    // (decode with rows that go through shared memory: every warp takes room for the rows it works on, as many warps as find
+    // both a slot and that room; one always does: its room is no larger than the guard area)
+    const bool row_bufs = !product && rows_through_smem(k->m[0]);
     auto warps_with = [&](uint64_t pair_bytes) -> uint64_t {
         uint64_t best = 0;
         for (uint64_t n = row_bufs ? max_w : 1; n > best; --n) {

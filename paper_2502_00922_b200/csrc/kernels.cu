@@ -82,9 +82,9 @@ __device__ __forceinline__ void store_piece(uint16_t *dst, const uint4 &p, int32
 
 // ------------------------------------------------------------------------------ the fused kernel
 
-// MODE 0: write the decoded weights (rows of a multiple of 8 columns: every lane's eight weights are one aligned store).
-// MODE 2: write the decoded weights of a matrix whose rows start anywhere (see store_piece).  MODE 1: y = W x for up to 8
-// activation vectors.
+// MODE 0: write the decoded weights, every lane its eight: one aligned store where rows have a multiple of 8 columns, one by one
+// otherwise (small matrices).  MODE 2: write the decoded weights of a matrix whose rows start anywhere (see store_piece).
+// MODE 1: y = W x for up to 8 activation vectors.
 // LB = table index bits (the blobs' lut_bits): 8 or 9; LB = 12 stands for every longer limit up to 12 (BF16: 10..12,
 // FP16: 9..12): two-level lookup, the number of bits is A.lut_bits.
 // FMT = 0: BF16 blobs; FMT = 1: FP16 {1,5,5,5} blobs (three lookups per weight, sign bits as the raw part); FMT = 2: the same
@@ -771,11 +771,9 @@ static cudaError_t launch_decode_mode(const KernelArgs &k, uint32_t grid, cudaSt
     if (k.lut_bits > 9) return launch_one<MODE, 12, kThreads, 0>(k, grid, stream);
     return k.lut_bits == 8 ? launch_slots<MODE, 8, 0>(k, grid, stream) : launch_one<MODE, 9, kThreads, 0>(k, grid, stream);
 }
-// Rows of a multiple of 8 columns start on 16-byte boundaries (the output does): every lane's eight weights are one store.
-// (Multiples of 8 that are not multiples of 16 stay there although rows then straddle sectors: 11008 x 4104 49.1 us against
-// 50 us with the rows going through shared memory, 28672 x 8184 248 against 227 us.)
+// (Where rows go through shared memory is decided with the launch's shared memory: part_bytes.)
 cudaError_t launch_decode(const KernelArgs &k, uint32_t grid, cudaStream_t stream) {
-    return k.m[0].cols % 8 == 0 ? launch_decode_mode<0>(k, grid, stream) : launch_decode_mode<2>(k, grid, stream);
+    return k.part_bytes ? launch_decode_mode<2>(k, grid, stream) : launch_decode_mode<0>(k, grid, stream);
 }
 
 cudaError_t launch_gemm(const KernelArgs &k, uint32_t grid, cudaStream_t stream) {

@@ -123,6 +123,25 @@ def test_decode_to_rows_that_start_off_a_16_byte_boundary(hl, torch, rows, cols,
     assert np.array_equal(gpu_decode(hl, torch, up), w)
 
 
+@pytest.mark.parametrize("cols", [63, 65, 249, 252, 509, 515, 774, 1030, 209717, 1048583])
+@pytest.mark.parametrize("ce,budget,dtype", [(512, 0, 0), (4096, 9, 0), (1024, 0, 1), (1024, 7, 1)])
+def test_decode_of_large_matrices_whose_rows_start_off_a_16_byte_boundary(hl, torch, cols, ce, budget, dtype):
+    """The same for matrices of 2^20 weights and more, whose rows go through shared memory from 64 columns on: every remainder
+    modulo 8, rows that end with a row group's first or last rows, outputs on and off 32-byte boundaries."""
+    rows = (1 << 20) // cols + 1
+    w = wl.gaussian_weights(rows, cols, 0.02, cols, "fp16") if dtype else make("gauss", rows, cols, cols)
+    up = Uploaded(hl, torch, w, ce, budget, dtype=dtype)
+    buf = torch.empty(rows * cols + 128, dtype=torch.int16, device="cuda")
+    for first in (64, 72):                         # weights in front of the output: 128 and 144 bytes
+        buf.fill_(0x5A5A)
+        hl.decode(up.desc, up.blob_dev, buf[first:], up.err)
+        torch.cuda.synchronize()
+        got = buf.cpu().numpy().view(np.uint16)
+        assert int(up.err.item()) == 0
+        assert np.all(got[:first] == 0x5A5A) and np.all(got[first + rows * cols:] == 0x5A5A)
+        assert np.array_equal(got[first:first + rows * cols].reshape(rows, cols), w)
+
+
 @pytest.mark.parametrize("rows,cols,ce,budget,gen,batch", [
     (1024, 1024, 4096, 0, "gauss", 1), (37, 300, 1024, 0, "student", 0), (256, 2048, 4096, 0, "patterns", 0),
     (512, 4096, 4096, 9, "student", 5), (272, 2080, 16384, 0, "gauss", 4), (16, 512, 512, 0, "constant", 2),
