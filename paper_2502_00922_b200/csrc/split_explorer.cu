@@ -17,6 +17,7 @@
 #include <algorithm>
 #include <cmath>
 #include <cstring>
+#include <type_traits>
 #include <vector>
 
 #include "internal.h"
@@ -65,18 +66,26 @@ __global__ void __launch_bounds__(kHistThreads, 2) split_histogram_kernel(const 
     // 16-byte vectors of eight weights, dealt to the grid's threads in turn; the last n % 8 weights go to one thread
     const uint64_t n_vec = A.n / 8, stride = (uint64_t)gridDim.x * blockDim.x;
     const uint4 *src = (const uint4 *)A.w;
-    // the n_in_word weights of a 32-bit word
-    auto count_word = [&](uint32_t word, uint32_t n_in_word) {
+    // n_words words of two weights each (one with `single`): a piece at a time, its plan read once for all of them
+    auto count_words = [&](const uint32_t *word, auto n_words, bool single) {
 #pragma unroll 1
         for (uint32_t pi = 0; pi < A.n_pieces; ++pi) {
             const PiecePlan &p = A.p[pi];
             const uint32_t lane_off = base + ((p.smem_off + (lane & ((1u << p.rep_log2) - 1u))) << 2);
-            const uint32_t step = 4u << p.rep_log2;
+            const uint32_t step = 4u << p.rep_log2, sh = p.shift, mask = p.mask, lo = p.bin_lo, nb = p.bin_n;
+            if (!p.ranged) {
 #pragma unroll
-            for (uint32_t j = 0; j < 2; ++j) {
-                if (j >= n_in_word) break;
-                uint32_t b = ((word >> (p.shift + 16 * j)) & p.mask) - p.bin_lo;
-                if (!p.ranged || b < p.bin_n) red_shared_inc(lane_off + b * step);
+                for (int i = 0; i < decltype(n_words)::value; ++i) {
+                    red_shared_inc(lane_off + ((word[i] >> sh) & mask) * step);
+                    if (!single) red_shared_inc(lane_off + ((word[i] >> (sh + 16)) & mask) * step);
+                }
+            } else {
+#pragma unroll
+                for (int i = 0; i < decltype(n_words)::value; ++i) {
+                    const uint32_t b0 = ((word[i] >> sh) & mask) - lo, b1 = ((word[i] >> (sh + 16)) & mask) - lo;
+                    if (b0 < nb) red_shared_inc(lane_off + b0 * step);
+                    if (!single && b1 < nb) red_shared_inc(lane_off + b1 * step);
+                }
             }
         }
     };
@@ -91,9 +100,11 @@ __global__ void __launch_bounds__(kHistThreads, 2) split_histogram_kernel(const 
     auto inc = [&](uint32_t table, uint32_t byte_off) { atomicAdd((uint32_t *)((char *)hist + table + byte_off), 1u); };
     auto count = [&](const uint4 &q) {
         const uint32_t word[4] = {q.x, q.y, q.z, q.w};
+        if constexpr (PIECES == 0) {
+            count_words(word, std::integral_constant<int, 4>{}, false);
+        } else {
 #pragma unroll
-        for (int i = 0; i < 4; ++i) {
-            if (PIECES) {
+            for (int i = 0; i < 4; ++i) {
                 // a counter's 32 copies are 128 bytes: the value, moved to bit 7, is its byte offset.  (The upper weight's
                 // value is moved down by at least 9, 16 + shift - 7; the lower one's up or down: as a 64-bit shift, one instruction.)
 #pragma unroll
@@ -101,22 +112,24 @@ __global__ void __launch_bounds__(kHistThreads, 2) split_histogram_kernel(const 
                     inc(off[pi], ((uint32_t)(((uint64_t)word[i] << 7) >> sh[pi]) & mask[pi]) | lane4);
                     inc(off[pi], ((word[i] >> (sh[pi] + 9u)) & mask[pi]) | lane4);
                 }
-            } else {
-                count_word(word[i], 2);
             }
         }
     };
     uint64_t v = (uint64_t)blockIdx.x * blockDim.x + tid;
-    for (; v + 3 * stride < n_vec; v += 4 * stride) {          // four loads in flight per thread
-        uint4 q[4];
+    if constexpr (PIECES != 0)
+        for (; v + 3 * stride < n_vec; v += 4 * stride) {      // four loads in flight per thread
+            uint4 q[4];
 #pragma unroll
-        for (int i = 0; i < 4; ++i) q[i] = __ldg(src + v + i * stride);
+            for (int i = 0; i < 4; ++i) q[i] = __ldg(src + v + i * stride);
 #pragma unroll
-        for (int i = 0; i < 4; ++i) count(q[i]);
-    }
+            for (int i = 0; i < 4; ++i) count(q[i]);
+        }
     for (; v < n_vec; v += stride) count(__ldg(src + v));
     if (blockIdx.x == 0 && tid == 0)
-        for (uint64_t i = n_vec * 8; i < A.n; ++i) count_word(A.w[i], 1);
+        for (uint64_t i = n_vec * 8; i < A.n; ++i) {
+            const uint32_t word = A.w[i];
+            count_words(&word, std::integral_constant<int, 1>{}, true);
+        }
     __syncthreads();
 
     // the copies of every value summed (into the first one, which no other thread reads)
