@@ -5,8 +5,8 @@
 //
 // Counting is one streaming pass over the weights (2 bytes per weight from HBM).  Every CTA keeps private counters in
 // shared memory and adds them to the global 64-bit counters at the end.  What bounds it is the shared-memory atomic unit,
-// one counter update per weight and counted piece, so neighbouring narrow fields are counted together, as one piece of up
-// to ten bits, and told apart when the CTA adds its counters up.  LLM weights are very skewed (a handful of exponent values
+// one counter update per weight and counted piece, so neighbouring narrow fields of a large tensor are counted together, as one
+// piece of up to ten bits, and told apart when the CTA adds its counters up.  LLM weights are very skewed (a handful of exponent values
 // cover almost all weights), so a piece's counters are replicated 32 times, one copy per lane: the lanes of a warp never
 // touch the same address or the same bank, whatever the data.  Wider fields get fewer copies; a field whose counters do
 // not fit is counted in several launches, each owning a range of values.
@@ -28,6 +28,10 @@ constexpr uint32_t kHistThreads = 1024;
 constexpr uint32_t kHistBudgetWords = 48u * 1024u;   // shared-memory counters of one launch (192 KB)
 constexpr uint32_t kFieldWords = 8u * 1024u;         // target size of a wide field's counters, copies included
 constexpr uint32_t kPieceBits = 10;                  // most bits of a piece of several fields: 1024 counters, 32 copies, 128 KB
+// From this many counter updates on (weights times fields) fields are counted together.  Below, clearing and adding up the larger
+// tables costs a CTA more than its weights do.  (Apart / together, us: 1-5-5-5 at 10^6 weights 10.0 / 14.4, at 4 10^6 14.3 / 16.3, at
+// 45 10^6 53 / 36; 1-8-7 10.2 / 12.2, 14.2 / 15.7, 45 / 33; sixteen fields of one bit 17.5 / 23.5, 33 / 25.6, 169 / 45.)
+constexpr uint64_t kMergeFrom = 1ull << 25;
 
 struct PiecePlan {
     uint32_t shift, mask;        // value of the piece = (word >> shift) & mask
@@ -132,28 +136,26 @@ __global__ void __launch_bounds__(kHistThreads, 2) split_histogram_kernel(const 
         }
     __syncthreads();
 
-    // the copies of every value summed (into the first one, which no other thread reads)
+    // add the CTA's counters to the global ones, copies of a value summed first, zero sums skipped: a piece of one field at
+    // once; of several, the copies are summed into the first one (which no other thread reads), then a thread or a warp per
+    // field value sums the piece's values that have it
+    bool several = false;
     for (uint32_t pi = 0; pi < A.n_pieces; ++pi) {
         const PiecePlan &p = A.p[pi];
         const uint32_t reps = 1u << p.rep_log2;
+        several = several || p.n_fields > 1;
         for (uint32_t b = tid; b < p.bin_n; b += blockDim.x) {
             uint32_t s = 0;
             for (uint32_t r = 0; r < reps; ++r) s += hist[p.smem_off + (b << p.rep_log2) + ((r + tid) & (reps - 1u))];
-            hist[p.smem_off + (b << p.rep_log2)] = s;
+            if (p.n_fields > 1) hist[p.smem_off + (b << p.rep_log2)] = s;
+            else if (s) atomicAdd(A.counts + A.f[p.field_first].out_off + p.bin_lo + b, (unsigned long long)s);
         }
     }
+    if (!several) return;
     __syncthreads();
-    // add the CTA's counters to the global ones (zero sums are skipped): a piece of one field as it stands, a piece of
-    // several with a thread or a warp per field value, which sums the piece's values that have it
     for (uint32_t pi = 0; pi < A.n_pieces; ++pi) {
         const PiecePlan &p = A.p[pi];
-        if (p.n_fields == 1) {
-            for (uint32_t b = tid; b < p.bin_n; b += blockDim.x) {
-                const uint32_t s = hist[p.smem_off + (b << p.rep_log2)];
-                if (s) atomicAdd(A.counts + A.f[p.field_first].out_off + p.bin_lo + b, (unsigned long long)s);
-            }
-            continue;
-        }
+        if (p.n_fields == 1) continue;
         for (uint32_t fi = p.field_first; fi < p.field_first + p.n_fields; ++fi) {
             const FieldPlan &f = A.f[fi];
             const uint32_t others = p.bin_n >> f.width;        // piece values with a given field value
@@ -221,15 +223,16 @@ extern "C" huffllm_status huffllm_split_histogram(const uint16_t *w_dev, uint64_
     if ((e = cudaGetDevice(&dev)) != cudaSuccess || (e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev)) != cudaSuccess)
         return fail(HUFFLLM_ERR_CUDA, "device query: %s", cudaGetErrorString(e));
 
-    // the pieces to count: neighbouring fields of up to kPieceBits bits together, a wider field, or a range of a wide
+    // the pieces to count: neighbouring fields of up to kPieceBits bits together (large tensors), a wider field, or a range of a wide
     // field's values, each with its counters' size.  (A split has 16 bits, so two pieces are the least there can be, and no
     // split of fields of up to ten bits needs more than three.)
     std::vector<PiecePlan> pieces;
     FieldPlan fields[HUFFLLM_MAX_FIELDS] = {};
     uint32_t hi = 16, out_off = 0;
+    const bool merge = n_weights * n_fields >= kMergeFrom;
     for (uint32_t i = 0; i < n_fields;) {
         uint32_t bits = widths[i], last = i + 1;
-        while (last < n_fields && bits + widths[last] <= kPieceBits) bits += widths[last++];
+        while (merge && last < n_fields && bits + widths[last] <= kPieceBits) bits += widths[last++];
         const uint32_t n_bins = 1u << bits;
         PiecePlan p = {};
         p.shift = hi - bits;
@@ -243,7 +246,7 @@ extern "C" huffllm_status huffllm_split_histogram(const uint16_t *w_dev, uint64_
             fields[i].out_off = out_off;
             out_off += 1u << widths[i];
         }
-        const uint32_t target = bits <= kPieceBits ? n_bins << 5 : kFieldWords;
+        const uint32_t target = merge && bits <= kPieceBits ? n_bins << 5 : kFieldWords;
         while (p.rep_log2 < 5u && (n_bins << (p.rep_log2 + 1u)) <= target) ++p.rep_log2;
         const uint32_t per_piece = std::min(n_bins, kHistBudgetWords / 2u >= n_bins ? n_bins : 32u * 1024u);
         for (uint32_t lo = 0; lo < n_bins; lo += per_piece) {

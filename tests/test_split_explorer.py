@@ -97,6 +97,18 @@ def test_device_counters_edge_sizes(hl):
 
 
 @pytest.mark.gpu
+@pytest.mark.parametrize("widths", [[1, 8, 7], [1, 5, 5, 5], [4, 4, 4, 4], [5, 6, 5], [2, 3, 1, 4, 6], [1] * 16, [10, 6], [3, 13]])
+def test_device_counters_of_fields_counted_together(hl, widths):
+    """Fields are counted together where weights times fields reach 2^25: both sides of that line, every pattern met."""
+    import torch
+    line = -(-(1 << 25) // len(widths))
+    w = np.random.default_rng(7).integers(0, 1 << 16, line + 5, dtype=np.uint16)
+    w[line // 2:] = w[line // 2:] & 0x83FF | 0x2000         # (and half of the tensor with few exponents)
+    for n in (line - 1, line, line + 5):
+        assert np.array_equal(device_counts(hl, torch, w[:n], widths), np.concatenate(orc.split_histograms(w[:n], widths)))
+
+
+@pytest.mark.gpu
 def test_full_size_matrix_reproduces_the_tables_rows(hl):
     """A full-size FFN matrix of the benchmark's layer, every split of the entropy table, counters exact."""
     import torch
