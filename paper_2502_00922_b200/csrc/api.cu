@@ -151,7 +151,7 @@ bool tc_fits(const huffllm_desc *const *d, uint32_t n, uint32_t npad, const TcSh
 }
 // The shapes a launch chooses from: 0 = one slice, as many tiles of rows as find room; 1 = one slice and a warp of its own for
 // the activations (at the widest batch padding: there the issuer, which carries them otherwise, bounds the CTA, 8192 x 28672
-// at 64 vectors 138 us against 122 with one decoder fewer); 2, 3 = two and four slices.  False: it does not fit or apply.
+// at 64 vectors 149 us against 133 with one decoder fewer); 2, 3 = two and four slices.  False: it does not fit or apply.
 constexpr uint32_t kTcShapes = 4;
 bool tc_shape(const huffllm_desc *const *d, uint32_t n, uint32_t npad, uint32_t which, bool flat, uint32_t dyn_smem, TcShape *sh) {
     const uint32_t slices = which < 2 ? 1 : which == 2 ? 2 : 4;
@@ -181,9 +181,13 @@ struct TcPlan {
 // Estimated costs, in 1/32 of the time that a CTA of one slice takes for a block of 32 columns (0.93 us, 31 decoders).  Time
 // stamps: with two slices (30 decoders) a block takes 0.99 us, with four (28) 1.14; an item's start and epilogue take 5 to 6 us,
 // with several slices, whose pieces are smaller, 4.5; the last CTA's sum of a row tile's pieces 9 us for 16 ranges of 16 columns
-// per warp, 5.5 for 5 of 16, 6 for 14 of 8.
+// per warp, 5.5 for 5 of 16, 6 for 14 of 8.  (The term for that sum is a line through the origin: 4.7 and 6.5 us for the last two;
+// 14.9 for the first, where it stands against plans of 16 ranges and one slice, which no measured shape was better off with.)
+// At the widest padding two slices leave one slice's activations to the issuer, beside 16 MMAs per stage: 36 instead of 34.  (With
+// 34, 28672 x 4096 at 64 vectors took two slices, 99 us, instead of one and a warp for the activations, 91; with 38, 25088 x 7168
+// in chunks of 2048 would go the other way, 153 instead of 141.)
 constexpr uint32_t kTcUnit = 32;
-uint32_t tc_block_cost(const TcShape &sh) { return sh.slices == 1 ? kTcUnit : sh.slices == 2 ? 34 : 39; }
+uint32_t tc_block_cost(const TcShape &sh, uint32_t npad) { return sh.slices == 1 ? kTcUnit : sh.slices == 2 ? (npad == 64 ? 36 : 34) : 39; }
 constexpr uint32_t kTcItemCost = 5 * kTcUnit;
 uint32_t tc_sum_cost(const TcShape &sh, uint32_t npad, uint32_t ks) { return ks > 1 ? 2 * ks * sh.piece_columns(npad) : 0; }
 // The longest any CTA works when `ks` column ranges of `m_tiles` row tiles are dealt to `sms` CTAs: CTA b takes items b,
@@ -191,11 +195,11 @@ uint32_t tc_sum_cost(const TcShape &sh, uint32_t npad, uint32_t ks) { return ks 
 // in the last round: one sum per residue instead of one per CTA.  (Walking every item of every candidate took 15 to 30 us
 // of host time per matrix and launch: the four launches of a 7B-shaped layer at 32 vectors were bound by it, 225 us a layer
 // for 165 us of GPU time.)
-uint64_t tc_span(const huffllm_desc *d, const TcShape &sh, uint32_t m_tiles, uint32_t ks, uint32_t sms) {
+uint64_t tc_span(const huffllm_desc *d, const TcShape &sh, uint32_t npad, uint32_t m_tiles, uint32_t ks, uint32_t sms) {
     const uint64_t items = (uint64_t)m_tiles * ks;
     const uint32_t grid = (uint32_t)(items < sms ? items : sms), rounds = (uint32_t)((items + grid - 1) / grid);
     const uint32_t in_last = (uint32_t)(items - (uint64_t)(rounds - 1) * grid);      // CTAs with an item in the last round: the first ones
-    const uint32_t chunk_cost = d->chunk_cols / kBlockCols * tc_block_cost(sh), step = grid % ks;
+    const uint32_t chunk_cost = d->chunk_cols / kBlockCols * tc_block_cost(sh, npad), step = grid % ks;
     uint64_t cost[16];                                                               // of an item of range r
     for (uint32_t r = 0, at = 0; r < ks; ++r) {
         const uint32_t end = d->col_chunks * (r + 1) / ks;       // (at most 2^26 chunks: the product fits)
@@ -231,7 +235,7 @@ TcPlan tc_plan(const huffllm_desc *d, uint32_t npad, uint32_t sms, const TcShape
         if (ks > 1 && ws_partial_offset(d) + (size_t)p.m_tiles * ks * item_bytes > max_bytes) break;
         const uint32_t range = (d->col_chunks + ks - 1) / ks;
         if ((range + sh.slices - 1) / sh.slices > max_chunks) continue;
-        const uint64_t span = tc_span(d, sh, p.m_tiles, ks, sms) + (base ? 0 : tc_sum_cost(sh, npad, ks));
+        const uint64_t span = tc_span(d, sh, npad, p.m_tiles, ks, sms) + (base ? 0 : tc_sum_cost(sh, npad, ks));
         if (span < best_span) { best_span = span; best = ks; }
     }
     p.ksplit = best;                                     // (0: no number of ranges is within the limits)
