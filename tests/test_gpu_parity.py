@@ -741,6 +741,66 @@ def tc_case(hl, torch, shapes, ce, batch, budget=0, dtype=0, seed=2100):
     return ups, xs
 
 
+@pytest.mark.parametrize("rows,cols,ce,batch,slices,more_than_sms", [
+    (12513, 160, 512, 64, 2, True), (4343, 480, 512, 17, 4, True), (240, 160, 512, 17, 4, False), (1040, 4096, 2048, 33, 2, False)])
+def test_column_slices_over_several_work_items(hl, torch, rows, cols, ce, batch, slices, more_than_sms):
+    """Two and four slices, with more work items than SMs (a CTA takes a second one: stages, accumulators, the shared
+    arrival flag and the records asked for ahead are used again) and with ranges that leave slices without a chunk."""
+    ups, xs = tc_case(hl, torch, [(rows, cols)], ce, batch)
+    plan = hl.gemm_launch_plan([ups[0].desc], batch, ups[0].ws_bytes)
+    sms = torch.cuda.get_device_properties(0).multi_processor_count
+    assert plan["column_slices"] == slices and plan["ranges"][0] > 1 and (plan["work_items"][0] > sms) == more_than_sms
+    y = gpu_gemm(hl, torch, ups[0], xs[0])
+    check_product(y, ups[0].w, xs[0])
+    for _ in range(3):
+        assert np.array_equal(y, gpu_gemm(hl, torch, ups[0], xs[0])), "results must be bitwise reproducible"
+
+
+@pytest.mark.parametrize("shapes,ce,batch,slices", [
+    ([(1040, 4096), (496, 8192), (300, 2080)], 2048, 32, 4), ([(1383, 800), (563, 3776)], 512, 17, 4), ([(2503, 544), (995, 2368)], 512, 32, 4),
+    ([(2726, 2080), (1655, 128), (873, 448)], 512, 20, 2), ([(2457, 544), (3717, 704)], 512, 64, 2)])
+def test_several_matrices_through_column_slices(hl, torch, shapes, ce, batch, slices):
+    """Launches over several matrices of which some have more work items than their share of the SMs."""
+    ups, xs = tc_case(hl, torch, shapes, ce, batch)
+    ws_each = max(u.ws_bytes for u in ups)
+    plan = hl.gemm_launch_plan([u.desc for u in ups], batch, ws_each)
+    assert plan["column_slices"] == slices and max(plan["ranges"]) > 1
+    x_devs = [torch.from_numpy(x.view(np.int16)).cuda() for x in xs]
+    wss = [torch.zeros(ws_each, dtype=torch.uint8, device="cuda") for _ in ups]
+    first = None
+    for _ in range(3):
+        ys = [torch.full((batch * u.w.shape[0],), float("nan"), dtype=torch.float32, device="cuda") for u in ups]
+        hl.decode_gemm_multi([u.desc for u in ups], [u.blob_dev for u in ups], x_devs, batch, ys, wss, ws_each, ups[0].err)
+        torch.cuda.synchronize()
+        assert int(ups[0].err.item()) == 0
+        got = [y.cpu().numpy().reshape(batch, -1) for y in ys]
+        if first is None:
+            first = got
+            for u, x, y in zip(ups, xs, got):
+                check_product(y, u.w, x)
+        for u, ws, y, y0 in zip(ups, wss, got, first):
+            assert np.array_equal(y, y0), "results must be bitwise reproducible"
+            assert int(ws[:hl.workspace_control_bytes(u.desc)].count_nonzero().item()) == 0
+
+
+@pytest.mark.parametrize("batch", [12, 33, 64])
+def test_products_in_workspaces_that_cut_the_plan(hl, torch, batch):
+    """Every workspace from the least that is accepted up: fewer column ranges, the same product; one of the size asked for, or of the
+    size for more vectors, gives the same bits as a larger one."""
+    ups, xs = tc_case(hl, torch, [(2080, 4096)], 2048, batch, budget=9)
+    up, full = ups[0], hl.workspace_bytes(ups[0].desc, batch)
+    least = hl.workspace_bytes(up.desc, 8)
+    asked_for = None
+    for ws_bytes in (least, least + (full - least) // 3, full - 256, full, hl.workspace_bytes(up.desc, 64), 3 * full):
+        up.ws_bytes, up.ws = ws_bytes, torch.zeros(ws_bytes, dtype=torch.uint8, device="cuda")
+        y = gpu_gemm(hl, torch, up, xs[0])
+        check_product(y, up.w, xs[0])
+        if ws_bytes == full:
+            asked_for = y
+        assert ws_bytes < full or np.array_equal(y, asked_for)
+    assert hl.gemm_launch_plan([up.desc], batch, least)["ranges"] < hl.gemm_launch_plan([up.desc], batch)["ranges"]
+
+
 @pytest.mark.parametrize("rows,cols,ce,dtype", [(5000, 2080, 8192, 0), (9000, 544, 4096, 1), (300, 4128, 8192, 0)])
 @pytest.mark.parametrize("batch", [17, 64])
 def test_fewer_tiles_than_four(hl, torch, rows, cols, ce, dtype, batch):
