@@ -4,7 +4,7 @@
 //
 // One thread per bit sequence (64 per chunk), as in the format: thread q of a chunk owns lane q / 2 and row half q % 2,
 // so neighbouring threads write neighbouring raw bytes and the two halves of a lane sit in one warp.
-//   pass 1  code lengths only -> words per sequence of every chunk, coded bits
+//   pass 1  code lengths only -> words per sequence of every chunk; words and coded bits of every 1024 chunks
 //   scan    record offsets (the index section), payload size, largest record
 //   pass 2  raw part and coded part of every record (nothing if the scan found the tensor or the buffer unfit)
 //   pass 3  the checksum term of every record, a warp each; the last warp completes the header
@@ -25,6 +25,9 @@ struct EncTotals {
     uint32_t summed;             // CTAs whose records' checksums are in
 };
 
+static_assert(sizeof(EncTotals) <= 64, "the sums of pass 1 follow in the scratch");
+
+constexpr uint32_t kScanThreads = 1024;      // chunks of a scan CTA
 constexpr uint32_t kNoCode = 1u << 20;       // length of a symbol without codeword: makes any sum it is part of stand out
 
 struct EncArgs {
@@ -32,7 +35,8 @@ struct EncArgs {
     uint64_t rows, cols, n_chunks;
     uint32_t Kc, KC, fp16, lag_bits, pad, vec_ok;
     uint64_t max_units;          // what the blob has room for
-    uint32_t *words, *chunk_bits, *index;
+    unsigned long long *groups;  // per kScanThreads chunks: their words | their coded bits << 32
+    uint32_t *words, *index;
     uint8_t *blob, *payload;
     EncTotals *totals;
     uint32_t code[256];          // stream bits of a symbol's codeword | its length << 16
@@ -164,26 +168,33 @@ __global__ void __launch_bounds__(kSizeThreads) encode_size_kernel(const __grid_
         atomicAdd(&s_sum[T.sub], bits);
     }
     __syncthreads();
-    if (T.active && T.q == 0) {
-        A.words[T.c] = max(1u, (s_max[T.sub] + 31) / 32);
-        A.chunk_bits[T.c] = s_sum[T.sub];
+    if (threadIdx.x >= 32) return;
+    const uint64_t c = (uint64_t)blockIdx.x * kSizeChunks + threadIdx.x;
+    unsigned long long sum = 0;                            // (1024 chunks: fewer than 2^19 words and 2^30 bits)
+    if (threadIdx.x < kSizeChunks && c < A.n_chunks) {
+        const uint32_t W = max(1u, (s_max[threadIdx.x] + 31) / 32);
+        A.words[c] = W;
+        sum = (unsigned long long)s_sum[threadIdx.x] << 32 | W;
     }
+#pragma unroll
+    for (uint32_t o = kSizeChunks / 2; o; o >>= 1) sum += __shfl_xor_sync(0xFFFFFFFFu, sum, o);
+    if (threadIdx.x == 0) atomicAdd(A.groups + c / kScanThreads, sum);
 }
 
-// Record offsets: an exclusive prefix sum of the record sizes (in 128-byte units).  A CTA takes 1024 chunks and sums the words
-// of every chunk in front of them itself (the raw parts in front are known without a sum), so that no CTA waits for another;
-// a single CTA walking all chunks took 20 us for the 11008 chunks of an 11008 x 4096 tensor, most of it barriers.
-constexpr uint32_t kScanThreads = 1024;
+// Record offsets: an exclusive prefix sum of the record sizes (in 128-byte units).  A CTA takes 1024 chunks and sums what pass 1
+// has left of every 1024 chunks in front of them itself (the raw parts in front are known without a sum), so that no CTA waits
+// for another; a single CTA walking all chunks took 20 us for the 11008 chunks of an 11008 x 4096 tensor, most of it barriers.
+// (At 11008 / 88064 / 1.05 M chunks: one CTA 20 / 142 / 1677 us; every chunk in front read by every CTA, which grows with the square
+// of the chunks, 6.8 / 13 / 130; this 5.7 / 6.7 / 31.)
 __global__ void __launch_bounds__(kScanThreads) encode_scan_kernel(const __grid_constant__ EncArgs A) {
     __shared__ unsigned long long s_warp[32], s_front[32];
     const uint32_t tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-    const uint64_t first = (uint64_t)blockIdx.x * kScanThreads, c = first + tid;
+    const uint64_t c = (uint64_t)blockIdx.x * kScanThreads + tid;
     const uint32_t raw_full = enc_raw_bytes(A, enc_blocks_of(A, 0)) / kRecordUnit, raw_last = enc_raw_bytes(A, enc_blocks_of(A, A.KC - 1)) / kRecordUnit;
     unsigned long long front = 0;                           // words of the chunks in front of the CTA's
-#pragma unroll 8
-    for (uint64_t i = tid; i < first; i += kScanThreads) front += __ldcg(A.words + i);
+    for (uint32_t i = tid; i < blockIdx.x; i += kScanThreads) front += (uint32_t)__ldcg(A.groups + i);
     const uint32_t W = c < A.n_chunks ? __ldcg(A.words + c) : 0u;
-    unsigned long long bits = c < A.n_chunks ? __ldcg(A.chunk_bits + c) : 0u, incl = W;
+    unsigned long long incl = W;
     uint32_t maxw = W;
 #pragma unroll
     for (int o = 1; o < 32; o <<= 1) {
@@ -193,13 +204,12 @@ __global__ void __launch_bounds__(kScanThreads) encode_scan_kernel(const __grid_
 #pragma unroll
     for (int o = 16; o; o >>= 1) {
         front += __shfl_xor_sync(0xFFFFFFFFu, front, o);
-        bits += __shfl_xor_sync(0xFFFFFFFFu, bits, o);
         maxw = max(maxw, __shfl_xor_sync(0xFFFFFFFFu, maxw, o));
     }
     if (lane == 31) s_warp[warp] = incl;
     if (lane == 0) {
         s_front[warp] = front;
-        if (bits) atomicAdd(&A.totals->coded_bits, bits);
+        if (tid == 0 && c < A.n_chunks) atomicAdd(&A.totals->coded_bits, __ldcg(A.groups + blockIdx.x) >> 32);
         if (maxw) atomicMax(&A.totals->max_words, maxw);
     }
     __syncthreads();
@@ -539,8 +549,9 @@ extern "C" huffllm_status huffllm_encode_device(const huffllm_codebook *cb, cons
     A.vec_ok = (cols % 8 == 0 && ((uintptr_t)w_dev & 15u) == 0) ? 1u : 0u;
     A.max_units = blob_cap >= d.off_payload + kTailSlack ? (blob_cap - d.off_payload - kTailSlack) / kRecordUnit : 0;
     A.totals = (EncTotals *)scr;
-    A.words = (uint32_t *)(scr + 256);
-    A.chunk_bits = A.words + d.n_chunks;
+    A.groups = (unsigned long long *)(scr + 64);               // (8 bytes per 1024 chunks: fewer than the 192 + 4 n in front of the words)
+    A.words = (uint32_t *)(scr + 256 + 4 * d.n_chunks);
+    const size_t cleared = 64 + 8 * ((d.n_chunks + kScanThreads - 1) / kScanThreads);
     A.index = (uint32_t *)(blob + d.off_index);
     A.blob = blob;
     A.payload = blob + d.off_payload;
@@ -567,7 +578,7 @@ extern "C" huffllm_status huffllm_encode_device(const huffllm_codebook *cb, cons
     write_fixed_sections(cb, d, fixed.data());
     memset(fixed.data(), 0, sizeof(d));
     if ((e = cudaMemcpyAsync(blob, fixed.data(), fixed.size(), cudaMemcpyHostToDevice, s)) != cudaSuccess) return cuda_fail("copy of the fixed sections");
-    if ((e = cudaMemsetAsync(scr, 0, 256, s)) != cudaSuccess) return cuda_fail("cudaMemsetAsync");
+    if ((e = cudaMemsetAsync(scr, 0, cleared, s)) != cudaSuccess) return cuda_fail("cudaMemsetAsync");
     size_kernel<<<(uint32_t)((d.n_chunks + kSizeChunks - 1) / kSizeChunks), kSizeThreads, 0, s>>>(A);
     encode_scan_kernel<<<(uint32_t)((d.n_chunks + 64 + kScanThreads - 1) / kScanThreads), kScanThreads, 0, s>>>(A);
     write_kernel<<<(uint32_t)d.n_chunks, kWriteThreads, smem, s>>>(A);
