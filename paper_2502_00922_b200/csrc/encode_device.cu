@@ -7,7 +7,7 @@
 //   pass 1  code lengths only -> words per sequence of every chunk; words and coded bits of every 1024 chunks
 //   scan    record offsets (the index section), payload size, largest record
 //   pass 2  raw part and coded part of every record (nothing if the scan found the tensor or the buffer unfit)
-//   pass 3  the checksum term of every record, a warp each; the last warp completes the header
+//   pass 3  the checksum term of every record, a warp each (many short records: a thread); the last one completes the header
 // The host waits once, behind the last pass.
 #include <cuda_runtime.h>
 
@@ -458,6 +458,17 @@ __host__ __device__ inline void enc_fill_totals(huffllm_desc &d, const volatile 
     d.payload_checksum = t.checksum;
 }
 
+// One thread of every checksum CTA, with the CTA's sum; the last one to come completes the header.
+__device__ __forceinline__ void finish_checksum(const EncArgs &A, unsigned long long term) {
+    atomicAdd(&A.totals->checksum, term);
+    __threadfence();
+    if (atomicAdd(&A.totals->summed, 1u) != gridDim.x - 1u) return;
+    __threadfence();
+    huffllm_desc d = A.desc;
+    enc_fill_totals(d, *(const volatile EncTotals *)A.totals);
+    *(huffllm_desc *)A.blob = d;
+}
+
 constexpr uint32_t kSumWarps = 8;
 
 __global__ void __launch_bounds__(32 * kSumWarps) encode_checksum_kernel(const __grid_constant__ EncArgs A) {
@@ -493,14 +504,41 @@ __global__ void __launch_bounds__(32 * kSumWarps) encode_checksum_kernel(const _
     if (threadIdx.x) return;
     unsigned long long term = 0;
     for (uint32_t i = 0; i < kSumWarps; ++i) term += s_term[i];
-    atomicAdd(&A.totals->checksum, term);
-    __threadfence();
-    if (atomicAdd(&A.totals->summed, 1u) != gridDim.x - 1u) return;
-    // every record is in: the header
-    __threadfence();
-    huffllm_desc d = A.desc;
-    enc_fill_totals(d, *(const volatile EncTotals *)A.totals);
-    *(huffllm_desc *)A.blob = d;
+    finish_checksum(A, term);
+}
+
+// The same with a thread per record, as the hash is written.  A record takes a thread some 30 ns per byte (one load in flight),
+// but a GPU full of threads takes less than half of what the warps above need per byte, who pay for whole steps of 1.5 KB whatever
+// the record's size: with enough records this is faster, the sooner the shorter they are.  (Warps / threads: 88064 records of 512
+// weights 159 / 44 us, 1.05 M of them 1.75 / 0.33 ms, 44032 of 1024 104 / 62 us; whole calls: 16384 of 512 114 / 106, 8192 of 1024
+// 90 / 117, 22016 of 2048 175 / 217, 114688 of 2048 648 / 573, 57344 of 4096 558 / 547, 28672 of 8192 542 / 688.)
+constexpr uint32_t kEachThreads = 128;
+inline bool checksum_each(uint64_t n_chunks, uint32_t chunk_elems) { return n_chunks >= 16384ull + 8ull * chunk_elems; }
+__global__ void __launch_bounds__(kEachThreads) encode_checksum_each_kernel(const __grid_constant__ EncArgs A) {
+    __shared__ unsigned long long s_term[kEachThreads / 32];
+    const uint64_t c = (uint64_t)blockIdx.x * kEachThreads + threadIdx.x;
+    if (!enc_fits(A)) return;
+    unsigned long long term = 0;
+    if (c < A.n_chunks) {
+        const uint32_t r0 = A.index[c], n = (A.index[c + 1] - r0) * (kRecordUnit / 16);
+        const uint4 *p = (const uint4 *)(A.payload + (uint64_t)r0 * kRecordUnit);
+        uint64_t h = kFnvStart;
+        for (uint32_t i = 0; i < n; ++i) {
+            const uint4 q = __ldcg(p + i);
+            const uint32_t x[4] = {q.x, q.y, q.z, q.w};
+#pragma unroll
+            for (int k = 0; k < 16; ++k) h = (h ^ ((x[k >> 2] >> (8 * (k & 3))) & 0xFFu)) * kFnvPrime;
+        }
+        term = n ? h * (2 * c + 1) : 0ull;
+    }
+#pragma unroll
+    for (int o = 16; o; o >>= 1) term += __shfl_xor_sync(0xFFFFFFFFu, term, o);
+    if ((threadIdx.x & 31) == 0) s_term[threadIdx.x >> 5] = term;
+    __syncthreads();
+    if (threadIdx.x) return;
+    term = 0;
+    for (uint32_t i = 0; i < kEachThreads / 32; ++i) term += s_term[i];
+    finish_checksum(A, term);
 }
 
 }  // namespace huffllm
@@ -582,7 +620,10 @@ extern "C" huffllm_status huffllm_encode_device(const huffllm_codebook *cb, cons
     size_kernel<<<(uint32_t)((d.n_chunks + kSizeChunks - 1) / kSizeChunks), kSizeThreads, 0, s>>>(A);
     encode_scan_kernel<<<(uint32_t)((d.n_chunks + 64 + kScanThreads - 1) / kScanThreads), kScanThreads, 0, s>>>(A);
     write_kernel<<<(uint32_t)d.n_chunks, kWriteThreads, smem, s>>>(A);
-    encode_checksum_kernel<<<(uint32_t)((d.n_chunks + kSumWarps - 1) / kSumWarps), 32 * kSumWarps, 0, s>>>(A);
+    if (checksum_each(d.n_chunks, chunk_elems))
+        encode_checksum_each_kernel<<<(uint32_t)((d.n_chunks + kEachThreads - 1) / kEachThreads), kEachThreads, 0, s>>>(A);
+    else
+        encode_checksum_kernel<<<(uint32_t)((d.n_chunks + kSumWarps - 1) / kSumWarps), 32 * kSumWarps, 0, s>>>(A);
     if ((e = cudaGetLastError()) != cudaSuccess) return cuda_fail("encoder launches");
     EncTotals tot;
     if ((e = cudaMemcpyAsync(&tot, scr, sizeof(tot), cudaMemcpyDeviceToHost, s)) != cudaSuccess || (e = cudaStreamSynchronize(s)) != cudaSuccess)

@@ -116,6 +116,7 @@ def test_device_encoder_writes_the_host_encoders_blob(hl, rows, cols, ce, kind, 
     (16, 32 * 1025, 512, "constant", 0, 0, 0),
     (1040, 1024, 512, "fp16", 1, 7, 0),              # 2080 chunks, records of an odd number of 128-byte units
     (33, 32 * 20011 - 5, 512, "gauss", 0, 0, 0),     # 60033 chunks: a scan CTA has 58 sums in front of it
+    (16, 32 * 20483, 512, "fp16", 1, 12, 2),         # 20483 chunks: a thread per record in the checksum pass
 ])
 def test_device_encoder_at_the_edges_of_its_passes(hl, rows, cols, ce, kind, dtype, budget, offset):
     """Loads that are not aligned, sequences that fill their rows, the scan's and the checksum's borders: host blob, byte for byte."""
