@@ -34,6 +34,7 @@ struct EncArgs {
     const uint16_t *w;
     uint64_t rows, cols, n_chunks;
     uint32_t Kc, KC, fp16, lag_bits, pad, vec_ok;
+    uint32_t most_words;         // rows of the largest record this code can give a full chunk
     uint64_t max_units;          // what the blob has room for
     unsigned long long *groups;  // per kScanThreads chunks: their words | their coded bits << 32
     uint32_t *words, *index;
@@ -226,23 +227,29 @@ __global__ void __launch_bounds__(kScanThreads) encode_scan_kernel(const __grid_
     }
 }
 
-// Pass 2.  A CTA of 64 threads takes a chunk and collects the coded part in shared memory, row by row as the record has it:
-// stored straight from the threads, whose streams run apart, the words went to L2 one by one as partial sectors.
-constexpr uint32_t kWriteThreads = 64;
-// coded part of the largest chunk (1024 columns) under the longest codes: FP16, three fields of 12 bits
-constexpr uint32_t kMostCodedBytes = (7 + 32 * 8 * 3 * 12 + 31) / 32 * 256;
-template <bool FP16>
-__global__ void __launch_bounds__(kWriteThreads) encode_write_kernel(const __grid_constant__ EncArgs A) {
+// Pass 2.  64 threads take a chunk and collect the coded part in shared memory (STAGED), row by row as the record has it: stored
+// straight from the threads, whose streams run apart, the words go to L2 one by one as partial sectors.  Short chunks share a
+// CTA of four, whose table and set-up they share too; above 512 columns, where shared memory leaves an SM few warps, straight
+// stores are the better choice.  (11008 x 4096: chunks of 512 / 1024 one to a CTA 185 / 97 us, four 90 / 56; FP16 16384 under codes of
+// up to 12 bits staged 157, straight 98.  Whole calls on 28672 x 8192, staged / straight: 2048 574 / 594, 4096 558 / 572, 16384 551 /
+// 526, FP16 995 / 831; at 8192 542 / 526 there, but 158 / 165 on 11008 x 4096.)
+template <bool FP16, uint32_t CHUNKS, bool STAGED>
+__global__ void __launch_bounds__(64 * CHUNKS) encode_write_kernel(const __grid_constant__ EncArgs A) {
     extern __shared__ __align__(16) uint32_t s_coded[];
     __shared__ uint32_t s_code[256];
 #pragma unroll
-    for (uint32_t i = 0; i < 256 / kWriteThreads; ++i) s_code[i * kWriteThreads + threadIdx.x] = A.code[i * kWriteThreads + threadIdx.x];
+    for (uint32_t i = threadIdx.x; i < 256; i += 64 * CHUNKS) s_code[i] = A.code[i];
     if (!enc_fits(A)) return;
     __syncthreads();
-    const EncThread T = enc_thread<1>(A);
+    const EncThread T = enc_thread<CHUNKS>(A);
+    if (CHUNKS > 1 && !T.active) {                                // (a chunk's two warps leave or stay together)
+        if (STAGED) __syncthreads();
+        return;
+    }
     const uint32_t W = A.words[T.c], raw_bytes = enc_raw_bytes(A, T.nkb);
     uint8_t *raw = A.payload + (uint64_t)A.index[T.c] * kRecordUnit;
-    uint32_t *out = s_coded + T.seq;                              // word j of this sequence at out[64 j]
+    uint32_t *const rows = STAGED ? s_coded + T.sub * A.most_words * 64 : (uint32_t *)(raw + raw_bytes);
+    uint32_t *out = rows + T.seq;                                 // word j of this sequence at out[64 j]
     uint32_t acc = 0, nacc = A.lag_bits;
     auto append = [&](uint32_t b, uint32_t len) {                 // len <= 24, nacc < 32
         acc |= b << nacc;
@@ -283,19 +290,30 @@ __global__ void __launch_bounds__(kWriteThreads) encode_write_kernel(const __gri
             *(uint2 *)(raw + kb * 512 + T.lane * 16 + T.half * 8) = make_uint2(word[0], word[1]);
         }
     }
-    uint32_t *const end = s_coded + T.seq + (size_t)64 * W;
+    uint32_t *const end = rows + T.seq + (size_t)64 * W;
     if (nacc) {
         *out = acc;
         out += 64;
     }
     for (; out < end; out += 64) *out = 0;
     if (FP16 && (T.nkb & 1u) && T.q < 32) *(uint16_t *)(raw + T.nkb * 64 + T.q * 2) = 0;   // padding of the sign plane
-    __syncthreads();
-    for (uint32_t i = T.q; i < W * 16; i += kWriteThreads) ((uint4 *)(raw + raw_bytes))[i] = ((const uint4 *)s_coded)[i];
+    if (STAGED) {
+        __syncthreads();
+        for (uint32_t i = T.q; i < W * 16; i += 64) ((uint4 *)(raw + raw_bytes))[i] = ((const uint4 *)rows)[i];
+    }
     if (T.c + 1 == A.n_chunks) {                                  // the zero bytes behind the payload
         uint4 *tail = (uint4 *)(A.payload + __ldcg(&A.totals->payload_units) * kRecordUnit);
-        for (uint32_t i = T.q; i < kTailSlack / 16; i += kWriteThreads) tail[i] = make_uint4(0, 0, 0, 0);
+        for (uint32_t i = T.q; i < kTailSlack / 16; i += 64) tail[i] = make_uint4(0, 0, 0, 0);
     }
+}
+
+inline uint32_t write_chunks(const EncArgs &A) { return A.Kc <= 128 ? 4 : 1; }
+inline bool write_staged(const EncArgs &A) { return A.Kc <= 512; }      // (at most 37 KB of shared memory)
+inline void (*write_kernel_of(bool fp16, uint32_t chunks, bool staged))(EncArgs) {
+    if (fp16) return chunks == 4 ? (staged ? encode_write_kernel<true, 4, true> : encode_write_kernel<true, 4, false>)
+                                 : (staged ? encode_write_kernel<true, 1, true> : encode_write_kernel<true, 1, false>);
+    return chunks == 4 ? (staged ? encode_write_kernel<false, 4, true> : encode_write_kernel<false, 4, false>)
+                       : (staged ? encode_write_kernel<false, 1, true> : encode_write_kernel<false, 1, false>);
 }
 
 // ------------------------------------------------------------------------------ checksum of the records
@@ -601,16 +619,13 @@ extern "C" huffllm_status huffllm_encode_device(const huffllm_codebook *cb, cons
         A.code[i] = bits[i] | (uint32_t)len[i] << 16;
         longest = std::max<uint32_t>(longest, len[i]);
     }
-    // rows of the largest record this code can give a full chunk (the sizes are known on the device only)
-    const uint32_t most_words = (d.lag_bits + Kc / kBlockCols * 8 * longest * (A.fp16 ? 3 : 1) + 31) / 32;
-    const size_t smem = (size_t)most_words * 256;
+    A.most_words = (d.lag_bits + Kc / kBlockCols * 8 * longest * (A.fp16 ? 3 : 1) + 31) / 32;    // (the sizes are known on the device only)
 
     cudaError_t e;
     auto cuda_fail = [&](const char *what) { return fail(HUFFLLM_ERR_CUDA, "%s: %s", what, cudaGetErrorString(e)); };
     const auto size_kernel = A.fp16 ? encode_size_kernel<true> : encode_size_kernel<false>;
-    const auto write_kernel = A.fp16 ? encode_write_kernel<true> : encode_write_kernel<false>;
-    if ((e = cudaFuncSetAttribute(write_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kMostCodedBytes)) != cudaSuccess)
-        return cuda_fail("cudaFuncSetAttribute");
+    const uint32_t chunks = write_chunks(A), smem = write_staged(A) ? chunks * A.most_words * 256 : 0;
+    const auto write_kernel = write_kernel_of(A.fp16 != 0, chunks, smem != 0);
     // code lengths and table, assembled on the host; the header's bytes stay zero until the last kernel writes them
     std::vector<uint8_t> fixed((size_t)d.off_index, 0);
     write_fixed_sections(cb, d, fixed.data());
@@ -619,7 +634,7 @@ extern "C" huffllm_status huffllm_encode_device(const huffllm_codebook *cb, cons
     if ((e = cudaMemsetAsync(scr, 0, cleared, s)) != cudaSuccess) return cuda_fail("cudaMemsetAsync");
     size_kernel<<<(uint32_t)((d.n_chunks + kSizeChunks - 1) / kSizeChunks), kSizeThreads, 0, s>>>(A);
     encode_scan_kernel<<<(uint32_t)((d.n_chunks + 64 + kScanThreads - 1) / kScanThreads), kScanThreads, 0, s>>>(A);
-    write_kernel<<<(uint32_t)d.n_chunks, kWriteThreads, smem, s>>>(A);
+    write_kernel<<<(uint32_t)((d.n_chunks + chunks - 1) / chunks), 64 * chunks, smem, s>>>(A);
     if (checksum_each(d.n_chunks, chunk_elems))
         encode_checksum_each_kernel<<<(uint32_t)((d.n_chunks + kEachThreads - 1) / kEachThreads), kEachThreads, 0, s>>>(A);
     else
