@@ -34,6 +34,7 @@ struct EncArgs {
     const uint16_t *w;
     uint64_t rows, cols, n_chunks;
     uint32_t Kc, KC, fp16, lag_bits, pad, vec_ok;
+    uint32_t size_groups;        // groups of kSizeChunks chunks that a CTA of pass 1 takes, one after the other
     uint32_t most_words;         // rows of the largest record this code can give a full chunk
     uint64_t max_units;          // what the blob has room for
     unsigned long long *groups;  // per kScanThreads chunks: their words | their coded bits << 32
@@ -106,16 +107,16 @@ struct EncThread {
     EncRow row;
     bool active;
 };
-// CHUNKS chunks per CTA, 64 threads each
+// 64 threads for each of the CHUNKS chunks of a group
 template <uint32_t CHUNKS>
-__device__ __forceinline__ EncThread enc_thread(const EncArgs &A) {
+__device__ __forceinline__ EncThread enc_thread(const EncArgs &A, uint32_t group) {
     EncThread T;
     T.sub = threadIdx.x >> 6;
     T.q = threadIdx.x & 63;
     T.lane = T.q >> 1;
     T.half = T.q & 1;
     T.seq = T.lane + 32 * T.half;
-    T.c = (uint64_t)blockIdx.x * CHUNKS + T.sub;
+    T.c = (uint64_t)group * CHUNKS + T.sub;
     T.active = T.c < A.n_chunks;
     const uint64_t cc = T.active ? T.c : 0;
     const uint32_t rg = (uint32_t)cc / A.KC, kc = (uint32_t)cc - rg * A.KC;       // (fewer than 2^31 chunks)
@@ -133,53 +134,64 @@ template <bool FP16>
 __global__ void __launch_bounds__(kSizeThreads) encode_size_kernel(const __grid_constant__ EncArgs A) {
     __shared__ uint32_t s_max[kSizeChunks], s_sum[kSizeChunks], s_len[256];
     s_len[threadIdx.x] = A.code[threadIdx.x] >> 16 ? A.code[threadIdx.x] >> 16 : kNoCode;
-    if (threadIdx.x < kSizeChunks) s_max[threadIdx.x] = s_sum[threadIdx.x] = 0;
-    __syncthreads();
-    const EncThread T = enc_thread<kSizeChunks>(A);
-    if (T.active) {
-        uint32_t bits = 0;
-        const char *len = (const char *)s_len;
-        auto at = [&](uint32_t byte_off) -> uint32_t { return *(const uint32_t *)(len + byte_off); };
-        auto add = [&](const uint4 &v) {
-            const uint32_t x[4] = {v.x, v.y, v.z, v.w};
+#pragma unroll 1
+    for (uint32_t it = 0; it < A.size_groups; ++it) {
+        const uint32_t group = blockIdx.x * A.size_groups + it;
+        if (threadIdx.x < kSizeChunks) s_max[threadIdx.x] = s_sum[threadIdx.x] = 0;
+        __syncthreads();
+        const EncThread T = enc_thread<kSizeChunks>(A, group);
+        if (T.active) {
+            uint32_t bits = 0;
+            const char *len = (const char *)s_len;
+            auto at = [&](uint32_t byte_off) -> uint32_t { return *(const uint32_t *)(len + byte_off); };
+            auto add = [&](const uint4 &v) {
+                const uint32_t x[4] = {v.x, v.y, v.z, v.w};
 #pragma unroll
-            for (int i = 0; i < 4; ++i) {
-                if (FP16) {
-                    bits += at((x[i] >> 8) & 0x7Cu) + at(128u + ((x[i] >> 3) & 0x7Cu)) + at(256u + ((x[i] << 2) & 0x7Cu));
-                    bits += at((x[i] >> 24) & 0x7Cu) + at(128u + ((x[i] >> 19) & 0x7Cu)) + at(256u + ((x[i] >> 14) & 0x7Cu));
-                } else {
-                    bits += at((x[i] >> 5) & 0x3FCu) + at((x[i] >> 21) & 0x3FCu);
+                for (int i = 0; i < 4; ++i) {
+                    if (FP16) {
+                        bits += at((x[i] >> 8) & 0x7Cu) + at(128u + ((x[i] >> 3) & 0x7Cu)) + at(256u + ((x[i] << 2) & 0x7Cu));
+                        bits += at((x[i] >> 24) & 0x7Cu) + at(128u + ((x[i] >> 19) & 0x7Cu)) + at(256u + ((x[i] >> 14) & 0x7Cu));
+                    } else {
+                        bits += at((x[i] >> 5) & 0x3FCu) + at((x[i] >> 21) & 0x3FCu);
+                    }
                 }
+            };
+            uint32_t kb = 0;
+            for (; kb + 4 <= T.nkb; kb += 4) {
+                uint4 v[4];
+#pragma unroll
+                for (int i = 0; i < 4; ++i) v[i] = enc_load8(A, T.row, kb + i);
+#pragma unroll
+                for (int i = 0; i < 4; ++i) add(v[i]);
             }
-        };
-        uint32_t kb = 0;
-        for (; kb + 4 <= T.nkb; kb += 4) {
-            uint4 v[4];
-#pragma unroll
-            for (int i = 0; i < 4; ++i) v[i] = enc_load8(A, T.row, kb + i);
-#pragma unroll
-            for (int i = 0; i < 4; ++i) add(v[i]);
+            for (; kb < T.nkb; ++kb) add(enc_load8(A, T.row, kb));
+            if (bits >= kNoCode) {
+                atomicOr(&A.totals->bad, 1u);
+                bits = 0;
+            }
+            atomicMax(&s_max[T.sub], bits + A.lag_bits);
+            atomicAdd(&s_sum[T.sub], bits);
         }
-        for (; kb < T.nkb; ++kb) add(enc_load8(A, T.row, kb));
-        if (bits >= kNoCode) {
-            atomicOr(&A.totals->bad, 1u);
-            bits = 0;
+        __syncthreads();
+        if (threadIdx.x >= 32) continue;
+        const uint64_t c = (uint64_t)group * kSizeChunks + threadIdx.x;
+        unsigned long long sum = 0;                        // (1024 chunks: fewer than 2^19 words and 2^30 bits)
+        if (threadIdx.x < kSizeChunks && c < A.n_chunks) {
+            const uint32_t W = max(1u, (s_max[threadIdx.x] + 31) / 32);
+            A.words[c] = W;
+            sum = (unsigned long long)s_sum[threadIdx.x] << 32 | W;
         }
-        atomicMax(&s_max[T.sub], bits + A.lag_bits);
-        atomicAdd(&s_sum[T.sub], bits);
-    }
-    __syncthreads();
-    if (threadIdx.x >= 32) return;
-    const uint64_t c = (uint64_t)blockIdx.x * kSizeChunks + threadIdx.x;
-    unsigned long long sum = 0;                            // (1024 chunks: fewer than 2^19 words and 2^30 bits)
-    if (threadIdx.x < kSizeChunks && c < A.n_chunks) {
-        const uint32_t W = max(1u, (s_max[threadIdx.x] + 31) / 32);
-        A.words[c] = W;
-        sum = (unsigned long long)s_sum[threadIdx.x] << 32 | W;
-    }
 #pragma unroll
-    for (uint32_t o = kSizeChunks / 2; o; o >>= 1) sum += __shfl_xor_sync(0xFFFFFFFFu, sum, o);
-    if (threadIdx.x == 0) atomicAdd(A.groups + c / kScanThreads, sum);
+        for (uint32_t o = kSizeChunks / 2; o; o >>= 1) sum += __shfl_xor_sync(0xFFFFFFFFu, sum, o);
+        if (threadIdx.x == 0 && sum) atomicAdd(A.groups + c / kScanThreads, sum);
+    }
+}
+
+// A group's threads have a block or two each where chunks are short, less than the table costs their CTA: eight blocks per thread
+// are worth going on for, as long as the GPU stays full.  (Chunks of 512: 11008 x 4096 88 -> 82 us, 65536 x 8192 1070 -> 847.)
+inline uint32_t size_groups(const EncArgs &A) {
+    const uint64_t full = A.n_chunks / (kSizeChunks * 8 * 148), want = 8 / (A.Kc / kBlockCols);
+    return (uint32_t)std::max<uint64_t>(1, std::min<uint64_t>(full, want));
 }
 
 // Record offsets: an exclusive prefix sum of the record sizes (in 128-byte units).  A CTA takes 1024 chunks and sums what pass 1
@@ -241,7 +253,7 @@ __global__ void __launch_bounds__(64 * CHUNKS) encode_write_kernel(const __grid_
     for (uint32_t i = threadIdx.x; i < 256; i += 64 * CHUNKS) s_code[i] = A.code[i];
     if (!enc_fits(A)) return;
     __syncthreads();
-    const EncThread T = enc_thread<CHUNKS>(A);
+    const EncThread T = enc_thread<CHUNKS>(A, blockIdx.x);
     if (CHUNKS > 1 && !T.active) {                                // (a chunk's two warps leave or stay together)
         if (STAGED) __syncthreads();
         return;
@@ -632,7 +644,9 @@ extern "C" huffllm_status huffllm_encode_device(const huffllm_codebook *cb, cons
     memset(fixed.data(), 0, sizeof(d));
     if ((e = cudaMemcpyAsync(blob, fixed.data(), fixed.size(), cudaMemcpyHostToDevice, s)) != cudaSuccess) return cuda_fail("copy of the fixed sections");
     if ((e = cudaMemsetAsync(scr, 0, cleared, s)) != cudaSuccess) return cuda_fail("cudaMemsetAsync");
-    size_kernel<<<(uint32_t)((d.n_chunks + kSizeChunks - 1) / kSizeChunks), kSizeThreads, 0, s>>>(A);
+    A.size_groups = size_groups(A);
+    const uint64_t per_cta = (uint64_t)kSizeChunks * A.size_groups;
+    size_kernel<<<(uint32_t)((d.n_chunks + per_cta - 1) / per_cta), kSizeThreads, 0, s>>>(A);
     encode_scan_kernel<<<(uint32_t)((d.n_chunks + 64 + kScanThreads - 1) / kScanThreads), kScanThreads, 0, s>>>(A);
     write_kernel<<<(uint32_t)((d.n_chunks + chunks - 1) / chunks), 64 * chunks, smem, s>>>(A);
     if (checksum_each(d.n_chunks, chunk_elems))
