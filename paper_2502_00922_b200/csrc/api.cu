@@ -708,7 +708,8 @@ huffllm_status huffllm_decode_gemm(const huffllm_desc *desc, const void *blob, c
         // 9..16 vectors: the tensor-core kernel, whose time does not grow with the batch below its padding of 16, is the
         // faster one for matrices that are at least as wide as tall (few row groups per SM make the register path's
         // cross-CTA sums of 16-vector pieces expensive), unless they have so few rows that it gets few row tiles; measured
-        // at 12 and 16 vectors on seven shapes from 1024 x 8192 to 28672 x 8192.  Above 16 vectors it is the only one.
+        // at 12 and 16 vectors on seven shapes from 1024 x 8192 to 28672 x 8192, before that kernel had column slices (the line has
+        // not been drawn again).  Above 16 vectors it is the only one.
         const bool wide = desc->cols >= desc->rows && desc->rows >= 2048;
         if (!wide && (st = two_tiles()) != HUFFLLM_OK) return st;
         if (!done && (st = tensor_core(wide && batch <= kTwoTileBatch && two_tile_blob(desc))) != HUFFLLM_OK) return st;
