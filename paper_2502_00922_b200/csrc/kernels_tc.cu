@@ -174,14 +174,14 @@ __global__ void __launch_bounds__(1024, 1) huff_gemm_tc_kernel(const __grid_cons
     // `rgi` there and decodes if the CTA has that many.  Where all 32 warps belong to slices (four tiles) a slice's warp that does
     // not decode carries its activations, the very last one, the issuer, only where its slice has no other; with fewer tiles
     // (one slice) the first warp behind the tiles carries them and the others in front of the issuer leave at once.  (With the
-    // issuer carrying them there too and issuing in a loop over the tiles, 8192 x 28672 in chunks of 8192 elements took 242 us
-    // at 64 vectors against 181, 12288 x 12288 148 against 115.)
+    // issuer carrying them there too, chunks of 8192 elements took, back to back, 230 us against 172 for 8192 x 28672 at 64 vectors,
+    // 111 against 94 for 12288 x 12288 at 32.)
     const uint32_t S = A.tc_stages, slices = A.tc_slices, na = A.tc_tiles, tiles = na * slices, issuer = 31u;
     const uint32_t n_rg = A.tc_row_groups, n_dec = n_rg * slices;
-    const uint32_t slice = min(warp / (8u * na), slices - 1u), li = warp - warp / (8u * na) * 8u * na;
+    const uint32_t slice = warp == issuer || warp >= tiles * 8u ? slices - 1u : warp / (8u * na), li = warp - warp / (8u * na) * 8u * na;
     const uint32_t tile = warp >> 3, q = warp & 3, h = (warp >> 2) & 1, rgi = (li & ~7u) + q * 2 + h;
-    const bool decodes = warp < tiles * 8u && rgi < n_rg, serves = warp != issuer && (warp < tiles * 8u ? rgi >= n_rg : warp == tiles * 8u);
-    const bool issuer_carries = n_rg == na * 8u - 1u;
+    const bool decodes = warp < tiles * 8u && rgi < n_rg, serves = warp != issuer && warp <= tiles * 8u && (rgi >= n_rg || warp == tiles * 8u);
+    const bool issuer_carries = tiles == 4u && n_rg == na * 8u - 1u;
     const uint32_t a_lane = (32u * q + 16u * h) << 16;
     const uint32_t KC = k.col_chunks, RG = (uint32_t)((k.rows + 15) / 16);
     const uint32_t *index = (const uint32_t *)(k.blob + k.off_index);
@@ -286,7 +286,7 @@ __global__ void __launch_bounds__(1024, 1) huff_gemm_tc_kernel(const __grid_cons
     __syncthreads();
     tc_fence_after();
     const uint32_t tmem = s_tmem_base;
-    if (!decodes && !serves && warp != issuer) {  // in no tile: only the teardown barrier is left
+    if (warp > tiles * 8u && warp != issuer) {    // in no tile: only the teardown barrier is left
         tc_fence_before();
         __syncthreads();
         return;
@@ -382,33 +382,30 @@ __global__ void __launch_bounds__(1024, 1) huff_gemm_tc_kernel(const __grid_cons
     // What bounds this warp is the number of instructions per MMA (its scheduler has seven decoding warps to serve, so each
     // costs some eight cycles): the thread is elected, not chosen by its number, and every operand is a base and a constant,
     // so that addresses and descriptors are worked out on the uniform datapath, where the MMA wants them.  (28672 x 8192 at
-    // 32 vectors: 154 us with a loop over runtime strides in lane 0, 127 so; a stage's 16 MMAs take 500 to 600 cycles.)
-    auto issue_tiles = [&](auto n_slices, bool first_of_item, uint32_t n_tiles) {  // a stage whose slices all have two blocks
+    // 32 vectors: 154 us with a loop over runtime strides in lane 0, 127 so; a stage's 16 MMAs take 500 to 600 cycles.
+    // Unrolled for fewer tiles too, those launches took 1 to 2 % less, but those of four tiles up to 1 % more.)
+    auto issue_tiles = [&](auto n_slices, bool first_of_item) {                    // a stage of four tiles whose slices all have two blocks
         constexpr uint32_t SL = decltype(n_slices)::value, NA = 4u / SL;
         const uint32_t ac = tmem + kACol0 + st_s * 128u;
         const uint32_t bd = smem_desc_lo(b_base + st_s * SL * kBStage, kLbo);
 #pragma unroll
-        for (uint32_t t = 0; t < 4; ++t) {
-            if (t >= n_tiles) break;
+        for (uint32_t t = 0; t < 4; ++t)
 #pragma unroll
             for (uint32_t j = 0; j < 4; ++j)
                 tc_mma_f16_tmem_a(tmem + t * NPAD, ac + t * 32u + j * 8u, smem_desc(bd + ((t / NA * kBStage + j * 2u * kLbo) >> 4), kSbo), kIdesc,
                                   j == 0 ? (first_of_item ? 0u : 1u) : 1u);
-        }
     };
-    auto issue_stage = [&](bool first_of_item, bool full, auto halves) {           // full: two blocks of every slice
+    auto issue_stage = [&](bool first_of_item, bool full, auto halves) {           // full: four tiles, two blocks of every slice
         bounded_wait(smem_u32(&full_bar[st_s]), st_use & 1u);
         if (elect_one()) {
             tc_fence_after();
             if (failed) {
-            } else if (full && tiles < 4u) {
-                issue_tiles(std::integral_constant<uint32_t, 1>{}, first_of_item, tiles);
             } else if (full && slices == 1u) {
-                issue_tiles(std::integral_constant<uint32_t, 1>{}, first_of_item, 4u);
+                issue_tiles(std::integral_constant<uint32_t, 1>{}, first_of_item);
             } else if (full && slices == 2u) {
-                issue_tiles(std::integral_constant<uint32_t, 2>{}, first_of_item, 4u);
+                issue_tiles(std::integral_constant<uint32_t, 2>{}, first_of_item);
             } else if (full) {
-                issue_tiles(std::integral_constant<uint32_t, 4>{}, first_of_item, 4u);
+                issue_tiles(std::integral_constant<uint32_t, 4>{}, first_of_item);
             } else {
                 uint32_t ac = tmem + kACol0 + st_s * 128u;
                 for (uint32_t sl = 0; sl < slices; ++sl) {
@@ -543,7 +540,7 @@ __global__ void __launch_bounds__(1024, 1) huff_gemm_tc_kernel(const __grid_cons
                 }
                 for (uint32_t p = 0; p < n_st; ++p) {
                     if (issuer_carries) x_landed();
-                    issue_stage(j == 0 && p == 0, least >= 2 * p + 2, [&](uint32_t sl) -> uint32_t {
+                    issue_stage(j == 0 && p == 0, tiles == 4u && least >= 2 * p + 2, [&](uint32_t sl) -> uint32_t {
                         return halves(sl == 0 ? nkb[0] : sl == 1 ? nkb[1] : sl == 2 ? nkb[2] : nkb[3], p);
                     });
                     if (!issuer_carries) continue;
