@@ -82,6 +82,16 @@ struct SmemNeeds {
     uint32_t checks_per_block;           // refill checks per bit sequence and block of 32 columns
     uint32_t guard_bytes;                // readable bytes kept behind the last slot
 };
+// Which mantissa halves of an FP16 blob carry the flat code and can be read without a table (codes of at most 8 bits).
+uint32_t flat_of(const huffllm_desc *d) {
+    if (d->dtype != HUFFLLM_FP16 || d->lut_bits > 8) return kFlatNone;
+    return (d->flat_fields & 6u) == 6u ? kFlatBoth : d->flat_fields & 2u ? kFlatUpper : kFlatNone;
+}
+// ... and of several blobs.
+uint32_t flat_of_both(uint32_t a, uint32_t b) { return a == b ? a : a == kFlatNone || b == kFlatNone ? kFlatNone : kFlatUpper; }
+// Bytes of the FP16 tables (first level): three of 16 KB; the exponent's with a copy per lane and the lower half's with
+// sixteen; the exponent's alone.
+uint32_t fp16_table_bytes(uint32_t flat) { return flat == kFlatBoth ? 32768u : 49152u; }
 SmemNeeds smem_needs(const huffllm_desc *desc) {
     SmemNeeds n;
     const bool fmt = desc->dtype == HUFFLLM_FP16;
@@ -89,11 +99,10 @@ SmemNeeds smem_needs(const huffllm_desc *desc) {
     // first 8 bits, then one copy of the whole table behind it
     // (FP16: three sixteen-fold tables of 8 bits; fields of 9 bits and more take the second level too)
     const bool two_level = desc->lut_bits > (fmt ? 8u : 9u);
-    // (FP16 blobs whose mantissa codes are flat need the exponent's table only; a launch over several matrices of which
-    // some are not marked takes all three, see fp16_table_bytes)
+    // (FP16 blobs with flat mantissa codes need fewer tables; a launch over several matrices takes what all of them allow, see
+    // fp16_table_bytes)
     n.table_align = fmt ? 16384u : 128u << (two_level ? 8u : desc->lut_bits);
-    const bool flat = fmt && desc->lut_bits == 8 && (desc->flat_fields & 6u) == 6u;
-    n.table_bytes = fmt ? (flat ? 16384u : 49152u) + (two_level ? 3u * (4u << desc->lut_bits) : 0u)
+    n.table_bytes = fmt ? fp16_table_bytes(two_level ? kFlatNone : flat_of(desc)) + (two_level ? 3u * (4u << desc->lut_bits) : 0u)
                         : (two_level ? (128u << 8) + (4u << desc->lut_bits) : 128u << desc->lut_bits);
     // a slot holds the W rows of a record; the window runs one row ahead of what it consumes, and that look-ahead
     // past the last row lands in the next slot, the table or the guard area and is never used
@@ -117,7 +126,7 @@ uint32_t planned_warps(uint32_t lut_align, uint32_t lut_size, uint64_t pair_byte
     uint64_t least = ~0ull;
     for (uint64_t base = 0; base <= kStaticSmem + 1024; base += 128) {
         const uint64_t lut = (base + lut_align - 1) / lut_align * lut_align;
-        const uint64_t n_a = lut > base ? (lut - base) / pair_bytes : 0;
+        const uint64_t slot_a = (base + 255) / 256 * 256, n_a = lut > slot_a ? (lut - slot_a) / pair_bytes : 0;
         const uint64_t slot_b = lut + lut_size, end = base + dyn_smem - part_bytes;
         const uint64_t n_b = end > slot_b + guard_extra ? (end - slot_b - guard_extra) / pair_bytes : 0;
         if (n_a + n_b < least) least = n_a + n_b;
@@ -135,13 +144,11 @@ struct TcShape {
     uint32_t piece_columns(uint32_t npad) const { return npad / (2 * slices); }        // columns of a warp's share of the accumulators
 };
 uint32_t tc_npad_of(uint32_t batch) { return batch <= 16 ? 16 : (batch <= 32 ? 32 : 64); }
-// (`flat`: every matrix of the launch has flat FP16 mantissa codes: the exponent's table alone is kept)
-bool flat_fp16(const huffllm_desc *d) { return d->dtype == HUFFLLM_FP16 && d->lut_bits == 8 && (d->flat_fields & 6u) == 6u; }
 // Do the slot pairs of the shape's decoder warps fit beside the tables and the stages of activations (the guard area may lie
 // over those), for the largest records among the launch's matrices?
-bool tc_fits(const huffllm_desc *const *d, uint32_t n, uint32_t npad, const TcShape &sh, bool flat, uint32_t dyn_smem) {
+bool tc_fits(const huffllm_desc *const *d, uint32_t n, uint32_t npad, const TcShape &sh, uint32_t flat, uint32_t dyn_smem) {
     SmemNeeds need = smem_needs(d[0]);
-    if (d[0]->dtype == HUFFLLM_FP16 && d[0]->lut_bits == 8) need.table_bytes = flat ? 16384u : 49152u;   // (a launch-wide choice)
+    if (d[0]->dtype == HUFFLLM_FP16 && d[0]->lut_bits <= 8) need.table_bytes = fp16_table_bytes(flat);   // (a launch-wide choice)
     for (uint32_t i = 1; i < n; ++i) {
         const SmemNeeds o = smem_needs(d[i]);
         if (o.slot_bytes > need.slot_bytes) need.slot_bytes = o.slot_bytes;
@@ -153,7 +160,7 @@ bool tc_fits(const huffllm_desc *const *d, uint32_t n, uint32_t npad, const TcSh
 // the activations (at the widest batch padding: there the issuer, which carries them otherwise, bounds the CTA, 8192 x 28672
 // at 64 vectors 149 us against 133 with one decoder fewer); 2, 3 = two and four slices.  False: it does not fit or apply.
 constexpr uint32_t kTcShapes = 4;
-bool tc_shape(const huffllm_desc *const *d, uint32_t n, uint32_t npad, uint32_t which, bool flat, uint32_t dyn_smem, TcShape *sh) {
+bool tc_shape(const huffllm_desc *const *d, uint32_t n, uint32_t npad, uint32_t which, uint32_t flat, uint32_t dyn_smem, TcShape *sh) {
     const uint32_t slices = which < 2 ? 1 : which == 2 ? 2 : 4;
     // three stages, two at the widest batch padding, where tensor memory holds no more; the CTA's last warp issues the MMAs
     *sh = TcShape{4 / slices, slices, npad == 64 ? 2u : 3u, 32 / slices - (which == 1 ? 2 : 1)};
@@ -256,7 +263,7 @@ TcPlan tc_plan(const huffllm_desc *d, uint32_t npad, uint32_t sms, const TcShape
 // plan that the workspace had already cut, 28672 x 4096 at 64 vectors in a workspace of exactly the size asked for added up 2048
 // columns instead of 1024.)  Only where no plan of any shape is within both, the cut shape-0 plan is the measure.
 // False: no shape fits.
-bool tc_best(const huffllm_desc *const *d, uint32_t n, uint32_t npad, const uint32_t *cta, bool flat, uint32_t dyn_smem, size_t max_bytes,
+bool tc_best(const huffllm_desc *const *d, uint32_t n, uint32_t npad, const uint32_t *cta, uint32_t flat, uint32_t dyn_smem, size_t max_bytes,
              TcShape *shape, TcPlan *plans) {
     TcShape base;
     if (!tc_shape(d, n, npad, 0, flat, dyn_smem, &base)) return false;
@@ -284,10 +291,6 @@ bool tc_best(const huffllm_desc *const *d, uint32_t n, uint32_t npad, const uint
         if (base_bytes == max_bytes) return false;
     }
 }
-
-// Bytes of the FP16 tables a launch keeps in shared memory: three sixteen-fold tables of 8-bit codes, or the exponent's
-// alone where every matrix of the launch has flat mantissa codes (those are read without tables).
-uint32_t fp16_table_bytes(const KernelArgs *k) { return k->lut_bits == 8 && k->fp16_flat ? 16384u : 49152u; }
 
 // Start a launch description.
 void begin_args(KernelArgs *k, uint32_t batch, const DeviceInfo &dev) {
@@ -322,9 +325,8 @@ huffllm_status add_matrix(KernelArgs *k, const huffllm_desc *desc, const void *b
     m.col_chunks = desc->col_chunks;
     k->total_chunks += m.n_chunks;
     k->lut_bits = desc->lut_bits;
-    // (flat mantissa codes: only if every matrix of the launch has them)
-    const uint32_t flat = fmt && (desc->flat_fields & 6u) == 6u ? 1u : 0u;
-    k->fp16_flat = k->n_mats == 1 ? flat : (k->fp16_flat & flat);
+    // (flat mantissa codes: those that every matrix of the launch has)
+    k->fp16_flat = k->n_mats == 1 ? flat_of(desc) : flat_of_both(k->fp16_flat, flat_of(desc));
     const SmemNeeds need = smem_needs(desc);
     k->lut_align = need.table_align;
     k->lut_size = need.table_bytes;
@@ -359,7 +361,7 @@ bool rows_through_smem(const MatArgs &m) { return m.cols % 8 && m.cols >= 64 && 
 huffllm_status finish_args(KernelArgs *k, bool product, const DeviceInfo &dev, uint32_t *grid, uint32_t *warps_at_least = nullptr) {
     // (pieces that warps of a CTA exchange: in shared memory up to 8 vectors, in the workspace above)
     if (product) k->part_bytes = k->batch <= kKernelBatch ? 2 * 32 * 16 * k->batch * (uint32_t)sizeof(float) : 0;
-    if (k->fmt && k->lut_bits <= 8) k->lut_size = fp16_table_bytes(k);
+    if (k->fmt && k->lut_bits <= 8) k->lut_size = fp16_table_bytes(k->fp16_flat);
     // Two slots per decoder warp, so that a warp's next record lands while it decodes this one.  Where records are so large
     // that this would leave fewer than 31 warps a slot pair, and single slots serve at least a quarter more warps, every
     // warp gets one slot: more decoders at work outweigh the wait for a copy at every chunk start.
@@ -433,14 +435,15 @@ huffllm_status huffllm_workspace_bytes(const huffllm_desc *desc, uint32_t batch,
         const uint32_t dyn = (have ? (uint32_t)dev.smem_optin : 232448u) - kStaticSmem;
         const uint32_t cta = (uint32_t)sms;
         // The plan that will run for this and for every smaller batch, and the shape-0 plan, which a launch over several matrices
-        // may fall back on; with all three FP16 tables, and with one.
+        // may fall back on; with all three FP16 tables, and with those that flat codes leave.
         for (uint32_t npad = 16; npad <= tc_npad_of(batch); npad *= 2)
-            for (uint32_t flat = 0; flat < (flat_fp16(desc) ? 2u : 1u); ++flat) {
+            for (uint32_t flat : {kFlatNone, kFlatBoth, kFlatUpper}) {
+                if (flat != kFlatNone && flat_of_both(flat, flat_of(desc)) != flat) continue;
                 TcShape sh;
                 TcPlan p;
-                if (!tc_best(&desc, 1, npad, &cta, flat != 0, dyn, ~(size_t)0, &sh, &p)) continue;
+                if (!tc_best(&desc, 1, npad, &cta, flat, dyn, ~(size_t)0, &sh, &p)) continue;
                 if (p.bytes > *bytes) *bytes = p.bytes;
-                if (!tc_shape(&desc, 1, npad, 0, flat != 0, dyn, &sh)) continue;
+                if (!tc_shape(&desc, 1, npad, 0, flat, dyn, &sh)) continue;
                 p = tc_plan(desc, npad, cta, sh, ~(size_t)0, ~0u);
                 if (p.bytes > *bytes) *bytes = p.bytes;
             }
@@ -514,7 +517,7 @@ huffllm_status huffllm_gemm_launch_plan(uint32_t n, const huffllm_desc *const *d
     for (uint32_t i = 0; i < n; ++i) cta[i] = n > 1 ? k.m[i].cta_count : (uint32_t)dev.sms;
     TcShape sh;
     TcPlan plans[kMaxMats];
-    if (!tc_best(descs, n, tc_npad_of(batch), cta, k.fp16_flat != 0, k.dyn_smem_bytes, workspace_bytes_each ? workspace_bytes_each : ~(size_t)0, &sh, plans))
+    if (!tc_best(descs, n, tc_npad_of(batch), cta, k.fp16_flat, k.dyn_smem_bytes, workspace_bytes_each ? workspace_bytes_each : ~(size_t)0, &sh, plans))
         return fail(HUFFLLM_ERR_UNSUPPORTED, "chunk records too large for the tensor-core kernel's slots");
     if (column_slices) *column_slices = sh.slices;
     if (row_groups) *row_groups = sh.row_groups;
@@ -590,7 +593,7 @@ huffllm_status huffllm_decode_gemm_multi(uint32_t n, const huffllm_desc *const *
         for (uint32_t i = 0; i < n; ++i) cta[i] = k.m[i].cta_count;
         TcShape sh;
         TcPlan plans[kMaxMats];
-        if (!tc_best(descs, n, npad, cta, k.fp16_flat != 0, k.dyn_smem_bytes, workspace_bytes_each, &sh, plans))
+        if (!tc_best(descs, n, npad, cta, k.fp16_flat, k.dyn_smem_bytes, workspace_bytes_each, &sh, plans))
             return fail(HUFFLLM_ERR_UNSUPPORTED, "chunk records too large for the tensor-core kernel's slots");
         set_tc_shape(&k, npad, sh);
         uint32_t first = 0;
@@ -676,7 +679,7 @@ huffllm_status huffllm_decode_gemm(const huffllm_desc *desc, const void *blob, c
         const uint32_t npad = tc_npad_of(batch), cta = (uint32_t)dev.sms;
         TcShape sh;
         TcPlan tp;
-        if (!tc_best(&desc, 1, npad, &cta, flat_fp16(desc), (uint32_t)dev.smem_optin - kStaticSmem, workspace_bytes, &sh, &tp))
+        if (!tc_best(&desc, 1, npad, &cta, flat_of(desc), (uint32_t)dev.smem_optin - kStaticSmem, workspace_bytes, &sh, &tp))
             return HUFFLLM_OK;      // records too large for this kernel's slots
         TcArgs t;
         memset(&t, 0, sizeof(t));

@@ -11,9 +11,10 @@ namespace huffllm {
 
 __device__ __forceinline__ uint32_t smem_u32(const void *p) { return (uint32_t)__cvta_generic_to_shared(p); }
 
+template <int OFF = 0>
 __device__ __forceinline__ uint32_t lds_stream(uint32_t addr) {
     uint32_t v;
-    asm volatile("ld.shared.u32 %0, [%1];" : "=r"(v) : "r"(addr));
+    asm volatile("ld.shared.u32 %0, [%1+%2];" : "=r"(v) : "r"(addr), "n"(OFF));
     return v;
 }
 // LUT reads: the table is constant once built, so the compiler may schedule these freely.
@@ -125,341 +126,306 @@ __device__ __forceinline__ void pdl_wait_prior_grid() { asm volatile("griddepcon
 
 // ------------------------------------------------------------------------------ lane decoder
 
-// State of the decoder of one bit sequence.  (hi:lo) holds 64 stream bits; the current codeword starts
-// at bit pos + 7 of that window (the 7 bits in front are the lag that makes the table address fall out
-// of a single AND/OR); nxt is the shared-memory address of the sequence's next 32-bit word.  Words of
-// one sequence are 256 bytes apart (a row of the record holds one word of each of the 64 sequences).
-struct LaneStream {
-    uint32_t lo, hi, pos, nxt;
-};
+// All that a decoder keeps of a bit sequence is its pointer: bits, counted from shared address 0 as if the sequence's rows
+// were all there is (a row of a record holds one 32-bit word of each of the 64 sequences, 256 bytes), so that bits 5 and up
+// times 8 are the address of the row that holds the next codeword and the low 5 bits say where in that word it starts.
+// Whenever window bits are wanted, the two or three words at the pointer are read again: one multiplication and one logic
+// operation for the address, and no registers from one step to the next.
+// The pointer is advanced by adding whole table entries, which hold the length in their low bits and the symbol above bit
+// 15 or higher: shared addresses have 18 bits, so bits 0..14 of the pointer are all that is read.
+// What bounds these loops is the number of instructions (the SMs issue in four of five cycles) with the shared-memory pipe
+// close behind (1.5 loads per BF16 weight).  Cycles per 32 weights and scheduler, 31 warps decoding from shared memory with
+// nothing around them: window words kept in registers and refilled under a predicate 8.4 (28 instructions per four
+// codewords), this 8.2 (27; and six registers fewer).
+// Memory safety: the shared-memory copies of the tables hold no length above what the table's index bits allow
+// (lut_entry), so a block moves a sequence by at most that many bits per codeword, whatever the stream and the table hold;
+// the guard area behind the last slot covers it.
+constexpr uint32_t kRowMask = 0x3FF00u;
 
-__device__ __forceinline__ void stream_open(LaneStream &s, uint32_t lane_word0, uint32_t pos0 = 0) {
-    s.lo = lds_stream(lane_word0);
-    s.hi = lds_stream(lane_word0 + 256);
-    s.nxt = lane_word0 + 512;
-    s.pos = pos0;
-}
-
-// One decoder step: returns the table entry (length << 16 | exponent << 7) and advances the start pointer.
-// The window is shifted as a 64-bit value, so the pointer may run past bit 32 between two refill
-// checks.  The table address is (window & index mask) | (table base + 4 * lane): one logic operation,
-// because the table sits on a boundary above the index bits.  Only byte 2 of the entry (the length)
-// is added to the pointer: dp4a with that byte selected does it in one instruction off the ALU pipe.
-__device__ __forceinline__ uint32_t stream_step(LaneStream &s, uint32_t idx_mask, uint32_t lut_lane) {
-    uint64_t win = ((uint64_t)s.hi << 32) | s.lo;
-    uint32_t t = (uint32_t)(win >> s.pos), addr;
-    asm("lop3.b32 %0, %1, %2, %3, 0xEA;" : "=r"(addr) : "r"(t), "r"(idx_mask), "r"(lut_lane));
-    uint32_t e = lds_lut(addr);
-    s.pos = __dp4a(e, 0x00010000u, s.pos);
-    return e;
-}
-
-// Tables of 10 to 12 index bits (Section 3.2 quotes L_max = 12) are looked up in two levels.  The first level is the
-// 256-entry table of the first 8 stream bits, replicated per lane like the 8-bit table; an entry whose codeword is longer
-// than 8 bits carries a mark (bit 31) instead of a result, and the lane then reads the entry from the whole table
-// (one copy in shared memory, indexed by all lut_bits bits; bank conflicts there do not matter: long codewords are
-// rare).  full_mask = ((1 << lut_bits) - 1) << 2 turns the shifted window into that table's byte offset.
-constexpr uint32_t kLongMark = 0x80000000u;
-__device__ __forceinline__ uint32_t stream_step_long(LaneStream &s, uint32_t lut_lane, uint32_t full_base, uint32_t full_mask) {
-    uint64_t win = ((uint64_t)s.hi << 32) | s.lo;
-    uint32_t t = (uint32_t)(win >> s.pos), addr;
-    asm("lop3.b32 %0, %1, %2, %3, 0xEA;" : "=r"(addr) : "r"(t), "r"(0xFFu << 7), "r"(lut_lane));
-    uint32_t e = lds_lut(addr);
-    if (e & kLongMark) e = lds_lut(full_base + ((t >> 5) & full_mask));   // (t >> 7) is the index: times 4 bytes
-    s.pos = __dp4a(e, 0x00010000u, s.pos);
-    return e;
-}
-
-// The decoder of 8-bit BF16 tables works on four codewords at a time.  Its pointer stands on the codeword itself (the
-// sequence's leading zero bits are skipped when the sequence is opened), so after a refill check, with the pointer
-// below 32, the low 32 bits of the shifted window are all valid: room for four codewords of at most 8 bits.
-//   * The 32 bits are taken out of the window once (one 64-bit shift) and then shifted in place by each codeword's
-//     length: the shared-memory copy of the table repeats the length in an entry's low 5 bits (lut_entry_inplace), and a
-//     wrapping shift reads just those.  The pointer is not on the chain from one lookup to the next.
-//   * The table index is byte 0 of that word, and index * 128 + table base is one byte dot product.
-//   * The pointer is advanced once per four codewords by two three-input additions of the whole entries.  Only its low
-//     6 bits mean anything (pointer + lengths <= 31 + 32; bits 5 and 6 of an entry are zero, the exponent starts at
-//     bit 7, so nothing carries into them and bit 6 stays zero); whatever piles up above bit 6 is never read: the
-//     refill check tests bit 5 and the funnel shift reads bits 0..4.
-__device__ __forceinline__ uint32_t lut_entry_inplace(uint32_t e) { return e | (e >> 16); }
-
-template <bool RELOAD = true>      // false: the low word is copied from the high one (where shared-memory bandwidth is the scarcer resource)
-__device__ __forceinline__ void stream_refill4(LaneStream &s) {
-    if (RELOAD) {
-        asm volatile(
-            "{\n\t.reg .pred p, q;\n\t.reg .b32 b;\n\t"
-            "setp.ne.u32 q, 0, 0;\n\t"
-            "lop3.or.b32 b|p, %2, 32, 0, 0xC0, q;\n\t"          // p = bit 5 of the pointer: 32 or more bits consumed
-            "@p ld.shared.u32 %0, [%3+-256];\n\t"
-            "@p ld.shared.u32 %1, [%3];\n\t"
-            "@p add.u32 %3, %3, 256;\n\t"
-            "@p add.u32 %2, %2, 0xFFFFFFE0;\n\t}"
-            : "+r"(s.lo), "+r"(s.hi), "+r"(s.pos), "+r"(s.nxt));
-    } else {
-        asm volatile(
-            "{\n\t.reg .pred p, q;\n\t.reg .b32 b;\n\t"
-            "setp.ne.u32 q, 0, 0;\n\t"
-            "lop3.or.b32 b|p, %2, 32, 0, 0xC0, q;\n\t"
-            "@p mov.u32 %0, %1;\n\t"
-            "@p ld.shared.u32 %1, [%3];\n\t"
-            "@p add.u32 %3, %3, 256;\n\t"
-            "@p add.u32 %2, %2, 0xFFFFFFE0;\n\t}"
-            : "+r"(s.lo), "+r"(s.hi), "+r"(s.pos), "+r"(s.nxt));
-    }
-}
-// The 32 window bits at the pointer, right after a refill check (pointer below 32: a 32-bit funnel shift is enough,
-// and it reads only the pointer's low 5 bits).
-__device__ __forceinline__ uint32_t window_at(const LaneStream &s) {
-    uint32_t t;
-    asm("shf.r.wrap.b32 %0, %1, %2, %3;" : "=r"(t) : "r"(s.lo), "r"(s.hi), "r"(s.pos));
-    return t;
-}
-__device__ __forceinline__ uint32_t lookup_byte0(uint32_t t, uint32_t lut_lane) { return lds_lut(__dp4a(t, 0x00000080u, lut_lane)); }
-__device__ __forceinline__ uint32_t shift_by_entry(uint32_t t, uint32_t e) {
+// Address of the row under the pointer, at byte `col` of it (4 * sequence).
+__device__ __forceinline__ uint32_t row_addr(uint32_t pos, uint32_t col) {
     uint32_t d;
-    asm("shf.r.wrap.b32 %0, %1, 0, %2;" : "=r"(d) : "r"(t), "r"(e));
+    asm("lop3.b32 %0, %1, %2, %3, 0xEA;" : "=r"(d) : "r"(pos * 8u), "n"(kRowMask), "r"(col));
     return d;
 }
-// Four codewords of each of a lane's two sequences, the two chains interleaved.
-__device__ __forceinline__ void stream_step4x2(LaneStream &sa, LaneStream &sb, uint32_t lut_lane, uint32_t *ea, uint32_t *eb) {
-    stream_refill4(sa);
-    stream_refill4(sb);
-    uint32_t ta = window_at(sa), tb = window_at(sb);
-#pragma unroll
-    for (int k = 0; k < 4; ++k) {
-        ea[k] = lookup_byte0(ta, lut_lane);
-        eb[k] = lookup_byte0(tb, lut_lane);
-        if (k < 3) {
-            ta = shift_by_entry(ta, ea[k]);
-            tb = shift_by_entry(tb, eb[k]);
-        }
-    }
-    sa.pos = (sa.pos + ea[0] + ea[1]) + (ea[2] + ea[3]);
-    sb.pos = (sb.pos + eb[0] + eb[1]) + (eb[2] + eb[3]);
+// 32 bits of (hi:lo) from bit n % 32 on.
+__device__ __forceinline__ uint32_t funnel(uint32_t lo, uint32_t hi, uint32_t n) {
+    uint32_t t;
+    asm("shf.r.wrap.b32 %0, %1, %2, %3;" : "=r"(t) : "r"(lo), "r"(hi), "r"(n));
+    return t;
+}
+// The 32 bits at the pointer.  OFF = 0: the lane's first sequence (row g), 128: its second one (row g + 8).
+template <int OFF>
+__device__ __forceinline__ uint32_t window32(uint32_t pos, uint32_t col) {
+    const uint32_t a = row_addr(pos, col);
+    const uint32_t lo = lds_stream<OFF>(a), hi = lds_stream<OFF + 256>(a);
+    return funnel(lo, hi, pos);
+}
+// The 64 bits at the pointer.
+struct Window {
+    uint32_t lo, hi;
+};
+template <int OFF>
+__device__ __forceinline__ Window window64(uint32_t pos, uint32_t col) {
+    const uint32_t a = row_addr(pos, col);
+    const uint32_t w0 = lds_stream<OFF>(a), w1 = lds_stream<OFF + 256>(a), w2 = lds_stream<OFF + 512>(a);
+    return {funnel(w0, w1, pos), funnel(w1, w2, pos)};
+}
+// A window shifted in place by an entry's length (its low 5 bits; the entry may be a sum of entries).
+__device__ __forceinline__ uint32_t shift_by(uint32_t t, uint32_t e) { return funnel(t, 0u, e); }
+// Table entry of the window's low byte: `stride` bytes per entry (byte dot product: index * stride + the lane's column).
+__device__ __forceinline__ uint32_t lookup_byte0(uint32_t t, uint32_t stride, uint32_t lut_lane) { return lds_lut(__dp4a(t, stride, lut_lane)); }
+
+// The decoders, by the blobs' format and code lengths (LB = index bits of the tables, 12 for all above 9; FMT: see huff_kernel).
+enum Decoder {
+    kBf8,      // BF16, codewords of at most 8 bits: table once per lane
+    kBf9,      // BF16, 9 bits: table once per lane
+    kBf12,     // BF16, up to 12 bits: two levels
+    kHalf,     // FP16, three tables of 8 bits, sixteen copies each
+    kHalf7,    // FP16, three tables of 7 bits, once per lane
+    kHalf12,   // FP16, up to 12 bits per field: two levels
+    kFlat,     // FP16, both mantissa halves carry the flat code (codewords of at most 8 bits)
+    kUpper,    // FP16, the upper mantissa half carries the flat code (codewords of at most 8 bits)
+};
+__host__ __device__ constexpr Decoder decoder_of(int lb, int fmt) {
+    return fmt == 0 ? (lb == 8 ? kBf8 : lb == 9 ? kBf9 : kBf12) : fmt == 1 ? (lb == 8 ? kHalf : lb == 7 ? kHalf7 : kHalf12) : fmt == 2 ? kFlat : kUpper;
+}
+// Where a sequence's pointer starts: on its first codeword, behind the leading zero bits (7, FP16: 6); kBf9 stays 7 bits
+// behind, so that the index stands where the address wants it.
+__host__ __device__ constexpr uint32_t lag_of(Decoder d) { return d <= kBf12 ? 7u : 6u; }
+__host__ __device__ constexpr uint32_t start_of(Decoder d) { return d == kBf9 ? 0u : lag_of(d); }
+// Longest codeword (per field).
+__host__ __device__ constexpr uint32_t longest_of(Decoder d) { return d == kBf9 ? 9u : d == kHalf7 ? 7u : d == kBf12 || d == kHalf12 ? 12u : 8u; }
+constexpr uint32_t kLongMark = 0x80000000u;
+
+// Shared-memory form of a blob's table entry (length << 16 | symbol bits): the length in the low bits, the symbol above.
+// BF16: exponent at bits 23..30.  FP16: the field where it belongs in the weight, 16 bits up; the exponent's entry of the
+// decoders that read flat codes without a table has their bits added to its length.  A codeword of more than the first
+// level's 8 bits is only marked there.
+template <Decoder D>
+__device__ __forceinline__ uint32_t lut_entry(uint32_t e, uint32_t field, bool first_level = true) {
+    const uint32_t len = e >> 16;
+    if ((D == kBf12 || D == kHalf12) && first_level && len > 8u) return kLongMark;
+    const uint32_t flat_bits = D == kFlat ? 10u : D == kUpper && field == 0 ? 5u : 0u;
+    return ((D <= kBf12 ? e & 0x7F80u : e & 0x7FFFu) << 16) | (min(len, longest_of(D)) + flat_bits);
 }
 
-// Refill: once 32 bits have been consumed, slide the window by one word.  Written with predicated
-// instructions so that lanes which need a word and lanes which do not stay converged.  The low word is
-// reloaded from shared memory rather than copied from the high word: a load is not an integer
-// instruction, and 32-bit integer issue is what bounds this kernel.
-// (A plain 32-bit addition costs one dispatch cycle; logic, shift, compare, select and byte-permute instructions two.
-// Adding the entry's length by multiply-high with a register holding 65536 is cheap in isolation, 1.35 cycles, but
-// made this kernel 20 % slower: the pointer advance sits on the decoder's dependency chain.)
-template <bool RELOAD = true>
-__device__ __forceinline__ void stream_refill(LaneStream &s) {
-    if (RELOAD) {
-        asm volatile(
-            "{\n\t.reg .pred p;\n\t"
-            "setp.ge.u32 p, %2, 32;\n\t"
-            "@p ld.shared.u32 %0, [%3+-256];\n\t"
-            "@p ld.shared.u32 %1, [%3];\n\t"
-            "@p add.u32 %3, %3, 256;\n\t"
-            "@p add.u32 %2, %2, 0xFFFFFFE0;\n\t}"
-            : "+r"(s.lo), "+r"(s.hi), "+r"(s.pos), "+r"(s.nxt));
-    } else {   // where shared-memory bandwidth is the scarcer resource (FP16 blobs): copy the register instead
-        asm volatile(
-            "{\n\t.reg .pred p;\n\t"
-            "setp.ge.u32 p, %2, 32;\n\t"
-            "@p mov.u32 %0, %1;\n\t"
-            "@p ld.shared.u32 %1, [%3];\n\t"
-            "@p add.u32 %3, %3, 256;\n\t"
-            "@p add.u32 %2, %2, 0xFFFFFFE0;\n\t}"
-            : "+r"(s.lo), "+r"(s.hi), "+r"(s.pos), "+r"(s.nxt));
-    }
-}
+// ---- BF16
 
-// Two table entries + the raw word of their group -> two bf16 weights packed in one register.
+// Two entries -> one word with the even weight's exponent at bits 7..14 and the odd one's at 23..30: the even entry's upper
+// half plus the odd entry (a 16-bit dot product: one instruction of the multiplying pipe, where a byte permute would join
+// the shifts on the integer pipe: 8.2 against 8.4 cycles).  Lengths end up among the mantissa bits.
+__device__ __forceinline__ uint32_t merge_exponents(uint32_t e_even, uint32_t e_odd) { return __dp2a_lo(e_even, 0x00000100u, e_odd); }
+// Exponents + the raw word of their group -> two bf16 weights packed in one register.
 // A raw word holds the sign and mantissa bits of four consecutive weights of a row, laid out so that the first pair's
 // bits already sit where a packed pair of bf16 words has them (mantissas at bits 0..6 and 16..22, signs at 15 and 31)
 // and the second pair's do after a rotation by one byte; the other pair's bits lie in the exponent positions, which
-// the select below takes from the table entries.  The exponent of the even weight is already in place (bits 7..14);
-// the odd entry times 65536 puts its exponent at bits 23..30 and pushes its length out of the word, so one
-// multiply-add merges the two.
-__device__ __forceinline__ uint32_t pack_pair(uint32_t e_even, uint32_t e_odd, uint32_t sm) {
-    uint32_t ex;
-    asm("mad.lo.u32 %0, %1, 65536, %2;" : "=r"(ex) : "r"(e_odd), "r"(e_even));
+// the select takes from the table entries.
+__device__ __forceinline__ uint32_t pack_pair(uint32_t ex, uint32_t sm) {
     uint32_t w;   // sign and mantissa bits from sm, exponent bits from ex
     asm("lop3.b32 %0, %1, %2, 0x807F807F, 0xE4;" : "=r"(w) : "r"(sm), "r"(ex));
     return w;
 }
 __device__ __forceinline__ uint32_t rotr8(uint32_t v) { return prmt(v, v, 0x0321u); }
 
-// Decode one block (16 weights of this lane) into 8 packed registers:
+// One codeword of a longer code.  9 bits: the window is 7 bits behind the codeword, so the masked window is the address
+// (the table lies on a boundary above the index bits).  Up to 12: the first level resolves codewords of up to 8 bits; a
+// marked entry sends the lane to the whole table (one copy, 1 << lut_bits entries; full_mask = ((1 << lut_bits) - 1) * 4).
+// Long codewords are rare, so the second level's bank conflicts do not matter.
+template <Decoder D>
+__device__ __forceinline__ uint32_t lookup_long(uint32_t t, uint32_t lut_lane, uint32_t full_base, uint32_t full_mask) {
+    if (D == kBf9) {
+        uint32_t addr;
+        asm("lop3.b32 %0, %1, %2, %3, 0xEA;" : "=r"(addr) : "r"(t), "n"(0x1FFu << 7), "r"(lut_lane));
+        return lds_lut(addr);
+    }
+    uint32_t e = lookup_byte0(t, D == kBf12 ? 128u : 64u, lut_lane);
+    asm("{\n\t.reg .pred p;\n\t.reg .b32 i;\n\t"
+        "setp.lt.s32 p, %0, 0;\n\t"
+        "mad.lo.u32 i, %1, 4, 0;\n\t"
+        "@p and.b32 i, i, %3;\n\t"
+        "@p add.u32 i, i, %2;\n\t"
+        "@p ld.shared.u32 %0, [i];\n\t}"
+        : "+r"(e)
+        : "r"(t), "r"(full_base), "r"(full_mask));
+    return e;
+}
+
+// Four codewords of each of a lane's two sequences, the two chains interleaved; x: two words of merged exponents each.
+// Codewords of up to 8 bits: the window's 32 bits hold four, taken out once and shifted in place; the pointer is not on
+// the chain from one lookup to the next.  Longer ones: 64 bits are taken out, two codewords (at most 24 bits, 25 with the
+// 9-bit table's lag) come from the low word, two from the 32 bits behind them.
+template <Decoder D>
+__device__ __forceinline__ void step4(uint32_t &pa, uint32_t &pb, uint32_t col, uint32_t lut_lane, uint32_t *xa, uint32_t *xb,
+                                      uint32_t full_base, uint32_t full_mask) {
+    uint32_t ea[4], eb[4];
+    if (D == kBf8) {
+        uint32_t ta = window32<0>(pa, col), tb = window32<128>(pb, col);
+#pragma unroll
+        for (int i = 0; i < 4; ++i) {
+            ea[i] = lookup_byte0(ta, 128u, lut_lane);
+            eb[i] = lookup_byte0(tb, 128u, lut_lane);
+            if (i < 3) {
+                ta = shift_by(ta, ea[i]);
+                tb = shift_by(tb, eb[i]);
+            }
+        }
+        pa = (pa + ea[0] + ea[1]) + (ea[2] + ea[3]);
+        pb = (pb + eb[0] + eb[1]) + (eb[2] + eb[3]);
+    } else {
+        const Window wa = window64<0>(pa, col), wb = window64<128>(pb, col);
+        uint32_t ta = wa.lo, tb = wb.lo;
+#pragma unroll
+        for (int h = 0; h < 2; ++h) {
+            ea[2 * h] = lookup_long<D>(ta, lut_lane, full_base, full_mask);
+            eb[2 * h] = lookup_long<D>(tb, lut_lane, full_base, full_mask);
+            ta = shift_by(ta, ea[2 * h]);
+            tb = shift_by(tb, eb[2 * h]);
+            ea[2 * h + 1] = lookup_long<D>(ta, lut_lane, full_base, full_mask);
+            eb[2 * h + 1] = lookup_long<D>(tb, lut_lane, full_base, full_mask);
+            const uint32_t da = ea[2 * h] + ea[2 * h + 1], db = eb[2 * h] + eb[2 * h + 1];
+            pa += da;
+            pb += db;
+            ta = funnel(wa.lo, wa.hi, da);
+            tb = funnel(wb.lo, wb.hi, db);
+        }
+    }
+#pragma unroll
+    for (int i = 0; i < 2; ++i) {
+        xa[i] = merge_exponents(ea[2 * i], ea[2 * i + 1]);
+        xb[i] = merge_exponents(eb[2 * i], eb[2 * i + 1]);
+    }
+}
+
+// ---- FP16 {1,5,5,5}
+
+// FP16 blobs code three fields per weight (exponent, upper and lower mantissa half: Section 3.1), each with its own table.
+// A weight's entries are added up: its low 15 bits stand in the sum's upper half, its length in the low bits, which is what
+// the next window and the pointer want.  Two weights come from one 64-bit window (at most 48 bits; the second one's 32 bits
+// are taken out behind the first).
+// The three tables of kHalf are 16 KB each, sixteen copies per entry (entry i of copy c at word 16 i + c; a lane uses copy
+// lane % 16: a lookup takes two passes).  kHalf7's have 128 entries and a copy per lane: no conflicts; seven bits are no
+// byte, so the window is moved up by 7 bits and masked.
+// A FLAT code (all 32 symbols, 5 bits each: the canonical codeword of symbol s is s, written first bit first) needs no
+// table: fp16-trained weights have it in both mantissa halves, bf16-trained ones in the upper half.  Its bits follow the
+// exponent's codeword in reverse order.  The exponent's entry has them in its length, and the window is ROTATED by that
+// length instead of shifted: what comes next (the second weight, or the lower half's codeword) stands at bit 0, and the flat
+// bits at the top, in the order in which a bit reversal of both weights' halves at once puts them where they belong.
+// The tables that are left have a copy per lane (kUpper's lower half: sixteen).
+template <Decoder D>
+__device__ __forceinline__ uint32_t lookup_field(uint32_t t, int field, uint32_t lut_lane, uint32_t full_base, uint32_t full_mask) {
+    if (D == kHalf7) {
+        uint32_t addr;
+        asm("lop3.b32 %0, %1, %2, %3, 0xEA;" : "=r"(addr) : "r"(t), "n"(0x7Fu << 7), "r"(lut_lane));
+        return lds_lut(addr + 16384u * field);
+    }
+    if (D == kHalf12) return lookup_long<D>(t, lut_lane + 16384u * field, full_base + (full_mask + 4u) * field, full_mask);
+    return lds_lut(__dp4a(t, 64u, lut_lane) + 16384u * field);
+}
+// One weight out of the 32 (kHalf12: 64) bits at its start: the sum of its entries, and the rotated window of the flat codes.
+template <Decoder D>
+__device__ __forceinline__ uint32_t weight_sum(const Window &w, uint32_t lut_lane, uint32_t lut_low, uint32_t full_base, uint32_t full_mask, uint32_t &rot) {
+    uint32_t t = D == kHalf7 ? w.lo << 7 : w.lo;
+    if (D == kFlat || D == kUpper) {
+        const uint32_t e0 = lookup_byte0(t, 128u, lut_lane);
+        rot = funnel(t, t, e0);
+        if (D == kFlat) return e0;
+        return e0 + lookup_byte0(rot, 64u, lut_low);
+    }
+    const uint32_t e0 = lookup_field<D>(t, 0, lut_lane, full_base, full_mask);
+    t = shift_by(t, e0);
+    const uint32_t e1 = lookup_field<D>(t, 1, lut_lane, full_base, full_mask);
+    if (D == kHalf12) t = funnel(w.lo, w.hi, e0 + e1);
+    else t = shift_by(t, e1);
+    return e0 + e1 + lookup_field<D>(t, 2, lut_lane, full_base, full_mask);
+}
+// Two weights of each of a lane's two sequences -> their 15 bits each, as packed pairs (the sign positions hold anything).
+template <Decoder D>
+__device__ __forceinline__ void step2_fp16(uint32_t &pa, uint32_t &pb, uint32_t col, uint32_t lut_lane, uint32_t lut_low, uint32_t &xa, uint32_t &xb,
+                                           uint32_t full_base, uint32_t full_mask) {
+    Window wa = window64<0>(pa, col), wb = window64<128>(pb, col);
+    uint32_t ea[2], eb[2], ra[2], rb[2];
+#pragma unroll
+    for (int i = 0; i < 2; ++i) {
+        if (D == kHalf12 && i) {                      // (36 bits at most: the second weight has a window of its own)
+            wa = window64<0>(pa, col);
+            wb = window64<128>(pb, col);
+        }
+        ea[i] = weight_sum<D>(wa, lut_lane, lut_low, full_base, full_mask, ra[i]);
+        eb[i] = weight_sum<D>(wb, lut_lane, lut_low, full_base, full_mask, rb[i]);
+        if (D == kHalf12) {
+            pa += ea[i];
+            pb += eb[i];
+        } else if (i == 0) {
+            wa.lo = funnel(wa.lo, wa.hi, ea[0]);
+            wb.lo = funnel(wb.lo, wb.hi, eb[0]);
+        }
+    }
+    if (D != kHalf12) {
+        pa += ea[0] + ea[1];
+        pb += eb[0] + eb[1];
+    }
+    auto pair = [&](const uint32_t *e, const uint32_t *r) -> uint32_t {
+        const uint32_t coded = D == kFlat ? merge_exponents(e[0], e[1]) : prmt(e[0], e[1], 0x7632u);
+        if (D != kFlat && D != kUpper) return coded;
+        const uint32_t flat = __brev(prmt(r[0], r[1], 0x3276u));      // bits 0..9 / 16..25 (kUpper: 0..4 / 16..20): mantissa bits
+        uint32_t x;
+        if (D == kFlat) asm("lop3.b32 %0, %1, %2, 0x03FF03FF, 0xE4;" : "=r"(x) : "r"(flat), "r"(coded));
+        else asm("lop3.b32 %0, %1, %2, 0x03E003E0, 0xE4;" : "=r"(x) : "r"(flat * 32u), "r"(coded));
+        return x;
+    };
+    xa = pair(ea, ra);
+    xb = pair(eb, rb);
+}
+
+// ---- a block of 32 columns: 16 weights of this lane as 8 packed registers
 // a[0..3] = row g, columns (0,1) (2,3) (4,5) (6,7);  a[4..7] = row g+8, same columns.
-// The lane's two sequences are stepped alternately.  Each window is checked for a refill before every
-// R-th step: after a check at least 26 bits are valid in front of the start pointer, enough for R
-// codewords of at most 26/R bits.
-template <int R, bool SKIP = false, bool LONG = false>
-__device__ __forceinline__ void decode_block(LaneStream &sa, LaneStream &sb, uint32_t idx_mask, uint32_t lut_lane,
-                                             const uint4 &raw, uint32_t (&a)[8], uint32_t full_base = 0, uint32_t full_mask = 0) {
-    uint32_t e[16];
-    if (SKIP) {
-        stream_step4x2(sa, sb, lut_lane, e, e + 8);
-        stream_step4x2(sa, sb, lut_lane, e + 4, e + 12);
-    } else
+// raw: the lane's raw bytes of the block.  BF16: four words of sign and mantissa bits.  FP16: raw.x is a uint16, bit p = sign of
+// the first weight of pair p, bit 8 + p = sign of its second weight.
+template <Decoder D>
+__device__ __forceinline__ void decode_block(uint32_t &pa, uint32_t &pb, uint32_t col, uint32_t lut_lane, uint32_t lut_low, const uint4 &raw,
+                                             uint32_t (&a)[8], uint32_t full_base, uint32_t full_mask) {
+    uint32_t x[8];
+    if (D <= kBf12) {
 #pragma unroll
-    for (int i = 0; i < 8; ++i) {
-        if (i % R == 0) {
-            stream_refill(sa);
-            stream_refill(sb);
-        }
-        if (LONG) {
-            e[i] = stream_step_long(sa, lut_lane, full_base, full_mask);
-            e[8 + i] = stream_step_long(sb, lut_lane, full_base, full_mask);
-        } else {
-            e[i] = stream_step(sa, idx_mask, lut_lane);
-            e[8 + i] = stream_step(sb, idx_mask, lut_lane);
-        }
+        for (int i = 0; i < 4; i += 2) step4<D>(pa, pb, col, lut_lane, x + i, x + 4 + i, full_base, full_mask);
+        const uint32_t sm[8] = {raw.x, rotr8(raw.x), raw.y, rotr8(raw.y), raw.z, rotr8(raw.z), raw.w, rotr8(raw.w)};
+#pragma unroll
+        for (int i = 0; i < 8; ++i) a[i] = pack_pair(x[i], sm[i]);
+    } else {
+#pragma unroll
+        for (int i = 0; i < 4; ++i) step2_fp16<D>(pa, pb, col, lut_lane, lut_low, x[i], x[4 + i], full_base, full_mask);
+        const uint32_t s32 = prmt(raw.x, 0u, 0x4140u);     // first-weight signs in bits 0..7, second-weight signs in bits 16..23
+#pragma unroll
+        for (int p = 0; p < 8; ++p)                        // their sign bits at bits 15 and 31; mask bit set: the pair's, else the sign
+            asm("lop3.b32 %0, %1, %2, 0x7FFF7FFF, 0xE4;" : "=r"(a[p]) : "r"(x[p]), "r"(s32 << (15 - p)));
     }
-    a[0] = pack_pair(e[0], e[1], raw.x);
-    a[1] = pack_pair(e[2], e[3], rotr8(raw.x));
-    a[2] = pack_pair(e[4], e[5], raw.y);
-    a[3] = pack_pair(e[6], e[7], rotr8(raw.y));
-    a[4] = pack_pair(e[8], e[9], raw.z);
-    a[5] = pack_pair(e[10], e[11], rotr8(raw.z));
-    a[6] = pack_pair(e[12], e[13], raw.w);
-    a[7] = pack_pair(e[14], e[15], rotr8(raw.w));
 }
 
-// ------------------------------------------------------------------------------ FP16 {1,5,5,5}
-
-// FP16 blobs code three fields per weight (exponent, upper and lower mantissa half: Section 3.1), each with its own
-// 256-entry table.  The tables sit 16 KB apart, each replicated sixteen times (entry i of copy c at word 16 i + c; a
-// lane uses copy lane % 16: two lanes share a copy and collide when their entries fall into the same bank, which the
-// measured 86 % shared-memory pipe load of an eight-fold version made worth halving), so the index bits of a lookup
-// address are bits 6..13 and the lag of the stream is 6 bits.
-// A table entry is length << 16 | symbol << (10, 5, 0): the three entries of a weight OR-ed together are its low
-// 15 bits.  One refill check per weight: after it the pointer is below 32, three codewords of at most 8 bits and the
-// lag of the last lookup end at bit 31 + 16 + 14 = 61 of the 64-bit window.
-__device__ __forceinline__ uint32_t fp16_field(LaneStream &s, uint32_t lut_lane, uint32_t table_off) {
-    uint64_t win = ((uint64_t)s.hi << 32) | s.lo;
-    uint32_t t = (uint32_t)(win >> s.pos), addr, e;
-    asm("lop3.b32 %0, %1, %2, %3, 0xEA;" : "=r"(addr) : "r"(t), "r"(0xFFu << 6), "r"(lut_lane));
-    asm("ld.shared.u32 %0, [%1];" : "=r"(e) : "r"(addr + table_off));
-    s.pos = __dp4a(e, 0x00010000u, s.pos);
-    return e;
-}
-__device__ __forceinline__ uint32_t fp16_weight(LaneStream &s, uint32_t lut_lane) {
-    uint32_t e0 = fp16_field(s, lut_lane, 0), e1 = fp16_field(s, lut_lane, 16384), e2 = fp16_field(s, lut_lane, 32768), w;
-    asm("lop3.b32 %0, %1, %2, %3, 0xFE;" : "=r"(w) : "r"(e0), "r"(e1), "r"(e2));
-    return w;                                      // low 16 bits: exponent and mantissa; above: the three lengths mixed
-}
-// Field codes of 9 to 12 bits (Section 3.2: L_max = 12 for the 5-bit fields): two levels, as for BF16.  The first level is
-// the field's sixteen-fold table of the first 8 bits; a marked entry sends the lane to the field's whole table
-// (1 << lut_bits entries, one copy; the three follow each other from full_base).  A codeword may now take 12 bits, so the
-// window is checked before every field (pointer below 32: lag 6 + 12 bits end inside the 64-bit window).
-__device__ __forceinline__ uint32_t fp16_field_long(LaneStream &s, uint32_t lut_lane, uint32_t table_off, uint32_t full_addr,
-                                                    uint32_t full_mask) {
-    stream_refill<false>(s);
-    uint64_t win = ((uint64_t)s.hi << 32) | s.lo;
-    uint32_t t = (uint32_t)(win >> s.pos), addr, e;
-    asm("lop3.b32 %0, %1, %2, %3, 0xEA;" : "=r"(addr) : "r"(t), "r"(0xFFu << 6), "r"(lut_lane));
-    asm("ld.shared.u32 %0, [%1];" : "=r"(e) : "r"(addr + table_off));
-    if (e & kLongMark) e = lds_lut(full_addr + ((t >> 4) & full_mask));     // (t >> 6) is the index: times 4 bytes
-    s.pos = __dp4a(e, 0x00010000u, s.pos);
-    return e;
-}
-__device__ __forceinline__ uint32_t fp16_weight_long(LaneStream &s, uint32_t lut_lane, uint32_t full_base, uint32_t full_mask) {
-    const uint32_t table_bytes = full_mask + 4u;                            // bytes of one field's whole table
-    uint32_t e0 = fp16_field_long(s, lut_lane, 0, full_base, full_mask);
-    uint32_t e1 = fp16_field_long(s, lut_lane, 16384, full_base + table_bytes, full_mask);
-    uint32_t e2 = fp16_field_long(s, lut_lane, 32768, full_base + 2u * table_bytes, full_mask), w;
-    asm("lop3.b32 %0, %1, %2, %3, 0xFE;" : "=r"(w) : "r"(e0), "r"(e1), "r"(e2));
-    return w;
-}
-// Field codes of at most 8 bits, three codewords at a time (the scheme of the 8-bit BF16 decoder): the pointer stands on the
-// codeword (the sequence's 6 leading zero bits are skipped when it is opened); after one check per weight it is below 32,
-// so the low 32 bits of the shifted window hold the weight's three codewords (at most 24 bits).  They are taken out of
-// the window once and shifted in place by each codeword's length, which the shared-memory copy of the tables keeps in an
-// entry's low byte: entry = symbol bits << 8 | length (fp16_entry_inplace), so the OR of a weight's three entries has the
-// weight's low 15 bits at bits 8..22.  The table address is byte 0 of the window times 64 plus the lane's column of the
-// field's table: one byte dot product.  The pointer is advanced once per weight by the sum of the three entries; only its
-// low 6 bits mean anything (lengths add up to at most 24, bits 4..7 of an entry are zero) and nothing reads above them.
-__device__ __forceinline__ uint32_t fp16_entry_inplace(uint32_t e) { return ((e & 0x7FFFu) << 8) | (e >> 16); }
-__device__ __forceinline__ uint32_t fp16_weight_inplace(LaneStream &s, uint32_t lut_lane) {
-    stream_refill4<false>(s);
-    uint32_t t = window_at(s);
-    const uint32_t e0 = lds_lut(__dp4a(t, 0x00000040u, lut_lane));
-    t = shift_by_entry(t, e0);
-    const uint32_t e1 = lds_lut(__dp4a(t, 0x00000040u, lut_lane) + 16384u);
-    t = shift_by_entry(t, e1);
-    const uint32_t e2 = lds_lut(__dp4a(t, 0x00000040u, lut_lane) + 32768u);
-    s.pos = (s.pos + e0) + (e1 + e2);
-    uint32_t w;
-    asm("lop3.b32 %0, %1, %2, %3, 0xFE;" : "=r"(w) : "r"(e0), "r"(e1), "r"(e2));
-    return w;                                      // bits 8..22: exponent and mantissa
-}
-// Both mantissa halves carry the FLAT code (all 32 symbols, 5 bits each: the canonical codeword of symbol s is s, written
-// first bit first), which is what fp16-trained weights give: their mantissa bits are incompressible.  The ten stream bits
-// behind the exponent's codeword are then the weight's ten mantissa bits in reverse order: one bit reversal replaces two
-// table lookups.  (The exponent's table and everything else is as in fp16_weight_inplace; bits 0..7 of the result hold
-// the exponent's length and later stream bits, which the packing step never looks at.)
-__device__ __forceinline__ uint32_t fp16_weight_flat(LaneStream &s, uint32_t lut_lane) {
-    stream_refill4<false>(s);
-    uint32_t t = window_at(s);
-    const uint32_t e0 = lds_lut(__dp4a(t, 0x00000040u, lut_lane));
-    t = shift_by_entry(t, e0);
-    s.pos = s.pos + e0 + 10u;
-    return e0 | (__brev(t) >> 14);                 // bits 8..17: the mantissa, bits 18..22: the exponent
-}
-// Field codes of at most 7 bits: the same three-at-a-time scheme on tables of 128 entries, which are small enough to keep
-// once per LANE (entry i of lane l at word 32 i + l, 16 KB per field: the footprint of the sixteen-fold 256-entry tables),
-// so that a warp-wide lookup never has a bank conflict.  Seven index bits are not a byte, so the window is moved up by 7
-// bits once per weight and the table address is (window & index mask) | lane column, one logic operation; the in-place
-// shifts keep the next codeword at bit 7 (25 window bits are valid there: three codewords take at most 21).
-__device__ __forceinline__ uint32_t fp16_weight_lane(LaneStream &s, uint32_t lut_lane) {
-    stream_refill4<false>(s);
-    uint32_t t = window_at(s) << 7, a0, a1, a2;
-    asm("lop3.b32 %0, %1, %2, %3, 0xEA;" : "=r"(a0) : "r"(t), "r"(0x7Fu << 7), "r"(lut_lane));
-    const uint32_t e0 = lds_lut(a0);
-    t = shift_by_entry(t, e0);
-    asm("lop3.b32 %0, %1, %2, %3, 0xEA;" : "=r"(a1) : "r"(t), "r"(0x7Fu << 7), "r"(lut_lane));
-    const uint32_t e1 = lds_lut(a1 + 16384u);
-    t = shift_by_entry(t, e1);
-    asm("lop3.b32 %0, %1, %2, %3, 0xEA;" : "=r"(a2) : "r"(t), "r"(0x7Fu << 7), "r"(lut_lane));
-    const uint32_t e2 = lds_lut(a2 + 32768u);
-    s.pos = (s.pos + e0) + (e1 + e2);
-    uint32_t w;
-    asm("lop3.b32 %0, %1, %2, %3, 0xFE;" : "=r"(w) : "r"(e0), "r"(e1), "r"(e2));
-    return w;                                      // bits 8..22: exponent and mantissa
-}
-// Decode one block of an FP16 chunk into 8 packed registers (same order as decode_block).  `signs` is the lane's
-// uint16 of the block: bit p = sign of the first weight of pair p, bit 8 + p = sign of its second weight.
-// INPLACE: the three-at-a-time decoders above: 1 = tables of 8 bits (sixteen-fold), 2 = tables of 7 bits (per lane),
-// 3 = tables of 8 bits with flat codes for both mantissa halves.
-template <bool LONG = false, int INPLACE = 0>
-__device__ __forceinline__ void decode_block_fp16(LaneStream &sa, LaneStream &sb, uint32_t lut_lane, uint32_t signs,
-                                                  uint32_t (&a)[8], uint32_t full_base = 0, uint32_t full_mask = 0) {
-    uint32_t w[16];
-#pragma unroll
-    for (int i = 0; i < 8; ++i) {
-        if (INPLACE == 3) {
-            w[i] = fp16_weight_flat(sa, lut_lane);
-            w[8 + i] = fp16_weight_flat(sb, lut_lane);
-        } else if (INPLACE == 2) {
-            w[i] = fp16_weight_lane(sa, lut_lane);
-            w[8 + i] = fp16_weight_lane(sb, lut_lane);
-        } else if (INPLACE == 1) {
-            w[i] = fp16_weight_inplace(sa, lut_lane);
-            w[8 + i] = fp16_weight_inplace(sb, lut_lane);
-        } else if (LONG) {
-            w[i] = fp16_weight_long(sa, lut_lane, full_base, full_mask);
-            w[8 + i] = fp16_weight_long(sb, lut_lane, full_base, full_mask);
-        } else {
-            stream_refill<false>(sa);
-            stream_refill<false>(sb);
-            w[i] = fp16_weight(sa, lut_lane);
-            w[8 + i] = fp16_weight(sb, lut_lane);
-        }
+// ---- the tables in shared memory, by decoder: words per thread of `threads`, in 16-byte pieces (copies of one entry)
+template <Decoder D>
+struct LutPlan {
+    // 16-byte pieces of the first level
+    static constexpr uint32_t kVecs = D == kBf9 ? 4096u : D <= kBf12 || D == kFlat ? 2048u : 3072u;
+    // entry index in the blob's tables (of 1 << lut_bits entries each) and field of piece v
+    static __device__ __forceinline__ uint32_t source(uint32_t v, uint32_t lut_bits) {
+        if (D <= kBf12) return v >> 3;
+        if (D == kHalf7) return (field(v) << lut_bits) + ((v >> 3) & 127u);
+        if (D == kHalf || D == kHalf12) return (field(v) << lut_bits) + ((v >> 2) & 255u);
+        // (tables of 7 bits serve as tables of 8 whose upper half repeats the lower one)
+        const uint32_t in = field(v) ? (v >> 2) & 255u : v >> 3;
+        return (field(v) << lut_bits) + (in & ((1u << lut_bits) - 1u));
     }
-    const uint32_t s32 = prmt(signs, 0u, 0x4140u);     // first-weight signs in bits 0..7, second-weight signs in bits 16..23
-#pragma unroll
-    for (int p = 0; p < 8; ++p) {
-        uint32_t pair = prmt(w[2 * p], w[2 * p + 1], INPLACE ? 0x6521u : 0x5410u);   // the two weights' 15 bits (in place: from bits 8..22)
-        uint32_t sh = s32 << (15 - p);                            // their sign bits at bits 15 and 31
-        asm("lop3.b32 %0, %1, %2, 0x7FFF7FFF, 0xE4;" : "=r"(a[p]) : "r"(pair), "r"(sh));   // mask bit set: pair, else sign
-    }
-}
+    static __device__ __forceinline__ uint32_t field(uint32_t v) { return D <= kBf12 || D == kFlat ? 0u : D == kUpper ? (v >> 11) * 2u : v >> 10; }
+};
+// A lane's column of the table(s), and of kUpper's second one.
+template <Decoder D>
+__device__ __forceinline__ uint32_t lut_column(uint32_t lut, uint32_t lane) { return lut | (D == kHalf || D == kHalf12 ? lane & 15u : lane) << 2; }
+template <Decoder D>
+__device__ __forceinline__ uint32_t lut_low_column(uint32_t lut, uint32_t lane) { return D == kUpper ? lut + 32768u + ((lane & 15u) << 2) : 0u; }
+// Bytes of the first level, behind which the whole tables of the two-level decoders lie.
+template <Decoder D>
+constexpr uint32_t kLutBytes = LutPlan<D>::kVecs * 16u;
 
 // ------------------------------------------------------------------------------ shared memory plan
 
@@ -480,7 +446,7 @@ struct SmemPlan {
 __device__ __forceinline__ SmemPlan plan_smem(uint32_t base, const KernelArgs &k, uint32_t max_warps, uint32_t slots = 2) {   // k: launch-wide fields only
     SmemPlan p;
     const uint32_t lut_bytes = k.lut_align;
-    uint32_t a0 = (base + 127u) & ~127u;
+    uint32_t a0 = (base + 255u) & ~255u;     // (slots are whole rows of 256 bytes, on 256-byte boundaries)
     p.lut = (base + lut_bytes - 1) & ~(lut_bytes - 1);        // lut_align is a power of two
     p.slotA = a0;
     // (divisions by the slot pair's size as a multiplication by its rounded-down reciprocal and one correction: this

@@ -44,24 +44,28 @@ namespace huffllm {
 // Measured (BF16, 11007 x 4099 / 28672 x 8191; 11008 x 4096 takes 38.9 us): every lane storing its eight weights one by
 // one, 320 partial sector writes per block of 512 weights, 178 us / -; pieces on 16-byte boundaries through quad shuffles,
 // 48 sectors per block, 57 / 293 us; through shared memory 56 / 291; on 32-byte boundaries (this) 48 / 227 us.
+template <int OFF>
 __device__ __forceinline__ void sts_row(uint32_t addr, const uint32_t *v) {
-    asm volatile("st.shared.v4.u32 [%0], {%1, %2, %3, %4};" ::"r"(addr), "r"(v[0]), "r"(v[1]), "r"(v[2]), "r"(v[3]) : "memory");
+    asm volatile("st.shared.v4.u32 [%0+%5], {%1, %2, %3, %4};" ::"r"(addr), "r"(v[0]), "r"(v[1]), "r"(v[2]), "r"(v[3]), "n"(OFF) : "memory");
 }
-__device__ __forceinline__ uint4 shifted_piece(uint32_t row_word0, uint32_t sel) {     // row_word0: address of the first of the five words
-    uint32_t u[5];
+// A lane's piece: five words from `from` on, moved down by half a word where `sel` says so.  (Two loads of 16 bytes and a
+// selection of five of their eight words instead: 52.7 us against 49.0, more instructions and no fewer passes.)
+template <int OFF>
+__device__ __forceinline__ uint4 shifted_piece(uint32_t from, uint32_t sel) {
+    uint32_t w[5];
 #pragma unroll
-    for (int j = 0; j < 5; ++j) u[j] = lds_stream(row_word0 + 4 * j);
-    return make_uint4(prmt(u[0], u[1], sel), prmt(u[1], u[2], sel), prmt(u[2], u[3], sel), prmt(u[3], u[4], sel));
+    for (int j = 0; j < 5; ++j) w[j] = lds_stream<OFF>(from + 4 * j);
+    return make_uint4(prmt(w[0], w[1], sel), prmt(w[1], w[2], sel), prmt(w[2], w[3], sel), prmt(w[3], w[4], sel));
 }
-// The part of a piece that lies in columns [0, lim) of its chunk, the piece starting in column c.  A piece that is cut at
+// The part of a piece that lies in columns [first, end), the piece starting in column c.  A piece that is cut at
 // one end only (all but those of rows shorter than a piece) takes three stores of 8, 4 and 2 bytes: n weights from its
 // front or up to its end fall into such stores by the bits of n.
-__device__ __forceinline__ void store_piece(uint16_t *dst, const uint4 &p, int32_t c, int32_t lim) {
-    if (c >= 0 && c + 8 <= lim) {
+__device__ __forceinline__ void store_piece(uint16_t *dst, const uint4 &p, int32_t c, int32_t first, int32_t end) {
+    if (c >= first && c + 8 <= end) {
         *(uint4 *)dst = p;
         return;
     }
-    const int32_t lo = max(-c, 0), hi = min(lim - c, 8);        // weights lo .. hi - 1 of the piece
+    const int32_t lo = max(first - c, 0), hi = min(end - c, 8);        // weights lo .. hi - 1 of the piece
     if (lo >= hi) return;
     const uint32_t w[4] = {p.x, p.y, p.z, p.w};
     if (hi == 8) {
@@ -110,23 +114,18 @@ __device__ __forceinline__ void store_piece(uint16_t *dst, const uint4 &p, int32
 template <int MODE, int LB, int THREADS, int FMT, int NT = 1, int SLOTS = 2>
 __global__ void __launch_bounds__(THREADS, 1) huff_kernel(const __grid_constant__ KernelArgs A) {
     constexpr int kV = NT == 2 ? 8 : 4;                       // values a lane holds of a row group's 16 x batch outputs
+    constexpr int kOut = NT == 0 ? 1 : kV;                    // outputs a lane adds up and stores
     constexpr uint32_t kRawBlock = FMT ? 64u : 512u;          // raw bytes of one block of a record
     constexpr uint32_t kRawLane = FMT ? 2u : 16u;             // of which one lane's share
     // raw part of a record with nkb blocks, in record units of 128 bytes (FP16: rounded up to whole units)
     auto raw_units = [](uint32_t nkb) -> uint32_t { return FMT ? (nkb + 1u) >> 1 : nkb * 4u; };
-    // 8-bit BF16 tables: the decoder starts behind the sequences' leading zero bits and works on four codewords at a
-    // time (stream_step4x2)
-    constexpr bool SKIP = LB == 8 && FMT == 0;
-    constexpr int SKIP16 = FMT ? (LB == 8 ? (FMT == 2 ? 3 : 1) : LB == 7 ? 2 : 0) : 0;   // the same scheme for FP16: three codewords (one weight) at a
-                                                             // time; 2 = field codes of 7 bits, tables once per lane
-    constexpr bool LONG = LB > 9;                            // first level of 8 bits, then the whole table (FP16: lut_bits 9..12)
-    constexpr uint32_t kLB1 = LONG ? 8u : (uint32_t)LB;      // index bits of the per-lane table
-    constexpr int R = SKIP ? 4 : LB == 8 ? 3 : 2;            // decoder steps between two refill checks
-    constexpr uint32_t kIdxMask = ((1u << kLB1) - 1u) << 7;
+    constexpr Decoder D = decoder_of(LB, FMT);
+    constexpr bool LONG = D == kBf12 || D == kHalf12;        // first level of 8 bits, then the whole table
     extern __shared__ __align__(128) uint8_t dyn_smem[];
-    // per decoder warp: "full" barriers of its two slots (the copy has landed), then the two "empty" ones (the decoder is done)
-    __shared__ __align__(16) uint64_t bars[kMaxWarps * 4];
-    __shared__ __align__(16) uint2 notes[kMaxWarps * 2];       // per slot: the record's first and last offset, or kBadRecord
+    // per decoder warp: "full" barriers of its two slots (the copy has landed), the two "empty" ones (the decoder is done), and
+    // a note per slot: the record's first and last offset, or kBadRecord
+    __shared__ __align__(16) uint64_t bars[kMaxWarps * 6];
+    constexpr uint32_t kBarWarp = 48u, kNote = 32u;            // bytes per warp, and where its notes start
     __shared__ uint32_t s_arrive[kMaxWarps];   // arrival counters of row groups shared by several warps
     __shared__ uint32_t s_stop;                // a decoder gave up waiting: the feeder stops too
     constexpr uint32_t kBadRecord = 0xFFFFFFFFu;
@@ -160,7 +159,7 @@ __global__ void __launch_bounds__(THREADS, 1) huff_kernel(const __grid_constant_
     // blocks of 32 columns in column chunk kc: every chunk is full except, possibly, the last one of a row
     const uint32_t nkb_full = k.chunk_cols >> 5, nkb_tail = ((uint32_t)k.cols - (KC - 1) * k.chunk_cols + 31u) >> 5;
 
-    const uint32_t bar_w = smem_u32(&bars[(warp == feeder ? lane : warp) * 4]);   // the four barriers of "my" decoder warp
+    const uint32_t bar_w = smem_u32(bars) + (warp == feeder ? lane : warp) * kBarWarp;   // barriers and notes of "my" decoder warp
     constexpr uint32_t kSetupBarrier = 1;       // hardware barrier of the set-up: the decoders wait at it, the feeder only arrives
 
     if (warp == feeder) {
@@ -186,7 +185,6 @@ __global__ void __launch_bounds__(THREADS, 1) huff_kernel(const __grid_constant_
         uint32_t f_kc = f_ci % KC;
         const uint32_t slot_units = A.slot_bytes >> 7, slot_w = SLOTS == 2 ? slot_addr(plan, lane < nw ? lane : 0u, 0, A.slot_bytes)
                                                                                 : slot_addr_single(plan, lane < nw ? lane : 0u, A.slot_bytes);
-        const uint32_t note_w = smem_u32(&notes[lane * 2]);
         uint32_t idle = 0;
         while (__any_sync(0xFFFFFFFFu, f_ci < f_ce)) {
             const uint32_t which = f_issued & 1u;
@@ -199,7 +197,7 @@ __global__ void __launch_bounds__(THREADS, 1) huff_kernel(const __grid_constant_
                 const uint32_t full = bar_w + 8 * which, nkb = f_kc + 1 == KC ? nkb_tail : nkb_full;
                 // a record is usable if it lies inside the payload, is longer than its raw part and its coded part fits a slot
                 const bool ok = f_rb <= k.payload_units && f_rb - f_ra - raw_units(nkb) - 1u < slot_units;
-                asm volatile("st.shared.v2.u32 [%0], {%1, %2};" ::"r"(note_w + 8 * which), "r"(ok ? f_ra : kBadRecord), "r"(f_rb) : "memory");
+                asm volatile("st.shared.v2.u32 [%0], {%1, %2};" ::"r"(full + kNote), "r"(ok ? f_ra : kBadRecord), "r"(f_rb) : "memory");
                 if (ok) {
                     const uint32_t bytes = (f_rb - f_ra - raw_units(nkb)) << 7;
                     mbar_expect_tx(full, bytes);
@@ -230,32 +228,21 @@ __global__ void __launch_bounds__(THREADS, 1) huff_kernel(const __grid_constant_
     // ====================================================================== the decoder warps
     // ---- set-up: the table loads are started first, then this warp's own values are worked out, then the table is
     // written to shared memory (by the decoder warps alone: the feeder is already asking for records)
-    // (FP16: three tables of 256 entries, sixteen copies each: word j holds entry j / 16 of its table)
     // The table goes to shared memory in 16-byte pieces: four neighbouring copies of one entry per piece.
-    // (FP16, 7 bits: 3 x 32 x 128, the same; flat mantissa codes: the exponent's table alone)
-    constexpr uint32_t kLutWords = FMT == 2 ? 16u * 256u : FMT ? 3u * 16u * 256u : 32u << kLB1;
-    constexpr uint32_t kLutRep = FMT && LB != 7 ? 4u : 5u; // log2 of the copies per entry
-    constexpr uint32_t kLutVecs = kLutWords / 4;
-    constexpr uint32_t kLutThreads = THREADS - 32;
+    constexpr uint32_t kLutVecs = LutPlan<D>::kVecs, kLutThreads = THREADS - 32;
     constexpr int kLutLoads = (kLutVecs + kLutThreads - 1) / kLutThreads;
     uint32_t lut_v[kLutLoads];
-    {
-        const uint32_t *lut_g = (const uint32_t *)(k.blob + k.off_lut);
+    const uint32_t *lut_g = (const uint32_t *)(k.blob + k.off_lut);
 #pragma unroll
-        for (int i = 0; i < kLutLoads; ++i) {
-            uint32_t v = tid + i * kLutThreads;
-            // (entry of vector v: BF16 v / 8; FP16 field v / 1024, entry v / 4 % 256 of that field's table of 1 << lut_bits)
-            const uint32_t src = FMT ? ((v >> 10) << A.lut_bits) + (LB == 7 ? (v >> 3) & 127u : (v >> 2) & 255u) : v >> (kLutRep - 2);
-            lut_v[i] = v < kLutVecs ? __ldg(lut_g + src) : 0u;
-            if (SKIP) lut_v[i] = lut_entry_inplace(lut_v[i]);   // the length once more, where an in-place shift reads it
-            if (SKIP16) lut_v[i] = fp16_entry_inplace(lut_v[i]);
-            if (LONG && (lut_v[i] >> 16) > 8u) lut_v[i] |= kLongMark;   // a codeword longer than the first level resolves
-        }
+    for (int i = 0; i < kLutLoads; ++i) {
+        const uint32_t v = tid + i * kLutThreads;
+        lut_v[i] = v < kLutVecs ? __ldg(lut_g + LutPlan<D>::source(v, A.lut_bits)) : 0u;
     }
-    // two-level lookup: the whole table (1 << lut_bits entries, one copy) sits behind the per-lane first level
-    const uint32_t full_base = plan.lut + (FMT ? 49152u : 128u << kLB1), full_mask = ((1u << A.lut_bits) - 1u) << 2;
-    uint32_t lut_lane = plan.lut | ((FMT && LB != 7 ? lane & 15u : lane) << 2);
+    // two-level lookup: the whole table (1 << lut_bits entries, one copy) sits behind the first level
+    const uint32_t full_base = plan.lut + kLutBytes<D>, full_mask = ((1u << A.lut_bits) - 1u) << 2;
+    uint32_t lut_lane = lut_column<D>(plan.lut, lane), lut_low = lut_low_column<D>(plan.lut, lane);
     asm volatile("mov.u32 %0, %0;" : "+r"(lut_lane));  // keep it in a register: it is an operand of every lookup
+    if (D == kUpper) asm volatile("mov.u32 %0, %0;" : "+r"(lut_low));
     const uint32_t g = lane >> 2, t = lane & 3;
     uint32_t c_beg = 0, c_end = 0;
     if (warp < nw) {
@@ -271,23 +258,23 @@ __global__ void __launch_bounds__(THREADS, 1) huff_kernel(const __grid_constant_
         if (FMT) return make_uint4(ldg_stream2(p), 0, 0, 0);
         return ldg_stream16(p);
     };
-    const uint8_t *raw_p = payload;
+    const uint8_t *const raw0 = payload + lane * kRawLane;     // the lane's place in a record at offset 0
+    const uint8_t *raw_p = raw0;
     {
         uint4 *lut_s = (uint4 *)(dyn_smem + (plan.lut - smem_base));
 #pragma unroll
         for (int i = 0; i < kLutLoads; ++i) {
-            uint32_t v = tid + i * kLutThreads;
-            if (v < kLutVecs) lut_s[v] = make_uint4(lut_v[i], lut_v[i], lut_v[i], lut_v[i]);
+            const uint32_t v = tid + i * kLutThreads, e = lut_entry<D>(lut_v[i], LutPlan<D>::field(v));
+            if (v < kLutVecs) lut_s[v] = make_uint4(e, e, e, e);
         }
         if (tid < kMaxWarps) s_arrive[tid] = 0;
         if (LONG) {
-            const uint32_t *lut_g = (const uint32_t *)(k.blob + k.off_lut);
             uint32_t *full_s = (uint32_t *)(dyn_smem + (full_base - smem_base));
-            for (uint32_t i = tid; i < (FMT ? 3u : 1u) << A.lut_bits; i += kLutThreads) full_s[i] = __ldg(lut_g + i);
+            for (uint32_t i = tid; i < (FMT ? 3u : 1u) << A.lut_bits; i += kLutThreads) full_s[i] = lut_entry<D>(__ldg(lut_g + i), 0u, false);
         }
     }
     if (r_first < k.payload_units) {        // (the blob keeps 4 KB behind the payload: a block's read stays inside it)
-        raw_p = payload + ((uint64_t)r_first << 7) + lane * kRawLane;
+        raw_p = raw0 + ((uint64_t)r_first << 7);
         raw_a = load_raw(raw_p);
         primed = true;
     }
@@ -299,7 +286,6 @@ __global__ void __launch_bounds__(THREADS, 1) huff_kernel(const __grid_constant_
     float acc[kV];
 #pragma unroll
     for (int j = 0; j < kV; ++j) acc[j] = 0.f;
-    int cur_rg = -1;
     if (NT == 2) part_val = k.ws_warp_pieces + (size_t)J * (2 * kMaxWarps) * vals;   // (same-SM traffic: it stays in L1 / L2)
 
     // ---- reduction of a finished row group, without any CTA-wide barrier.
@@ -312,53 +298,13 @@ __global__ void __launch_bounds__(THREADS, 1) huff_kernel(const __grid_constant_
         const uint32_t big = k.cta_extra * (k.cta_chunks + 1);
         return ch < big ? ch / (k.cta_chunks + 1) : k.cta_extra + (ch - big) / k.cta_chunks;
     };
-    // lanes 0..vals-1 (looping if vals > 32) hold or produce the value of output o = column * 16 + row
-    auto finish_cta_sum = [&](int rg, float (&v)[kV]) {      // v[i] = value of output o = lane + 32 i
-        const uint32_t g_lo = (uint32_t)rg * KC, g_hi = g_lo + KC;
-        if (cta_beg <= g_lo && cta_end >= g_hi) {             // the CTA held the whole row group
-#pragma unroll
-            for (int i = 0; i < kV; ++i) {
-                uint32_t o = lane + 32 * i;
-                uint64_t r = (uint64_t)rg * 16 + (o & 15);
-                if (o < vals && r < k.rows) k.y[(uint64_t)(o >> 4) * k.rows + r] = v[i];
-            }
-            return;
-        }
-        // slot 0 holds the piece of the CTA's first row group in this matrix, slot 1 the piece of its last one
-        const uint32_t my_slot = (uint32_t)rg == cta_beg / KC ? 0u : 1u;
-#pragma unroll
-        for (int i = 0; i < kV; ++i) {
-            uint32_t o = lane + 32 * i;
-            if (o < vals) k.ws_partial[((size_t)J * 2 + my_slot) * vals + o] = v[i];
-        }
-        __syncwarp();
-        const uint32_t c0 = cta_of_chunk(g_lo), c1 = cta_of_chunk(g_hi - 1);
-        uint32_t last = 0;
-        if (lane == 0) {
-            last = arrive_acq_rel(k.ws_ticket + c0) == c1 - c0 ? 1u : 0u;
-            if (last) k.ws_ticket[c0] = 0;                    // leave the counter as it was found
-        }
-        if (!__shfl_sync(0xFFFFFFFFu, last, 0)) return;       // somebody else will arrive later and add us in
-#pragma unroll
-        for (int i = 0; i < kV; ++i) {
-            uint32_t o = lane + 32 * i;
-            if (o >= vals) continue;
-            float sum = 0.f;
-            for (uint32_t c = c0; c <= c1; ++c) {
-                uint32_t slot = cta_cut(c) / KC == (uint32_t)rg ? 0u : 1u;
-                sum += __ldcg(k.ws_partial + ((size_t)c * 2 + slot) * vals + o);
-            }
-            uint64_t r = (uint64_t)rg * 16 + (o & 15);
-            if (r < k.rows) k.y[(uint64_t)(o >> 4) * k.rows + r] = sum;
-        }
-    };
-    auto flush = [&](int rg, uint32_t first_c, uint32_t last_c_excl) {
-        if (rg < 0) return;
-        const uint32_t g_lo = max((uint32_t)rg * KC, cta_beg), g_hi = min((uint32_t)(rg + 1) * KC, cta_end);  // this CTA's part
-        const bool alone = first_c <= g_lo && last_c_excl >= g_hi;   // no other warp of this CTA holds a piece
-        // D fragment -> output order (o = column * 16 + row) through this warp's shared-memory entry
-        const uint32_t ent = warp * 2 + ((uint32_t)rg == c_beg / KC ? 0u : 1u);
-        float *mine = part_val + (size_t)ent * vals;
+    // Called at one place, in code that is short: it runs once or twice per warp, from instruction memory that is cold by then.
+    auto flush = [&](uint32_t rg, uint32_t first_c, uint32_t last_c_excl) {
+        const uint32_t g_lo = rg * KC, g_hi = g_lo + KC, my_lo = max(g_lo, cta_beg), my_hi = min(g_hi, cta_end);  // its chunks, and this CTA's part
+        const bool alone = first_c <= my_lo && last_c_excl >= my_hi;   // no other warp of this CTA holds a piece
+        // D fragment -> output order (o = column * 16 + row) through this warp's shared-memory entry: the first one for the
+        // row group that the warp's range starts in front of or at, the second for the one it starts inside of
+        const uint32_t mine = warp * 2 + (c_beg >= g_lo ? 0u : 1u);
         if (NT == 0) {
             // acc[0]: this lane's eight columns of row g; acc[2]: of row g + 8.  The four lanes of a row add theirs
             // (always in this order), and lane t = 0 then holds what the D fragment's column 0 would hold.
@@ -367,48 +313,74 @@ __global__ void __launch_bounds__(THREADS, 1) huff_kernel(const __grid_constant_
             s_hi += __shfl_xor_sync(0xFFFFFFFFu, s_hi, 1);
             s_lo += __shfl_xor_sync(0xFFFFFFFFu, s_lo, 2);
             s_hi += __shfl_xor_sync(0xFFFFFFFFu, s_hi, 2);
-            acc[0] = s_lo;
-            acc[2] = s_hi;
-        }
+            if (t == 0) {
+                part_val[mine * vals + g] = s_lo;
+                part_val[mine * vals + g + 8] = s_hi;
+            }
+        } else {
 #pragma unroll
-        for (int j = 0; j < kV; ++j) {      // (tile j / 4 of the activations: columns 8 (j / 4) + 2 t, + 1)
-            uint32_t col = 8 * (j >> 2) + 2 * t + (j & 1), row = g + 8 * ((j >> 1) & 1);
-            if (col < A.batch) mine[col * 16 + row] = acc[j];
+            for (int j = 0; j < kV; ++j) {      // (tile j / 4 of the activations: columns 8 (j / 4) + 2 t, + 1)
+                uint32_t col = 8 * (j >> 2) + 2 * t + (j & 1), row = g + 8 * ((j >> 1) & 1);
+                if (col < A.batch) part_val[mine * vals + col * 16 + row] = acc[j];
+            }
         }
 #pragma unroll
         for (int j = 0; j < kV; ++j) acc[j] = 0.f;
         __syncwarp();
-        float v[kV];
-        if (alone) {
-#pragma unroll
-            for (int i = 0; i < kV; ++i) v[i] = lane + 32 * i < vals ? mine[lane + 32 * i] : 0.f;
-            __syncwarp();
-            finish_cta_sum(rg, v);
-            return;
+        uint32_t mask = 1u << warp, entry = mine;            // the warps with a piece of this row group; lane l: warp l's entry
+        if (!alone) {
+            const uint32_t wb = warp_beg(lane), we = warp_beg(lane + 1);
+            mask = __ballot_sync(0xFFFFFFFFu, lane < nw && wb < we && wb < my_hi && we > my_lo);
+            entry = lane * 2 + (wb >= g_lo ? 0u : 1u);
+            uint32_t last = 0;
+            if (lane == 0) {
+                __threadfence_block();
+                last = atomicAdd(&s_arrive[__ffs(mask) - 1], 1u) == __popc(mask) - 1u ? 1u : 0u;
+                if (last) __threadfence_block();
+            }
+            if (!__shfl_sync(0xFFFFFFFFu, last, 0)) return;
         }
-        // which warps of this CTA hold a piece of this row group (lane l answers for warp l)
-        const uint32_t wb = warp_beg(lane), we = warp_beg(lane + 1);
-        const bool holds = lane < nw && wb < we && wb < g_hi && we > g_lo;
-        const uint32_t mask = __ballot_sync(0xFFFFFFFFu, holds);
-        const uint32_t w_first = __ffs(mask) - 1, n_hold = __popc(mask);
-        const uint32_t slot_of_lane = (uint32_t)rg == wb / KC ? 0u : 1u;
-        uint32_t last = 0;
-        if (lane == 0) {
-            __threadfence_block();
-            last = atomicAdd(&s_arrive[w_first], 1u) == n_hold - 1 ? 1u : 0u;
-            if (last) __threadfence_block();
-        }
-        if (!__shfl_sync(0xFFFFFFFFu, last, 0)) return;
+        // outputs o = lane + 32 i
+        float v[kOut];
 #pragma unroll
-        for (int i = 0; i < kV; ++i) v[i] = 0.f;
+        for (int i = 0; i < kOut; ++i) v[i] = 0.f;
+#pragma unroll 1
         for (uint32_t m = mask; m; m &= m - 1) {              // pieces in warp order
-            const uint32_t w = __ffs(m) - 1;
-            const float *piece = part_val + (size_t)(w * 2 + __shfl_sync(0xFFFFFFFFu, slot_of_lane, w)) * vals;
+            const float *piece = part_val + __shfl_sync(0xFFFFFFFFu, entry, __ffs(m) - 1) * vals + lane;
 #pragma unroll
-            for (int i = 0; i < kV; ++i)
-                if (lane + 32 * i < vals) v[i] += piece[lane + 32 * i];
+            for (int i = 0; i < kOut; ++i)
+                if (lane + 32 * i < vals) v[i] += piece[32 * i];
         }
-        finish_cta_sum(rg, v);
+        if (cta_beg > g_lo || cta_end < g_hi) {               // other CTAs have pieces too
+            // slot 0 holds the piece of the row group that a CTA's range starts in front of or at, slot 1 of the other one
+            float *const parts = k.ws_partial + lane;
+            float *const to = parts + ((size_t)J * 2 + (cta_beg >= g_lo ? 0u : 1u)) * vals;
+#pragma unroll
+            for (int i = 0; i < kOut; ++i)
+                if (lane + 32 * i < vals) to[32 * i] = v[i];
+            __syncwarp();
+            const uint32_t c0 = cta_of_chunk(g_lo), c1 = cta_of_chunk(g_hi - 1);
+            uint32_t last = 0;
+            if (lane == 0) {
+                last = arrive_acq_rel(k.ws_ticket + c0) == c1 - c0 ? 1u : 0u;
+                if (last) k.ws_ticket[c0] = 0;                // leave the counter as it was found
+            }
+            if (!__shfl_sync(0xFFFFFFFFu, last, 0)) return;   // somebody else will arrive later and add us in
+#pragma unroll
+            for (int i = 0; i < kOut; ++i) v[i] = 0.f;
+#pragma unroll 2
+            for (uint32_t c = c0; c <= c1; ++c) {             // pieces in CTA order
+                const float *piece = parts + ((size_t)c * 2 + (cta_cut(c) >= g_lo ? 0u : 1u)) * vals;
+#pragma unroll
+                for (int i = 0; i < kOut; ++i)
+                    if (lane + 32 * i < vals) v[i] += __ldcg(piece + 32 * i);
+            }
+        }
+        const uint64_t r = (uint64_t)rg * 16 + (lane & 15);
+        float *const y = k.y + (uint64_t)(lane >> 4) * k.rows + r;
+#pragma unroll
+        for (int i = 0; i < kOut; ++i)
+            if (lane + 32 * i < vals && r < k.rows) y[2 * i * k.rows] = v[i];
     };
 
     if (c_beg < c_end) {
@@ -417,32 +389,63 @@ __global__ void __launch_bounds__(THREADS, 1) huff_kernel(const __grid_constant_
         const uint16_t *xq = k.x + (MODE == 1 ? (uint64_t)min(g, A.batch - 1) * k.cols + kc * k.chunk_cols + t * 8u : 0);
         // (second tile of activations, vectors 8 .. 15: lane g's vector 8 + g lies this many elements further on)
         const uint64_t x_tile2 = NT == 2 ? (uint64_t)(min(g + 8u, A.batch - 1) - min(g, A.batch - 1)) * k.cols : 0;
-        // this chunk's slot (the lane's column of it), its barrier and its note, toggled by XOR from chunk to chunk; parity
-        // of the barrier's next completion (each of the two "full" barriers completes every second chunk)
-        // (With two tiles of activations, where registers are shortest, the five are worked out from the chunk's number at
-        // every chunk instead of being carried along: 4 % faster there, 3 % slower in the other kernels.)
-        constexpr bool kDerive = NT == 2;
-        uint32_t slot_cur = (SLOTS == 2 ? slot_addr(plan, warp, 0, A.slot_bytes) : slot_addr_single(plan, warp, A.slot_bytes)) + (lane << 2);
-        uint32_t bar_cur = bar_w, par = 0, which = 0;
-        const uint32_t slot_tog = SLOTS == 2 ? slot_cur ^ (slot_cur + A.slot_bytes) : 0u;   // (one slot: every chunk lands in the same place)
-        uint32_t note_cur = smem_u32(&notes[warp * 2]);
-        const uint32_t slot0 = slot_cur, note0 = note_cur;      // (used where the five are worked out anew)
+        // where this chunk's sequences start in its slot, and the slot's barrier, toggled by XOR from chunk to chunk; parity of
+        // the barrier's next completion (each of the two "full" barriers completes every second chunk)
+        const uint32_t slot0 = SLOTS == 2 ? slot_addr(plan, warp, 0, A.slot_bytes) : slot_addr_single(plan, warp, A.slot_bytes);
+        const uint32_t pos_tog = SLOTS == 2 ? (slot0 >> 3) ^ ((slot0 + A.slot_bytes) >> 3) : 0u;   // (one slot: every chunk lands in the same place)
+        uint32_t pos_cur = (slot0 >> 3) + start_of(D), bar_cur = bar_w, par = 0, which = 0;
+        const uint32_t col = lane << 2;
+        // MODE 2: where row g of the warp's buffer keeps what is left of the block before, and the block's 64 bytes
+        const uint32_t row_left = MODE == 2 ? smem_base + A.dyn_smem_bytes - A.part_bytes + (warp * 16u + g) * kRowBuf : 0u;
+        const uint32_t row_new = row_left + 32u;
+        constexpr int kRowHalf = 8 * kRowBuf;           // rows g + 8: as much further on
+        // The columns that a warp has decoded of a row group without a gap, from run_first on, are stored as one run: a chunk's
+        // last row_off columns wait in the row buffers for the next chunk's first pieces.
+        int32_t run_first = 0;
+        bool left_over = false;
+        struct Rows {                                   // rows g and g + 8, which start 8 * cols weights apart, at the same place in a sector
+            uint32_t off, from, sel;                    // row_off; the piece's five words start (row_off + 1) / 2 words in front of the
+                                                        // lane's own weights, its weights half a word further where row_off is odd
+            int64_t first;                              // the row's first weight in the output
+            bool ok[2];
+        };
+        auto rows_of = [&]() -> Rows {
+            Rows R;
+            R.off = ((rg * 16u + g) * (uint32_t)k.cols + (uint32_t)((uintptr_t)k.out >> 1)) & 15u;
+            R.from = row_new + t * 16u - ((R.off + 1u) >> 1) * 4u;
+            R.sel = (R.off & 1u) ? 0x5432u : 0x3210u;
+            R.first = (int64_t)(((uint64_t)rg * 16 + g) * k.cols);
+            R.ok[0] = (uint64_t)rg * 16 + g < k.rows;
+            R.ok[1] = (uint64_t)rg * 16 + g + 8 < k.rows;
+            return R;
+        };
+        // the end of a run: what the row buffers still hold of the columns in front of chunk kc
+        auto store_left_over = [&]() {
+            __syncwarp();
+            const Rows R = rows_of();
+            const int32_t end = (int32_t)min((uint64_t)kc * k.chunk_cols, k.cols), c = ((end + 31) & ~31) + (int32_t)(t * 8u) - (int32_t)R.off;
+            if (left_over && t * 8u < R.off) {
+                uint16_t *const dst = k.out + (R.first + c);
+                if (R.ok[0]) store_piece(dst, shifted_piece<0>(R.from, R.sel), c, run_first, end);
+                if (R.ok[1]) store_piece(dst + 8 * k.cols, shifted_piece<kRowHalf>(R.from, R.sel), c, run_first, end);
+            }
+            left_over = false;
+            __syncwarp();
+        };
 
 #pragma unroll 1
-        for (uint32_t c = c_beg; c < c_end; ++c) {
+        for (uint32_t c = c_beg;; ++c) {
+            if (c == c_end || (MODE != 0 && kc == KC)) {      // a row group, or the warp's part of it, ended with chunk c - 1
+                if (MODE == 1) flush(rg, c_beg, c);
+                if (MODE == 2) store_left_over();
+                if (c == c_end) break;
+            }
+            if (kc == KC) {                                   // the next row group: back to column 0
+                kc = 0;
+                ++rg;
+                if (MODE == 1) xq -= k.cols;
+            }
             const uint32_t nkb = kc + 1 == KC ? nkb_tail : nkb_full;
-            if (kDerive) {
-                const uint32_t ci = c - c_beg;
-                which = ci & 1u;
-                par = (ci >> 1) & 1u;
-                bar_cur = bar_w + 8u * which;
-                note_cur = note0 + 8u * which;
-                slot_cur = slot0 + (SLOTS == 2 ? which * A.slot_bytes : 0u);
-            }
-            if (MODE == 1 && (int)rg != cur_rg) {
-                flush(cur_rg, c_beg, c);  // the previous row group ended with chunk c - 1
-                cur_rg = (int)rg;
-            }
 
             // wait, with a limit, for the coded part; the outcome is made uniform across the warp
             if (!failed) {
@@ -465,77 +468,52 @@ __global__ void __launch_bounds__(THREADS, 1) huff_kernel(const __grid_constant_
                 waited_prior = true;
             }
             uint32_t r0, r1;            // the feeder's note: the record's first and last offset
-            asm volatile("ld.shared.v2.u32 {%0, %1}, [%2];" : "=r"(r0), "=r"(r1) : "r"(note_cur));
+            asm volatile("ld.shared.v2.u32 {%0, %1}, [%2];" : "=r"(r0), "=r"(r1) : "r"(bar_cur + kNote));
             if (failed || r0 == kBadRecord) {  // record offsets out of range: report, produce nothing for this chunk, touch no memory
                 if (!failed && A.err && lane == 0) atomicExch(A.err, (int32_t)min(c + 1, 0x7FFFFFFFu));
                 primed = false;
                 if (MODE == 1) xq += nkb * 32u;
+                if (MODE == 2) store_left_over();
             } else {
                 if (!primed) {
-                    raw_p = payload + ((uint64_t)r0 << 7) + lane * kRawLane;
+                    raw_p = raw0 + ((uint64_t)r0 << 7);
                     raw_a = load_raw(raw_p);
                 }
                 // the record behind this one is the next chunk's: its first raw block is fetched from inside this chunk's last
                 // block (the address lies inside the blob whatever that record's offsets turn out to be)
                 const bool has_next = c + 1 < c_end;
-                const uint32_t coded_bytes = (r1 - r0 - raw_units(nkb)) << 7;
-                // from the end of the record's last raw block to the next record: the coded part and, in FP16 records with an
-                // odd number of blocks, the 64 bytes that pad the raw part to a whole unit
-                const uint32_t to_next = FMT ? ((r1 - r0) << 7) - nkb * kRawBlock : coded_bytes;
-                LaneStream sa, sb;
-                stream_open(sa, slot_cur, SKIP ? 7u : SKIP16 ? 6u : 0u);
-                stream_open(sb, slot_cur + 128u, SKIP ? 7u : SKIP16 ? 6u : 0u);
+                const uint8_t *const raw_next = raw0 + ((uint64_t)r1 << 7);
+                uint32_t pa = pos_cur, pb = pos_cur;
                 const uint32_t col0 = kc * k.chunk_cols + t * 8u;
                 // (activations: lanes of unused output columns repeat the last vector; cols is a multiple of 32
                 // here, so every block of the chunk lies inside the row and xq ends the chunk where the next begins)
-                // (MODE 2: the chunk's first column, moved back to the 32-byte boundary in front of it; rows g + 8 h)
-                uint32_t row_off[2] = {0u, 0u};
-                if (MODE == 2)
-#pragma unroll
-                    for (int h = 0; h < 2; ++h)
-                        row_off[h] = ((uint32_t)((uint64_t)rg * 16 + g + 8 * h) * (uint32_t)k.cols + (uint32_t)((uintptr_t)k.out >> 1)) & 15u;
-                const int32_t lim = MODE == 2 ? (int32_t)min(k.chunk_cols, (uint32_t)k.cols - kc * k.chunk_cols) : 0;
-                // (MODE 2: this lane's sixteen bytes of row g in the warp's buffer; rows g + 8 follow 8 rows further on; the piece's
-                // five words start (row_off + 1) / 2 words in front of them, its weights half a word further where row_off is odd)
-                const uint32_t row_buf = MODE == 2 ? smem_base + A.dyn_smem_bytes - A.part_bytes + (warp * 16u + g) * kRowBuf + 32u + t * 16u : 0u;
-                const uint32_t half_sel = (row_off[0] & 1u) ? 0x5432u : 0x3210u;       // (rows g and g + 8 start 8 * cols weights apart)
-                uint16_t *out0 = MODE != 1 ? k.out + ((uint64_t)rg * 16 + g) * k.cols + col0 : nullptr;
-                const uint32_t last = nkb - 1;
-
-                // one block: start the fetch of the next block's raw bytes into `nxt`, decode with `cur`
-                // (may_be_last = false: the caller knows that another block of this chunk follows)
-                // Every block asks L2 for the 16 bytes per lane that lie four blocks further on in the record stream (the
-                // loads that bring raw bytes to registers run one block ahead of the decoder, too short for a miss in
-                // DRAM).  In a record's first half that is the raw part of its second half; in the second half it is the
-                // coded part and, at its end, the start of the next record.  The request ends at most 2 KB behind the
-                // record it is issued in: inside the blob, whose format keeps 4 KB of zero bytes behind the payload for this.
-                // (products of BF16 blobs only: the decode-only kernel has no register to spare for it, and an FP16 record's
-                // raw part is a sixteenth of its bytes)
-                constexpr bool kPrefetchRaw = false;
-                auto block = [&](uint32_t kb, const uint4 &cur, uint4 &nxt, auto may_be_last) {
-                    raw_p += kRawBlock;
-                    if (kPrefetchRaw) asm volatile("prefetch.global.L2 [%0];" ::"l"(raw_p + 3u * kRawBlock));
-                    if (decltype(may_be_last)::value) {
-                        if (kb == last) raw_p += to_next;           // the next record's first block
-                        if (kb != last || has_next) nxt = load_raw(raw_p);
-                    } else {
-                        nxt = load_raw(raw_p);
-                    }
+                uint16_t *out0 = MODE == 0 ? k.out + ((uint64_t)rg * 16 + g) * k.cols + col0 : nullptr;
+                Rows R;
+                uint32_t inner_from = 0, inner_to = 0;           // MODE 2: the blocks all of whose pieces are stored whole
+                if (MODE != 1) {
+                    R = rows_of();
+                    if (MODE == 2) out0 = k.out + (R.first + (int32_t)col0 - (int32_t)R.off);
+                    if (!left_over) run_first = (int32_t)(kc * k.chunk_cols);
+                    inner_from = left_over ? 0u : 1u;
+                    inner_to = ((uint32_t)k.cols - kc * k.chunk_cols) >> 5;
+                    left_over = true;
+                }
+                // one block, number kb of the chunk and `i` behind where raw_p and xq stand: decode with `cur` while the raw bytes
+                // of the next one, at `from`, are on their way to `nxt`
+                auto block = [&](uint32_t kb, int i, const uint4 &cur, uint4 &nxt, const uint8_t *from, bool fetch) {
+                    if (fetch) nxt = load_raw(from);
+                    const uint16_t *const xi = xq + 32 * i;
                     uint4 xv;
-                    if (MODE == 1) {
-                        if (NT <= 1) xv = __ldg((const uint4 *)xq);   // (two tiles: both are fetched behind the decoder, registers are short)
-                        xq += 32;
-                    }
+                    if (MODE == 1 && NT <= 1) xv = __ldg((const uint4 *)xi);   // (two tiles: both are fetched behind the decoder, registers are short)
 
                     uint32_t a[8];
-                    if (FMT) decode_block_fp16<LONG, SKIP16>(sa, sb, lut_lane, cur.x, a, full_base, full_mask);
-                    else decode_block<R, SKIP, LONG>(sa, sb, kIdxMask, lut_lane, cur, a, full_base, full_mask);
+                    decode_block<D>(pa, pb, col, lut_lane, lut_low, cur, a, full_base, full_mask);
 
                     if (MODE == 1) {
                         uint4 xw;
                         if (NT == 2) {
-                            xv = __ldg((const uint4 *)(xq - 32));
-                            xw = __ldg((const uint4 *)(xq - 32 + x_tile2));
+                            xv = __ldg((const uint4 *)xi);
+                            xw = __ldg((const uint4 *)(xi + x_tile2));
                         }
                         float (&acc0)[4] = *reinterpret_cast<float (*)[4]>(&acc[0]);
                         if (NT == 0) {
@@ -570,19 +548,23 @@ __global__ void __launch_bounds__(THREADS, 1) huff_kernel(const __grid_constant_
                             }
                         }
                     } else if (MODE == 2) {
-#pragma unroll
-                        for (int h = 0; h < 2; ++h) sts_row(row_buf + 8 * kRowBuf * h, a + 4 * h);
+                        sts_row<0>(row_new + t * 16u, a);
+                        sts_row<kRowHalf>(row_new + t * 16u, a + 4);
                         __syncwarp();
-#pragma unroll
-                        for (int h = 0; h < 2; ++h) {
-                            const uint4 piece = shifted_piece(row_buf + 8 * kRowBuf * h - ((row_off[h] + 1u) >> 1) * 4u, half_sel);
-                            if ((uint64_t)rg * 16 + g + 8 * h < k.rows)
-                                store_piece(out0 + (uint64_t)(8 * h) * k.cols + kb * 32u - row_off[h], piece, (int32_t)(kb * 32u + t * 8u - row_off[h]), lim);
+                        const uint4 p0 = shifted_piece<0>(R.from, R.sel), p1 = shifted_piece<kRowHalf>(R.from, R.sel);
+                        if (kb >= inner_from && kb < inner_to) {
+                            if (R.ok[0]) *(uint4 *)out0 = p0;
+                            if (R.ok[1]) *(uint4 *)(out0 + 8 * k.cols) = p1;
+                        } else {
+                            const int32_t c = (int32_t)(col0 + kb * 32u) - (int32_t)R.off;
+                            if (R.ok[0]) store_piece(out0, p0, c, run_first, (int32_t)k.cols);
+                            if (R.ok[1]) store_piece(out0 + 8 * k.cols, p1, c, run_first, (int32_t)k.cols);
                         }
+                        out0 += 32;
                         __syncwarp();
                         if (t >= 2) {                        // the row's last sixteen weights, for the next block's first pieces
-#pragma unroll
-                            for (int h = 0; h < 2; ++h) sts_row(row_buf + 8 * kRowBuf * h - 64u, a + 4 * h);
+                            sts_row<0>(row_left + t * 16u - 32u, a);
+                            sts_row<kRowHalf>(row_left + t * 16u - 32u, a + 4);
                         }
                     } else {
                         // (With the one-by-one stores left out of this kernel, which one branch skips, the compiler ordered the
@@ -591,7 +573,7 @@ __global__ void __launch_bounds__(THREADS, 1) huff_kernel(const __grid_constant_
                         const uint32_t col = col0 + kb * 32u;
 #pragma unroll
                         for (int h = 0; h < 2; ++h) {
-                            if ((uint64_t)rg * 16 + g + 8 * h >= k.rows || col >= (uint32_t)k.cols) continue;
+                            if (!R.ok[h] || col >= (uint32_t)k.cols) continue;
                             uint16_t *dst = out0 + (uint64_t)(8 * h) * k.cols + kb * 32u;
                             if (k.cols % 8 == 0) {
                                 *(uint4 *)dst = make_uint4(a[4 * h], a[4 * h + 1], a[4 * h + 2], a[4 * h + 3]);
@@ -603,57 +585,43 @@ __global__ void __launch_bounds__(THREADS, 1) huff_kernel(const __grid_constant_
                         }
                     }
                 };
-                constexpr std::integral_constant<bool, false> inner{};
-                constexpr std::integral_constant<bool, true> maybe_last{};
-                uint32_t kb = 0;
+                // Blocks in pairs, which keeps the loop short: an SM's warps, all somewhere else in it, share the instruction cache.
+                // (7B-shaped layer as four launches: groups of four 86.3 us, of two 82.5, single blocks 89.6, two blocks with a
+                // way out between them 86.6.  Rows through shared memory: pairs 49.0 us, single blocks 46.8.)
+                uint32_t left = nkb;
 #pragma unroll 1
-                for (; kb + 4 <= nkb; kb += 4) {                    // the usual case: groups of four blocks
-                    block(kb, raw_a, raw_b, inner);
-                    block(kb + 1, raw_b, raw_a, inner);
-                    block(kb + 2, raw_a, raw_b, inner);
-                    block(kb + 3, raw_b, raw_a, maybe_last);
+                for (; MODE != 2 && left >= 2u; left -= 2u) {
+                    const uint32_t kb = nkb - left;
+                    const uint8_t *const behind = left == 2u ? raw_next : raw_p + 2u * kRawBlock;
+                    block(kb, 0, raw_a, raw_b, raw_p + kRawBlock, true);
+                    block(kb + 1u, 1, raw_b, raw_a, behind, left != 2u || has_next);
+                    raw_p = behind;
+                    if (MODE == 1) xq += 64;
                 }
 #pragma unroll 1
-                for (; kb < nkb; kb += 2) {
-                    block(kb, raw_a, raw_b, maybe_last);
-                    if (kb + 1 < nkb) block(kb + 1, raw_b, raw_a, maybe_last);
+                while (left) {
+                    raw_p = left == 1u ? raw_next : raw_p + kRawBlock;
+                    block(nkb - left, 0, raw_a, raw_b, raw_p, left != 1u || has_next);
+                    if (MODE == 1) xq += 32;
+                    raw_a = raw_b;
+                    --left;
                 }
-                if (MODE == 2) {                 // the chunk's last row_off columns: no lane's piece ends behind them
-                    __syncwarp();
-#pragma unroll
-                    for (int h = 0; h < 2; ++h)
-                        if (t * 8u < row_off[h] && (uint64_t)rg * 16 + g + 8 * h < k.rows)
-                            store_piece(out0 + (uint64_t)(8 * h) * k.cols + nkb * 32u - row_off[h],
-                                        shifted_piece(row_buf + 8 * kRowBuf * h - ((row_off[h] + 1u) >> 1) * 4u, half_sel),
-                                        (int32_t)(nkb * 32u + t * 8u - row_off[h]), min(lim, (int32_t)(nkb * 32u)));
-                    __syncwarp();
-                }
-                if (nkb & 1u) raw_a = raw_b;     // the next chunk's first block always starts in raw_a
                 primed = has_next;
-                // A sequence of a sound record ends inside the record's W rows, so its next-row pointer stands at most two
-                // rows behind them.  Bits that made the decoder run further (a damaged coded part) are reported; what was
-                // decoded from them is wrong, but every read stayed inside shared memory (one row per refill check at most).
-                const uint32_t row_limit = slot_cur + 512u + coded_bytes;
-                if (__any_sync(0xFFFFFFFFu, sa.nxt > row_limit || sb.nxt > row_limit + 128u)) {
+                // A sequence of a sound record ends inside the record's W rows.  Bits that made the decoder run further (a damaged
+                // coded part) are reported; what was decoded from them is wrong, but every read stayed inside shared memory.
+                const uint32_t end = pos_cur - lag_of(D) + (r1 - r0 - raw_units(nkb)) * 16u;     // (128 bytes of the record: 16 bits of every sequence)
+                if (__any_sync(0xFFFFFFFFu, (pa & 0x7FFFu) > end || (pb & 0x7FFFu) > end)) {
                     if (A.err && lane == 0) atomicExch(A.err, (int32_t)(kErrOverrun | min(c + 1, kErrOverrun - 1u)));
                 }
             }
             __syncwarp();
             if (lane == 0) mbar_arrive(bar_cur + 16);                 // the slot goes back to the feeder
-            if (!kDerive) {
-                par ^= which;                                     // 0, 0, 1, 1, 0, 0, ...
-                which ^= 1u;
-                if (SLOTS == 2) slot_cur ^= slot_tog;
-                bar_cur ^= 8u;
-                note_cur ^= 8u;
-            }
-            kc = kc + 1 == KC ? 0u : kc + 1;
-            if (kc == 0) {                                        // the next chunk starts the next row group: back to column 0
-                ++rg;
-                if (MODE == 1) xq -= k.cols;
-            }
+            par ^= which;                                         // 0, 0, 1, 1, 0, 0, ...
+            which ^= 1u;
+            pos_cur ^= pos_tog;
+            bar_cur ^= 8u;
+            ++kc;
         }
-        if (MODE == 1) flush(cur_rg, c_beg, c_end);
     }
 }
 
@@ -763,35 +731,27 @@ static cudaError_t launch_slots(const KernelArgs &k, uint32_t grid, cudaStream_t
     return launch_one<MODE, LB, kThreads, FMT, NT, 2>(k, grid, stream);
 }
 
-template <int MODE>
-static cudaError_t launch_decode_mode(const KernelArgs &k, uint32_t grid, cudaStream_t stream) {
-    if (k.fmt && k.lut_bits == 7) return launch_slots<MODE, 7, 1>(k, grid, stream);
-    if (k.fmt && k.lut_bits == 8 && k.fp16_flat) return launch_slots<MODE, 8, 2>(k, grid, stream);
-    if (k.fmt) return k.lut_bits > 8 ? launch_slots<MODE, 12, 1>(k, grid, stream) : launch_slots<MODE, 8, 1>(k, grid, stream);
-    if (k.lut_bits > 9) return launch_one<MODE, 12, kThreads, 0>(k, grid, stream);
-    return k.lut_bits == 8 ? launch_slots<MODE, 8, 0>(k, grid, stream) : launch_one<MODE, 9, kThreads, 0>(k, grid, stream);
+// The kernel of a launch's blobs: format, code lengths, flat codes (kernels.h).
+template <int MODE, int NT>
+static cudaError_t launch_format(const KernelArgs &k, uint32_t grid, cudaStream_t stream) {
+    if (k.fmt) {
+        if (k.lut_bits > 8) return launch_slots<MODE, 12, 1, NT>(k, grid, stream);
+        if (k.fp16_flat == kFlatBoth) return launch_slots<MODE, 8, 2, NT>(k, grid, stream);
+        if (k.fp16_flat == kFlatUpper) return launch_slots<MODE, 8, 3, NT>(k, grid, stream);
+        return k.lut_bits == 7 ? launch_slots<MODE, 7, 1, NT>(k, grid, stream) : launch_slots<MODE, 8, 1, NT>(k, grid, stream);
+    }
+    if (k.lut_bits > 9) return launch_one<MODE, 12, kThreads, 0, NT>(k, grid, stream);
+    return k.lut_bits == 8 ? launch_slots<MODE, 8, 0, NT>(k, grid, stream) : launch_one<MODE, 9, kThreads, 0, NT>(k, grid, stream);
 }
 // (Where rows go through shared memory is decided with the launch's shared memory: part_bytes.)
 cudaError_t launch_decode(const KernelArgs &k, uint32_t grid, cudaStream_t stream) {
-    return k.part_bytes ? launch_decode_mode<2>(k, grid, stream) : launch_decode_mode<0>(k, grid, stream);
+    return k.part_bytes ? launch_format<2, 1>(k, grid, stream) : launch_format<0, 1>(k, grid, stream);
 }
 
 cudaError_t launch_gemm(const KernelArgs &k, uint32_t grid, cudaStream_t stream) {
-    if (k.batch == 1 && k.fmt) {                  // one vector: multiply-adds on the FMA pipe
-        if (k.lut_bits == 7) return launch_slots<1, 7, 1, 0>(k, grid, stream);
-        if (k.lut_bits == 8 && k.fp16_flat) return launch_slots<1, 8, 2, 0>(k, grid, stream);
-        return k.lut_bits > 8 ? launch_slots<1, 12, 1, 0>(k, grid, stream) : launch_slots<1, 8, 1, 0>(k, grid, stream);
-    }
-    if (k.batch == 1) {
-        if (k.lut_bits > 9) return launch_one<1, 12, kThreads, 0, 0>(k, grid, stream);
-        return k.lut_bits == 8 ? launch_slots<1, 8, 0, 0>(k, grid, stream) : launch_one<1, 9, kThreads, 0, 0>(k, grid, stream);
-    }
-    if (k.batch > 8) return launch_slots<1, 8, 0, 2>(k, grid, stream);   // (the entry point sends only BF16 blobs of 8-bit tables here)
-    if (k.fmt && k.lut_bits == 7) return launch_slots<1, 7, 1>(k, grid, stream);
-    if (k.fmt && k.lut_bits == 8 && k.fp16_flat) return launch_slots<1, 8, 2>(k, grid, stream);
-    if (k.fmt) return k.lut_bits > 8 ? launch_slots<1, 12, 1>(k, grid, stream) : launch_slots<1, 8, 1>(k, grid, stream);
-    if (k.lut_bits > 9) return launch_one<1, 12, kThreads, 0>(k, grid, stream);
-    return k.lut_bits == 8 ? launch_slots<1, 8, 0>(k, grid, stream) : launch_one<1, 9, kThreads, 0>(k, grid, stream);
+    if (k.batch == 1) return launch_format<1, 0>(k, grid, stream);           // one vector: multiply-adds on the FMA pipe
+    if (k.batch > 8) return launch_slots<1, 8, 0, 2>(k, grid, stream);       // (the entry point sends only BF16 blobs of 8-bit tables here)
+    return launch_format<1, 1>(k, grid, stream);
 }
 
 cudaError_t launch_plain_gemv(const PlainArgs &a, uint32_t sms, cudaStream_t stream) {

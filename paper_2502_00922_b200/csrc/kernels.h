@@ -53,8 +53,9 @@ struct KernelArgs {
     uint32_t slots;            // slots per decoder warp: 2 (the next record lands while this one is decoded), or 1 where two would
                                // leave too few warps a slot (large records: the feeder then waits for a slot before every copy).
                                // Kernels with single slots exist for FP16 blobs and for BF16 blobs with 8-bit tables.
-    uint32_t fp16_flat;        // FP16 blobs: both mantissa halves of every matrix of the launch carry the flat 5-bit code
+    uint32_t fp16_flat;        // FP16 blobs: which mantissa halves of every matrix of the launch carry the flat 5-bit code
 };
+constexpr uint32_t kFlatNone = 0, kFlatBoth = 1, kFlatUpper = 2;    // (the lower half alone is not made use of)
 
 // Arguments of the tensor-core kernel: the launch description plus, per matrix, its work items and where their pieces meet.
 // (The CTAs of a launch are dealt to the matrices as in the other kernels: m[i].cta_first / cta_count.)

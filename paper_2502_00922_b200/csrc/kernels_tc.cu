@@ -142,12 +142,7 @@ __global__ void __launch_bounds__(1024, 1) huff_gemm_tc_kernel(const __grid_cons
         if (FMT) return make_uint4(ldg_stream2(p), 0, 0, 0);
         return ldg_stream16(p);
     };
-    // the decoder that starts behind the leading zero bits and takes four codewords at a time (see huff_kernel)
-    constexpr bool SKIP = LB == 8 && FMT == 0;
-    // FP16 (8-bit tables only here): three codewords at a time with in-place shifts; FMT = 2: flat codes for both mantissa halves
-    constexpr int SKIP16 = FMT ? (FMT == 2 ? 3 : 1) : 0;
-    constexpr int R = SKIP ? 4 : LB == 8 ? 3 : 2;
-    constexpr uint32_t kIdxMask = ((1u << LB) - 1u) << 7;
+    constexpr Decoder D = decoder_of(LB, FMT);
     constexpr uint32_t kBStage = NPAD * 128;                // bytes of B per slice and stage: NPAD rows x 64 columns (two blocks) of bf16
     constexpr uint32_t kLbo = 128, kSbo = 1024;             // core matrices: 8 along K side by side, then the next 8 rows
     constexpr uint32_t kACol0 = kTcTiles * NPAD;            // first tensor-memory column of the A stages
@@ -225,8 +220,9 @@ __global__ void __launch_bounds__(1024, 1) huff_gemm_tc_kernel(const __grid_cons
         return;
     }
     const uint32_t b_base = smem_base + A.dyn_smem_bytes - A.part_bytes;   // the stages of B behind everything else
-    uint32_t lut_lane = plan.lut | ((FMT ? lane & 15u : lane) << 2);
+    uint32_t lut_lane = lut_column<D>(plan.lut, lane), lut_low = lut_low_column<D>(plan.lut, lane);
     asm volatile("mov.u32 %0, %0;" : "+r"(lut_lane));
+    if (D == kUpper) asm volatile("mov.u32 %0, %0;" : "+r"(lut_low));
     const uint32_t bar0 = smem_u32(&bars[warp * 2]);
     const uint32_t slot0 = slot_addr(plan, decodes ? slice * n_rg + rgi : 0u, 0, A.slot_bytes);    // (this kernel always runs with two slots per warp)
     auto record_ok = [&](uint32_t r0, uint32_t r1, uint32_t nkb) -> bool {
@@ -250,15 +246,14 @@ __global__ void __launch_bounds__(1024, 1) huff_gemm_tc_kernel(const __grid_cons
             mbar_init(bar0 + 8, 1);
         }
         // the table goes to shared memory in 16-byte pieces: four neighbouring copies of one entry per piece
-        // (FP16: three tables of 256 entries, sixteen copies each; flat mantissa codes: the exponent's table alone)
-        constexpr uint32_t kLutVecs = FMT == 2 ? 4u * 256u : FMT ? 3u * 4u * 256u : 8u << LB;
+        constexpr uint32_t kLutVecs = LutPlan<D>::kVecs;
         constexpr int kLutLoads = (kLutVecs + 1023) / 1024;
         const uint32_t *lut_g = (const uint32_t *)(k.blob + k.off_lut);
         uint32_t lut_v[kLutLoads];
 #pragma unroll
         for (int i = 0; i < kLutLoads; ++i) {
             const uint32_t v = tid + i * 1024u;
-            lut_v[i] = v < kLutVecs ? __ldg(lut_g + (v >> (FMT ? 2 : 3))) : 0u;
+            lut_v[i] = v < kLutVecs ? __ldg(lut_g + LutPlan<D>::source(v, A.lut_bits)) : 0u;
         }
         if (tid < S) {
             mbar_init(smem_u32(&empty_bar[tid]), 1);
@@ -278,7 +273,7 @@ __global__ void __launch_bounds__(1024, 1) huff_gemm_tc_kernel(const __grid_cons
         uint4 *lut_s = (uint4 *)(dyn_smem + (plan.lut - smem_base));
 #pragma unroll
         for (int i = 0; i < kLutLoads; ++i) {
-            const uint32_t v = tid + i * 1024u, e = SKIP ? lut_entry_inplace(lut_v[i]) : SKIP16 ? fp16_entry_inplace(lut_v[i]) : lut_v[i];
+            const uint32_t v = tid + i * 1024u, e = lut_entry<D>(lut_v[i], LutPlan<D>::field(v));
             if (v < kLutVecs) lut_s[v] = make_uint4(e, e, e, e);
         }
     }
@@ -578,7 +573,8 @@ __global__ void __launch_bounds__(1024, 1) huff_gemm_tc_kernel(const __grid_cons
             // one before: a chunk's start waits for neither
             uint32_t r0 = __ldg(index + c_beg), r1 = __ldg(index + c_beg + 1), r2 = c_beg + 1 < c_end ? __ldg(index + c_beg + 2) : r1;
             bool raw_there = false;
-            const uint8_t *raw_p = payload;
+            const uint8_t *const raw0 = payload + lane * kRawLane;
+            const uint8_t *raw_p = raw0;
             uint4 raw_cur = make_uint4(0, 0, 0, 0), raw_b = make_uint4(0, 0, 0, 0);
 #pragma unroll 1
             for (uint32_t c = c_beg; c < c_end; ++c, ++kc) {
@@ -587,7 +583,7 @@ __global__ void __launch_bounds__(1024, 1) huff_gemm_tc_kernel(const __grid_cons
                 const bool ok = record_ok(r0, r1, nkb), has_next = c + 1 < c_end;
                 const uint32_t r3 = c + 2 < c_end ? __ldg(index + c + 3) : r2;
                 if (ok && !raw_there) {
-                    raw_p = payload + (uint64_t)r0 * 128u + lane * kRawLane;
+                    raw_p = raw0 + (uint64_t)r0 * 128u;
                     raw_cur = load_raw(raw_p);
                 }
                 bounded_wait(bar0 + which * 8, (phase >> which) & 1u);
@@ -599,19 +595,16 @@ __global__ void __launch_bounds__(1024, 1) huff_gemm_tc_kernel(const __grid_cons
                     for (uint32_t kb = 0; kb < nkb; ++kb) stage_block(zero, kb & 1u, (kb & 1u) || kb + 1 < nkb ? 2u : 1u);
                     raw_there = false;
                 } else {
-                    LaneStream sa, sb;
-                    stream_open(sa, slot0 + which * A.slot_bytes + (lane << 2), SKIP ? 7u : SKIP16 ? 6u : 0u);
-                    stream_open(sb, slot0 + which * A.slot_bytes + 128u + (lane << 2), SKIP ? 7u : SKIP16 ? 6u : 0u);
+                    uint32_t pa = (slot0 + which * A.slot_bytes) / 8u + start_of(D), pb = pa;
                     // one block: fetch the next block's raw bytes into the other register set (behind the record's last one: the
                     // next record's first, an address inside the blob whatever its offsets turn out to be), decode this one, hand
                     // it to the tensor core
                     auto block = [&](const uint4 &raw_c, uint4 &raw_n, bool last, uint32_t half, uint32_t nblk) {
                         raw_p += kRawBlock;
-                        if (last) raw_p = payload + (uint64_t)r1 * 128u + lane * kRawLane;
+                        if (last) raw_p = raw0 + (uint64_t)r1 * 128u;
                         if (!last || has_next) raw_n = load_raw(raw_p);
                         uint32_t a[8];
-                        if (FMT) decode_block_fp16<false, SKIP16>(sa, sb, lut_lane, raw_c.x, a);
-                        else decode_block<R, SKIP>(sa, sb, kIdxMask, lut_lane, raw_c, a);
+                        decode_block<D>(pa, pb, lane << 2, lut_lane, lut_low, raw_c, a, 0u, 0u);
                         stage_block(a, half, nblk);
                     };
                     uint32_t kb = 0;
@@ -705,7 +698,12 @@ static cudaError_t launch_tc_one(const TcArgs &t, uint32_t grid, cudaStream_t st
 
 cudaError_t launch_gemm_tc(const TcArgs &t, uint32_t grid, cudaStream_t stream) {
     const KernelArgs &k = t.k;
-    if (k.fmt && k.fp16_flat) {
+    if (k.fmt && k.fp16_flat == kFlatUpper) {
+        if (k.tc_npad == 16) return launch_tc_one<8, 16, 3>(t, grid, stream);
+        if (k.tc_npad == 32) return launch_tc_one<8, 32, 3>(t, grid, stream);
+        return launch_tc_one<8, 64, 3>(t, grid, stream);
+    }
+    if (k.fmt && k.fp16_flat == kFlatBoth) {
         if (k.tc_npad == 16) return launch_tc_one<8, 16, 2>(t, grid, stream);
         if (k.tc_npad == 32) return launch_tc_one<8, 32, 2>(t, grid, stream);
         return launch_tc_one<8, 64, 2>(t, grid, stream);
