@@ -245,7 +245,7 @@ __global__ void __launch_bounds__(kScanThreads) encode_scan_kernel(const __grid_
 // stores are the better choice.  (11008 x 4096: chunks of 512 / 1024 one to a CTA 185 / 97 us, four 90 / 56; FP16 16384 under codes of
 // up to 12 bits staged 157, straight 98.  Whole calls on 28672 x 8192, staged / straight: 2048 574 / 594, 4096 558 / 572, 16384 551 /
 // 526, FP16 995 / 831; at 8192 542 / 526 there, but 158 / 165 on 11008 x 4096.)
-template <bool FP16, uint32_t CHUNKS, bool STAGED>
+template <bool FP16, uint32_t CHUNKS, bool STAGED, bool SHORT>
 __global__ void __launch_bounds__(64 * CHUNKS) encode_write_kernel(const __grid_constant__ EncArgs A) {
     extern __shared__ __align__(16) uint32_t s_coded[];
     __shared__ uint32_t s_code[256];
@@ -263,7 +263,7 @@ __global__ void __launch_bounds__(64 * CHUNKS) encode_write_kernel(const __grid_
     uint32_t *const rows = STAGED ? s_coded + T.sub * A.most_words * 64 : (uint32_t *)(raw + raw_bytes);
     uint32_t *out = rows + T.seq;                                 // word j of this sequence at out[64 j]
     uint32_t acc = 0, nacc = A.lag_bits;
-    auto append = [&](uint32_t b, uint32_t len) {                 // len <= 24, nacc < 32
+    auto append = [&](uint32_t b, uint32_t len) {                 // len <= 32, nacc < 32
         acc |= b << nacc;
         const uint32_t over = __funnelshift_rc(b, 0u, 32u - nacc);         // (nacc = 0: a shift by 32, nothing left over)
         nacc += len;
@@ -275,7 +275,18 @@ __global__ void __launch_bounds__(64 * CHUNKS) encode_write_kernel(const __grid_
         }
     };
     auto code = [&](uint32_t byte_off) -> uint32_t { return *(const uint32_t *)((const char *)s_code + byte_off); };
-    auto append2 = [&](uint32_t e0, uint32_t e1) { append((e0 & 0xFFFFu) | (e1 & 0xFFFFu) << (e0 >> 16), (e0 >> 16) + (e1 >> 16)); };
+    // entries are stream bits and length << 16: two codewords joined, up to 24 bits, or, where none has more than 8 (SHORT), three or four
+    // (whole calls on 11008 x 4096: FP16 442 -> 434 us, BF16 229 -> 228)
+    auto bits2 = [](uint32_t e0, uint32_t e1) -> uint32_t { return (e0 & 0xFFFFu) | (e1 & 0xFFFFu) << (e0 >> 16); };
+    auto append2 = [&](uint32_t e0, uint32_t e1) { append(bits2(e0, e1), (e0 >> 16) + (e1 >> 16)); };
+    auto append3 = [&](uint32_t e0, uint32_t e1, uint32_t e2) {
+        const uint32_t l2 = (e0 >> 16) + (e1 >> 16);
+        append(bits2(e0, e1) | (e2 & 0xFFFFu) << l2, l2 + (e2 >> 16));
+    };
+    auto append4 = [&](uint32_t e0, uint32_t e1, uint32_t e2, uint32_t e3) {
+        const uint32_t l2 = (e0 >> 16) + (e1 >> 16);
+        append(bits2(e0, e1) | bits2(e2, e3) << l2, l2 + (e2 >> 16) + (e3 >> 16));
+    };
     uint4 next = enc_load8(A, T.row, 0);
     for (uint32_t kb = 0; kb < T.nkb; ++kb) {
         const uint32_t x[4] = {next.x, next.y, next.z, next.w};
@@ -286,9 +297,16 @@ __global__ void __launch_bounds__(64 * CHUNKS) encode_write_kernel(const __grid_
 #pragma unroll
             for (int i = 0; i < 4; ++i) {
                 sg |= (x[i] >> 15 & 1u) << (i + 4 * T.half) | (x[i] >> 31) << (i + 4 * T.half + 8);
-                append2(code((x[i] >> 8) & 0x7Cu), code(128u + ((x[i] >> 3) & 0x7Cu)));
-                append2(code(256u + ((x[i] << 2) & 0x7Cu)), code((x[i] >> 24) & 0x7Cu));
-                append2(code(128u + ((x[i] >> 19) & 0x7Cu)), code(256u + ((x[i] >> 14) & 0x7Cu)));
+                const uint32_t e0 = code((x[i] >> 8) & 0x7Cu), e1 = code(128u + ((x[i] >> 3) & 0x7Cu)), e2 = code(256u + ((x[i] << 2) & 0x7Cu));
+                const uint32_t e3 = code((x[i] >> 24) & 0x7Cu), e4 = code(128u + ((x[i] >> 19) & 0x7Cu)), e5 = code(256u + ((x[i] >> 14) & 0x7Cu));
+                if (SHORT) {
+                    append3(e0, e1, e2);
+                    append3(e3, e4, e5);
+                } else {
+                    append2(e0, e1);
+                    append2(e2, e3);
+                    append2(e4, e5);
+                }
             }
             sg |= __shfl_xor_sync(0xFFFFFFFFu, sg, 1);
             if (T.half == 0) *(uint16_t *)(raw + kb * 64 + T.lane * 2) = (uint16_t)sg;
@@ -298,7 +316,16 @@ __global__ void __launch_bounds__(64 * CHUNKS) encode_write_kernel(const __grid_
             for (int i = 0; i < 2; ++i)                           // bytes in the raw layout's order: low bytes' mantissas, high bytes' signs
                 word[i] = (__byte_perm(x[2 * i], x[2 * i + 1], kRawMantSel) & 0x7F7F7F7Fu) | (__byte_perm(x[2 * i], x[2 * i + 1], kRawSignSel) & 0x80808080u);
 #pragma unroll
-            for (int i = 0; i < 4; ++i) append2(code((x[i] >> 5) & 0x3FCu), code((x[i] >> 21) & 0x3FCu));
+            for (int i = 0; i < 4; i += 2) {
+                const uint32_t e0 = code((x[i] >> 5) & 0x3FCu), e1 = code((x[i] >> 21) & 0x3FCu);
+                const uint32_t e2 = code((x[i + 1] >> 5) & 0x3FCu), e3 = code((x[i + 1] >> 21) & 0x3FCu);
+                if (SHORT) {
+                    append4(e0, e1, e2, e3);
+                } else {
+                    append2(e0, e1);
+                    append2(e2, e3);
+                }
+            }
             *(uint2 *)(raw + kb * 512 + T.lane * 16 + T.half * 8) = make_uint2(word[0], word[1]);
         }
     }
@@ -321,11 +348,12 @@ __global__ void __launch_bounds__(64 * CHUNKS) encode_write_kernel(const __grid_
 
 inline uint32_t write_chunks(const EncArgs &A) { return A.Kc <= 128 ? 4 : 1; }
 inline bool write_staged(const EncArgs &A) { return A.Kc <= 512; }      // (at most 37 KB of shared memory)
+template <bool SHORT>
 inline void (*write_kernel_of(bool fp16, uint32_t chunks, bool staged))(EncArgs) {
-    if (fp16) return chunks == 4 ? (staged ? encode_write_kernel<true, 4, true> : encode_write_kernel<true, 4, false>)
-                                 : (staged ? encode_write_kernel<true, 1, true> : encode_write_kernel<true, 1, false>);
-    return chunks == 4 ? (staged ? encode_write_kernel<false, 4, true> : encode_write_kernel<false, 4, false>)
-                       : (staged ? encode_write_kernel<false, 1, true> : encode_write_kernel<false, 1, false>);
+    if (fp16) return chunks == 4 ? (staged ? encode_write_kernel<true, 4, true, SHORT> : encode_write_kernel<true, 4, false, SHORT>)
+                                 : (staged ? encode_write_kernel<true, 1, true, SHORT> : encode_write_kernel<true, 1, false, SHORT>);
+    return chunks == 4 ? (staged ? encode_write_kernel<false, 4, true, SHORT> : encode_write_kernel<false, 4, false, SHORT>)
+                       : (staged ? encode_write_kernel<false, 1, true, SHORT> : encode_write_kernel<false, 1, false, SHORT>);
 }
 
 // ------------------------------------------------------------------------------ checksum of the records
@@ -379,6 +407,7 @@ struct FnvWeights {
     }
 };
 __device__ const FnvWeights<7> g_fnv7{};
+__device__ const FnvWeights<6> g_fnv6{};
 __device__ const FnvWeights<3> g_fnv3{};
 
 __device__ __forceinline__ uint32_t xor_and(uint32_t a, uint32_t b, uint32_t m) {       // (a ^ b) & m
@@ -499,40 +528,78 @@ __device__ __forceinline__ void finish_checksum(const EncArgs &A, unsigned long 
     *(huffllm_desc *)A.blob = d;
 }
 
-constexpr uint32_t kSumWarps = 8;
-
-__global__ void __launch_bounds__(32 * kSumWarps) encode_checksum_kernel(const __grid_constant__ EncArgs A) {
-    __shared__ uint32_t s_words[kSumWarps][7 * 128];
+// A warp goes through its records a step (7, 6 or 3 times 512 bytes) at a time, while the next step's bytes are on their way to its
+// other buffer.  Bound by the integer pipe.  (11008 records of 1600 to 1664 words: a warp per record that waits for every step's
+// bytes, steps of 7 and 3 times 512, 55 us; so 51.  Beside the packing in one kernel, which would leave the record in shared memory,
+// 110 us instead of 46 + 51: 80 registers a thread leave an SM too few warps to pack with.)
+constexpr uint32_t kSumWarps = 8, kSumCtas = 3, kSumBuf = 7 * 128;       // CTAs of an SM (80 registers); words of a step
+constexpr uint32_t kSumSmem = kSumWarps * 2 * kSumBuf * 4;
+struct SumStep {
+    uint64_t c;                  // record
+    uint32_t n, done;            // its words, and those in front of this step
+    const uint32_t *src;
+};
+__global__ void __launch_bounds__(32 * kSumWarps, kSumCtas) encode_checksum_kernel(const __grid_constant__ EncArgs A) {
+    extern __shared__ __align__(16) uint32_t s_steps[];
     __shared__ unsigned long long s_term[kSumWarps];
     const uint32_t lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-    const uint64_t c = (uint64_t)blockIdx.x * kSumWarps + warp;
+    const uint64_t stride = (uint64_t)gridDim.x * kSumWarps;
     if (!enc_fits(A)) return;
-    const uint32_t r0 = c < A.n_chunks ? A.index[c] : 0u, r1 = c < A.n_chunks ? A.index[c + 1] : 0u;
-    const uint32_t *src = (const uint32_t *)(A.payload + (uint64_t)r0 * kRecordUnit);
-    uint32_t *buf = s_words[warp];
-    const uint32_t n = (r1 - r0) * (kRecordUnit / 4);       // words of the record; what is read behind them is zero and adds nothing
-    uint64_t h = kFnvStart;
-    uint32_t done = 0;
+    uint32_t *const buf = s_steps + warp * 2 * kSumBuf;
     // 3, as a value the compiler does not know: times 3 as a shifted addition would join the logic instructions on the
     // integer pipe that bounds this kernel, as a multiplication it runs beside them
     const uint32_t three = 3u + (uint32_t)(A.n_chunks >> 32);
-    while (done < n) {
-        const uint32_t m = n - done > 3 * 128 ? 7u : 3u;
+    auto open = [&](uint64_t c) -> SumStep {
+        if (c >= A.n_chunks) return {c, 0u, 0u, nullptr};
+        const uint32_t r0 = __ldg(A.index + c), r1 = __ldg(A.index + c + 1);
+        return {c, (r1 - r0) * (kRecordUnit / 4), 0u, (const uint32_t *)(A.payload + (uint64_t)r0 * kRecordUnit)};
+    };
+    auto size_of = [](const SumStep &S) -> uint32_t { return S.n - S.done > 6 * 128 ? 7u : S.n - S.done > 3 * 128 ? 6u : 3u; };
+    auto fetch = [&](const SumStep &S, uint32_t *to) {       // (words behind the record are zero and add nothing; it has a multiple of 32)
+        if (S.c < A.n_chunks) {
+            const uint32_t pieces = size_of(S) * 32u, at = (uint32_t)__cvta_generic_to_shared(to);
+            for (uint32_t i = lane; i < pieces; i += 32) {
+                const uint32_t bytes = S.done + 4 * i < S.n ? 16u : 0u;
+                asm volatile("cp.async.cg.shared.global [%0], [%1], 16, %2;" ::"r"(at + 16 * i), "l"(bytes ? S.src + S.done + 4 * i : S.src), "r"(bytes) : "memory");
+            }
+        }
+        asm volatile("cp.async.commit_group;" ::: "memory");
+    };
+    unsigned long long term = 0;
+    uint64_t h = kFnvStart;
+    SumStep cur = open((uint64_t)blockIdx.x * kSumWarps + warp), after = open(cur.c + stride);
+    uint32_t which = 0;
+    fetch(cur, buf);
+#pragma unroll 1
+    while (cur.c < A.n_chunks) {
+        const uint32_t m = size_of(cur);
+        SumStep next = cur;
+        next.done += m * 128;
+        const bool last = next.done >= cur.n;
+        if (last) {
+            next = after;
+            after = open(next.c + stride);                   // (wanted a record later)
+        }
         __syncwarp();
-#pragma unroll
-        for (int i = 0; i < 7 * 4; ++i)
-            if (i < (int)m * 4) buf[i * 32 + lane] = done + i * 32 < n ? __ldcg(src + done + i * 32 + lane) : 0u;
+        fetch(next, buf + (which ^ 1u) * kSumBuf);
+        asm volatile("cp.async.wait_group 1;" ::: "memory");
         __syncwarp();
-        h = m == 7u ? fnv_step<7>(h, buf, g_fnv7, lane, three) : fnv_step<3>(h, buf, g_fnv3, lane, three);
-        done += m * 128;
+        const uint32_t *const words = buf + which * kSumBuf;
+        h = m == 7u ? fnv_step<7>(h, words, g_fnv7, lane, three) : m == 6u ? fnv_step<6>(h, words, g_fnv6, lane, three) : fnv_step<3>(h, words, g_fnv3, lane, three);
+        if (last) {
+            // the zero bytes behind the record multiplied h by P each: a multiple of 32 words
+            constexpr uint64_t kUnitBack = fnv_pow(kFnvInverse, kRecordUnit);
+            for (uint32_t p = cur.n; p < cur.done + m * 128; p += kRecordUnit / 4) h *= kUnitBack;
+            term += h * (2 * cur.c + 1);
+            h = kFnvStart;
+        }
+        cur = next;
+        which ^= 1u;
     }
-    // the zero bytes behind the record multiplied h by P each: (done - n) words, a multiple of 32
-    constexpr uint64_t kUnitBack = fnv_pow(kFnvInverse, kRecordUnit);
-    for (uint32_t p = n; p < done; p += kRecordUnit / 4) h *= kUnitBack;
-    if (lane == 0) s_term[warp] = n ? h * (2 * c + 1) : 0ull;
+    if (lane == 0) s_term[warp] = term;
     __syncthreads();
     if (threadIdx.x) return;
-    unsigned long long term = 0;
+    term = 0;
     for (uint32_t i = 0; i < kSumWarps; ++i) term += s_term[i];
     finish_checksum(A, term);
 }
@@ -637,7 +704,7 @@ extern "C" huffllm_status huffllm_encode_device(const huffllm_codebook *cb, cons
     auto cuda_fail = [&](const char *what) { return fail(HUFFLLM_ERR_CUDA, "%s: %s", what, cudaGetErrorString(e)); };
     const auto size_kernel = A.fp16 ? encode_size_kernel<true> : encode_size_kernel<false>;
     const uint32_t chunks = write_chunks(A), smem = write_staged(A) ? chunks * A.most_words * 256 : 0;
-    const auto write_kernel = write_kernel_of(A.fp16 != 0, chunks, smem != 0);
+    const auto write_kernel = longest <= 8 ? write_kernel_of<true>(A.fp16 != 0, chunks, smem != 0) : write_kernel_of<false>(A.fp16 != 0, chunks, smem != 0);
     // code lengths and table, assembled on the host; the header's bytes stay zero until the last kernel writes them
     std::vector<uint8_t> fixed((size_t)d.off_index, 0);
     write_fixed_sections(cb, d, fixed.data());
@@ -651,8 +718,10 @@ extern "C" huffllm_status huffllm_encode_device(const huffllm_codebook *cb, cons
     write_kernel<<<(uint32_t)((d.n_chunks + chunks - 1) / chunks), 64 * chunks, smem, s>>>(A);
     if (checksum_each(d.n_chunks, chunk_elems))
         encode_checksum_each_kernel<<<(uint32_t)((d.n_chunks + kEachThreads - 1) / kEachThreads), kEachThreads, 0, s>>>(A);
-    else
-        encode_checksum_kernel<<<(uint32_t)((d.n_chunks + kSumWarps - 1) / kSumWarps), 32 * kSumWarps, 0, s>>>(A);
+    else {
+        if ((e = cudaFuncSetAttribute(encode_checksum_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kSumSmem)) != cudaSuccess) return cuda_fail("cudaFuncSetAttribute");
+        encode_checksum_kernel<<<(uint32_t)std::min<uint64_t>(kSumCtas * 148, (d.n_chunks + kSumWarps - 1) / kSumWarps), 32 * kSumWarps, kSumSmem, s>>>(A);
+    }
     if ((e = cudaGetLastError()) != cudaSuccess) return cuda_fail("encoder launches");
     EncTotals tot;
     if ((e = cudaMemcpyAsync(&tot, scr, sizeof(tot), cudaMemcpyDeviceToHost, s)) != cudaSuccess || (e = cudaStreamSynchronize(s)) != cudaSuccess)
