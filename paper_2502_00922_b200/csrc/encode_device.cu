@@ -705,15 +705,15 @@ extern "C" huffllm_status huffllm_encode_device(const huffllm_codebook *cb, cons
     const auto size_kernel = A.fp16 ? encode_size_kernel<true> : encode_size_kernel<false>;
     const uint32_t chunks = write_chunks(A), smem = write_staged(A) ? chunks * A.most_words * 256 : 0;
     const auto write_kernel = longest <= 8 ? write_kernel_of<true>(A.fp16 != 0, chunks, smem != 0) : write_kernel_of<false>(A.fp16 != 0, chunks, smem != 0);
-    // code lengths and table, assembled on the host; the header's bytes stay zero until the last kernel writes them
-    std::vector<uint8_t> fixed((size_t)d.off_index, 0);
-    write_fixed_sections(cb, d, fixed.data());
-    memset(fixed.data(), 0, sizeof(d));
-    if ((e = cudaMemcpyAsync(blob, fixed.data(), fixed.size(), cudaMemcpyHostToDevice, s)) != cudaSuccess) return cuda_fail("copy of the fixed sections");
     if ((e = cudaMemsetAsync(scr, 0, cleared, s)) != cudaSuccess) return cuda_fail("cudaMemsetAsync");
     A.size_groups = size_groups(A);
     const uint64_t per_cta = (uint64_t)kSizeChunks * A.size_groups;
     size_kernel<<<(uint32_t)((d.n_chunks + per_cta - 1) / per_cta), kSizeThreads, 0, s>>>(A);
+    // code lengths and table, assembled on the host while pass 1 runs; the header's bytes stay zero until the last kernel writes them
+    std::vector<uint8_t> fixed((size_t)d.off_index, 0);
+    write_fixed_sections(cb, d, fixed.data());
+    memset(fixed.data(), 0, sizeof(d));
+    if ((e = cudaMemcpyAsync(blob, fixed.data(), fixed.size(), cudaMemcpyHostToDevice, s)) != cudaSuccess) return cuda_fail("copy of the fixed sections");
     encode_scan_kernel<<<(uint32_t)((d.n_chunks + 64 + kScanThreads - 1) / kScanThreads), kScanThreads, 0, s>>>(A);
     write_kernel<<<(uint32_t)((d.n_chunks + chunks - 1) / chunks), 64 * chunks, smem, s>>>(A);
     if (checksum_each(d.n_chunks, chunk_elems))

@@ -70,7 +70,7 @@ huffllm_status check_desc(const huffllm_desc *d) {
 
 // ------------------------------------------------------------------ code construction
 
-// Optimal prefix-code lengths with every length <= cap, by exhaustive dynamic programming over
+// Optimal prefix-code lengths with every length <= cap, by dynamic programming over
 // the Kraft budget: state = (symbols placed, budget spent in units of 2^-cap).
 static bool limited_lengths(const uint64_t *counts, int nsym, int cap, uint8_t *len) {
     std::vector<int> used;
@@ -83,30 +83,37 @@ static bool limited_lengths(const uint64_t *counts, int nsym, int cap, uint8_t *
     if (n == 1) { len[used[0]] = 1; return true; }
     if (cap < 1 || cap > 15 || (1 << cap) < n) return false;
     std::stable_sort(used.begin(), used.end(), [&](int a, int b) { return counts[a] > counts[b]; });
+    // Of the states with the symbols placed so far only those are gone on from that no state of less budget spent equals in cost:
+    // whatever completes the others completes that one too, at no more cost and less budget, which is what the last choice
+    // (least cost, then least budget) prefers.  States that leave the symbols still to come less than one unit each cannot be
+    // completed.  (Codebooks from counts, us: all states / these, BF16 at 8 and 12 bits 33 / 20 and 926 / 220, FP16 179 / 97 and
+    // 6150 / 630.)
     const int U = 1 << cap;
     const uint64_t INF = ~0ull;
-    std::vector<uint64_t> cost((size_t)(n + 1) * (U + 1), INF);
-    std::vector<uint8_t> choice((size_t)(n + 1) * (U + 1), 0);
-    cost[0] = 0;
-    for (int i = 0; i < n; ++i)
-        for (int b = 0; b <= U; ++b) {
-            uint64_t c = cost[(size_t)i * (U + 1) + b];
-            if (c == INF) continue;
-            for (int l = 1; l <= cap; ++l) {
-                int nb = b + (U >> l);
-                if (nb > U) continue;
-                uint64_t v = c + counts[used[i]] * (uint64_t)l;
-                size_t k = (size_t)(i + 1) * (U + 1) + nb;
-                if (v < cost[k]) { cost[k] = v; choice[k] = (uint8_t)l; }
+    std::vector<uint64_t> cost((size_t)2 * (U + 1));         // of the symbols so far, and with one more
+    std::vector<uint8_t> choice((size_t)(n + 1) * (U + 1));
+    std::vector<int> open(1, 0);
+    uint64_t *from = cost.data(), *to = from + U + 1;
+    from[0] = 0;
+    for (int i = 0; i < n; ++i) {
+        uint8_t *pick = &choice[(size_t)(i + 1) * (U + 1)];
+        const int most = U - (n - 1 - i);
+        std::fill(to, to + U + 1, INF);
+        for (int b : open)
+            for (int l = cap; l >= 1; --l) {
+                const int nb = b + (U >> l);
+                if (nb > most) break;
+                const uint64_t v = from[b] + counts[used[i]] * (uint64_t)l;
+                if (v < to[nb]) { to[nb] = v; pick[nb] = (uint8_t)l; }
             }
-        }
-    int best_b = -1;
-    for (int b = 0; b <= U; ++b)
-        if (cost[(size_t)n * (U + 1) + b] != INF &&
-            (best_b < 0 || cost[(size_t)n * (U + 1) + b] < cost[(size_t)n * (U + 1) + best_b]))
-            best_b = b;
-    if (best_b < 0) return false;
-    for (int i = n, b = best_b; i > 0; --i) {
+        open.clear();
+        uint64_t least = INF;
+        for (int b = 0; b <= most; ++b)
+            if (to[b] < least) { least = to[b]; open.push_back(b); }
+        std::swap(from, to);
+    }
+    if (open.empty()) return false;
+    for (int i = n, b = open.back(); i > 0; --i) {
         int l = choice[(size_t)i * (U + 1) + b];
         len[used[i - 1]] = (uint8_t)l;
         b -= U >> l;
@@ -305,12 +312,17 @@ static huffllm_status codebook_from_counts(huffllm_dtype dtype, huffllm_split sp
     }
 
     bool have = false;
-    uint64_t best = 0;
+    uint64_t best = 0, least0 = 0;
     uint8_t l0[32], l1[32];
     for (uint32_t c0 = 1; c0 < budget; ++c0) {
         uint32_t c1 = budget - c0;
-        if (!limited_lengths(cb->counts[0], 16, (int)c0, l0) || !limited_lengths(cb->counts[1], 16, (int)c1, l1)) continue;
-        uint64_t cost = code_cost(cb->counts[0], l0, 16) + code_cost(cb->counts[1], l1, 16);
+        if (!limited_lengths(cb->counts[0], 16, (int)c0, l0)) continue;
+        // (the lower nibbles' cost does not fall as their cap does: where the upper ones gain nothing, neither does the sum)
+        const uint64_t cost0 = code_cost(cb->counts[0], l0, 16);
+        if (have && cost0 >= least0) continue;
+        if (!limited_lengths(cb->counts[1], 16, (int)c1, l1)) continue;
+        least0 = cost0;
+        uint64_t cost = cost0 + code_cost(cb->counts[1], l1, 16);
         if (!have || cost < best) {
             have = true;
             best = cost;

@@ -1,0 +1,83 @@
+"""The codebook builder goes on from the least-cost states of its dynamic programme only; the lengths must be those of the
+programme over all states, ties included (a blob's bytes depend on them).  CPU only."""
+import numpy as np
+import pytest
+
+INF = 1 << 62
+
+
+def lengths_over_all_states(counts, cap):
+    """State = (symbols placed, most frequent first; budget spent in units of 2^-cap).  Among equal costs the shortest last
+    length, at the end the least budget."""
+    used = sorted((s for s in range(len(counts)) if counts[s]), key=lambda s: -counts[s])
+    out = [0] * len(counts)
+    if len(used) == 1:
+        out[used[0]] = 1
+        return out
+    U = 1 << cap
+    if U < len(used):
+        return None
+    cost, choice = [0] + [INF] * U, []
+    for s in used:
+        to, pick = [INF] * (U + 1), [0] * (U + 1)
+        for b in range(U + 1):
+            for l in range(1, cap + 1) if cost[b] < INF else ():
+                nb = b + (U >> l)
+                if nb <= U and cost[b] + counts[s] * l < to[nb]:
+                    to[nb], pick[nb] = cost[b] + counts[s] * l, l
+        cost = to
+        choice.append(pick)
+    b = cost.index(min(cost))
+    for s, pick in zip(reversed(used), reversed(choice)):
+        out[s] = pick[b]
+        b -= U >> pick[b]
+    return out
+
+
+def draw(kind, n, rng):
+    if kind == "equal":
+        return [7] * n
+    if kind == "few values":
+        return [int(v) for v in rng.integers(0, 4, n)]
+    if kind == "few symbols":
+        return [int(v) if rng.random() < 0.2 else 0 for v in rng.integers(1, 1000, n)]
+    if kind == "halving":
+        return [int(1e8 * 0.5 ** abs(i - 11)) for i in range(n)]
+    return [int(2.0 ** v) for v in rng.uniform(0, 30, n)]
+
+
+KINDS = ["equal", "few values", "few symbols", "halving", "wide"]
+
+
+@pytest.mark.parametrize("kind", KINDS)
+@pytest.mark.parametrize("limit", [7, 8, 9])
+def test_fp16_field_lengths(kind, limit):
+    import paper_2502_00922_b200 as hl
+    rng = np.random.default_rng(limit)
+    fields = [draw(kind, 32, rng) for _ in range(3)]
+    for f in fields:
+        f[5] += 1                                            # (an empty field has no code)
+    cb = hl.build_codebook_from_counts(np.array(sum(fields, []), dtype=np.uint64), hl.FP16, limit)
+    for i, f in enumerate(fields):
+        assert list(cb.get(i)[2][:32]) == lengths_over_all_states(f, limit)
+    cb.free()
+
+
+@pytest.mark.parametrize("kind", KINDS)
+@pytest.mark.parametrize("budget", [8, 9, 12])
+def test_bf16_nibble_lengths_over_every_split_of_the_budget(kind, budget):
+    import paper_2502_00922_b200 as hl
+    counts = draw(kind, 256, np.random.default_rng(budget))
+    counts[121] += 1
+    hi = [sum(counts[16 * h:16 * h + 16]) for h in range(16)]
+    lo = [sum(counts[l::16]) for l in range(16)]
+    best = None
+    for c0 in range(1, budget):                              # least cost, ties to the smaller cap of the upper nibble
+        a, b = lengths_over_all_states(hi, c0), lengths_over_all_states(lo, budget - c0)
+        if a and b:
+            cost = sum(x * y for x, y in zip(hi, a)) + sum(x * y for x, y in zip(lo, b))
+            if best is None or cost < best[0]:
+                best = (cost, a, b)
+    cb = hl.build_codebook_from_counts(np.array(counts, dtype=np.uint64), hl.BF16, budget)
+    assert list(cb.get(0)[2][:16]) == best[1] and list(cb.get(1)[2][:16]) == best[2]
+    cb.free()
