@@ -236,7 +236,7 @@ huffllm_status huffllm_workspace_control_bytes(const huffllm_desc *desc, size_t 
  * product calls) is left alone by a sound blob and otherwise set to: c + 1 if chunk c's record offsets point outside
  * the payload or do not fit (that chunk is skipped, nothing is read through them); 0x40000000 + c + 1 if chunk c's bits
  * made the decoder run past the end of its record (a damaged coded part: the chunk's output is wrong, but no read left
- * the CTA's shared memory: a sequence moves on by at most one row per refill check, and room for that is kept, see
+ * the CTA's shared memory: a sequence moves on by at most its tables' longest codewords, and room for that is kept, see
  * huffllm_decode_smem_plan); -1 if a copy never arrived within the wait limit.  A damaged coded part that still ends
  * inside its record is not detectable here: huffllm_validate_blob (host, checksum) is the check for that.
  */
@@ -246,8 +246,9 @@ huffllm_status huffllm_decode(const huffllm_desc *desc, const void *blob_dev, ui
 /*
  * The shared-memory budget a decoder CTA keeps for this blob (host call, no device needed; any pointer may be null):
  * bytes of the decode table(s), bytes of one slot (the coded rows of the largest record: max_words * 256), the number
- * of refill checks per bit sequence and block of 32 columns, and the readable bytes kept behind the last slot,
- * 256 * (3 + checks * blocks per chunk): the furthest row any stream, sound or not, can make the decoder touch.
+ * of rows budgeted per bit sequence and block of 32 columns (its name is from decoders that checked for a refill once a
+ * row), and the readable bytes kept behind the last slot, 256 * (3 + that * blocks per chunk): beyond the furthest row any
+ * stream, sound or not, can make the decoder touch.
  */
 huffllm_status huffllm_decode_smem_plan(const huffllm_desc *desc, uint32_t *table_bytes, uint32_t *slot_bytes,
                                         uint32_t *refill_checks_per_block, uint32_t *guard_bytes);

@@ -79,7 +79,7 @@ size_t ws_bytes_for(const huffllm_desc *d, uint32_t batch) {
 struct SmemNeeds {
     uint32_t table_align, table_bytes;   // window of the decode table(s)
     uint32_t slot_bytes;                 // one slot: the W rows of the largest record
-    uint32_t checks_per_block;           // refill checks per bit sequence and block of 32 columns
+    uint32_t checks_per_block;           // rows a sequence may move on in a block of 32 columns, as budgeted
     uint32_t guard_bytes;                // readable bytes kept behind the last slot
 };
 // Which mantissa halves of an FP16 blob carry the flat code and can be read without a table (codes of at most 8 bits).
@@ -104,13 +104,13 @@ SmemNeeds smem_needs(const huffllm_desc *desc) {
     n.table_align = fmt ? 16384u : 128u << (two_level ? 8u : desc->lut_bits);
     n.table_bytes = fmt ? fp16_table_bytes(two_level ? kFlatNone : flat_of(desc)) + (two_level ? 3u * (4u << desc->lut_bits) : 0u)
                         : (two_level ? (128u << 8) + (4u << desc->lut_bits) : 128u << desc->lut_bits);
-    // a slot holds the W rows of a record; the window runs one row ahead of what it consumes, and that look-ahead
-    // past the last row lands in the next slot, the table or the guard area and is never used
+    // a slot holds the W rows of a record; the windows run up to two rows ahead of the pointer, and what they read
+    // past the last row lies in the next slot, the table or the guard area and is never used
     n.slot_bytes = desc->max_words * 256;
-    // A stream can move its read pointer by one row per refill check and no further, whatever its bits and whatever the
-    // table says: a sequence opens on rows 0 and 1, and every check loads at most the next row.  The furthest row a
-    // chunk's decoder can touch is therefore 1 + checks, counted from the slot's first row, and the bytes kept readable
-    // behind the last slot cover that for a slot of any size.
+    // No table in shared memory holds a length above what its index bits allow (lut_entry), so a block moves a sequence by
+    // 64 bits (8-bit BF16 tables) to 288 (FP16, fields of up to 12 bits), two to nine rows, whatever its bits and whatever
+    // the blob's table says.  The budget is that of decoders that took a check per row (three to 24 a block): it covers
+    // these too, for a slot of any size.
     n.checks_per_block = fmt ? (two_level ? 24 : 8) : (desc->lut_bits == 8 ? 3 : 4);
     n.guard_bytes = 256 * (3 + n.checks_per_block * (desc->chunk_cols / kBlockCols));
     return n;
