@@ -92,7 +92,8 @@ __device__ __forceinline__ void store_piece(uint16_t *dst, const uint4 &p, int32
 // LB = table index bits (the blobs' lut_bits): 8 or 9; LB = 12 stands for every longer limit up to 12 (BF16: 10..12,
 // FP16: 9..12): two-level lookup, the number of bits is A.lut_bits.
 // FMT = 0: BF16 blobs; FMT = 1: FP16 {1,5,5,5} blobs (three lookups per weight, sign bits as the raw part); FMT = 2: the same
-// where both mantissa halves carry the flat 5-bit code (8-bit tables only: one lookup and a bit reversal per weight).
+// where both mantissa halves carry the flat 5-bit code (codes of up to 8 bits: one lookup per weight and a bit reversal per two);
+// FMT = 3: where the upper half does (two lookups).
 //
 // One launch works through a LIST of matrices (A.n_mats, usually the matrices of one decoder layer that
 // may run together).  The CTAs are dealt out to the matrices in proportion to their chunks, so every CTA
@@ -303,7 +304,7 @@ __global__ void __launch_bounds__(THREADS, 1) huff_kernel(const __grid_constant_
         const uint32_t g_lo = rg * KC, g_hi = g_lo + KC, my_lo = max(g_lo, cta_beg), my_hi = min(g_hi, cta_end);  // its chunks, and this CTA's part
         const bool alone = first_c <= my_lo && last_c_excl >= my_hi;   // no other warp of this CTA holds a piece
         // D fragment -> output order (o = column * 16 + row) through this warp's shared-memory entry: the first one for the
-        // row group that the warp's range starts in front of or at, the second for the one it starts inside of
+        // row group that the warp's range starts in, the second for those behind it
         const uint32_t mine = warp * 2 + (c_beg >= g_lo ? 0u : 1u);
         if (NT == 0) {
             // acc[0]: this lane's eight columns of row g; acc[2]: of row g + 8.  The four lanes of a row add theirs
@@ -352,7 +353,7 @@ __global__ void __launch_bounds__(THREADS, 1) huff_kernel(const __grid_constant_
                 if (lane + 32 * i < vals) v[i] += piece[32 * i];
         }
         if (cta_beg > g_lo || cta_end < g_hi) {               // other CTAs have pieces too
-            // slot 0 holds the piece of the row group that a CTA's range starts in front of or at, slot 1 of the other one
+            // slot 0 holds the piece of the row group that a CTA's range starts in, slot 1 that of its last one
             float *const parts = k.ws_partial + lane;
             float *const to = parts + ((size_t)J * 2 + (cta_beg >= g_lo ? 0u : 1u)) * vals;
 #pragma unroll

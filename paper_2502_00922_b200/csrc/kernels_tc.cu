@@ -129,7 +129,7 @@ __device__ __forceinline__ bool elect_one() {
     return p != 0;
 }
 
-// LB = table index bits; NPAD = batch rounded up to 16, 32 or 64 (the MMA's N); FMT = 0: BF16 blobs, 1: FP16 {1,5,5,5} blobs, 2: FP16 blobs with flat mantissa codes
+// LB = table index bits; NPAD = batch rounded up to 16, 32 or 64 (the MMA's N); FMT = 0: BF16 blobs, 1: FP16 {1,5,5,5} blobs, 2 / 3: those with flat mantissa codes, see huff_kernel
 // (three tables, sign words as the raw part, f16 operands).
 // MULTI: the launch works through several matrices (a launch over one matrix reads its arguments without an index).
 template <int LB, int NPAD, int FMT, bool MULTI>
