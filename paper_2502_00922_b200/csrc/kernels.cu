@@ -30,6 +30,7 @@
 #include <type_traits>
 
 #include "decode_common.cuh"
+#include "row_pieces.h"
 
 namespace huffllm {
 
@@ -61,11 +62,12 @@ __device__ __forceinline__ uint4 shifted_piece(uint32_t from, uint32_t sel) {
 // one end only (all but those of rows shorter than a piece) takes three stores of 8, 4 and 2 bytes: n weights from its
 // front or up to its end fall into such stores by the bits of n.
 __device__ __forceinline__ void store_piece(uint16_t *dst, const uint4 &p, int32_t c, int32_t first, int32_t end) {
-    if (c >= first && c + 8 <= end) {
+    const PieceCut cut = piece_cut(c, first, end);
+    const int32_t lo = cut.lo, hi = cut.hi;
+    if (lo == 0 && hi == 8) {
         *(uint4 *)dst = p;
         return;
     }
-    const int32_t lo = max(first - c, 0), hi = min(end - c, 8);        // weights lo .. hi - 1 of the piece
     if (lo >= hi) return;
     const uint32_t w[4] = {p.x, p.y, p.z, p.w};
     if (hi == 8) {
@@ -400,9 +402,8 @@ __global__ void __launch_bounds__(THREADS, 1) huff_kernel(const __grid_constant_
         const uint32_t row_left = MODE == 2 ? smem_base + A.dyn_smem_bytes - A.part_bytes + (warp * 16u + g) * kRowBuf : 0u;
         const uint32_t row_new = row_left + 32u;
         constexpr int kRowHalf = 8 * kRowBuf;           // rows g + 8: as much further on
-        // The columns that a warp has decoded of a row group without a gap, from run_first on, are stored as one run: a chunk's
-        // last row_off columns wait in the row buffers for the next chunk's first pieces.
-        int32_t run_first = 0;
+        // The columns that a warp has decoded of a row group without a gap are stored as one run: a chunk's last row_off columns
+        // wait in the row buffers for the next chunk's first pieces.
         bool left_over = false;
         struct Rows {                                   // rows g and g + 8, which start 8 * cols weights apart, at the same place in a sector
             uint32_t off, from, sel;                    // row_off; the piece's five words start (row_off + 1) / 2 words in front of the
@@ -424,11 +425,12 @@ __global__ void __launch_bounds__(THREADS, 1) huff_kernel(const __grid_constant_
         auto store_left_over = [&]() {
             __syncwarp();
             const Rows R = rows_of();
-            const int32_t end = (int32_t)min((uint64_t)kc * k.chunk_cols, k.cols), c = ((end + 31) & ~31) + (int32_t)(t * 8u) - (int32_t)R.off;
             if (left_over && t * 8u < R.off) {
-                uint16_t *const dst = k.out + (R.first + c);
-                if (R.ok[0]) store_piece(dst, shifted_piece<0>(R.from, R.sel), c, run_first, end);
-                if (R.ok[1]) store_piece(dst + 8 * k.cols, shifted_piece<kRowHalf>(R.from, R.sel), c, run_first, end);
+                const uint32_t at = (kc - 1u) * k.chunk_cols;       // the run's last chunk
+                const int32_t end = min(columns_left(k.cols, at), (int32_t)k.chunk_cols), c = last_piece_column(end, t, R.off);
+                uint16_t *const dst = k.out + (R.first + at + c);
+                if (R.ok[0]) store_piece(dst, shifted_piece<0>(R.from, R.sel), c, 0, end);
+                if (R.ok[1]) store_piece(dst + 8 * k.cols, shifted_piece<kRowHalf>(R.from, R.sel), c, 0, end);
             }
             left_over = false;
             __syncwarp();
@@ -490,13 +492,13 @@ __global__ void __launch_bounds__(THREADS, 1) huff_kernel(const __grid_constant_
                 // here, so every block of the chunk lies inside the row and xq ends the chunk where the next begins)
                 uint16_t *out0 = MODE == 0 ? k.out + ((uint64_t)rg * 16 + g) * k.cols + col0 : nullptr;
                 Rows R;
-                uint32_t inner_from = 0, inner_to = 0;           // MODE 2: the blocks all of whose pieces are stored whole
+                uint32_t inner_from = 0;                         // MODE 2: the blocks all of whose pieces are stored whole start here ...
+                int32_t row_left_cols = 0;                       // ... and end with the columns that are left of the row
                 if (MODE != 1) {
                     R = rows_of();
-                    if (MODE == 2) out0 = k.out + (R.first + (int32_t)col0 - (int32_t)R.off);
-                    if (!left_over) run_first = (int32_t)(kc * k.chunk_cols);
+                    if (MODE == 2) out0 = k.out + (R.first + kc * k.chunk_cols + piece_column(0, t, R.off));
                     inner_from = left_over ? 0u : 1u;
-                    inner_to = ((uint32_t)k.cols - kc * k.chunk_cols) >> 5;
+                    row_left_cols = columns_left(k.cols, kc * k.chunk_cols);
                     left_over = true;
                 }
                 // one block, number kb of the chunk and `i` behind where raw_p and xq stand: decode with `cur` while the raw bytes
@@ -553,13 +555,13 @@ __global__ void __launch_bounds__(THREADS, 1) huff_kernel(const __grid_constant_
                         sts_row<kRowHalf>(row_new + t * 16u, a + 4);
                         __syncwarp();
                         const uint4 p0 = shifted_piece<0>(R.from, R.sel), p1 = shifted_piece<kRowHalf>(R.from, R.sel);
-                        if (kb >= inner_from && kb < inner_to) {
+                        if (kb >= inner_from && (int32_t)(kb * 32u + 32u) <= row_left_cols) {
                             if (R.ok[0]) *(uint4 *)out0 = p0;
                             if (R.ok[1]) *(uint4 *)(out0 + 8 * k.cols) = p1;
                         } else {
-                            const int32_t c = (int32_t)(col0 + kb * 32u) - (int32_t)R.off;
-                            if (R.ok[0]) store_piece(out0, p0, c, run_first, (int32_t)k.cols);
-                            if (R.ok[1]) store_piece(out0 + 8 * k.cols, p1, c, run_first, (int32_t)k.cols);
+                            const int32_t c = piece_column(kb, t, R.off), run_first = run_start(inner_from == 0u);
+                            if (R.ok[0]) store_piece(out0, p0, c, run_first, row_left_cols);
+                            if (R.ok[1]) store_piece(out0 + 8 * k.cols, p1, c, run_first, row_left_cols);
                         }
                         out0 += 32;
                         __syncwarp();
