@@ -40,11 +40,13 @@ namespace huffllm {
 // behind its start.  What bounds the output is L2's handling of sector writes, so the warp stores whole sectors: each of its
 // 16 rows has 96 bytes of shared memory (the row's last sixteen weights of the block before, then the block's 32); a lane
 // writes its own eight weights there and reads back, moved on by row_off weights, the five words that its 16-byte piece of
-// the output covers (a word offset, then half a word by byte permutation).  A quad's four pieces are two whole sectors.
-// Only the pieces at the two ends of a chunk's columns are stored in parts.
-// Measured (BF16, 11007 x 4099 / 28672 x 8191; 11008 x 4096 takes 38.9 us): every lane storing its eight weights one by
+// the output covers (a word offset, then half a word by byte permutation).  A quad's four pieces are two whole sectors, in
+// rows g and g + 8 alike: with an odd column count those lie half a sector apart and have offsets of their own.
+// Only the pieces at the two ends of a run of chunks are stored in parts.
+// Measured (BF16, 11007 x 4099 / 28672 x 8191; 11008 x 4096 takes 33.0 us): every lane storing its eight weights one by
 // one, 320 partial sector writes per block of 512 weights, 178 us / -; pieces on 16-byte boundaries through quad shuffles,
-// 48 sectors per block, 57 / 293 us; through shared memory 56 / 291; on 32-byte boundaries (this) 48 / 227 us.
+// 48 sectors per block, 57 / 293 us; through shared memory 56 / 291; all this by the decoder of the time.  Rows g + 8 on
+// 16-byte boundaries 49.8 / 250 us; all on 32-byte boundaries (this) 42.8 / 196 us.
 template <int OFF>
 __device__ __forceinline__ void sts_row(uint32_t addr, const uint32_t *v) {
     asm volatile("st.shared.v4.u32 [%0+%5], {%1, %2, %3, %4};" ::"r"(addr), "r"(v[0]), "r"(v[1]), "r"(v[2]), "r"(v[3]), "n"(OFF) : "memory");
@@ -405,17 +407,20 @@ __global__ void __launch_bounds__(THREADS, 1) huff_kernel(const __grid_constant_
         // The columns that a warp has decoded of a row group without a gap are stored as one run: a chunk's last row_off columns
         // wait in the row buffers for the next chunk's first pieces.
         bool left_over = false;
-        struct Rows {                                   // rows g and g + 8, which start 8 * cols weights apart, at the same place in a sector
-            uint32_t off, from, sel;                    // row_off; the piece's five words start (row_off + 1) / 2 words in front of the
-                                                        // lane's own weights, its weights half a word further where row_off is odd
-            int64_t first;                              // the row's first weight in the output
+        struct Rows {                                   // rows g and g + 8
+            uint32_t off, from, sel;                    // row g's row_off; the piece's five words start (row_off + 1) / 2 words in front of
+                                                        // the lane's own weights, its weights half a word further where row_off is odd
+            int32_t half;                               // row g + 8's pieces start so many columns further on (see row_half)
+            int64_t first;                              // row g's first weight in the output
             bool ok[2];
         };
+        auto row_off = [&]() -> uint32_t { return ((rg * 16u + g) * (uint32_t)k.cols + (uint32_t)((uintptr_t)k.out >> 1)) & 15u; };
         auto rows_of = [&]() -> Rows {
             Rows R;
-            R.off = ((rg * 16u + g) * (uint32_t)k.cols + (uint32_t)((uintptr_t)k.out >> 1)) & 15u;
+            R.off = row_off();
             R.from = row_new + t * 16u - ((R.off + 1u) >> 1) * 4u;
             R.sel = (R.off & 1u) ? 0x5432u : 0x3210u;
+            R.half = row_half(R.off, (uint32_t)k.cols);
             R.first = (int64_t)(((uint64_t)rg * 16 + g) * k.cols);
             R.ok[0] = (uint64_t)rg * 16 + g < k.rows;
             R.ok[1] = (uint64_t)rg * 16 + g + 8 < k.rows;
@@ -425,12 +430,15 @@ __global__ void __launch_bounds__(THREADS, 1) huff_kernel(const __grid_constant_
         auto store_left_over = [&]() {
             __syncwarp();
             const Rows R = rows_of();
-            if (left_over && t * 8u < R.off) {
-                const uint32_t at = (kc - 1u) * k.chunk_cols;       // the run's last chunk
-                const int32_t end = min(columns_left(k.cols, at), (int32_t)k.chunk_cols), c = last_piece_column(end, t, R.off);
-                uint16_t *const dst = k.out + (R.first + at + c);
-                if (R.ok[0]) store_piece(dst, shifted_piece<0>(R.from, R.sel), c, 0, end);
-                if (R.ok[1]) store_piece(dst + 8 * k.cols, shifted_piece<kRowHalf>(R.from, R.sel), c, 0, end);
+            if (left_over) {                            // (the block behind the run's last one: nothing of it was decoded)
+                const uint32_t at = (kc - 1u) * k.chunk_cols;
+                const int32_t cols = min(columns_left((uint32_t)k.cols, at), (int32_t)k.chunk_cols), block = (cols + 31) & ~31;
+                auto store_last = [&](const uint4 &p, int32_t h, uint32_t off) {
+                    const int32_t c = piece_column(t, off);
+                    if (R.ok[h] && c < 0) store_piece(k.out + (R.first + 8 * h * (int64_t)k.cols + at + (block + c)), p, c, run_start(false), cols - block);
+                };
+                store_last(shifted_piece<0>(R.from, R.sel), 0, R.off);
+                store_last(shifted_piece<kRowHalf>(R.from + 2 * R.half, R.sel), 1, R.off - R.half);
             }
             left_over = false;
             __syncwarp();
@@ -492,13 +500,13 @@ __global__ void __launch_bounds__(THREADS, 1) huff_kernel(const __grid_constant_
                 // here, so every block of the chunk lies inside the row and xq ends the chunk where the next begins)
                 uint16_t *out0 = MODE == 0 ? k.out + ((uint64_t)rg * 16 + g) * k.cols + col0 : nullptr;
                 Rows R;
-                uint32_t inner_from = 0;                         // MODE 2: the blocks all of whose pieces are stored whole start here ...
-                int32_t row_left_cols = 0;                       // ... and end with the columns that are left of the row
+                bool opens = false;                              // MODE 2: no block of the run has been stored yet
+                int32_t cols_left = 0;                           // and the columns from the block in hand to the row's end
                 if (MODE != 1) {
                     R = rows_of();
-                    if (MODE == 2) out0 = k.out + (R.first + kc * k.chunk_cols + piece_column(0, t, R.off));
-                    inner_from = left_over ? 0u : 1u;
-                    row_left_cols = columns_left(k.cols, kc * k.chunk_cols);
+                    if (MODE == 2) out0 = k.out + (R.first + kc * k.chunk_cols + piece_column(t, R.off));
+                    opens = !left_over;
+                    cols_left = columns_left((uint32_t)k.cols, kc * k.chunk_cols);
                     left_over = true;
                 }
                 // one block, number kb of the chunk and `i` behind where raw_p and xq stand: decode with `cur` while the raw bytes
@@ -554,15 +562,19 @@ __global__ void __launch_bounds__(THREADS, 1) huff_kernel(const __grid_constant_
                         sts_row<0>(row_new + t * 16u, a);
                         sts_row<kRowHalf>(row_new + t * 16u, a + 4);
                         __syncwarp();
-                        const uint4 p0 = shifted_piece<0>(R.from, R.sel), p1 = shifted_piece<kRowHalf>(R.from, R.sel);
-                        if (kb >= inner_from && (int32_t)(kb * 32u + 32u) <= row_left_cols) {
+                        const uint4 p0 = shifted_piece<0>(R.from, R.sel), p1 = shifted_piece<kRowHalf>(R.from + 2 * R.half, R.sel);
+                        uint16_t *const out1 = out0 + 8 * k.cols;
+                        if (!opens && cols_left >= 32) {     // (the usual block: every piece whole)
                             if (R.ok[0]) *(uint4 *)out0 = p0;
-                            if (R.ok[1]) *(uint4 *)(out0 + 8 * k.cols) = p1;
+                            if (R.ok[1]) *(uint4 *)(out1 + R.half) = p1;
                         } else {
-                            const int32_t c = piece_column(kb, t, R.off), run_first = run_start(inner_from == 0u);
-                            if (R.ok[0]) store_piece(out0, p0, c, run_first, row_left_cols);
-                            if (R.ok[1]) store_piece(out0 + 8 * k.cols, p1, c, run_first, row_left_cols);
+                            asm volatile("" : "+r"(rg));     // (row_off again, instead of a register through the loop)
+                            const int32_t c = piece_column(t, row_off()), first = run_start(opens);
+                            if (R.ok[0]) store_piece(out0, p0, c, first, cols_left);
+                            if (R.ok[1]) store_piece(out1 + R.half, p1, c + R.half, first, cols_left);
                         }
+                        opens = false;
+                        cols_left -= 32;
                         out0 += 32;
                         __syncwarp();
                         if (t >= 2) {                        // the row's last sixteen weights, for the next block's first pieces
@@ -603,7 +615,12 @@ __global__ void __launch_bounds__(THREADS, 1) huff_kernel(const __grid_constant_
                 }
 #pragma unroll 1
                 while (left) {
-                    raw_p = left == 1u ? raw_next : raw_p + kRawBlock;
+                    if (MODE == 2) {                              // (worked out from r1 again, instead of two registers through the loop)
+                        asm volatile("" : "+r"(r1));
+                        raw_p = left == 1u ? raw0 + ((uint64_t)r1 << 7) : raw_p + kRawBlock;
+                    } else {
+                        raw_p = left == 1u ? raw_next : raw_p + kRawBlock;
+                    }
                     block(nkb - left, 0, raw_a, raw_b, raw_p, left != 1u || has_next);
                     if (MODE == 1) xq += 32;
                     raw_a = raw_b;

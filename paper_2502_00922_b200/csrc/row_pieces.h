@@ -11,18 +11,19 @@
 
 namespace huffllm {
 
-// Columns are counted from the first column of the chunk in hand, in front of which they are negative: a row has up to 2^31 of
-// them, a chunk at most 1024, and no sum of theirs leaves 32 bits.
+// Columns are counted from the first one of the block in hand (32 columns), those in front of it are negative: a row has up to 2^31
+// columns, and no sum of these leaves 32 bits.
 
 // Columns from `at` to the row's end, or as many as no chunk has.
-HUFFLLM_HD int32_t columns_left(uint64_t cols, uint32_t at) { return (int32_t)(cols - at < (1u << 20) ? cols - at : 1u << 20); }
-// The run's first column: the chunk's own, or, where the row buffers still hold columns of the chunk in front, which has at least a
-// block, one in front of all that is left of it.
-HUFFLLM_HD int32_t run_start(bool left_over) { return left_over ? -32 : 0; }
-// First column of quad lane t's piece of block kb, in a row that starts `off` weights behind a sector's start ...
-HUFFLLM_HD int32_t piece_column(uint32_t kb, uint32_t t, uint32_t off) { return (int32_t)(kb * 32u + t * 8u) - (int32_t)off; }
-// ... and of the piece behind a run that ends in column `end` (lanes with 8 t < off have one).
-HUFFLLM_HD int32_t last_piece_column(int32_t end, uint32_t t, uint32_t off) { return ((end + 31) & ~31) + (int32_t)(t * 8u) - (int32_t)off; }
+HUFFLLM_HD int32_t columns_left(uint32_t cols, uint32_t at) { return (int32_t)(cols - at < (1u << 20) ? cols - at : 1u << 20); }
+// The run's first column: that of its first block, or, behind it, one in front of all that the row buffers hold.
+HUFFLLM_HD int32_t run_start(bool opens) { return opens ? 0 : -32; }
+// First column of quad lane t's piece, in a row that starts `off` weights behind a sector's start.
+HUFFLLM_HD int32_t piece_column(uint32_t t, uint32_t off) { return (int32_t)(t * 8u) - (int32_t)off; }
+
+// A row 8 further down starts 8 * cols weights further on: with an odd column count half a sector off, and its pieces, which are to
+// lie on sectors too, start so many columns further on than those of the row that starts `off` weights behind a sector's start.
+HUFFLLM_HD int32_t row_half(uint32_t off, uint32_t cols) { return cols & 1u ? (off & 8u ? 8 : -8) : 0; }
 
 // The weights lo .. hi - 1 of the piece in column c that lie in columns [first, end); none if lo >= hi.
 struct PieceCut {
