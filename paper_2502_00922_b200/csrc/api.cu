@@ -90,8 +90,8 @@ uint32_t flat_of(const huffllm_desc *d) {
 // ... and of several blobs.
 uint32_t flat_of_both(uint32_t a, uint32_t b) { return a == b ? a : a == kFlatNone || b == kFlatNone ? kFlatNone : kFlatUpper; }
 // Bytes of the FP16 tables (first level): three of 16 KB; the exponent's with a copy per lane and the lower half's with
-// sixteen; the exponent's alone.
-uint32_t fp16_table_bytes(uint32_t flat) { return flat == kFlatBoth ? 32768u : 49152u; }
+// sixteen; the exponent's alone, with sixteen or with one per lane (a launch's choice, see finish_args and tc_choose).
+uint32_t fp16_table_bytes(uint32_t flat) { return flat == kFlatBoth ? 16384u : flat == kFlatBothLanes ? 32768u : 49152u; }
 SmemNeeds smem_needs(const huffllm_desc *desc) {
     SmemNeeds n;
     const bool fmt = desc->dtype == HUFFLLM_FP16;
@@ -122,16 +122,17 @@ SmemNeeds smem_needs(const huffllm_desc *desc) {
 // which the host does not know exactly: the smallest count over every 128-byte start within kStaticSmem + 1 KB is taken.
 uint32_t planned_warps(uint32_t lut_align, uint32_t lut_size, uint64_t pair_bytes, uint32_t dyn_smem, uint32_t part_bytes,
                        uint32_t guard_bytes) {
-    const uint64_t guard_extra = guard_bytes > part_bytes ? guard_bytes - part_bytes : 0;
-    uint64_t least = ~0ull;
-    for (uint64_t base = 0; base <= kStaticSmem + 1024; base += 128) {
-        const uint64_t lut = (base + lut_align - 1) / lut_align * lut_align;
-        const uint64_t slot_a = (base + 255) / 256 * 256, n_a = lut > slot_a ? (lut - slot_a) / pair_bytes : 0;
-        const uint64_t slot_b = lut + lut_size, end = base + dyn_smem - part_bytes;
-        const uint64_t n_b = end > slot_b + guard_extra ? (end - slot_b - guard_extra) / pair_bytes : 0;
+    // (32-bit arithmetic, whose divisions are cheap: a launch asks this a dozen times; check_desc bounds the records)
+    const uint32_t guard_extra = guard_bytes > part_bytes ? guard_bytes - part_bytes : 0, pair = (uint32_t)pair_bytes;
+    uint32_t least = 64;
+    for (uint32_t base = 0; base <= kStaticSmem + 1024; base += 128) {
+        const uint32_t lut = (base + lut_align - 1) / lut_align * lut_align;
+        const uint32_t slot_a = (base + 255) / 256 * 256, n_a = lut > slot_a ? (lut - slot_a) / pair : 0;
+        const uint32_t slot_b = lut + lut_size, end = base + dyn_smem - part_bytes;
+        const uint32_t n_b = end > slot_b + guard_extra ? (end - slot_b - guard_extra) / pair : 0;
         if (n_a + n_b < least) least = n_a + n_b;
     }
-    return (uint32_t)(least > 64 ? 64 : least);
+    return least;
 }
 
 // ---- the tensor-core small-batch path (batch 9..64)
@@ -292,6 +293,34 @@ bool tc_best(const huffllm_desc *const *d, uint32_t n, uint32_t npad, const uint
     }
 }
 
+// The same with the choice of the exponent's table where FP16 mantissa codes are flat: a copy per lane where no accumulator adds up
+// more chunks for the 16 KB (the workspace at hand does not decide).  With fewer tiles a CTA because of it, 12288 x 12288 at 32
+// vectors in chunks of 2048 took 121.5 us and was 4.9e-6 from 64 bits, with sixteen copies 117.8 and 1.7e-6; in chunks of 1024, where
+// all tiles fit either way, 8192 x 8192 at 24 took 56.0 us with a copy per lane and 58.0 with sixteen.
+bool tc_choose(const huffllm_desc *const *d, uint32_t n, uint32_t npad, const uint32_t *cta, uint32_t *flat, uint32_t dyn_smem, size_t max_bytes,
+               TcShape *shape, TcPlan *plans) {
+    // (room for 32 decoders beside the larger table and the most stages that a shape has: every shape fits beside either table, and
+    // so the plans are the same)
+    const uint32_t slices = npad == 64 ? 2 : 4;
+    if (*flat == kFlatBoth && tc_fits(d, n, npad, TcShape{4 / slices, slices, npad == 64 ? 2u : 3u, 32 / slices}, kFlatBothLanes, dyn_smem))
+        *flat = kFlatBothLanes;
+    if (*flat != kFlatBoth) return tc_best(d, n, npad, cta, *flat, dyn_smem, max_bytes, shape, plans);
+    TcShape wide;
+    TcPlan wide_plans[kMaxMats];
+    const bool tight = tc_best(d, n, npad, cta, kFlatBoth, dyn_smem, ~(size_t)0, shape, plans);
+    bool lanes = tc_best(d, n, npad, cta, kFlatBothLanes, dyn_smem, ~(size_t)0, &wide, wide_plans);
+    for (uint32_t i = 0; lanes && tight && i < n; ++i) lanes = wide_plans[i].chunks <= plans[i].chunks;
+    if (!lanes && !tight) return false;
+    if (lanes) {
+        *flat = kFlatBothLanes;
+        *shape = wide;
+        for (uint32_t i = 0; i < n; ++i) plans[i] = wide_plans[i];
+    }
+    for (uint32_t i = 0; i < n; ++i)
+        if (plans[i].bytes > max_bytes) return tc_best(d, n, npad, cta, *flat, dyn_smem, max_bytes, shape, plans);
+    return true;
+}
+
 // Start a launch description.
 void begin_args(KernelArgs *k, uint32_t batch, const DeviceInfo &dev) {
     memset(k, 0, sizeof(*k));
@@ -336,7 +365,9 @@ huffllm_status add_matrix(KernelArgs *k, const huffllm_desc *desc, const void *b
 }
 
 // The tensor-core kernel's part of a launch description.
-void set_tc_shape(KernelArgs *k, uint32_t npad, const TcShape &sh) {
+void set_tc_shape(KernelArgs *k, uint32_t npad, const TcShape &sh, uint32_t flat) {
+    k->fp16_flat = flat;
+    if (k->fmt) k->lut_size = fp16_table_bytes(flat);
     k->part_bytes = sh.part_bytes(npad);
     k->slots = 2;
     k->pair_recip = (uint32_t)(0x100000000ull / (2ull * k->slot_bytes));
@@ -361,7 +392,6 @@ bool rows_through_smem(const MatArgs &m) { return m.cols % 8 && m.cols >= 64 && 
 huffllm_status finish_args(KernelArgs *k, bool product, const DeviceInfo &dev, uint32_t *grid, uint32_t *warps_at_least = nullptr) {
     // (pieces that warps of a CTA exchange: in shared memory up to 8 vectors, in the workspace above)
     if (product) k->part_bytes = k->batch <= kKernelBatch ? 2 * 32 * 16 * k->batch * (uint32_t)sizeof(float) : 0;
-    if (k->fmt && k->lut_bits <= 8) k->lut_size = fp16_table_bytes(k->fp16_flat);
     // Two slots per decoder warp, so that a warp's next record lands while it decodes this one.  Where records are so large
     // that this would leave fewer than 31 warps a slot pair, and single slots serve at least a quarter more warps, every
     // warp gets one slot: more decoders at work outweigh the wait for a copy at every chunk start.
@@ -380,14 +410,19 @@ huffllm_status finish_args(KernelArgs *k, bool product, const DeviceInfo &dev, u
         }
         return best;
     };
-    const uint64_t w2 = warps_with(2ull * k->slot_bytes), w1 = warps_with(k->slot_bytes);
-    const bool single_ok = k->fmt || k->lut_bits == 8;                // (the kernels that exist with single slots)
-    k->slots = single_ok && w2 < max_w && 4 * w1 >= 5 * w2 ? 1u : 2u;
-    if ((k->slots == 2 ? w2 : w1) == 0)
-        return fail(HUFFLLM_ERR_UNSUPPORTED, "chunk records too large for shared memory (slot %u bytes)", k->slot_bytes);
-    if (row_bufs) k->part_bytes = (uint32_t)(k->slots == 1 ? w1 : w2) * 16 * kRowBuf;
-    if (warps_at_least) *warps_at_least = (uint32_t)(k->slots == 1 ? w1 : w2);
-    k->pair_recip = (uint32_t)(0x100000000ull / ((uint64_t)k->slots * k->slot_bytes));
+    // slots and warps with the table(s) that `flat` asks for; false: not even one warp finds its slots
+    uint32_t warps = 0;
+    auto fit = [&](uint32_t flat) -> bool {
+        k->fp16_flat = flat;
+        if (k->fmt && k->lut_bits <= 8) k->lut_size = fp16_table_bytes(flat);
+        const uint64_t w2 = warps_with(2ull * k->slot_bytes), w1 = warps_with(k->slot_bytes);
+        const bool single_ok = k->fmt || k->lut_bits == 8;            // (the kernels that exist with single slots)
+        k->slots = single_ok && w2 < max_w && 4 * w1 >= 5 * w2 ? 1u : 2u;
+        warps = (uint32_t)(k->slots == 1 ? w1 : w2);
+        if (row_bufs) k->part_bytes = warps * 16 * kRowBuf;
+        return warps != 0;
+    };
+    if (!fit(k->fp16_flat)) return fail(HUFFLLM_ERR_UNSUPPORTED, "chunk records too large for shared memory (slot %u bytes)", k->slot_bytes);
     uint64_t g = k->total_chunks < (uint64_t)dev.sms ? k->total_chunks : (uint64_t)dev.sms;
     *grid = (uint32_t)(g < kMaxGrid ? g : kMaxGrid);
     // deal the CTAs out to the matrices: one each, then always to the matrix with the most chunks per CTA, so that
@@ -413,6 +448,26 @@ huffllm_status finish_args(KernelArgs *k, bool product, const DeviceInfo &dev, u
         first += cnt[i];
     }
     *grid = first;
+    // Flat FP16 mantissa codes: the exponent's table with a copy per lane has no bank conflicts, but takes 16 KB that decoder warps
+    // want for their slots.  It is taken where no warp's accumulators add up more chunks for it, nor, in chunks so long that warps
+    // have single slots, any warp is lost (decode adds up nothing).  FP16 11008 x 4096, sixteen copies / one per lane, us and the
+    // relative error against 64 bits: one vector, chunks of 4096 (26 / 24 warps) 29.2, 2.30e-7 / 31.4, 2.39e-7, chunks of 2048 (27 /
+    // 25, six chunks a warp either way) 27.0, 2.31e-7 / 29.5, 2.11e-7; 8 vectors, chunks of 1024 (31 / 31) 36.6 / 35.8 and no
+    // difference, of 4096 (24 / 22) 35.6, 9.5e-7 / 32.0, 10.3e-7, of 8192 (12 / 10) 42.7, 1.76e-6 / 41.0, 2.05e-6.
+    if (k->fp16_flat == kFlatBoth) {
+        auto longest_sum = [&](const MatArgs &m) -> uint32_t {
+            const uint32_t chunks = (m.cta_chunks + (m.cta_extra ? 1u : 0u) + warps - 1) / warps;
+            return chunks < m.col_chunks ? chunks : m.col_chunks;
+        };
+        uint32_t most[kMaxMats];
+        for (uint32_t i = 0; i < k->n_mats; ++i) most[i] = longest_sum(k->m[i]);
+        const uint32_t needed = k->slots == 1 ? warps : 1;
+        bool lanes = fit(kFlatBothLanes) && (!product || warps >= needed);
+        for (uint32_t i = 0; lanes && product && i < k->n_mats; ++i) lanes = longest_sum(k->m[i]) <= most[i];
+        if (!lanes) fit(kFlatBoth);
+    }
+    if (warps_at_least) *warps_at_least = warps;
+    k->pair_recip = (uint32_t)(0x100000000ull / ((uint64_t)k->slots * k->slot_bytes));
     return HUFFLLM_OK;
 }
 
@@ -437,8 +492,9 @@ huffllm_status huffllm_workspace_bytes(const huffllm_desc *desc, uint32_t batch,
         // The plan that will run for this and for every smaller batch, and the shape-0 plan, which a launch over several matrices
         // may fall back on; with all three FP16 tables, and with those that flat codes leave.
         for (uint32_t npad = 16; npad <= tc_npad_of(batch); npad *= 2)
-            for (uint32_t flat : {kFlatNone, kFlatBoth, kFlatUpper}) {
-                if (flat != kFlatNone && flat_of_both(flat, flat_of(desc)) != flat) continue;
+            for (uint32_t flat : {kFlatNone, kFlatUpper, kFlatBoth, kFlatBothLanes}) {
+                const uint32_t have_flat = flat == kFlatBothLanes ? kFlatBoth : flat;
+                if (flat != kFlatNone && flat_of_both(have_flat, flat_of(desc)) != have_flat) continue;
                 TcShape sh;
                 TcPlan p;
                 if (!tc_best(&desc, 1, npad, &cta, flat, dyn, ~(size_t)0, &sh, &p)) continue;
@@ -513,11 +569,12 @@ huffllm_status huffllm_gemm_launch_plan(uint32_t n, const huffllm_desc *const *d
         if ((st = add_matrix(&k, descs[i], (const void *)256)) != HUFFLLM_OK) return st;     // (the pointer is only checked for alignment)
         if (!tc_blob(descs[i])) return fail(HUFFLLM_ERR_UNSUPPORTED, "the tensor-core path takes tables of up to 9 bits (FP16: 8)");
     }
+    uint32_t flat = k.fp16_flat;
     if (n > 1 && (st = finish_args(&k, true, dev, &grid)) != HUFFLLM_OK) return st;
     for (uint32_t i = 0; i < n; ++i) cta[i] = n > 1 ? k.m[i].cta_count : (uint32_t)dev.sms;
     TcShape sh;
     TcPlan plans[kMaxMats];
-    if (!tc_best(descs, n, tc_npad_of(batch), cta, k.fp16_flat, k.dyn_smem_bytes, workspace_bytes_each ? workspace_bytes_each : ~(size_t)0, &sh, plans))
+    if (!tc_choose(descs, n, tc_npad_of(batch), cta, &flat, k.dyn_smem_bytes, workspace_bytes_each ? workspace_bytes_each : ~(size_t)0, &sh, plans))
         return fail(HUFFLLM_ERR_UNSUPPORTED, "chunk records too large for the tensor-core kernel's slots");
     if (column_slices) *column_slices = sh.slices;
     if (row_groups) *row_groups = sh.row_groups;
@@ -587,15 +644,16 @@ huffllm_status huffllm_decode_gemm_multi(uint32_t n, const huffllm_desc *const *
             k.m[i].x = xs[i];
             k.m[i].y = ys[i];
         }
+        uint32_t flat = k.fp16_flat;
         if ((st = finish_args(&k, true, dev, &grid)) != HUFFLLM_OK) return st;      // (deals the CTAs to the matrices by their chunks)
         const uint32_t npad = tc_npad_of(batch);
         uint32_t cta[kMaxMats];
         for (uint32_t i = 0; i < n; ++i) cta[i] = k.m[i].cta_count;
         TcShape sh;
         TcPlan plans[kMaxMats];
-        if (!tc_best(descs, n, npad, cta, k.fp16_flat, k.dyn_smem_bytes, workspace_bytes_each, &sh, plans))
+        if (!tc_choose(descs, n, npad, cta, &flat, k.dyn_smem_bytes, workspace_bytes_each, &sh, plans))
             return fail(HUFFLLM_ERR_UNSUPPORTED, "chunk records too large for the tensor-core kernel's slots");
-        set_tc_shape(&k, npad, sh);
+        set_tc_shape(&k, npad, sh, flat);
         uint32_t first = 0;
         for (uint32_t i = 0; i < n; ++i) {
             const TcPlan &tp = plans[i];
@@ -679,7 +737,8 @@ huffllm_status huffllm_decode_gemm(const huffllm_desc *desc, const void *blob, c
         const uint32_t npad = tc_npad_of(batch), cta = (uint32_t)dev.sms;
         TcShape sh;
         TcPlan tp;
-        if (!tc_best(&desc, 1, npad, &cta, flat_of(desc), (uint32_t)dev.smem_optin - kStaticSmem, workspace_bytes, &sh, &tp))
+        uint32_t flat = flat_of(desc);
+        if (!tc_choose(&desc, 1, npad, &cta, &flat, (uint32_t)dev.smem_optin - kStaticSmem, workspace_bytes, &sh, &tp))
             return HUFFLLM_OK;      // records too large for this kernel's slots
         TcArgs t;
         memset(&t, 0, sizeof(t));
@@ -687,7 +746,7 @@ huffllm_status huffllm_decode_gemm(const huffllm_desc *desc, const void *blob, c
         begin_args(&k, batch, dev);
         huffllm_status s2 = add_matrix(&k, desc, blob);
         if (s2 != HUFFLLM_OK) return s2;
-        set_tc_shape(&k, npad, sh);
+        set_tc_shape(&k, npad, sh, flat);
         if (workspace_bytes < tp.bytes) {
             if (other_path_left) return HUFFLLM_OK;     // (the register path needs less)
             return fail(HUFFLLM_ERR_BUFFER_TOO_SMALL, "workspace too small for batch %u", batch);

@@ -184,11 +184,12 @@ enum Decoder {
     kHalf,     // FP16, three tables of 8 bits, sixteen copies each
     kHalf7,    // FP16, three tables of 7 bits, once per lane
     kHalf12,   // FP16, up to 12 bits per field: two levels
-    kFlat,     // FP16, both mantissa halves carry the flat code (codewords of at most 8 bits)
+    kFlat,     // FP16, both mantissa halves carry the flat code (codewords of at most 8 bits): sixteen copies
+    kFlatLanes, // the same, table once per lane
     kUpper,    // FP16, the upper mantissa half carries the flat code (codewords of at most 8 bits)
 };
 __host__ __device__ constexpr Decoder decoder_of(int lb, int fmt) {
-    return fmt == 0 ? (lb == 8 ? kBf8 : lb == 9 ? kBf9 : kBf12) : fmt == 1 ? (lb == 8 ? kHalf : lb == 7 ? kHalf7 : kHalf12) : fmt == 2 ? kFlat : kUpper;
+    return fmt == 0 ? (lb == 8 ? kBf8 : lb == 9 ? kBf9 : kBf12) : fmt == 1 ? (lb == 8 ? kHalf : lb == 7 ? kHalf7 : kHalf12) : fmt == 2 ? kFlat : fmt == 4 ? kFlatLanes : kUpper;
 }
 // Where a sequence's pointer starts: on its first codeword, behind the leading zero bits (7, FP16: 6); kBf9 stays 7 bits
 // behind, so that the index stands where the address wants it.
@@ -196,6 +197,8 @@ __host__ __device__ constexpr uint32_t lag_of(Decoder d) { return d <= kBf12 ? 7
 __host__ __device__ constexpr uint32_t start_of(Decoder d) { return d == kBf9 ? 0u : lag_of(d); }
 // Longest codeword (per field).
 __host__ __device__ constexpr uint32_t longest_of(Decoder d) { return d == kBf9 ? 9u : d == kHalf7 ? 7u : d == kBf12 || d == kHalf12 ? 12u : 8u; }
+// FP16 with both mantissa halves flat.
+__host__ __device__ constexpr bool both_flat(Decoder d) { return d == kFlat || d == kFlatLanes; }
 constexpr uint32_t kLongMark = 0x80000000u;
 
 // Shared-memory form of a blob's table entry (length << 16 | symbol bits): the length in the low bits, the symbol above.
@@ -206,7 +209,7 @@ template <Decoder D>
 __device__ __forceinline__ uint32_t lut_entry(uint32_t e, uint32_t field, bool first_level = true) {
     const uint32_t len = e >> 16;
     if ((D == kBf12 || D == kHalf12) && first_level && len > 8u) return kLongMark;
-    const uint32_t flat_bits = D == kFlat ? 10u : D == kUpper && field == 0 ? 5u : 0u;
+    const uint32_t flat_bits = both_flat(D) ? 10u : D == kUpper && field == 0 ? 5u : 0u;
     return ((D <= kBf12 ? e & 0x7F80u : e & 0x7FFFu) << 16) | (min(len, longest_of(D)) + flat_bits);
 }
 
@@ -311,7 +314,7 @@ __device__ __forceinline__ void step4(uint32_t &pa, uint32_t &pb, uint32_t col, 
 // exponent's codeword in reverse order.  The exponent's entry has them in its length, and the window is ROTATED by that
 // length instead of shifted: what comes next (the second weight, or the lower half's codeword) stands at bit 0, and the flat
 // bits at the top, in the order in which a bit reversal of both weights' halves at once puts them where they belong.
-// The tables that are left have a copy per lane (kUpper's lower half: sixteen).
+// The tables that are left have a copy per lane (kUpper's lower half and kFlat's one: sixteen).
 template <Decoder D>
 __device__ __forceinline__ uint32_t lookup_field(uint32_t t, int field, uint32_t lut_lane, uint32_t full_base, uint32_t full_mask) {
     if (D == kHalf7) {
@@ -326,10 +329,10 @@ __device__ __forceinline__ uint32_t lookup_field(uint32_t t, int field, uint32_t
 template <Decoder D>
 __device__ __forceinline__ uint32_t weight_sum(const Window &w, uint32_t lut_lane, uint32_t lut_low, uint32_t full_base, uint32_t full_mask, uint32_t &rot) {
     uint32_t t = D == kHalf7 ? w.lo << 7 : w.lo;
-    if (D == kFlat || D == kUpper) {
-        const uint32_t e0 = lookup_byte0(t, 128u, lut_lane);
+    if (both_flat(D) || D == kUpper) {
+        const uint32_t e0 = lookup_byte0(t, D == kFlat ? 64u : 128u, lut_lane);
         rot = funnel(t, t, e0);
-        if (D == kFlat) return e0;
+        if (both_flat(D)) return e0;
         return e0 + lookup_byte0(rot, 64u, lut_low);
     }
     const uint32_t e0 = lookup_field<D>(t, 0, lut_lane, full_base, full_mask);
@@ -366,11 +369,11 @@ __device__ __forceinline__ void step2_fp16(uint32_t &pa, uint32_t &pb, uint32_t 
         pb += eb[0] + eb[1];
     }
     auto pair = [&](const uint32_t *e, const uint32_t *r) -> uint32_t {
-        const uint32_t coded = D == kFlat ? merge_exponents(e[0], e[1]) : prmt(e[0], e[1], 0x7632u);
-        if (D != kFlat && D != kUpper) return coded;
+        const uint32_t coded = both_flat(D) ? merge_exponents(e[0], e[1]) : prmt(e[0], e[1], 0x7632u);
+        if (!both_flat(D) && D != kUpper) return coded;
         const uint32_t flat = __brev(prmt(r[0], r[1], 0x3276u));      // bits 0..9 / 16..25 (kUpper: 0..4 / 16..20): mantissa bits
         uint32_t x;
-        if (D == kFlat) asm("lop3.b32 %0, %1, %2, 0x03FF03FF, 0xE4;" : "=r"(x) : "r"(flat), "r"(coded));
+        if (both_flat(D)) asm("lop3.b32 %0, %1, %2, 0x03FF03FF, 0xE4;" : "=r"(x) : "r"(flat), "r"(coded));
         else asm("lop3.b32 %0, %1, %2, 0x03E003E0, 0xE4;" : "=r"(x) : "r"(flat * 32u), "r"(coded));
         return x;
     };
@@ -406,21 +409,21 @@ __device__ __forceinline__ void decode_block(uint32_t &pa, uint32_t &pb, uint32_
 template <Decoder D>
 struct LutPlan {
     // 16-byte pieces of the first level
-    static constexpr uint32_t kVecs = D == kBf9 ? 4096u : D <= kBf12 || D == kFlat ? 2048u : 3072u;
+    static constexpr uint32_t kVecs = D == kBf9 ? 4096u : D <= kBf12 || D == kFlatLanes ? 2048u : D == kFlat ? 1024u : 3072u;
     // entry index in the blob's tables (of 1 << lut_bits entries each) and field of piece v
     static __device__ __forceinline__ uint32_t source(uint32_t v, uint32_t lut_bits) {
         if (D <= kBf12) return v >> 3;
         if (D == kHalf7) return (field(v) << lut_bits) + ((v >> 3) & 127u);
         if (D == kHalf || D == kHalf12) return (field(v) << lut_bits) + ((v >> 2) & 255u);
         // (tables of 7 bits serve as tables of 8 whose upper half repeats the lower one)
-        const uint32_t in = field(v) ? (v >> 2) & 255u : v >> 3;
+        const uint32_t in = D == kFlat ? v >> 2 : field(v) ? (v >> 2) & 255u : v >> 3;
         return (field(v) << lut_bits) + (in & ((1u << lut_bits) - 1u));
     }
-    static __device__ __forceinline__ uint32_t field(uint32_t v) { return D <= kBf12 || D == kFlat ? 0u : D == kUpper ? (v >> 11) * 2u : v >> 10; }
+    static __device__ __forceinline__ uint32_t field(uint32_t v) { return D <= kBf12 || both_flat(D) ? 0u : D == kUpper ? (v >> 11) * 2u : v >> 10; }
 };
 // A lane's column of the table(s), and of kUpper's second one.
 template <Decoder D>
-__device__ __forceinline__ uint32_t lut_column(uint32_t lut, uint32_t lane) { return lut | (D == kHalf || D == kHalf12 ? lane & 15u : lane) << 2; }
+__device__ __forceinline__ uint32_t lut_column(uint32_t lut, uint32_t lane) { return lut | (D == kHalf || D == kHalf12 || D == kFlat ? lane & 15u : lane) << 2; }
 template <Decoder D>
 __device__ __forceinline__ uint32_t lut_low_column(uint32_t lut, uint32_t lane) { return D == kUpper ? lut + 32768u + ((lane & 15u) << 2) : 0u; }
 // Bytes of the first level, behind which the whole tables of the two-level decoders lie.

@@ -96,8 +96,8 @@ __device__ __forceinline__ void store_piece(uint16_t *dst, const uint4 &p, int32
 // LB = table index bits (the blobs' lut_bits): 8 or 9; LB = 12 stands for every longer limit up to 12 (BF16: 10..12,
 // FP16: 9..12): two-level lookup, the number of bits is A.lut_bits.
 // FMT = 0: BF16 blobs; FMT = 1: FP16 {1,5,5,5} blobs (three lookups per weight, sign bits as the raw part); FMT = 2: the same
-// where both mantissa halves carry the flat 5-bit code (codes of up to 8 bits: one lookup per weight and a bit reversal per two);
-// FMT = 3: where the upper half does (two lookups).
+// where both mantissa halves carry the flat 5-bit code (codes of up to 8 bits: one lookup per weight and a bit reversal per two),
+// FMT = 4: with the table once per lane; FMT = 3: where the upper half does (two lookups).
 //
 // One launch works through a LIST of matrices (A.n_mats, usually the matrices of one decoder layer that
 // may run together).  The CTAs are dealt out to the matrices in proportion to their chunks, so every CTA
@@ -757,6 +757,7 @@ static cudaError_t launch_format(const KernelArgs &k, uint32_t grid, cudaStream_
     if (k.fmt) {
         if (k.lut_bits > 8) return launch_slots<MODE, 12, 1, NT>(k, grid, stream);
         if (k.fp16_flat == kFlatBoth) return launch_slots<MODE, 8, 2, NT>(k, grid, stream);
+        if (k.fp16_flat == kFlatBothLanes) return launch_slots<MODE, 8, 4, NT>(k, grid, stream);
         if (k.fp16_flat == kFlatUpper) return launch_slots<MODE, 8, 3, NT>(k, grid, stream);
         return k.lut_bits == 7 ? launch_slots<MODE, 7, 1, NT>(k, grid, stream) : launch_slots<MODE, 8, 1, NT>(k, grid, stream);
     }

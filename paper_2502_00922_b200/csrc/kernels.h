@@ -55,7 +55,8 @@ struct KernelArgs {
                                // Kernels with single slots exist for FP16 blobs and for BF16 blobs with 8-bit tables.
     uint32_t fp16_flat;        // FP16 blobs: which mantissa halves of every matrix of the launch carry the flat 5-bit code
 };
-constexpr uint32_t kFlatNone = 0, kFlatBoth = 1, kFlatUpper = 2;    // (the lower half alone is not made use of)
+// (kFlatBoth: the exponent's table with sixteen copies of an entry, kFlatBothLanes: with one per lane; the lower half alone is not made use of)
+constexpr uint32_t kFlatNone = 0, kFlatBoth = 1, kFlatUpper = 2, kFlatBothLanes = 3;
 
 // Arguments of the tensor-core kernel: the launch description plus, per matrix, its work items and where their pieces meet.
 // (The CTAs of a launch are dealt to the matrices as in the other kernels: m[i].cta_first / cta_count.)

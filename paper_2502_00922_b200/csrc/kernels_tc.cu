@@ -129,7 +129,7 @@ __device__ __forceinline__ bool elect_one() {
     return p != 0;
 }
 
-// LB = table index bits; NPAD = batch rounded up to 16, 32 or 64 (the MMA's N); FMT = 0: BF16 blobs, 1: FP16 {1,5,5,5} blobs, 2 / 3: those with flat mantissa codes, see huff_kernel
+// LB = table index bits; NPAD = batch rounded up to 16, 32 or 64 (the MMA's N); FMT = 0: BF16 blobs, 1: FP16 {1,5,5,5} blobs, 2 to 4: those with flat mantissa codes, see huff_kernel
 // (three tables, sign words as the raw part, f16 operands).
 // MULTI: the launch works through several matrices (a launch over one matrix reads its arguments without an index).
 template <int LB, int NPAD, int FMT, bool MULTI>
@@ -714,6 +714,11 @@ cudaError_t launch_gemm_tc(const TcArgs &t, uint32_t grid, cudaStream_t stream) 
         if (k.tc_npad == 16) return launch_tc_one<8, 16, 2>(t, grid, stream);
         if (k.tc_npad == 32) return launch_tc_one<8, 32, 2>(t, grid, stream);
         return launch_tc_one<8, 64, 2>(t, grid, stream);
+    }
+    if (k.fmt && k.fp16_flat == kFlatBothLanes) {
+        if (k.tc_npad == 16) return launch_tc_one<8, 16, 4>(t, grid, stream);
+        if (k.tc_npad == 32) return launch_tc_one<8, 32, 4>(t, grid, stream);
+        return launch_tc_one<8, 64, 4>(t, grid, stream);
     }
     if (k.fmt) {
         if (k.tc_npad == 16) return launch_tc_one<8, 16, 1>(t, grid, stream);
