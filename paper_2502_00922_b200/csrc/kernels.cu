@@ -514,15 +514,20 @@ __global__ void __launch_bounds__(THREADS, 1) huff_kernel(const __grid_constant_
                 auto block = [&](uint32_t kb, int i, const uint4 &cur, uint4 &nxt, const uint8_t *from, bool fetch) {
                     if (fetch) nxt = load_raw(from);
                     const uint16_t *const xi = xq + 32 * i;
-                    uint4 xv;
-                    if (MODE == 1 && NT <= 1) xv = __ldg((const uint4 *)xi);   // (two tiles: both are fetched behind the decoder, registers are short)
+                    // Activations are on their way while the block is decoded.  Two tiles with two slots a warp: both are fetched behind
+                    // the decoder, registers are short (11008 x 4096 at 16 vectors 31.4 us, ahead of it 32.5).  With single slots fewer
+                    // registers are taken, and a wait in a block holds the slot's next copy up as well (ahead / behind: 28672 x 8192 in
+                    // chunks of 8192 at 9 vectors 105.3 / 123.5 us, at 16 118.1 / 129.8, in chunks of 16384 132 / 175).
+                    constexpr bool kAhead = NT <= 1 || SLOTS == 1;
+                    uint4 xv, xw;
+                    if (MODE == 1 && kAhead) xv = __ldg((const uint4 *)xi);
+                    if (MODE == 1 && kAhead && NT == 2) xw = __ldg((const uint4 *)(xi + x_tile2));
 
                     uint32_t a[8];
                     decode_block<D>(pa, pb, col, lut_lane, lut_low, cur, a, full_base, full_mask);
 
                     if (MODE == 1) {
-                        uint4 xw;
-                        if (NT == 2) {
+                        if (!kAhead) {
                             xv = __ldg((const uint4 *)xi);
                             xw = __ldg((const uint4 *)(xi + x_tile2));
                         }

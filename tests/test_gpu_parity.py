@@ -811,3 +811,17 @@ def test_fewer_tiles_than_four(hl, torch, rows, cols, ce, dtype, batch):
     y = gpu_gemm(hl, torch, ups[0], xs[0])
     check_product(y, ups[0].w, xs[0], dtype)
     assert np.array_equal(y, gpu_gemm(hl, torch, ups[0], xs[0])), "results must be bitwise reproducible"
+
+
+@pytest.mark.parametrize("ce", [8192, 16384])
+@pytest.mark.parametrize("batch", [9, 16])
+def test_two_tiles_of_activations_with_single_slots(hl, torch, ce, batch):
+    """9 and 16 vectors on records so large that warps have single slots, some of which are used more than once; ragged last chunks."""
+    rows, cols = 16393, 2592
+    w = wl.gaussian_weights(rows, cols, 0.02, ce)
+    up = Uploaded(hl, torch, w, ce, batch=batch)
+    assert hl.decode_launch_plan(up.desc, 8)["slots_per_warp"] == 1
+    x = wl.activations(batch, cols, 60 + batch)
+    y = gpu_gemm(hl, torch, up, x)
+    pick = np.unique(np.r_[np.arange(0, rows, 97), np.arange(rows - 20, rows)])
+    check_product(np.ascontiguousarray(y[:, pick]), w[pick], x)
