@@ -12,6 +12,7 @@
 #include <cuda_runtime.h>
 
 #include <algorithm>
+#include <atomic>
 #include <cstring>
 #include <vector>
 
@@ -604,6 +605,19 @@ __global__ void __launch_bounds__(32 * kSumWarps, kSumCtas) encode_checksum_kern
     finish_checksum(A, term);
 }
 
+// The device's SMs, whose number the checksum's CTAs go by, and the kernel's shared memory allowed, once per device.
+static cudaError_t prepare_checksum(int *sms) {
+    static std::atomic<int> known[64];               // set twice by racing threads at worst: to the same value
+    int dev = 0;
+    cudaError_t e = cudaGetDevice(&dev);
+    if (e != cudaSuccess) return e;
+    if (dev >= 0 && dev < 64 && (*sms = known[dev].load(std::memory_order_acquire)) != 0) return cudaSuccess;
+    if ((e = cudaDeviceGetAttribute(sms, cudaDevAttrMultiProcessorCount, dev)) != cudaSuccess) return e;
+    if ((e = cudaFuncSetAttribute(encode_checksum_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kSumSmem)) != cudaSuccess) return e;
+    if (dev >= 0 && dev < 64) known[dev].store(*sms, std::memory_order_release);
+    return cudaSuccess;
+}
+
 // The same with a thread per record, as the hash is written.  A record takes a thread some 30 ns per byte (one load in flight),
 // but a GPU full of threads takes less than half of what the warps above need per byte, who pay for whole steps of 1.5 KB whatever
 // the record's size: with enough records this is faster, the sooner the shorter they are.  (Warps / threads: 88064 records of 512
@@ -705,12 +719,16 @@ extern "C" huffllm_status huffllm_encode_device(const huffllm_codebook *cb, cons
     const auto size_kernel = A.fp16 ? encode_size_kernel<true> : encode_size_kernel<false>;
     const uint32_t chunks = write_chunks(A), smem = write_staged(A) ? chunks * A.most_words * 256 : 0;
     const auto write_kernel = longest <= 8 ? write_kernel_of<true>(A.fp16 != 0, chunks, smem != 0) : write_kernel_of<false>(A.fp16 != 0, chunks, smem != 0);
+    int sms = 0;
+    if ((e = prepare_checksum(&sms)) != cudaSuccess) return cuda_fail("device attributes");
+    std::vector<uint8_t> fixed;
+    fixed.reserve((size_t)d.off_index);                          // (what can fail without a launch does so before the first one)
     if ((e = cudaMemsetAsync(scr, 0, cleared, s)) != cudaSuccess) return cuda_fail("cudaMemsetAsync");
     A.size_groups = size_groups(A);
     const uint64_t per_cta = (uint64_t)kSizeChunks * A.size_groups;
     size_kernel<<<(uint32_t)((d.n_chunks + per_cta - 1) / per_cta), kSizeThreads, 0, s>>>(A);
     // code lengths and table, assembled on the host while pass 1 runs; the header's bytes stay zero until the last kernel writes them
-    std::vector<uint8_t> fixed((size_t)d.off_index, 0);
+    fixed.assign((size_t)d.off_index, 0);
     write_fixed_sections(cb, d, fixed.data());
     memset(fixed.data(), 0, sizeof(d));
     if ((e = cudaMemcpyAsync(blob, fixed.data(), fixed.size(), cudaMemcpyHostToDevice, s)) != cudaSuccess) return cuda_fail("copy of the fixed sections");
@@ -718,10 +736,8 @@ extern "C" huffllm_status huffllm_encode_device(const huffllm_codebook *cb, cons
     write_kernel<<<(uint32_t)((d.n_chunks + chunks - 1) / chunks), 64 * chunks, smem, s>>>(A);
     if (checksum_each(d.n_chunks, chunk_elems))
         encode_checksum_each_kernel<<<(uint32_t)((d.n_chunks + kEachThreads - 1) / kEachThreads), kEachThreads, 0, s>>>(A);
-    else {
-        if ((e = cudaFuncSetAttribute(encode_checksum_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kSumSmem)) != cudaSuccess) return cuda_fail("cudaFuncSetAttribute");
-        encode_checksum_kernel<<<(uint32_t)std::min<uint64_t>(kSumCtas * 148, (d.n_chunks + kSumWarps - 1) / kSumWarps), 32 * kSumWarps, kSumSmem, s>>>(A);
-    }
+    else
+        encode_checksum_kernel<<<(uint32_t)std::min<uint64_t>((uint64_t)kSumCtas * sms, (d.n_chunks + kSumWarps - 1) / kSumWarps), 32 * kSumWarps, kSumSmem, s>>>(A);
     if ((e = cudaGetLastError()) != cudaSuccess) return cuda_fail("encoder launches");
     EncTotals tot;
     if ((e = cudaMemcpyAsync(&tot, scr, sizeof(tot), cudaMemcpyDeviceToHost, s)) != cudaSuccess || (e = cudaStreamSynchronize(s)) != cudaSuccess)

@@ -27,7 +27,6 @@
 #include <cuda_runtime.h>
 #include <atomic>
 #include <cstdint>
-#include <type_traits>
 
 #include "decode_common.cuh"
 #include "row_pieces.h"
