@@ -3,11 +3,7 @@
 #pragma once
 #include <cstdint>
 
-#ifdef __CUDACC__
-#define HUFFLLM_HD __host__ __device__ __forceinline__
-#else
-#define HUFFLLM_HD inline
-#endif
+#include "host_device.h"
 
 namespace huffllm {
 
