@@ -209,7 +209,8 @@ def workspace_control_bytes(desc: Desc) -> int:
 
 
 def decode_smem_plan(desc: Desc) -> dict:
-    """huffllm_decode_smem_plan: table bytes, slot bytes, refill checks per block and guard bytes of a decoder CTA."""
+    """huffllm_decode_smem_plan: table bytes, slot bytes, rows budgeted per bit sequence and block (under the name of the
+    refill checks that former decoders made), and guard bytes of a decoder CTA."""
     t, sl, ch, g = C.c_uint32(), C.c_uint32(), C.c_uint32(), C.c_uint32()
     _check(lib().huffllm_decode_smem_plan(C.byref(desc), C.byref(t), C.byref(sl), C.byref(ch), C.byref(g)))
     return {"table_bytes": t.value, "slot_bytes": sl.value, "refill_checks_per_block": ch.value, "guard_bytes": g.value}

@@ -230,7 +230,8 @@ def test_fp16_long_field_codes_decode_and_product(hl, torch, rows, cols, ce, bud
     (128, 1024, 1024, "fp16", 16),                # batch above 8: passes of 8 vectors
 ])
 def test_fp16_seven_bit_field_codes(hl, torch, rows, cols, ce, gen, batch):
-    """FP16 {1,5,5,5} blobs whose field codes are limited to 7 bits: 128-entry tables that the device keeps once per lane."""
+    """FP16 {1,5,5,5} blobs whose field codes are limited to 7 bits: 128-entry tables that the device keeps once per lane, or,
+    where mantissa halves are flat, doubled for the decoders that read those without a table."""
     w = FP16_GENS[gen](rows, cols, 1500 + rows)
     up = Uploaded(hl, torch, w, ce, 7, max(batch, 1), dtype=hl.FP16)
     assert (up.desc.dtype, up.desc.lut_bits) == (hl.FP16, 7)
@@ -456,7 +457,7 @@ def test_bad_record_offsets_are_reported_not_followed(hl, torch):
 def test_damaged_coded_part_is_reported_and_contained(hl, torch):
     """The coded rows of one chunk are overwritten (on the host) with the longest codeword over and over, so that the
     chunk's sequences run far past their record.  The kernels must say so in the error flag, stay inside their shared
-    memory (the read pointer moves one row per refill check at most, and room for that is kept), and decode every
+    memory (a sequence moves on by at most its tables' longest codewords, and room for that is kept), and decode every
     other chunk as before."""
     rows, cols = 64, 2048
     w = wl.gaussian_weights(rows, cols, 0.02, 21)
@@ -825,3 +826,31 @@ def test_two_tiles_of_activations_with_single_slots(hl, torch, ce, batch):
     y = gpu_gemm(hl, torch, up, x)
     pick = np.unique(np.r_[np.arange(0, rows, 97), np.arange(rows - 20, rows)])
     check_product(np.ascontiguousarray(y[:, pick]), w[pick], x)
+
+
+@pytest.mark.parametrize("cols,ce,budget,dtype", [(1027, 512, 0, 0), (1030, 512, 9, 0), (1027, 1024, 0, 0), (1029, 1024, 0, 1), (2051, 8192, 0, 0)])
+def test_bad_record_offsets_between_runs_of_chunks(hl, torch, cols, ce, budget, dtype):
+    """Rows that go through shared memory, warps with several chunks: records in the middle of a run, at its ends and at the ends
+    of a row lie outside the payload (an index made on the host).  Their columns stay as they were, everything else is decoded."""
+    rows = 9003
+    w = wl.gaussian_weights(rows, cols, 0.02, cols + ce, "fp16") if dtype else make("gauss", rows, cols, cols + ce)
+    up = Uploaded(hl, torch, w, ce, budget, dtype=dtype)
+    d = up.desc
+    blob = up.blob.copy()
+    idx = blob[d.off_index:d.off_index + 4 * (d.n_chunks + 1)].view(np.uint32)
+    KC, n = d.col_chunks, d.n_chunks
+    victims = {0, KC // 2, 2 * KC - 1, 3 * KC, 5 * KC + 1, n // 2, n // 2 + 2, n - 1}
+    for c in victims:
+        idx[c] = 0x7FFFFFF0                        # chunks c - 1 and c are unusable
+    dev = torch.from_numpy(blob).cuda()
+    out = torch.full((rows * cols + 64,), 0x5A5A, dtype=torch.int16, device="cuda")
+    hl.decode(d, dev, out, up.err)
+    torch.cuda.synchronize()
+    assert int(up.err.item()) != 0
+    got = out.cpu().numpy().view(np.uint16)
+    assert np.all(got[rows * cols:] == 0x5A5A)
+    want = w.copy()
+    for c in victims | {c - 1 for c in victims if c}:
+        rg, kc = divmod(c, KC)
+        want[rg * 16:rg * 16 + 16, kc * d.chunk_cols:(kc + 1) * d.chunk_cols] = 0x5A5A
+    assert np.array_equal(got[:rows * cols].reshape(rows, cols), want)

@@ -53,8 +53,8 @@ def test_fp16_decoders_by_their_flat_codes(hl, kind, flat, limit, rows, cols, ch
     cb = hl.build_codebook(w, hl.FP16, limit)
     blob, desc = hl.encode(cb, w, chunk)
     cb.free()
-    if flat is not None and rows * cols > 100000:
-        assert desc.flat_fields & 6 == flat
+    if rows * cols > 100000:
+        assert desc.flat_fields & 6 == flat if flat is not None else desc.flat_fields & 2 == 0
     dev, err = torch.from_numpy(blob).cuda(), torch.zeros(1, dtype=torch.int32, device="cuda")
     out = torch.zeros(rows * cols, dtype=torch.int16, device="cuda")
     hl.decode(desc, dev, out, err)
@@ -62,6 +62,29 @@ def test_fp16_decoders_by_their_flat_codes(hl, kind, flat, limit, rows, cols, ch
     if kind == "no field flat":                                       # (infinities and NaN among them)
         return
     for batch in (1, 3, 24):
+        x = wl.activations(batch, cols, 7, "fp16")
+        xd, y = torch.from_numpy(x.view(np.int16)).cuda(), torch.zeros((batch, rows), dtype=torch.float32, device="cuda")
+        n = hl.workspace_bytes(desc, batch)
+        ws = torch.zeros(n, dtype=torch.uint8, device="cuda")
+        hl.decode_gemm(desc, dev, xd, batch, y, ws, n, err) if batch > 1 else hl.decode_gemv(desc, dev, xd, y, ws, n, err)
+        want, size = orc.matmul(w, x, orc.FP16)
+        assert np.all(np.abs(y.cpu().numpy().astype(np.float64) - want) <= cols * 2.0**-23 * size)
+    assert int(err.item()) == 0
+
+
+@pytest.mark.gpu
+@pytest.mark.parametrize("limit", [7, 8, 12])
+@pytest.mark.parametrize("rows,cols,chunk", [(250, 1024, 512), (129, 2080, 1024), (37, 4128, 2048)])
+def test_fp16_products_through_three_tables(hl, limit, rows, cols, chunk):
+    """Fields none of which is flat: every product goes through the tables of all three, on the register path and the tensor cores."""
+    import torch
+    w = wl.skewed_exponent_weights(rows, cols, rows + limit, dtype="fp16")
+    cb = hl.build_codebook(w, hl.FP16, limit)
+    blob, desc = hl.encode(cb, w, chunk)
+    cb.free()
+    assert desc.flat_fields & 6 == 0 and desc.lut_bits == limit
+    dev, err = torch.from_numpy(blob).cuda(), torch.zeros(1, dtype=torch.int32, device="cuda")
+    for batch in (1, 3, 8, 12, 24, 40):
         x = wl.activations(batch, cols, 7, "fp16")
         xd, y = torch.from_numpy(x.view(np.int16)).cuda(), torch.zeros((batch, rows), dtype=torch.float32, device="cuda")
         n = hl.workspace_bytes(desc, batch)
