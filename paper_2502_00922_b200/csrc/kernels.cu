@@ -92,7 +92,7 @@ __device__ __forceinline__ void store_piece(uint16_t *dst, const uint4 &p, int32
 // MODE 0: write the decoded weights, every lane its eight: one aligned store where rows have a multiple of 8 columns, one by one
 // otherwise (small matrices).  MODE 2: write the decoded weights of a matrix whose rows start anywhere (see store_piece).
 // MODE 1: y = W x for up to 8 activation vectors.
-// LB = table index bits (the blobs' lut_bits): 8 or 9; LB = 12 stands for every longer limit up to 12 (BF16: 10..12,
+// LB = table index bits (the blobs' lut_bits): BF16 8 or 9, FP16 7 or 8; LB = 12 stands for every longer limit up to 12 (BF16: 10..12,
 // FP16: 9..12): two-level lookup, the number of bits is A.lut_bits.
 // FMT = 0: BF16 blobs; FMT = 1: FP16 {1,5,5,5} blobs (three lookups per weight, sign bits as the raw part); FMT = 2: the same
 // where both mantissa halves carry the flat 5-bit code (codes of up to 8 bits: one lookup per weight and a bit reversal per two),

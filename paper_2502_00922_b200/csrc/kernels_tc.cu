@@ -607,8 +607,10 @@ __global__ void __launch_bounds__(1024, 1) huff_gemm_tc_kernel(const __grid_cons
                         // lie in the coded part or behind the record, up to 1 KB behind the payload: the blob has 4 KB there.)
                         // Not at the widest padding, whose blocks take longer, nor for FP16, whose raw part is a sixteenth.
                         // (us, without / with it / two blocks further on: 4096 x 14336 at 16 vectors 35.1 / 34.2 / 35.1, 7B-shaped
-                        // layer at 32 135.5 / 133.1 / 135.1, 11008 x 4096 at 48 34.7 / 35.9 / 36.0, 8192 x 28672 at 64 124.5 / 125.9 /
-                        // 129.2.  The record's whole raw part at once, with its copy: 36.8 and 139.6 for the first two.)
+                        // layer at 32 135.5 / 133.1 / 135.1; padding 64: 11008 x 4096 at 48 34.7 / 35.9 / 36.0, 8192 x 28672 at 64
+                        // 124.5 / 125.9 / 129.2.  Without / with it: 4096 x 14336 at 32 38.3 / 37.3, 28672 x 8192 at 24 116.2 / 113.9, at 32
+                        // 117.7 / 117.9, in chunks of 8192 160.5 / 148.6, 8192 x 28672 at 32 116.0 / 115.3, 16384 x 4096 at 20 in chunks of
+                        // 1024 45.6 / 46.0.  The record's whole raw part at once, with its copy: 36.8 and 139.6 for the first two.)
                         if (NPAD < 64 && FMT == 0) asm volatile("prefetch.global.L2 [%0];" ::"l"(raw_p + kRawBlock));
                         uint32_t a[8];
                         decode_block<D>(pa, pb, lane << 2, lut_lane, lut_low, raw_c, a, 0u, 0u);
