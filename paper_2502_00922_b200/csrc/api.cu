@@ -126,7 +126,7 @@ uint32_t planned_warps(uint32_t lut_align, uint32_t lut_size, uint64_t pair_byte
     const uint32_t guard_extra = guard_bytes > part_bytes ? guard_bytes - part_bytes : 0, pair = (uint32_t)pair_bytes;
     uint32_t least = 64;
     for (uint32_t base = 0; base <= kStaticSmem + 1024; base += 128) {
-        const uint32_t lut = (base + lut_align - 1) / lut_align * lut_align;
+        const uint32_t lut = (base + lut_align - 1) & ~(lut_align - 1);      // (a power of two)
         const uint32_t slot_a = (base + 255) / 256 * 256, n_a = lut > slot_a ? (lut - slot_a) / pair : 0;
         const uint32_t slot_b = lut + lut_size, end = base + dyn_smem - part_bytes;
         const uint32_t n_b = end > slot_b + guard_extra ? (end - slot_b - guard_extra) / pair : 0;
@@ -415,14 +415,19 @@ huffllm_status finish_args(KernelArgs *k, bool product, const DeviceInfo &dev, u
     auto fit = [&](uint32_t flat) -> bool {
         k->fp16_flat = flat;
         if (k->fmt && k->lut_bits <= 8) k->lut_size = fp16_table_bytes(flat);
-        const uint64_t w2 = warps_with(2ull * k->slot_bytes), w1 = warps_with(k->slot_bytes);
         const bool single_ok = k->fmt || k->lut_bits == 8;            // (the kernels that exist with single slots)
-        k->slots = single_ok && w2 < max_w && 4 * w1 >= 5 * w2 ? 1u : 2u;
+        const uint64_t w2 = warps_with(2ull * k->slot_bytes), w1 = single_ok && w2 < max_w ? warps_with(k->slot_bytes) : 0;
+        k->slots = w1 && 4 * w1 >= 5 * w2 ? 1u : 2u;
         warps = (uint32_t)(k->slots == 1 ? w1 : w2);
         if (row_bufs) k->part_bytes = warps * 16 * kRowBuf;
         return warps != 0;
     };
-    if (!fit(k->fp16_flat)) return fail(HUFFLLM_ERR_UNSUPPORTED, "chunk records too large for shared memory (slot %u bytes)", k->slot_bytes);
+    // (flat FP16 mantissa codes, see below: a table per lane that leaves decode a warp, or a product all of them, needs no comparison)
+    const uint32_t flat = k->fp16_flat;
+    bool lanes = flat == kFlatBoth && fit(kFlatBothLanes);
+    const uint32_t lanes_warps = lanes ? warps : 0, lanes_slots = k->slots;
+    lanes = lanes && (!product || warps == max_w);
+    if (!lanes && !fit(flat)) return fail(HUFFLLM_ERR_UNSUPPORTED, "chunk records too large for shared memory (slot %u bytes)", k->slot_bytes);
     uint64_t g = k->total_chunks < (uint64_t)dev.sms ? k->total_chunks : (uint64_t)dev.sms;
     *grid = (uint32_t)(g < kMaxGrid ? g : kMaxGrid);
     // deal the CTAs out to the matrices: one each, then always to the matrix with the most chunks per CTA, so that
@@ -454,17 +459,19 @@ huffllm_status finish_args(KernelArgs *k, bool product, const DeviceInfo &dev, u
     // relative error against 64 bits: one vector, chunks of 4096 (26 / 24 warps) 29.2, 2.30e-7 / 31.4, 2.39e-7, chunks of 2048 (27 /
     // 25, six chunks a warp either way) 27.0, 2.31e-7 / 29.5, 2.11e-7; 8 vectors, chunks of 1024 (31 / 31) 36.6 / 35.8 and no
     // difference, of 4096 (24 / 22) 35.6, 9.5e-7 / 32.0, 10.3e-7, of 8192 (12 / 10) 42.7, 1.76e-6 / 41.0, 2.05e-6.
-    if (k->fp16_flat == kFlatBoth) {
-        auto longest_sum = [&](const MatArgs &m) -> uint32_t {
-            const uint32_t chunks = (m.cta_chunks + (m.cta_extra ? 1u : 0u) + warps - 1) / warps;
+    if (flat == kFlatBoth && !lanes && lanes_warps) {
+        auto longest_sum = [&](const MatArgs &m, uint32_t with) -> uint32_t {
+            const uint32_t chunks = (m.cta_chunks + (m.cta_extra ? 1u : 0u) + with - 1) / with;
             return chunks < m.col_chunks ? chunks : m.col_chunks;
         };
-        uint32_t most[kMaxMats];
-        for (uint32_t i = 0; i < k->n_mats; ++i) most[i] = longest_sum(k->m[i]);
-        const uint32_t needed = k->slots == 1 ? warps : 1;
-        bool lanes = fit(kFlatBothLanes) && (!product || warps >= needed);
-        for (uint32_t i = 0; lanes && product && i < k->n_mats; ++i) lanes = longest_sum(k->m[i]) <= most[i];
-        if (!lanes) fit(kFlatBoth);
+        lanes = k->slots == 2 || lanes_warps >= warps;
+        for (uint32_t i = 0; lanes && i < k->n_mats; ++i) lanes = longest_sum(k->m[i], lanes_warps) <= longest_sum(k->m[i], warps);
+        if (lanes) {
+            k->fp16_flat = kFlatBothLanes;
+            k->lut_size = fp16_table_bytes(kFlatBothLanes);
+            k->slots = lanes_slots;
+            warps = lanes_warps;
+        }
     }
     if (warps_at_least) *warps_at_least = warps;
     k->pair_recip = (uint32_t)(0x100000000ull / ((uint64_t)k->slots * k->slot_bytes));
