@@ -2,8 +2,8 @@
 // device memory.  Compression is an offline, one-time step (Section 3.1); on the host it takes seconds per decoder
 // layer, here it is three short passes over the tensor, so a model can be compressed while it is being loaded.
 //
-// One thread per bit sequence (64 per chunk), as in the format: thread q of a chunk owns lane q / 2 and row half q % 2,
-// so neighbouring threads write neighbouring raw bytes and the two halves of a lane sit in one warp.
+// A warp takes a chunk, its lanes the format's lanes: two bit sequences each (rows g and g + 8), one after the other in the loops
+// below, so that a lane has two chains under way and what a chunk costs besides its weights is paid once per 128 of a lane's.
 //   pass 1  code lengths only -> words per sequence of every chunk; words and coded bits of every 1024 chunks
 //   scan    record offsets (the index section), payload size, largest record
 //   pass 2  raw part and coded part of every record (nothing if the scan found the tensor or the buffer unfit)
@@ -14,6 +14,7 @@
 #include <algorithm>
 #include <atomic>
 #include <cstring>
+#include <type_traits>
 #include <vector>
 
 #include "internal.h"
@@ -29,20 +30,21 @@ struct EncTotals {
 static_assert(sizeof(EncTotals) <= 64, "the sums of pass 1 follow in the scratch");
 
 constexpr uint32_t kScanThreads = 1024;      // chunks of a scan CTA
-constexpr uint32_t kNoCode = 1u << 20;       // length of a symbol without codeword: makes any sum it is part of stand out
+constexpr uint32_t kWriteWarps = 4;          // of a CTA of pass 2
+__host__ __device__ constexpr uint32_t write_ctas(bool vec) { return vec ? 6 : 5; }     // of an SM (80 and 96 registers)
+constexpr uint32_t kNoCode = 1u << 14;       // length of a symbol without codeword: no sum of a sequence's codewords reaches it (768 of 12 bits)
 
 struct EncArgs {
     const uint16_t *w;
     uint64_t rows, cols, n_chunks;
     uint32_t Kc, KC, fp16, lag_bits, pad, vec_ok;
-    uint32_t size_groups;        // groups of kSizeChunks chunks that a CTA of pass 1 takes, one after the other
-    uint32_t most_words;         // rows of the largest record this code can give a full chunk
+    uint32_t stage_rows;         // rows of a record that a warp of pass 2 has room for in shared memory
     uint64_t max_units;          // what the blob has room for
     unsigned long long *groups;  // per kScanThreads chunks: their words | their coded bits << 32
     uint32_t *words, *index;
     uint8_t *blob, *payload;
     EncTotals *totals;
-    uint32_t code[256];          // stream bits of a symbol's codeword | its length << 16
+    uint32_t code[256];          // a symbol's codeword, first bit in bit 31 | its length (FP16: three fields of 32 symbols)
     huffllm_desc desc;           // the header, but for what the totals say
 };
 
@@ -73,25 +75,33 @@ __device__ __forceinline__ uint32_t enc_raw_bytes(const EncArgs &A, uint32_t nkb
     return A.fp16 ? (nkb * 64u + 127u) & ~127u : nkb * 512u;
 }
 
-// A thread's weights: eight in every block of 32 columns, from `p` on, `left` columns (at most) before the row ends.
-struct EncRow {
-    const uint16_t *p;
-    int32_t left;               // 0 for rows outside the tensor
+// A lane of the warp that takes chunk c: its weights are, in every block of 32 columns, eight in row g and eight in row g + 8.
+struct EncLane {
+    uint32_t nkb, whole;        // blocks of the chunk; those that lie inside the tensor, with the 16-byte pieces around their rows' ends
+    const uint16_t *row[2];     // the weights in the first block
+    int32_t left[2];            // columns (at most) before the row ends, 0 for rows outside the tensor
+    uint32_t off;               // bytes from a 16-byte boundary to the weights, in both rows
 };
-// The eight weights of block kb as four words, pad words outside the tensor.  Rows that do not start on 16-byte boundaries
-// are read in words; where those straddle the weights, the first and the last weight are read alone: nothing outside the
-// eight is touched (the word's other half may lie in front of the tensor or behind it).
-__device__ __forceinline__ uint4 enc_load8(const EncArgs &A, const EncRow &R, uint32_t kb) {
-    const uint16_t *p = R.p + kb * 32u;
-    const int32_t left = R.left - (int32_t)(kb * 32u);
-    if (left >= 8) {
-        if (A.vec_ok) return __ldg((const uint4 *)p);
-        const bool odd = ((uintptr_t)p & 2u) != 0;
-        const uint32_t *q = (const uint32_t *)(p + (odd ? 1 : 0)), sel = odd ? 0x5432u : 0x7654u;
-        const uint32_t u0 = __ldg(q), u1 = __ldg(q + 1), u2 = __ldg(q + 2);
-        const uint32_t first = odd ? __ldg(p) : 0u, u3 = odd ? __ldg(p + 7) : __ldg(q + 3);
-        return make_uint4(__byte_perm(first, u0, odd ? 0x5410u : 0x7654u), __byte_perm(u0, u1, sel), __byte_perm(u1, u2, sel), __byte_perm(u2, u3, sel));
-    }
+__device__ __forceinline__ EncLane enc_lane(const EncArgs &A, uint32_t c, uint32_t lane) {           // (fewer than 2^31 chunks)
+    EncLane L;
+    const uint32_t rg = c / A.KC, kc = c - rg * A.KC;
+    const uint64_t r = (uint64_t)rg * 16 + (lane >> 2), first = (uint64_t)kc * A.Kc, col0 = first + (lane & 3) * 8;
+    const uint32_t cols = (uint32_t)min(A.cols - first, (uint64_t)A.Kc);
+    L.nkb = (cols + 31) / 32;
+    L.whole = (uint64_t)rg * 16 + 16 <= A.rows ? cols / 32 : 0u;
+    // (nothing outside the tensor is read: off 16-byte boundaries the pieces of its first row begin in front of it, and those of its last
+    // row may reach up to eight weights behind the chunk)
+    if (!A.vec_ok && (c == 0 || ((uint64_t)rg * 16 + 16 >= A.rows && first + cols + 8 > A.cols))) L.whole = 0;
+    L.row[0] = A.w + r * A.cols + col0;
+    L.row[1] = L.row[0] + 8 * A.cols;
+    const int32_t left = (int32_t)cols - (int32_t)(lane & 3) * 8;
+    L.left[0] = r < A.rows ? left : 0;
+    L.left[1] = r + 8 < A.rows ? left : 0;
+    L.off = (uint32_t)(uintptr_t)L.row[0] & 15u;
+    return L;
+}
+// A block's eight weights of one row as four words, weight by weight, pad words outside the tensor.
+__device__ __forceinline__ uint4 enc_edge(const EncArgs &A, const uint16_t *p, int32_t left) {
     uint32_t x[4];
 #pragma unroll
     for (int i = 0; i < 4; ++i) {
@@ -100,99 +110,124 @@ __device__ __forceinline__ uint4 enc_load8(const EncArgs &A, const EncRow &R, ui
     }
     return make_uint4(x[0], x[1], x[2], x[3]);
 }
-
-struct EncThread {
-    uint32_t sub, q, lane, half, seq;
-    uint64_t c;
-    uint32_t nkb;
-    EncRow row;
-    bool active;
-};
-// 64 threads for each of the CHUNKS chunks of a group
-template <uint32_t CHUNKS>
-__device__ __forceinline__ EncThread enc_thread(const EncArgs &A, uint32_t group) {
-    EncThread T;
-    T.sub = threadIdx.x >> 6;
-    T.q = threadIdx.x & 63;
-    T.lane = T.q >> 1;
-    T.half = T.q & 1;
-    T.seq = T.lane + 32 * T.half;
-    T.c = (uint64_t)group * CHUNKS + T.sub;
-    T.active = T.c < A.n_chunks;
-    const uint64_t cc = T.active ? T.c : 0;
-    const uint32_t rg = (uint32_t)cc / A.KC, kc = (uint32_t)cc - rg * A.KC;       // (fewer than 2^31 chunks)
-    T.nkb = enc_blocks_of(A, kc);
-    const uint64_t r = (uint64_t)rg * 16 + (T.lane >> 2) + 8 * T.half, col0 = (uint64_t)kc * A.Kc + (T.lane & 3) * 8;
-    T.row.p = A.w + r * A.cols + col0;
-    T.row.left = r < A.rows && col0 < A.cols ? (int32_t)min(A.cols - col0, (uint64_t)A.Kc) : 0;
-    return T;
+// The 16 bytes that start `off` bytes (an even number) into two neighbouring pieces.
+__device__ __forceinline__ uint4 enc_shifted(const uint4 &p, const uint4 &n, uint32_t off) {
+    const bool two = off & 8u, one = off & 4u;
+    const uint32_t sel = (off & 2u) ? 0x5432u : 0x3210u;
+    const uint32_t a0 = two ? p.z : p.x, a1 = two ? p.w : p.y, a2 = two ? n.x : p.z, a3 = two ? n.y : p.w, a4 = two ? n.z : n.x, a5 = two ? n.w : n.y;
+    const uint32_t b0 = one ? a1 : a0, b1 = one ? a2 : a1, b2 = one ? a3 : a2, b3 = one ? a4 : a3, b4 = one ? a5 : a4;
+    return make_uint4(__byte_perm(b0, b1, sel), __byte_perm(b1, b2, sel), __byte_perm(b2, b3, sel), __byte_perm(b3, b4, sel));
 }
-
-// Pass 1.  Bound by the read of the tensor: four blocks' loads are in flight per thread (one at a time took 30 us on an
-// 11008 x 4096 tensor), and a weight costs a shift, a mask, a table read and an addition.
-constexpr uint32_t kSizeThreads = 256, kSizeChunks = kSizeThreads / 64;
-template <bool FP16>
-__global__ void __launch_bounds__(kSizeThreads) encode_size_kernel(const __grid_constant__ EncArgs A) {
-    __shared__ uint32_t s_max[kSizeChunks], s_sum[kSizeChunks], s_len[256];
-    s_len[threadIdx.x] = A.code[threadIdx.x] >> 16 ? A.code[threadIdx.x] >> 16 : kNoCode;
+// f(weights in row g, weights in row g + 8) for every block of the chunk in turn, the loads of the next AHEAD blocks under way.  VEC: rows
+// start on 16-byte boundaries; otherwise a row's weights are cut out of two pieces.
+template <bool VEC, int AHEAD, typename F>
+__device__ __forceinline__ void enc_blocks(const EncArgs &A, const EncLane &L, F &&f) {
+    const uint4 *pa = (const uint4 *)((const char *)L.row[0] - (VEC ? 0u : L.off)), *pb = (const uint4 *)((const char *)L.row[1] - (VEC ? 0u : L.off));
+    uint4 a[AHEAD], b[AHEAD], a1[AHEAD], b1[AHEAD];
+    auto load = [&](int i) {
+        a[i] = __ldg(pa + 4 * i);
+        b[i] = __ldg(pb + 4 * i);
+        if (!VEC) {
+            a1[i] = __ldg(pa + 4 * i + 1);
+            b1[i] = __ldg(pb + 4 * i + 1);
+        }
+    };
+#pragma unroll
+    for (int i = 0; i < AHEAD; ++i)
+        if ((uint32_t)i < L.whole) load(i);
+    uint32_t left = L.whole;
 #pragma unroll 1
-    for (uint32_t it = 0; it < A.size_groups; ++it) {
-        const uint32_t group = blockIdx.x * A.size_groups + it;
-        if (threadIdx.x < kSizeChunks) s_max[threadIdx.x] = s_sum[threadIdx.x] = 0;
-        __syncthreads();
-        const EncThread T = enc_thread<kSizeChunks>(A, group);
-        if (T.active) {
-            uint32_t bits = 0;
-            const char *len = (const char *)s_len;
-            auto at = [&](uint32_t byte_off) -> uint32_t { return *(const uint32_t *)(len + byte_off); };
-            auto add = [&](const uint4 &v) {
-                const uint32_t x[4] = {v.x, v.y, v.z, v.w};
+    while (left) {
+        pa += 4 * AHEAD;
+        pb += 4 * AHEAD;
 #pragma unroll
-                for (int i = 0; i < 4; ++i) {
-                    if (FP16) {
-                        bits += at((x[i] >> 8) & 0x7Cu) + at(128u + ((x[i] >> 3) & 0x7Cu)) + at(256u + ((x[i] << 2) & 0x7Cu));
-                        bits += at((x[i] >> 24) & 0x7Cu) + at(128u + ((x[i] >> 19) & 0x7Cu)) + at(256u + ((x[i] >> 14) & 0x7Cu));
-                    } else {
-                        bits += at((x[i] >> 5) & 0x3FCu) + at((x[i] >> 21) & 0x3FCu);
-                    }
-                }
-            };
-            uint32_t kb = 0;
-            for (; kb + 4 <= T.nkb; kb += 4) {
-                uint4 v[4];
-#pragma unroll
-                for (int i = 0; i < 4; ++i) v[i] = enc_load8(A, T.row, kb + i);
-#pragma unroll
-                for (int i = 0; i < 4; ++i) add(v[i]);
+        for (int i = 0; i < AHEAD; ++i) {
+            if (VEC) {
+                f(a[i], b[i]);
+                if (left > AHEAD) load(i);
+            } else {
+                const uint4 va = enc_shifted(a[i], a1[i], L.off), vb = enc_shifted(b[i], b1[i], L.off);
+                if (left > AHEAD) load(i);
+                f(va, vb);
             }
-            for (; kb < T.nkb; ++kb) add(enc_load8(A, T.row, kb));
-            if (bits >= kNoCode) {
-                atomicOr(&A.totals->bad, 1u);
-                bits = 0;
-            }
-            atomicMax(&s_max[T.sub], bits + A.lag_bits);
-            atomicAdd(&s_sum[T.sub], bits);
+            if (--left == 0) break;
         }
-        __syncthreads();
-        if (threadIdx.x >= 32) continue;
-        const uint64_t c = (uint64_t)group * kSizeChunks + threadIdx.x;
-        unsigned long long sum = 0;                        // (1024 chunks: fewer than 2^19 words and 2^30 bits)
-        if (threadIdx.x < kSizeChunks && c < A.n_chunks) {
-            const uint32_t W = max(1u, (s_max[threadIdx.x] + 31) / 32);
-            A.words[c] = W;
-            sum = (unsigned long long)s_sum[threadIdx.x] << 32 | W;
-        }
-#pragma unroll
-        for (uint32_t o = kSizeChunks / 2; o; o >>= 1) sum += __shfl_xor_sync(0xFFFFFFFFu, sum, o);
-        if (threadIdx.x == 0 && sum) atomicAdd(A.groups + c / kScanThreads, sum);
     }
+#pragma unroll 1
+    for (uint32_t kb = L.whole; kb < L.nkb; ++kb)
+        f(enc_edge(A, L.row[0] + kb * 32u, L.left[0] - (int32_t)(kb * 32u)), enc_edge(A, L.row[1] + kb * 32u, L.left[1] - (int32_t)(kb * 32u)));
 }
+__device__ __forceinline__ uint32_t lds32(uint32_t addr) {
+    uint32_t v;
+    asm("ld.shared.u32 %0, [%1];" : "=r"(v) : "r"(addr));
+    return v;
+}
+__device__ __forceinline__ uint32_t lds16(uint32_t addr) {
+    uint16_t v;
+    asm("ld.shared.u16 %0, [%1];" : "=h"(v) : "r"(addr));
+    return v;
+}
+// FP16: the exponent and the upper mantissa half of a weight, its bits 5 .. 14, are looked up together: a table of 1024 entries in front of
+// the lower half's 32.
+constexpr uint32_t kPairEntries = 1024;
 
-// A group's threads have a block or two each where chunks are short, less than the table costs their CTA: eight blocks per thread
-// are worth going on for, as long as the GPU stays full.  (Chunks of 512: 11008 x 4096 88 -> 82 us, 65536 x 8192 1070 -> 847.)
-inline uint32_t size_groups(const EncArgs &A) {
-    const uint64_t full = A.n_chunks / (kSizeChunks * 8 * 148), want = 8 / (A.Kc / kBlockCols);
-    return (uint32_t)std::max<uint64_t>(1, std::min<uint64_t>(full, want));
+// Pass 1.  Bound by the read of the tensor (BF16) and by the lookups, whose addresses are byte or halfword dot products of the weights
+// as they are, so that a BF16 weight costs 5.5 instructions (8.7 with a shift and a mask per weight, 64 threads a chunk and the
+// table read anew for every few of them).  FP16 lengths are 16 bits wide: half as many words for the lanes to meet in.
+// Four blocks' loads are in flight (two: 18.7 us instead of 17.3).  Rows off 16-byte boundaries are cut out of two 16-byte loads.
+// (11008 x 4096, in a whole call, before / now, us: BF16 23.6 / 17.3, 11007 x 4099 in chunks of 2048 42.9 / 27, FP16 41.6 / 29.0, chunks
+// of 512 79 / 50.)
+constexpr uint32_t kSizeWarps = 8;           // of a CTA of pass 1
+__host__ __device__ constexpr uint32_t size_ctas(bool vec) { return vec ? 3 : 4; }      // of an SM (80 and 64 registers)
+template <bool FP16, bool VEC>
+__global__ void __launch_bounds__(32 * kSizeWarps, size_ctas(VEC)) encode_size_kernel(const __grid_constant__ EncArgs A) {
+    __shared__ __align__(4) typename std::conditional<FP16, uint16_t, uint32_t>::type s_len[FP16 ? kPairEntries + 32 : 256];
+    const uint32_t lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    auto length = [&](uint32_t i) -> uint32_t { return A.code[i] ? A.code[i] & 31u : kNoCode; };
+    if (FP16) {
+        const uint32_t upper = length(32 + lane);
+        for (uint32_t e = warp; e < 32; e += kSizeWarps) s_len[32 * e + lane] = min(length(e) + upper, kNoCode);
+        if (warp == 0) s_len[kPairEntries + lane] = length(64 + lane);
+    } else {
+        s_len[threadIdx.x] = length(threadIdx.x);
+    }
+    __syncthreads();
+    const uint32_t table = (uint32_t)__cvta_generic_to_shared(s_len), low = table + 2 * kPairEntries;
+    auto bits_of = [&](const uint4 &v) -> uint32_t {
+        const uint32_t x[4] = {v.x, v.y, v.z, v.w};
+        uint32_t bits = 0;
+#pragma unroll
+        for (int i = 0; i < 4; ++i) {
+            if (FP16) {
+                const uint32_t u = x[i] >> 5 & 0x03FF03FFu, l = x[i] & 0x001F001Fu;
+                bits += lds16(__dp2a_lo(u, 0x0002u, table)) + lds16(__dp2a_lo(u, 0x0200u, table));
+                bits += lds16(__dp2a_lo(l, 0x0002u, low)) + lds16(__dp2a_lo(l, 0x0200u, low));
+            } else {
+                const uint32_t y = x[i] * 2u;                                // exponents in bytes 1 and 3
+                bits += lds32(__dp4a(y, 0x00000400u, table)) + lds32(__dp4a(y, 0x04000000u, table));
+            }
+        }
+        return bits;
+    };
+#pragma unroll 1
+    for (uint32_t c = blockIdx.x * kSizeWarps + warp; c < A.n_chunks; c += gridDim.x * kSizeWarps) {
+        const EncLane L = enc_lane(A, c, lane);
+        uint32_t ba = 0, bb = 0;
+        enc_blocks<VEC, VEC ? 4 : 1>(A, L, [&](const uint4 &va, const uint4 &vb) {
+            ba += bits_of(va);
+            bb += bits_of(vb);
+        });
+        if (ba >= kNoCode || bb >= kNoCode) {
+            atomicOr(&A.totals->bad, 1u);
+            ba = bb = 0;
+        }
+        const uint32_t most = __reduce_max_sync(0xFFFFFFFFu, max(ba, bb) + A.lag_bits), sum = __reduce_add_sync(0xFFFFFFFFu, ba + bb);
+        if (lane == 0) {
+            const uint32_t W = max(1u, (most + 31) / 32);
+            A.words[c] = W;
+            atomicAdd(A.groups + c / kScanThreads, (unsigned long long)sum << 32 | W);   // (1024 chunks: fewer than 2^19 words and 2^30 bits)
+        }
+    }
 }
 
 // Record offsets: an exclusive prefix sum of the record sizes (in 128-byte units).  A CTA takes 1024 chunks and sums what pass 1
@@ -240,121 +275,178 @@ __global__ void __launch_bounds__(kScanThreads) encode_scan_kernel(const __grid_
     }
 }
 
-// Pass 2.  64 threads take a chunk and collect the coded part in shared memory (STAGED), row by row as the record has it: stored
-// straight from the threads, whose streams run apart, the words go to L2 one by one as partial sectors.  Short chunks share a
-// CTA of four, whose table and set-up they share too; above 512 columns, where shared memory leaves an SM few warps, straight
-// stores are the better choice.  (11008 x 4096: chunks of 512 / 1024 one to a CTA 185 / 97 us, four 90 / 56; FP16 16384 under codes of
-// up to 12 bits staged 157, straight 98.  Whole calls on 28672 x 8192, staged / straight: 2048 574 / 594, 4096 558 / 572, 16384 551 /
-// 526, FP16 995 / 831; at 8192 542 / 526 there, but 158 / 165 on 11008 x 4096.)
-template <bool FP16, uint32_t CHUNKS, bool STAGED, bool SHORT>
-__global__ void __launch_bounds__(64 * CHUNKS) encode_write_kernel(const __grid_constant__ EncArgs A) {
+__device__ __forceinline__ uint32_t shl_pair(uint32_t hi, uint32_t lo, uint32_t n) {       // upper word of (hi:lo) << n % 32
+    uint32_t d;
+    asm("shf.l.wrap.b32 %0, %1, %2, %3;" : "=r"(d) : "r"(lo), "r"(hi), "r"(n));
+    return d;
+}
+__device__ __forceinline__ uint32_t shr_pair(uint32_t hi, uint32_t lo, uint32_t n) {       // lower word of (hi:lo) >> n % 32
+    uint32_t d;
+    asm("shf.r.wrap.b32 %0, %1, %2, %3;" : "=r"(d) : "r"(lo), "r"(hi), "r"(n));
+    return d;
+}
+// A sequence being written: its last 64 bits, the newest in bit 0, how many there are so far (bits 0 .. 5 are looked at), and where its
+// next word goes, 256 bytes behind the one before: in shared memory (STAGED, the word's first bit on top) or in the record.
+template <bool STAGED>
+struct EncSequence {
+    uint32_t hi, lo, n;
+    typename std::conditional<STAGED, uint32_t, uint64_t>::type out;
+    __device__ __forceinline__ void push(uint32_t e) {                 // the codeword of a table entry
+        hi = shl_pair(hi, lo, e);
+        lo = shl_pair(lo, e, e);
+    }
+    __device__ __forceinline__ void advance(uint32_t by) {             // up to 32 bits were pushed: if that made a word full, out with it
+        const uint32_t was = n;
+        n += by;
+        const uint32_t word = shr_pair(hi, lo, n);
+        if constexpr (STAGED)
+            asm volatile("{\n\t.reg .pred p, q;\n\t.reg .b32 t;\n\tsetp.ne.u32 q, 0, 0;\n\tlop3.or.b32 t|p, %1, %2, 32, 0x28, q;\n\t"
+                         "@p st.shared.u32 [%0], %3;\n\t@p add.u32 %0, %0, 256;\n\t}" : "+r"(out) : "r"(was), "r"(n), "r"(word) : "memory");
+        else
+            asm volatile("{\n\t.reg .pred p, q;\n\t.reg .b32 t;\n\tsetp.ne.u32 q, 0, 0;\n\tlop3.or.b32 t|p, %1, %2, 32, 0x28, q;\n\t"
+                         "@p st.global.u32 [%0], %3;\n\t@p add.u64 %0, %0, 256;\n\t}" : "+l"(out) : "r"(was), "r"(n), "r"(__brev(word)) : "memory");
+    }
+    __device__ __forceinline__ void put(uint32_t word) {
+        if constexpr (STAGED) asm volatile("st.shared.u32 [%0], %1;" ::"r"(out), "r"(word) : "memory");
+        else asm volatile("st.global.u32 [%0], %1;" ::"l"(out), "r"(__brev(word)) : "memory");
+        out += 256;
+    }
+    template <typename P>
+    __device__ __forceinline__ void finish(P end) {                    // what is left of the last word, and zeros up to the record's end
+        if (n & 31u) put(shr_pair(lo, 0u, n));
+        while (out < end) put(0u);
+    }
+    template <bool SHORT>
+    __device__ __forceinline__ void append_bf16(const uint4 &v, uint32_t table) {
+        const uint32_t x[4] = {v.x, v.y, v.z, v.w};
+#pragma unroll
+        for (int i = 0; i < 4; i += 2) {
+            const uint32_t y0 = x[i] * 2u, y1 = x[i + 1] * 2u;                            // exponents in bytes 1 and 3
+            const uint32_t e0 = lds32(__dp4a(y0, 0x00000400u, table)), e1 = lds32(__dp4a(y0, 0x04000000u, table));
+            const uint32_t e2 = lds32(__dp4a(y1, 0x00000400u, table)), e3 = lds32(__dp4a(y1, 0x04000000u, table));
+            push(e0);
+            push(e1);
+            if (!SHORT) advance(e0 + e1);
+            push(e2);
+            push(e3);
+            advance(SHORT ? e0 + e1 + e2 + e3 : e2 + e3);
+        }
+    }
+    template <bool SHORT>
+    __device__ __forceinline__ void append_fp16(const uint4 &v, uint32_t table) {
+        const uint32_t x[4] = {v.x, v.y, v.z, v.w}, low = table + 4 * kPairEntries;
+#pragma unroll
+        for (int i = 0; i < 4; ++i) {
+            const uint32_t u = x[i] >> 5 & 0x03FF03FFu, l = x[i] & 0x001F001Fu;
+            const uint32_t e0 = lds32(__dp2a_lo(u, 0x0004u, table)), e1 = lds32(__dp2a_lo(l, 0x0004u, low));
+            const uint32_t e2 = lds32(__dp2a_lo(u, 0x0400u, table)), e3 = lds32(__dp2a_lo(l, 0x0400u, low));
+            push(e0);
+            if (!SHORT) advance(e0);
+            push(e1);
+            advance(SHORT ? e0 + e1 : e1);
+            push(e2);
+            if (!SHORT) advance(e2);
+            push(e3);
+            advance(SHORT ? e2 + e3 : e3);
+        }
+    }
+};
+
+// Pass 2.  The coded part is collected in shared memory, row by row as the record has it: stored straight from the lanes, whose sequences
+// run apart, the words go to L2 one by one as partial sectors.  Only records of more rows than a warp has room for (stage_rows, 32 or what
+// the code can reach: chunks of 4096 stay below it, 12.7 bits a weight among FP16-trained ones included) are.
+// An entry has its codeword on top and its length in the low bits, which is where a funnel shift wants both: two of them move the last
+// 64 bits on by a codeword.  Whether a word is full shows in bit 5 of the count; four codewords of up to 8 bits (two of up to 12, an FP16
+// weight) are pushed between two such looks.  The words' bits are turned around on their way from shared memory to the record.
+// BF16 moves 161 MB in 29.2 us, 0.84 of a copy's rate; FP16 is bound by instruction issue (24 per weight).
+// (11008 x 4096, in a whole call, codewords shifted and or-ed into a word / this, us: BF16 42.0 / 29.2, codes of 12 bits 44 / 30.3, 11007 x 4099
+// 52 / 37, FP16 in chunks of 2048 83.9 / 52.9, chunks of 512 91 / 57; 28672 x 8192 188 / 141.  Two warps a chunk that meet at a barrier 42.9; stores
+// through generic addresses, which one loop could share with the straight ones, 31.8 and 61.6 (FP16).)
+template <bool FP16, bool SHORT, bool VEC>
+__global__ void __launch_bounds__(32 * kWriteWarps, write_ctas(VEC)) encode_write_kernel(const __grid_constant__ EncArgs A) {
     extern __shared__ __align__(16) uint32_t s_coded[];
-    __shared__ uint32_t s_code[256];
-#pragma unroll
-    for (uint32_t i = threadIdx.x; i < 256; i += 64 * CHUNKS) s_code[i] = A.code[i];
+    __shared__ uint32_t s_code[FP16 ? kPairEntries + 32 : 256];
     if (!enc_fits(A)) return;
+    const uint32_t lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    if (FP16) {
+        const uint32_t h = A.code[32 + lane];
+        for (uint32_t i = warp; i < 32; i += kWriteWarps) {
+            const uint32_t e = A.code[i];
+            s_code[32 * i + lane] = (e & ~31u) | ((h & ~31u) >> (e & 31u)) | ((e & 31u) + (h & 31u));
+        }
+        if (warp == 0) s_code[kPairEntries + lane] = A.code[64 + lane];
+    } else {
+        for (uint32_t i = threadIdx.x; i < 256; i += 32 * kWriteWarps) s_code[i] = A.code[i];
+    }
     __syncthreads();
-    const EncThread T = enc_thread<CHUNKS>(A, blockIdx.x);
-    if (CHUNKS > 1 && !T.active) {                                // (a chunk's two warps leave or stay together)
-        if (STAGED) __syncthreads();
-        return;
-    }
-    const uint32_t W = A.words[T.c], raw_bytes = enc_raw_bytes(A, T.nkb);
-    uint8_t *raw = A.payload + (uint64_t)A.index[T.c] * kRecordUnit;
-    uint32_t *const rows = STAGED ? s_coded + T.sub * A.most_words * 64 : (uint32_t *)(raw + raw_bytes);
-    uint32_t *out = rows + T.seq;                                 // word j of this sequence at out[64 j]
-    uint32_t acc = 0, nacc = A.lag_bits;
-    auto append = [&](uint32_t b, uint32_t len) {                 // len <= 32, nacc < 32
-        acc |= b << nacc;
-        const uint32_t over = __funnelshift_rc(b, 0u, 32u - nacc);         // (nacc = 0: a shift by 32, nothing left over)
-        nacc += len;
-        if (nacc >= 32u) {
-            *out = acc;
-            out += 64;
-            acc = over;
-            nacc -= 32u;
-        }
-    };
-    auto code = [&](uint32_t byte_off) -> uint32_t { return *(const uint32_t *)((const char *)s_code + byte_off); };
-    // entries are stream bits and length << 16: two codewords joined, up to 24 bits, or, where none has more than 8 (SHORT), three or four
-    // (whole calls on 11008 x 4096: FP16 442 -> 434 us, BF16 229 -> 228)
-    auto bits2 = [](uint32_t e0, uint32_t e1) -> uint32_t { return (e0 & 0xFFFFu) | (e1 & 0xFFFFu) << (e0 >> 16); };
-    auto append2 = [&](uint32_t e0, uint32_t e1) { append(bits2(e0, e1), (e0 >> 16) + (e1 >> 16)); };
-    auto append3 = [&](uint32_t e0, uint32_t e1, uint32_t e2) {
-        const uint32_t l2 = (e0 >> 16) + (e1 >> 16);
-        append(bits2(e0, e1) | (e2 & 0xFFFFu) << l2, l2 + (e2 >> 16));
-    };
-    auto append4 = [&](uint32_t e0, uint32_t e1, uint32_t e2, uint32_t e3) {
-        const uint32_t l2 = (e0 >> 16) + (e1 >> 16);
-        append(bits2(e0, e1) | bits2(e2, e3) << l2, l2 + (e2 >> 16) + (e3 >> 16));
-    };
-    uint4 next = enc_load8(A, T.row, 0);
-    for (uint32_t kb = 0; kb < T.nkb; ++kb) {
-        const uint32_t x[4] = {next.x, next.y, next.z, next.w};
-        if (kb + 1 < T.nkb) next = enc_load8(A, T.row, kb + 1);
-        if (FP16) {
-            // sign bit of weight i: pair p = i / 2 (+ 4 for the row g + 8 sequence), bit p (+ 8 if i is odd)
-            uint32_t sg = 0;
+    const uint32_t table = (uint32_t)__cvta_generic_to_shared(s_code);
+    uint32_t *const stage = s_coded + warp * A.stage_rows * 64;
+#pragma unroll 1
+    for (uint32_t c = blockIdx.x * kWriteWarps + warp; c < A.n_chunks; c += gridDim.x * kWriteWarps) {
+        const EncLane L = enc_lane(A, c, lane);
+        const uint32_t W = __ldg(A.words + c), raw_bytes = enc_raw_bytes(A, L.nkb);
+        uint8_t *const raw = A.payload + (uint64_t)__ldg(A.index + c) * kRecordUnit;
+        uint8_t *raw_to = raw + lane * (FP16 ? 2 : 16);
+        auto write = [&](auto &sa, auto &sb) {
+            sb.out = sa.out + 128;
+            const auto end = sa.out + W * 256u;
+            sa.hi = sa.lo = sb.hi = sb.lo = 0;
+            sa.n = sb.n = A.lag_bits;
+            enc_blocks<VEC, VEC ? 2 : 1>(A, L, [&](const uint4 &va, const uint4 &vb) {
+                const uint32_t x[8] = {va.x, va.y, va.z, va.w, vb.x, vb.y, vb.z, vb.w};
+                if (FP16) {
+                    // signs: bit p for the first weight of pair p, bit 8 + p for its second, row g's pairs first
+                    uint32_t u = x[0] & 0x80008000u;
 #pragma unroll
-            for (int i = 0; i < 4; ++i) {
-                sg |= (x[i] >> 15 & 1u) << (i + 4 * T.half) | (x[i] >> 31) << (i + 4 * T.half + 8);
-                const uint32_t e0 = code((x[i] >> 8) & 0x7Cu), e1 = code(128u + ((x[i] >> 3) & 0x7Cu)), e2 = code(256u + ((x[i] << 2) & 0x7Cu));
-                const uint32_t e3 = code((x[i] >> 24) & 0x7Cu), e4 = code(128u + ((x[i] >> 19) & 0x7Cu)), e5 = code(256u + ((x[i] >> 14) & 0x7Cu));
-                if (SHORT) {
-                    append3(e0, e1, e2);
-                    append3(e3, e4, e5);
+                    for (int i = 1; i < 8; ++i) u = u >> 1 | (x[i] & 0x80008000u);
+                    *(uint16_t *)raw_to = (uint16_t)__byte_perm(u, 0u, 0x4431);
+                    raw_to += 64;
+                    sa.template append_fp16<SHORT>(va, table);
+                    sb.template append_fp16<SHORT>(vb, table);
                 } else {
-                    append2(e0, e1);
-                    append2(e2, e3);
-                    append2(e4, e5);
+                    uint32_t word[4];
+#pragma unroll
+                    for (int i = 0; i < 4; ++i) {                     // bytes in the raw layout's order: low bytes' mantissas, high bytes' signs
+                        const uint32_t m = __byte_perm(x[2 * i], x[2 * i + 1], kRawMantSel), sg = __byte_perm(x[2 * i], x[2 * i + 1], kRawSignSel);
+                        asm("lop3.b32 %0, %1, %2, 0x7F7F7F7F, 0xE4;" : "=r"(word[i]) : "r"(m), "r"(sg));
+                    }
+                    *(uint4 *)raw_to = make_uint4(word[0], word[1], word[2], word[3]);
+                    raw_to += 512;
+                    sa.template append_bf16<SHORT>(va, table);
+                    sb.template append_bf16<SHORT>(vb, table);
                 }
+            });
+            sa.finish(end);
+            sb.finish(end + 128);
+        };
+        if (W <= A.stage_rows) {
+            EncSequence<true> sa, sb;
+            sa.out = (uint32_t)__cvta_generic_to_shared(stage + lane);
+            write(sa, sb);
+            __syncwarp();
+            for (uint32_t i = lane; i < W * 16; i += 32) {
+                const uint4 v = ((const uint4 *)stage)[i];
+                ((uint4 *)(raw + raw_bytes))[i] = make_uint4(__brev(v.x), __brev(v.y), __brev(v.z), __brev(v.w));
             }
-            sg |= __shfl_xor_sync(0xFFFFFFFFu, sg, 1);
-            if (T.half == 0) *(uint16_t *)(raw + kb * 64 + T.lane * 2) = (uint16_t)sg;
+            __syncwarp();                                             // (the next chunk's words go to the same place)
         } else {
-            uint32_t word[2];
-#pragma unroll
-            for (int i = 0; i < 2; ++i)                           // bytes in the raw layout's order: low bytes' mantissas, high bytes' signs
-                word[i] = (__byte_perm(x[2 * i], x[2 * i + 1], kRawMantSel) & 0x7F7F7F7Fu) | (__byte_perm(x[2 * i], x[2 * i + 1], kRawSignSel) & 0x80808080u);
-#pragma unroll
-            for (int i = 0; i < 4; i += 2) {
-                const uint32_t e0 = code((x[i] >> 5) & 0x3FCu), e1 = code((x[i] >> 21) & 0x3FCu);
-                const uint32_t e2 = code((x[i + 1] >> 5) & 0x3FCu), e3 = code((x[i + 1] >> 21) & 0x3FCu);
-                if (SHORT) {
-                    append4(e0, e1, e2, e3);
-                } else {
-                    append2(e0, e1);
-                    append2(e2, e3);
-                }
-            }
-            *(uint2 *)(raw + kb * 512 + T.lane * 16 + T.half * 8) = make_uint2(word[0], word[1]);
+            EncSequence<false> sa, sb;
+            sa.out = (uint64_t)(raw + raw_bytes) + 4 * lane;
+            write(sa, sb);
         }
-    }
-    uint32_t *const end = rows + T.seq + (size_t)64 * W;
-    if (nacc) {
-        *out = acc;
-        out += 64;
-    }
-    for (; out < end; out += 64) *out = 0;
-    if (FP16 && (T.nkb & 1u) && T.q < 32) *(uint16_t *)(raw + T.nkb * 64 + T.q * 2) = 0;   // padding of the sign plane
-    if (STAGED) {
-        __syncthreads();
-        for (uint32_t i = T.q; i < W * 16; i += 64) ((uint4 *)(raw + raw_bytes))[i] = ((const uint4 *)rows)[i];
-    }
-    if (T.c + 1 == A.n_chunks) {                                  // the zero bytes behind the payload
-        uint4 *tail = (uint4 *)(A.payload + __ldcg(&A.totals->payload_units) * kRecordUnit);
-        for (uint32_t i = T.q; i < kTailSlack / 16; i += 64) tail[i] = make_uint4(0, 0, 0, 0);
+        if (FP16 && (L.nkb & 1u)) *(uint16_t *)(raw + L.nkb * 64 + lane * 2) = 0;      // padding of the sign plane
+        if (c + 1 == A.n_chunks) {                                    // the zero bytes behind the payload
+            uint4 *tail = (uint4 *)(A.payload + __ldcg(&A.totals->payload_units) * kRecordUnit);
+            for (uint32_t i = lane; i < kTailSlack / 16; i += 32) tail[i] = make_uint4(0, 0, 0, 0);
+        }
     }
 }
 
-inline uint32_t write_chunks(const EncArgs &A) { return A.Kc <= 128 ? 4 : 1; }
-inline bool write_staged(const EncArgs &A) { return A.Kc <= 512; }      // (at most 37 KB of shared memory)
-template <bool SHORT>
-inline void (*write_kernel_of(bool fp16, uint32_t chunks, bool staged))(EncArgs) {
-    if (fp16) return chunks == 4 ? (staged ? encode_write_kernel<true, 4, true, SHORT> : encode_write_kernel<true, 4, false, SHORT>)
-                                 : (staged ? encode_write_kernel<true, 1, true, SHORT> : encode_write_kernel<true, 1, false, SHORT>);
-    return chunks == 4 ? (staged ? encode_write_kernel<false, 4, true, SHORT> : encode_write_kernel<false, 4, false, SHORT>)
-                       : (staged ? encode_write_kernel<false, 1, true, SHORT> : encode_write_kernel<false, 1, false, SHORT>);
+inline void (*write_kernel_of(bool fp16, bool short_codes, bool vec))(EncArgs) {
+    if (fp16) return short_codes ? (vec ? encode_write_kernel<true, true, true> : encode_write_kernel<true, true, false>)
+                                 : (vec ? encode_write_kernel<true, false, true> : encode_write_kernel<true, false, false>);
+    return short_codes ? (vec ? encode_write_kernel<false, true, true> : encode_write_kernel<false, true, false>)
+                       : (vec ? encode_write_kernel<false, false, true> : encode_write_kernel<false, false, false>);
 }
 
 // ------------------------------------------------------------------------------ checksum of the records
@@ -709,31 +801,34 @@ extern "C" huffllm_status huffllm_encode_device(const huffllm_codebook *cb, cons
     uint32_t bits[256], longest = 1;
     encoder_tables(cb, len, bits);
     for (int i = 0; i < 256; ++i) {
-        A.code[i] = bits[i] | (uint32_t)len[i] << 16;
+        uint32_t first = 0;                                      // the first bit in bit 31
+        for (uint32_t b = 0; b < len[i]; ++b) first |= (bits[i] >> b & 1u) << (31 - b);
+        A.code[i] = first | len[i];
         longest = std::max<uint32_t>(longest, len[i]);
     }
-    A.most_words = (d.lag_bits + Kc / kBlockCols * 8 * longest * (A.fp16 ? 3 : 1) + 31) / 32;    // (the sizes are known on the device only)
+    const uint32_t steps = Kc / kBlockCols * 8 * (A.fp16 ? 3 : 1), most_words = (d.lag_bits + steps * longest + 31) / 32;
+    A.stage_rows = std::min(most_words, 32u);
 
     cudaError_t e;
     auto cuda_fail = [&](const char *what) { return fail(HUFFLLM_ERR_CUDA, "%s: %s", what, cudaGetErrorString(e)); };
-    const auto size_kernel = A.fp16 ? encode_size_kernel<true> : encode_size_kernel<false>;
-    const uint32_t chunks = write_chunks(A), smem = write_staged(A) ? chunks * A.most_words * 256 : 0;
-    const auto write_kernel = longest <= 8 ? write_kernel_of<true>(A.fp16 != 0, chunks, smem != 0) : write_kernel_of<false>(A.fp16 != 0, chunks, smem != 0);
+    const auto size_kernel = A.fp16 ? (A.vec_ok ? encode_size_kernel<true, true> : encode_size_kernel<true, false>)
+                                    : (A.vec_ok ? encode_size_kernel<false, true> : encode_size_kernel<false, false>);
+    const auto write_kernel = write_kernel_of(A.fp16 != 0, longest <= 8, A.vec_ok != 0);
+    const uint32_t smem = kWriteWarps * A.stage_rows * 256;
     int sms = 0;
     if ((e = prepare_checksum(&sms)) != cudaSuccess) return cuda_fail("device attributes");
     std::vector<uint8_t> fixed;
     fixed.reserve((size_t)d.off_index);                          // (what can fail without a launch does so before the first one)
     if ((e = cudaMemsetAsync(scr, 0, cleared, s)) != cudaSuccess) return cuda_fail("cudaMemsetAsync");
-    A.size_groups = size_groups(A);
-    const uint64_t per_cta = (uint64_t)kSizeChunks * A.size_groups;
-    size_kernel<<<(uint32_t)((d.n_chunks + per_cta - 1) / per_cta), kSizeThreads, 0, s>>>(A);
+    auto ctas = [&](uint32_t warps, uint32_t per_sm) { return (uint32_t)std::min<uint64_t>((d.n_chunks + warps - 1) / warps, (uint64_t)per_sm * sms); };
+    size_kernel<<<ctas(kSizeWarps, size_ctas(A.vec_ok)), 32 * kSizeWarps, 0, s>>>(A);
     // code lengths and table, assembled on the host while pass 1 runs; the header's bytes stay zero until the last kernel writes them
     fixed.assign((size_t)d.off_index, 0);
     write_fixed_sections(cb, d, fixed.data());
     memset(fixed.data(), 0, sizeof(d));
     if ((e = cudaMemcpyAsync(blob, fixed.data(), fixed.size(), cudaMemcpyHostToDevice, s)) != cudaSuccess) return cuda_fail("copy of the fixed sections");
     encode_scan_kernel<<<(uint32_t)((d.n_chunks + 64 + kScanThreads - 1) / kScanThreads), kScanThreads, 0, s>>>(A);
-    write_kernel<<<(uint32_t)((d.n_chunks + chunks - 1) / chunks), 64 * chunks, smem, s>>>(A);
+    write_kernel<<<ctas(kWriteWarps, write_ctas(A.vec_ok)), 32 * kWriteWarps, smem, s>>>(A);
     if (checksum_each(d.n_chunks, chunk_elems))
         encode_checksum_each_kernel<<<(uint32_t)((d.n_chunks + kEachThreads - 1) / kEachThreads), kEachThreads, 0, s>>>(A);
     else

@@ -145,6 +145,32 @@ def test_device_encoder_at_the_edges_of_its_passes(hl, rows, cols, ce, kind, dty
 
 
 @pytest.mark.gpu
+@pytest.mark.parametrize("dtype,budget,ce", [(0, 0, 4096), (0, 12, 16384), (1, 0, 2048), (1, 12, 8192)])
+@pytest.mark.parametrize("offset", range(8))
+def test_device_encoder_takes_rows_on_any_boundary(hl, dtype, budget, ce, offset):
+    """Rows that start on every 2-byte boundary, one to nine whole blocks and a ragged one per chunk, a ragged last row group;
+    long codes in long chunks: records of more rows than are collected in shared memory.  Host blob, byte for byte."""
+    import torch
+    kind = "fp16" if dtype else "student"
+    for rows, cols in ((37, 2 * ce // 16 + 32 * (1 + offset) + 8 * (offset % 4) + offset % 2), (16, 40 + 32 * offset)):
+        w = gen(kind, rows, cols, 20 + offset)
+        buf = torch.zeros(rows * cols + 16, dtype=torch.int16, device="cuda")
+        w_dev = buf[offset:offset + rows * cols]
+        w_dev.copy_(torch.from_numpy(w.view(np.int16).reshape(-1)))
+        cb = hl.build_codebook(w, dtype, budget)
+        cap = hl.encode_bound(rows, cols, dtype, ce)
+        blob_dev = torch.full((cap + 256,), 0xA5, dtype=torch.uint8, device="cuda")
+        n_scr = hl.encode_device_scratch_bytes(rows, cols, ce)
+        scratch = torch.full((n_scr,), 0x5A, dtype=torch.uint8, device="cuda")
+        desc = hl.encode_device(cb, w_dev, rows, cols, ce, blob_dev, cap, scratch, n_scr)
+        want, desc_host = hl.encode(cb, w, ce)
+        got = blob_dev.cpu().numpy()
+        assert bytes(desc) == bytes(desc_host) and np.array_equal(got[:desc.blob_bytes], want)
+        assert np.all(got[desc.blob_bytes:] == 0xA5)
+        cb.free()
+
+
+@pytest.mark.gpu
 def test_full_size_matrix_on_the_device_equals_the_host_blob(hl):
     """A full-size FFN matrix of the benchmark's layer (45 M weights, 11008 chunks)."""
     import torch
