@@ -17,13 +17,14 @@
 #include <type_traits>
 #include <vector>
 
+#include "decode_common.cuh"
 #include "internal.h"
 
 namespace huffllm {
 
 struct EncTotals {
     unsigned long long payload_units, coded_bits, checksum;
-    uint32_t max_words, bad;     // bad: 1 = a symbol without codeword, 2 = payload beyond the 32-bit record index
+    uint32_t max_words, bad;     // bad: 1 = a symbol without codeword, 2 = payload beyond the 32-bit record index, 4 = a wait ran out
     uint32_t summed;             // CTAs whose records' checksums are in
 };
 
@@ -157,11 +158,6 @@ __device__ __forceinline__ void enc_blocks(const EncArgs &A, const EncLane &L, F
     for (uint32_t kb = L.whole; kb < L.nkb; ++kb)
         f(enc_edge(A, L.row[0] + kb * 32u, L.left[0] - (int32_t)(kb * 32u)), enc_edge(A, L.row[1] + kb * 32u, L.left[1] - (int32_t)(kb * 32u)));
 }
-__device__ __forceinline__ uint32_t lds32(uint32_t addr) {
-    uint32_t v;
-    asm("ld.shared.u32 %0, [%1];" : "=r"(v) : "r"(addr));
-    return v;
-}
 __device__ __forceinline__ uint32_t lds16(uint32_t addr) {
     uint16_t v;
     asm("ld.shared.u16 %0, [%1];" : "=h"(v) : "r"(addr));
@@ -204,7 +200,7 @@ __global__ void __launch_bounds__(32 * kSizeWarps, size_ctas(VEC)) encode_size_k
                 bits += lds16(__dp2a_lo(l, 0x0002u, low)) + lds16(__dp2a_lo(l, 0x0200u, low));
             } else {
                 const uint32_t y = x[i] * 2u;                                // exponents in bytes 1 and 3
-                bits += lds32(__dp4a(y, 0x00000400u, table)) + lds32(__dp4a(y, 0x04000000u, table));
+                bits += lds_lut(__dp4a(y, 0x00000400u, table)) + lds_lut(__dp4a(y, 0x04000000u, table));
             }
         }
         return bits;
@@ -322,8 +318,8 @@ struct EncSequence {
 #pragma unroll
         for (int i = 0; i < 4; i += 2) {
             const uint32_t y0 = x[i] * 2u, y1 = x[i + 1] * 2u;                            // exponents in bytes 1 and 3
-            const uint32_t e0 = lds32(__dp4a(y0, 0x00000400u, table)), e1 = lds32(__dp4a(y0, 0x04000000u, table));
-            const uint32_t e2 = lds32(__dp4a(y1, 0x00000400u, table)), e3 = lds32(__dp4a(y1, 0x04000000u, table));
+            const uint32_t e0 = lds_lut(__dp4a(y0, 0x00000400u, table)), e1 = lds_lut(__dp4a(y0, 0x04000000u, table));
+            const uint32_t e2 = lds_lut(__dp4a(y1, 0x00000400u, table)), e3 = lds_lut(__dp4a(y1, 0x04000000u, table));
             push(e0);
             push(e1);
             if (!SHORT) advance(e0 + e1);
@@ -338,8 +334,8 @@ struct EncSequence {
 #pragma unroll
         for (int i = 0; i < 4; ++i) {
             const uint32_t u = x[i] >> 5 & 0x03FF03FFu, l = x[i] & 0x001F001Fu;
-            const uint32_t e0 = lds32(__dp2a_lo(u, 0x0004u, table)), e1 = lds32(__dp2a_lo(l, 0x0004u, low));
-            const uint32_t e2 = lds32(__dp2a_lo(u, 0x0400u, table)), e3 = lds32(__dp2a_lo(l, 0x0400u, low));
+            const uint32_t e0 = lds_lut(__dp2a_lo(u, 0x0004u, table)), e1 = lds_lut(__dp2a_lo(l, 0x0004u, low));
+            const uint32_t e2 = lds_lut(__dp2a_lo(u, 0x0400u, table)), e3 = lds_lut(__dp2a_lo(l, 0x0400u, low));
             push(e0);
             if (!SHORT) advance(e0);
             push(e1);
@@ -462,10 +458,15 @@ inline void (*write_kernel_of(bool fp16, bool short_codes, bool vec))(EncArgs) {
 //     bytes is bit k at its start, exclusive-or a value that the stretch alone determines: an exclusive-or scan over the
 //     stretches gives bit k at the start of each.  Eight rounds, one per bit, give every stretch its starting x.
 // A warp takes a record; a lane walks four stretches of 4 M bytes at a time, one in each byte of a register (stretch 32 s + l
-// in byte s of lane l).  The rounds for bits 1 to 3 need two instructions per four bytes (P mod 16 = 3: four 4-bit values in
-// the bytes of a word times 3 stay in their bytes); from bit 5 on even and odd bytes are multiplied apart.  The weighted sum
-// goes to the tensor cores as an 8-bit product: the record's bytes (and x & b) times the eight byte limbs of the powers of P,
-// exact in 32-bit integers.  Bound by the integer pipe: some 28 instructions per four bytes.
+// in byte s of lane l), each in two halves, which gives it two chains.  A round of a bit takes two instructions per four bytes: the
+// low four bits times 3 (P mod 16) stay in their bytes, and so do the upper four, whose two bits of overflow end among the bits that
+// the next mask takes away, once what the lower four add to them has been worked out for every byte (C below).  The weighted sum
+// goes to the tensor cores as an 8-bit product: the record's bytes (and x & b, lower and upper four bits apart) times the eight byte limbs
+// of the powers of P, exact in 32-bit integers.
+// Bound by the integer pipe and what keeps it waiting: 40 instructions per four bytes, 20 of them there, at 57 % of its rate (a round
+// settles its bit in six dependent shuffles).  (11008 records of 1600 to 1664 words 48.4 -> 43.8 us, 22016 FP16 records 74.6 -> 60, 5504 of twice the
+// size 58 -> 41.7, against rounds of four instructions for the upper bits, even and odd bytes apart, in one chain, steps of 7, 6 and 3
+// copied piece by piece.  Steps of 5 and 4 only, 24 warps an SM instead of 16: 50.)
 constexpr uint64_t kFnvPrime = 1099511628211ull, kFnvStart = 1469598103934665603ull;
 __host__ __device__ constexpr uint64_t fnv_pow(uint64_t base, uint32_t e) {
     uint64_t r = 1;
@@ -481,9 +482,9 @@ constexpr uint64_t fnv_inverse() {                 // P^-1 mod 2^64 (Newton's it
 constexpr uint64_t kFnvInverse = fnv_inverse();
 static_assert(kFnvInverse * kFnvPrime == 1, "inverse of the hash's multiplier");
 // The sum's weights for stretches of M words: byte j of stretch 32 s + 4 g + t has weight P^(512 M - (32 s + 4 g + t) 4 M - j).
-// The factor of g is taken out (row_factor); limb n of the rest is the B operand: for the product of bytes j = 4 i .. 4 i + 3
-// (A registers in this order), lane 4 n + t holds in byte s of word 0 the limb for j = 4 i, of word 1 for j = 4 i + 2; the odd
-// j, rows g + 8 of A, carry one factor P^-1 more.
+// The factor of g is taken out (row_factor); limb n of the rest is the B operand: for the product of bytes j = 2 i, 2 i + 1 and
+// the same of the stretch's other half, 2 M further on (A registers in this order), lane 4 n + t holds in byte s of word 0 the limb
+// for the first, of word 1 for the third; the odd j, rows g + 8 of A, carry one factor P^-1 more.
 template <int M>
 struct FnvWeights {
     uint32_t b[M][32][2];
@@ -493,7 +494,7 @@ struct FnvWeights {
             for (int h = 0; h < 2; ++h)
                 for (int t = 0; t < 4; ++t)
                     for (int s = 0; s < 4; ++s) {
-                        const uint64_t w = fnv_pow(kFnvPrime, 512 * M - (32 * s + t) * 4 * M - (4 * i + 2 * h));
+                        const uint64_t w = fnv_pow(kFnvPrime, 512 * M - (32 * s + t) * 4 * M - (2 * i + 2 * M * h));
                         for (int n = 0; n < 8; ++n) b[i][4 * n + t][h] |= (uint32_t)(w >> (8 * n) & 0xFFu) << (8 * s);
                     }
         for (int g = 0; g < 8; ++g) row_factor[g] = fnv_pow(kFnvInverse, 16 * M * g);
@@ -501,6 +502,7 @@ struct FnvWeights {
 };
 __device__ const FnvWeights<7> g_fnv7{};
 __device__ const FnvWeights<6> g_fnv6{};
+__device__ const FnvWeights<4> g_fnv4{};
 __device__ const FnvWeights<3> g_fnv3{};
 
 __device__ __forceinline__ uint32_t xor_and(uint32_t a, uint32_t b, uint32_t m) {       // (a ^ b) & m
@@ -515,13 +517,19 @@ __device__ __forceinline__ void mma_u8(int32_t (&d)[4], uint32_t a0, uint32_t a1
                  : "r"(a0), "r"(a1), "r"(a2), "r"(a3), "r"(b0), "r"(b1));
 }
 
-// 512 M bytes of a record (`words`, in shared memory): hash `h` moved on over them.  All lanes hold the same h.
+// A record's hash on its way: every lane's part of it as if the record ended here (their sum is the hash), and the low byte, the same in
+// all lanes.
+struct FnvState {
+    uint64_t part;
+    uint32_t low;
+};
+// 512 M bytes of a record (`words`, in shared memory).
 template <int M>
-__device__ __forceinline__ uint64_t fnv_step(uint64_t h, const uint32_t *words, const FnvWeights<M> &wt, uint32_t lane, uint32_t three) {
-    constexpr int N = 4 * M;                       // bytes of a stretch
-    constexpr uint32_t kEven = 0x00FF00FFu, kOdd = 0xFF00FF00u;
+__device__ __forceinline__ void fnv_step(FnvState &F, const uint32_t *words, const FnvWeights<M> &wt, uint32_t lane, uint32_t three) {
+    constexpr int N = 4 * M, H = 2 * M;            // bytes of a stretch, of its halves
+    constexpr uint32_t kLow = 0x0F0F0F0Fu, kHigh = 0xF0F0F0F0u;
     uint32_t G[N];                                 // G[j]: byte j of the lane's four stretches
-    uint32_t all = 0;
+    uint32_t all[2] = {0, 0};
 #pragma unroll
     for (int m = 0; m < M; ++m) {
         const uint32_t a = words[lane * M + m], b = words[(32 + lane) * M + m], c = words[(64 + lane) * M + m], d = words[(96 + lane) * M + m];
@@ -530,75 +538,86 @@ __device__ __forceinline__ uint64_t fnv_step(uint64_t h, const uint32_t *words, 
         G[4 * m + 1] = byte_perm(t0, t1, 0x7632);
         G[4 * m + 2] = byte_perm(t2, t3, 0x5410);
         G[4 * m + 3] = byte_perm(t2, t3, 0x7632);
-        all ^= G[4 * m] ^ G[4 * m + 1] ^ G[4 * m + 2] ^ G[4 * m + 3];
     }
-    uint32_t X = 0;                                // the stretches' starting low bytes, as far as they are known
-    // e: bit k of each byte = bit k at the end of the stretch if it were 0 at its start; settles bit k of X
-    auto settle = [&](uint32_t e, uint32_t k) {
-        const uint32_t own = e & (0x01010101u << k);
+#pragma unroll
+    for (int j = 0; j < N; ++j) all[j / H] ^= G[j];
+    const uint32_t first = F.low * 0x01010101u;
+    uint32_t X[2] = {0, 0};                        // the halves' starting low bytes, as far as they are known
+    // e: the bits `bits` of each byte at the end of a half if they were 0 at its start; settles them in X
+    auto settle = [&](const uint32_t (&e)[2], uint32_t bits, bool two = false) {
+        const uint32_t own = xor_and(e[0], e[1], bits);
         uint32_t v = own;
 #pragma unroll
-        for (int o = 1; o < 32; o <<= 1) {
-            const uint32_t up = __shfl_up_sync(0xFFFFFFFFu, v, o);
-            if (lane >= (uint32_t)o) v ^= up;
-        }
-        const uint32_t tot = __shfl_sync(0xFFFFFFFFu, v, 31);
-        const uint32_t in = ((uint32_t)h & (1u << k)) * 0x01010101u;
-        X |= v ^ own ^ in ^ (tot << 8) ^ (tot << 16) ^ (tot << 24);
+        for (int o = 1; o < 32; o <<= 1)
+            asm volatile("{\n\t.reg .pred p;\n\t.reg .b32 up;\n\tshfl.sync.up.b32 up|p, %0, %1, 0, 0xFFFFFFFF;\n\t@p xor.b32 %0, %0, up;\n\t}" : "+r"(v) : "r"(o));
+        // what the stretches in the bytes below add (one bit: the lowest of the sum of their up to three totals is the exclusive or)
+        const uint32_t total = __shfl_sync(0xFFFFFFFFu, v, 31);
+        const uint32_t before = two ? total << 8 ^ total << 16 ^ total << 24 : total * 0x01010100u;
+        const uint32_t at = v ^ own ^ before ^ first;
+        X[0] |= at & bits;
+        X[1] |= xor_and(at, e[0], bits);
     };
-    settle(all, 0);
+    // (bits 0 and 1 together: what bit 0 adds to bit 1 over a half's even number of bytes does not depend on where it started)
 #pragma unroll
     for (uint32_t k = 1; k <= 3; ++k) {
-        uint32_t z = X;
+        uint32_t z[2] = {X[0], X[1]};
 #pragma unroll
-        for (int j = 0; j < N; ++j) z = xor_and(z, G[j], 0x0F0F0F0Fu) * three;
-        settle(z, k);
-    }
-    {   // bit 4 of the product with P mod 32 = 19: bit 4 of 3 times the low four bits, bit 4 and bit 0 of x ^ b
-        uint32_t z = X, acc = all, low = 0;
+        for (int j = 0; j < H; ++j)
 #pragma unroll
-        for (int j = 0; j < N; j += 2) {
-            const uint32_t y0 = xor_and(z, G[j], 0x0F0F0F0Fu), z0 = y0 * three, y1 = xor_and(z0, G[j + 1], 0x0F0F0F0Fu);
-            z = y1 * three;
-            acc ^= z0 ^ z;
-            low ^= y0 ^ y1;
-        }
-        settle(acc ^ (low << 4), 4);
+            for (int h = 0; h < 2; ++h) z[h] = xor_and(z[h], G[h * H + j], kLow) * three;
+        settle(z, k == 1 ? 0x03030303u : 0x01010101u << k, k == 1);
     }
-#pragma unroll 1
-    for (uint32_t k = 5; k <= 7; ++k) {
-        uint32_t ze = X, zo = X;
-#pragma unroll
-        for (int j = 0; j < N; ++j) {
-            ze = xor_and(ze, G[j], kEven) * 0xB3u;
-            zo = xor_and(zo, G[j], kOdd) * 0xB3u;
-        }
-        settle((ze & kEven) | (zo & kOdd), k);
-    }
+    // The low four bits are known.  What they add to the upper four of (x ^ b) * P mod 256 is worked out once: P mod 256 is 16 * 11 + 3.
     int32_t sb[4] = {0, 0, 0, 0}, sv[4] = {0, 0, 0, 0};
-    uint32_t ze = X, zo = X;
+    uint32_t C[N], zl[2] = {X[0], X[1]}, odd[2] = {all[0], all[1]};
+    auto weights = [&](int i) -> uint2 { return __ldg((const uint2 *)&wt.b[i][lane][0]); };
+    // four bytes j of half h: f(v's, number of the first byte)
 #pragma unroll
-    for (int i = 0; i < M; ++i) {
+    for (int j = 0; j < H; j += 2) {
         uint32_t v[4];
 #pragma unroll
-        for (int j = 0; j < 4; ++j) {
-            const uint32_t g = G[4 * i + j];
-            v[j] = ((ze & kEven) | (zo & kOdd)) & g;
-            ze = xor_and(ze, g, kEven) * 0xB3u;
-            zo = xor_and(zo, g, kOdd) * 0xB3u;
+        for (int i = 0; i < 4; ++i) {
+            const int h = i >> 1, n = h * H + j + (i & 1);
+            const uint32_t g = G[n], y = xor_and(zl[h], g, kLow);
+            v[i] = zl[h] & g & kLow;
+            zl[h] = y * three;
+            C[n] = y * 176u + (zl[h] & kHigh);
+            odd[h] ^= C[n];
         }
-        const uint2 w = __ldg((const uint2 *)&wt.b[i][lane][0]);
-        mma_u8(sb, G[4 * i], G[4 * i + 1], G[4 * i + 2], G[4 * i + 3], w.x, w.y);
+        const uint2 w = weights(j / 2);
+        mma_u8(sb, G[j], G[j + 1], G[H + j], G[H + j + 1], w.x, w.y);
         mma_u8(sv, v[0], v[1], v[2], v[3], w.x, w.y);
     }
+    settle(odd, 0x10101010u);
+#pragma unroll 1
+    for (uint32_t k = 5; k <= 7; ++k) {
+        uint32_t z[2] = {X[0], X[1]};
+#pragma unroll
+        for (int j = 0; j < H; ++j)
+#pragma unroll
+            for (int h = 0; h < 2; ++h) z[h] = xor_and(z[h], G[h * H + j], kHigh) * three + C[h * H + j];
+        settle(z, 0x01010101u << k);
+    }
+    uint32_t z[2] = {X[0], X[1]};
+#pragma unroll
+    for (int j = 0; j < H; j += 2) {
+        uint32_t v[4];
+#pragma unroll
+        for (int i = 0; i < 4; ++i) {
+            const int h = i >> 1, n = h * H + j + (i & 1);
+            v[i] = z[h] & G[n] & kHigh;
+            z[h] = xor_and(z[h], G[n], kHigh) * three + C[n];
+        }
+        const uint2 w = weights(j / 2);
+        mma_u8(sv, v[0], v[1], v[2], v[3], w.x, w.y);
+    }
+    F.low = __shfl_sync(0xFFFFFFFFu, (z[1] & kHigh) | (zl[1] & kLow), 31) >> 24;
     const uint32_t t = lane & 3u;
     auto limbs = [&](int32_t lo, int32_t hi) -> uint64_t { return ((uint64_t)(int64_t)lo + ((uint64_t)(int64_t)hi << 8)) << (16u * t); };
-    uint64_t sum = (limbs(sb[0] - 2 * sv[0], sb[1] - 2 * sv[1]) + limbs(sb[2] - 2 * sv[2], sb[3] - 2 * sv[3]) * kFnvInverse) *
-                   __ldg((const unsigned long long *)&wt.row_factor[lane >> 2]);
-#pragma unroll
-    for (int o = 16; o; o >>= 1) sum += __shfl_xor_sync(0xFFFFFFFFu, (unsigned long long)sum, o);
+    const uint64_t sum = (limbs(sb[0] - 2 * sv[0], sb[1] - 2 * sv[1]) + limbs(sb[2] - 2 * sv[2], sb[3] - 2 * sv[3]) * kFnvInverse) *
+                         __ldg((const unsigned long long *)&wt.row_factor[lane >> 2]);
     constexpr uint64_t kOver = fnv_pow(kFnvPrime, 512 * M);
-    return h * kOver + sum;
+    F.part = F.part * kOver + sum;
 }
 
 // What the totals add to the header.
@@ -621,78 +640,94 @@ __device__ __forceinline__ void finish_checksum(const EncArgs &A, unsigned long 
     *(huffllm_desc *)A.blob = d;
 }
 
-// A warp goes through its records a step (7, 6 or 3 times 512 bytes) at a time, while the next step's bytes are on their way to its
-// other buffer.  Bound by the integer pipe.  (11008 records of 1600 to 1664 words: a warp per record that waits for every step's
-// bytes, steps of 7 and 3 times 512, 55 us; so 51.  Beside the packing in one kernel, which would leave the record in shared memory,
-// 110 us instead of 46 + 51: 80 registers a thread leave an SM too few warps to pack with.)
-constexpr uint32_t kSumWarps = 8, kSumCtas = 3, kSumBuf = 7 * 128;       // CTAs of an SM (80 registers); words of a step
+// A warp goes through its records a step (7, 6, 4 or 3 times 512 bytes) at a time, while a bulk copy brings the next step's bytes to its
+// other buffer.  (Beside the packing in one kernel, which would leave the record in shared memory, 110 us instead of 46 + 51 by the kernels
+// of the time: too few warps to pack with.)
+constexpr uint32_t kSumWarps = 4, kSumCtas = 4, kSumBuf = 7 * 128;       // CTAs of an SM (128 registers); words of a step
 constexpr uint32_t kSumSmem = kSumWarps * 2 * kSumBuf * 4;
-struct SumStep {
-    uint64_t c;                  // record
-    uint32_t n, done;            // its words, and those in front of this step
-    const uint32_t *src;
-};
 __global__ void __launch_bounds__(32 * kSumWarps, kSumCtas) encode_checksum_kernel(const __grid_constant__ EncArgs A) {
     extern __shared__ __align__(16) uint32_t s_steps[];
     __shared__ unsigned long long s_term[kSumWarps];
-    const uint32_t lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-    const uint64_t stride = (uint64_t)gridDim.x * kSumWarps;
+    __shared__ __align__(8) uint64_t s_landed[kSumWarps][2];
+    const uint32_t lane = threadIdx.x & 31, warp = threadIdx.x >> 5, n_chunks = (uint32_t)A.n_chunks, stride = gridDim.x * kSumWarps;
     if (!enc_fits(A)) return;
     uint32_t *const buf = s_steps + warp * 2 * kSumBuf;
+    const uint32_t bar = smem_u32(&s_landed[warp][0]);
+    if (lane == 0) {
+        mbar_init(bar, 1);
+        mbar_init(bar + 8, 1);
+        asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+    }
+    __syncwarp();
     // 3, as a value the compiler does not know: times 3 as a shifted addition would join the logic instructions on the
     // integer pipe that bounds this kernel, as a multiplication it runs beside them
     const uint32_t three = 3u + (uint32_t)(A.n_chunks >> 32);
-    auto open = [&](uint64_t c) -> SumStep {
-        if (c >= A.n_chunks) return {c, 0u, 0u, nullptr};
-        const uint32_t r0 = __ldg(A.index + c), r1 = __ldg(A.index + c + 1);
-        return {c, (r1 - r0) * (kRecordUnit / 4), 0u, (const uint32_t *)(A.payload + (uint64_t)r0 * kRecordUnit)};
+    // a step's size: two of 4 rather than 7 and 3, FP16 records of 4 KB among others
+    auto step_of = [](uint32_t left) -> uint32_t { return left > 32u ? 7u : left > 28u ? 4u : left > 24u ? 7u : left > 16u ? 6u : left > 12u ? 4u : 3u; };
+    // (sizes and places in the format's units of 128 bytes: `at`, from the payload on; as many of the `left` as a step may have)
+    auto fetch = [&](uint32_t at, uint32_t left, uint32_t to) {
+        if (lane) return;
+        const uint32_t bytes = min(left, 4 * step_of(left)) * kRecordUnit;
+        asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
+        mbar_expect_tx(bar + 8 * to, bytes);
+        bulk_g2s(smem_u32(buf + to * kSumBuf), A.payload + (uint64_t)at * kRecordUnit, bytes, bar + 8 * to);
     };
-    auto size_of = [](const SumStep &S) -> uint32_t { return S.n - S.done > 6 * 128 ? 7u : S.n - S.done > 3 * 128 ? 6u : 3u; };
-    auto fetch = [&](const SumStep &S, uint32_t *to) {       // (words behind the record are zero and add nothing; it has a multiple of 32)
-        if (S.c < A.n_chunks) {
-            const uint32_t pieces = size_of(S) * 32u, at = (uint32_t)__cvta_generic_to_shared(to);
-            for (uint32_t i = lane; i < pieces; i += 32) {
-                const uint32_t bytes = S.done + 4 * i < S.n ? 16u : 0u;
-                asm volatile("cp.async.cg.shared.global [%0], [%1], 16, %2;" ::"r"(at + 16 * i), "l"(bytes ? S.src + S.done + 4 * i : S.src), "r"(bytes) : "memory");
-            }
-        }
-        asm volatile("cp.async.commit_group;" ::: "memory");
+    auto open = [&](uint32_t r, uint32_t &at, uint32_t &left) {
+        left = 0;
+        if (r >= n_chunks) return;
+        at = __ldg(A.index + r);
+        left = __ldg(A.index + r + 1) - at;
     };
-    unsigned long long term = 0;
-    uint64_t h = kFnvStart;
-    SumStep cur = open((uint64_t)blockIdx.x * kSumWarps + warp), after = open(cur.c + stride);
-    uint32_t which = 0;
-    fetch(cur, buf);
+    const FnvState start = {lane == 0 ? kFnvStart : 0ull, (uint32_t)kFnvStart & 0xFFu};
+    FnvState F = start;
+    // the record at hand, from the step at hand on, and the warp's next one
+    uint32_t c = blockIdx.x * kSumWarps + warp, step = 0, at = 0, left, next_at = 0, next_left;
+    open(c, at, left);
+    open(c + stride, next_at, next_left);
+    if (lane == 0) s_term[warp] = 0;
+    if (left) fetch(at, left, 0);
 #pragma unroll 1
-    while (cur.c < A.n_chunks) {
-        const uint32_t m = size_of(cur);
-        SumStep next = cur;
-        next.done += m * 128;
-        const bool last = next.done >= cur.n;
-        if (last) {
-            next = after;
-            after = open(next.c + stride);                   // (wanted a record later)
+    for (; left; ++step) {
+        const uint32_t which = step & 1u, m = step_of(left), here = min(left, 4 * m);
+        const bool last = left <= 4 * m;
+        __syncwarp();                                        // (all lanes are done with the other buffer)
+        if (!last) fetch(at + 4 * m, left - 4 * m, which ^ 1u);
+        else if (next_left) fetch(next_at, next_left, which ^ 1u);
+        uint32_t spins = 0;
+        bool done = mbar_try_wait(bar + 8 * which, step >> 1 & 1u);
+        while (!__all_sync(0xFFFFFFFFu, done) && ++spins < kWaitLimit) done = mbar_try_wait(bar + 8 * which, step >> 1 & 1u);
+        if (spins == kWaitLimit) {                           // (the copy never came: the call fails)
+            atomicOr(&A.totals->bad, 4u);
+            break;
         }
+        uint32_t *const words = buf + which * kSumBuf;
+        for (uint32_t i = here * 32 + lane; i < m * 128; i += 32) words[i] = 0;        // (zeros behind the record add nothing)
         __syncwarp();
-        fetch(next, buf + (which ^ 1u) * kSumBuf);
-        asm volatile("cp.async.wait_group 1;" ::: "memory");
-        __syncwarp();
-        const uint32_t *const words = buf + which * kSumBuf;
-        h = m == 7u ? fnv_step<7>(h, words, g_fnv7, lane, three) : m == 6u ? fnv_step<6>(h, words, g_fnv6, lane, three) : fnv_step<3>(h, words, g_fnv3, lane, three);
+        if (m == 7u) fnv_step<7>(F, words, g_fnv7, lane, three);
+        else if (m == 6u) fnv_step<6>(F, words, g_fnv6, lane, three);
+        else if (m == 4u) fnv_step<4>(F, words, g_fnv4, lane, three);
+        else fnv_step<3>(F, words, g_fnv3, lane, three);
         if (last) {
-            // the zero bytes behind the record multiplied h by P each: a multiple of 32 words
+            uint64_t h = F.part;
+#pragma unroll
+            for (int o = 16; o; o >>= 1) h += __shfl_xor_sync(0xFFFFFFFFu, (unsigned long long)h, o);
+            // the zero bytes behind the record multiplied h by P each
             constexpr uint64_t kUnitBack = fnv_pow(kFnvInverse, kRecordUnit);
-            for (uint32_t p = cur.n; p < cur.done + m * 128; p += kRecordUnit / 4) h *= kUnitBack;
-            term += h * (2 * cur.c + 1);
-            h = kFnvStart;
+            for (uint32_t p = here; p < 4 * m; ++p) h *= kUnitBack;
+            if (lane == 0) s_term[warp] += h * (2ull * c + 1);
+            F = start;
+            c += stride;
+            at = next_at;
+            left = next_left;
+            open(c + stride, next_at, next_left);            // (wanted a record later)
+        } else {
+            at += 4 * m;
+            left -= 4 * m;
         }
-        cur = next;
-        which ^= 1u;
     }
-    if (lane == 0) s_term[warp] = term;
     __syncthreads();
     if (threadIdx.x) return;
-    term = 0;
+    unsigned long long term = 0;
     for (uint32_t i = 0; i < kSumWarps; ++i) term += s_term[i];
     finish_checksum(A, term);
 }
@@ -710,29 +745,57 @@ static cudaError_t prepare_checksum(int *sms) {
     return cudaSuccess;
 }
 
-// The same with a thread per record, as the hash is written.  A record takes a thread some 30 ns per byte (one load in flight),
-// but a GPU full of threads takes less than half of what the warps above need per byte, who pay for whole steps of 1.5 KB whatever
-// the record's size: with enough records this is faster, the sooner the shorter they are.  (Warps / threads: 88064 records of 512
-// weights 159 / 44 us, 1.05 M of them 1.75 / 0.33 ms, 44032 of 1024 104 / 62 us; whole calls: 16384 of 512 114 / 106, 8192 of 1024
-// 90 / 117, 22016 of 2048 175 / 217, 114688 of 2048 648 / 573, 57344 of 4096 558 / 547, 28672 of 8192 542 / 688.)
+// The same with a thread per record, as the hash is written: six instructions per byte where the warps above spend ten, but one byte
+// after the other, 20 cycles each (16 of them the exclusive-or and the multiplication that wait for one another), which is
+// the time of a launch as long as every scheduler has a warp at most.  Four pieces of 32 bytes are on their way to registers (with
+// one of 16 bytes, 28672 x 8192 took 215 us instead of 145).  Both grow with the record, so the line is a number of records, which rises
+// with their size because from 19000 on threads share schedulers.  (Warps / threads, us, 11008 x 4096: chunks of 512 119 / 33, 1024 66 / 35,
+// 2048 45.5 / 47.0 and FP16 60.0 / 51.8, 4096 43.8 / 70; 28672 x 8192 in chunks of 4096 180 / 145, 28672 x 4096 in chunks of 8192 91 / 126.)
 constexpr uint32_t kEachThreads = 128;
-inline bool checksum_each(uint64_t n_chunks, uint32_t chunk_elems) { return n_chunks >= 16384ull + 8ull * chunk_elems; }
+inline bool checksum_each(uint64_t n_chunks, uint32_t chunk_elems) { return n_chunks >= 13000ull + 4ull * chunk_elems; }
+inline uint32_t each_threads(uint64_t n_chunks) { return n_chunks >= 65536 ? kEachThreads : 32; }       // (few records: a warp for every scheduler)
+struct Piece32 {
+    uint32_t w[8];
+};
+__device__ __forceinline__ Piece32 ldg_32(const uint8_t *p) {
+    Piece32 v;
+    asm volatile("ld.global.v8.b32 {%0, %1, %2, %3, %4, %5, %6, %7}, [%8];"
+                 : "=r"(v.w[0]), "=r"(v.w[1]), "=r"(v.w[2]), "=r"(v.w[3]), "=r"(v.w[4]), "=r"(v.w[5]), "=r"(v.w[6]), "=r"(v.w[7])
+                 : "l"(p)
+                 : "memory");
+    return v;
+}
 __global__ void __launch_bounds__(kEachThreads) encode_checksum_each_kernel(const __grid_constant__ EncArgs A) {
     __shared__ unsigned long long s_term[kEachThreads / 32];
-    const uint64_t c = (uint64_t)blockIdx.x * kEachThreads + threadIdx.x;
+    const uint64_t c = (uint64_t)blockIdx.x * blockDim.x + threadIdx.x;
     if (!enc_fits(A)) return;
     unsigned long long term = 0;
     if (c < A.n_chunks) {
-        const uint32_t r0 = A.index[c], n = (A.index[c + 1] - r0) * (kRecordUnit / 16);
-        const uint4 *p = (const uint4 *)(A.payload + (uint64_t)r0 * kRecordUnit);
-        uint64_t h = kFnvStart;
-        for (uint32_t i = 0; i < n; ++i) {
-            const uint4 q = __ldcg(p + i);
-            const uint32_t x[4] = {q.x, q.y, q.z, q.w};
+        constexpr uint32_t kPrimeLow = (uint32_t)kFnvPrime;          // P = 2^40 + this
+        static_assert(kFnvPrime == (1ull << 40) + kPrimeLow, "the hash's multiplier");
+        const uint32_t r0 = A.index[c];
+        uint32_t units = A.index[c + 1] - r0;                        // (at least one)
+        const uint8_t *p = A.payload + (uint64_t)r0 * kRecordUnit;
+        uint32_t lo = (uint32_t)kFnvStart, hi = (uint32_t)(kFnvStart >> 32);
+        Piece32 v[4];
 #pragma unroll
-            for (int k = 0; k < 16; ++k) h = (h ^ ((x[k >> 2] >> (8 * (k & 3))) & 0xFFu)) * kFnvPrime;
+        for (int s = 0; s < 4; ++s) v[s] = ldg_32(p + 32 * s);
+#pragma unroll 1
+        for (; units; --units) {
+            p += kRecordUnit;
+#pragma unroll
+            for (int s = 0; s < 4; ++s) {
+#pragma unroll
+                for (int k = 0; k < 32; ++k) {
+                    const uint32_t x = lo ^ ((v[s].w[k >> 2] >> (8 * (k & 3))) & 0xFFu);
+                    const uint64_t m = (uint64_t)x * kPrimeLow;
+                    lo = (uint32_t)m;
+                    hi = hi * kPrimeLow + (uint32_t)(m >> 32) + (x << 8);
+                }
+                if (units > 1) v[s] = ldg_32(p + 32 * s);
+            }
         }
-        term = n ? h * (2 * c + 1) : 0ull;
+        term = ((unsigned long long)hi << 32 | lo) * (2 * c + 1);
     }
 #pragma unroll
     for (int o = 16; o; o >>= 1) term += __shfl_xor_sync(0xFFFFFFFFu, term, o);
@@ -740,7 +803,7 @@ __global__ void __launch_bounds__(kEachThreads) encode_checksum_each_kernel(cons
     __syncthreads();
     if (threadIdx.x) return;
     term = 0;
-    for (uint32_t i = 0; i < kEachThreads / 32; ++i) term += s_term[i];
+    for (uint32_t i = 0; i < blockDim.x / 32; ++i) term += s_term[i];
     finish_checksum(A, term);
 }
 
@@ -829,14 +892,16 @@ extern "C" huffllm_status huffllm_encode_device(const huffllm_codebook *cb, cons
     if ((e = cudaMemcpyAsync(blob, fixed.data(), fixed.size(), cudaMemcpyHostToDevice, s)) != cudaSuccess) return cuda_fail("copy of the fixed sections");
     encode_scan_kernel<<<(uint32_t)((d.n_chunks + 64 + kScanThreads - 1) / kScanThreads), kScanThreads, 0, s>>>(A);
     write_kernel<<<ctas(kWriteWarps, write_ctas(A.vec_ok)), 32 * kWriteWarps, smem, s>>>(A);
+    const uint32_t each = each_threads(d.n_chunks);
     if (checksum_each(d.n_chunks, chunk_elems))
-        encode_checksum_each_kernel<<<(uint32_t)((d.n_chunks + kEachThreads - 1) / kEachThreads), kEachThreads, 0, s>>>(A);
+        encode_checksum_each_kernel<<<(uint32_t)((d.n_chunks + each - 1) / each), each, 0, s>>>(A);
     else
         encode_checksum_kernel<<<(uint32_t)std::min<uint64_t>((uint64_t)kSumCtas * sms, (d.n_chunks + kSumWarps - 1) / kSumWarps), 32 * kSumWarps, kSumSmem, s>>>(A);
     if ((e = cudaGetLastError()) != cudaSuccess) return cuda_fail("encoder launches");
     EncTotals tot;
     if ((e = cudaMemcpyAsync(&tot, scr, sizeof(tot), cudaMemcpyDeviceToHost, s)) != cudaSuccess || (e = cudaStreamSynchronize(s)) != cudaSuccess)
         return cuda_fail("encoder");
+    if (tot.bad & 4u) return fail(HUFFLLM_ERR_CUDA, "a copy of a record did not arrive");
     if (tot.bad & 1u) return fail(HUFFLLM_ERR_INVALID_ARG, "a weight uses a symbol the codebook has no codeword for");
     if (tot.bad & 2u) return fail(HUFFLLM_ERR_UNSUPPORTED, "payload exceeds the 32-bit record index");
     enc_fill_totals(d, tot);

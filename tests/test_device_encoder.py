@@ -171,6 +171,28 @@ def test_device_encoder_takes_rows_on_any_boundary(hl, dtype, budget, ce, offset
 
 
 @pytest.mark.gpu
+@pytest.mark.parametrize("dtype,kind,rows,cols,ce", [
+    (0, "constant", 16, 512, 512), (0, "gauss", 32, 1000, 512), (0, "gauss", 100, 2048, 1024), (1, "fp16", 48, 1024, 1024),
+    (0, "gauss", 48, 1040, 2048), (1, "fp16", 48, 1040, 2048), (0, "student", 64, 2100, 4096), (1, "fp16_from_bf16", 64, 2100, 4096),
+    (0, "gauss", 33, 4100, 8192), (1, "fp16", 33, 4100, 8192),
+    (0, "gauss", 16, 32 * 15047, 512), (0, "gauss", 16, 32 * 15048 - 3, 512),     # 15047 records: a warp each; 15048: a thread each
+])
+def test_checksums_of_records_of_every_size(hl, dtype, kind, rows, cols, ce):
+    """Records that take one to four steps of every size, ends inside a step, more records than warps; the host encoder's checksum."""
+    import torch
+    w = gen(kind, rows, cols, 31)
+    w_dev = torch.from_numpy(w.view(np.int16)).cuda()
+    cb = hl.build_codebook(w, dtype)
+    cap, n_scr = hl.encode_bound(rows, cols, dtype, ce), hl.encode_device_scratch_bytes(rows, cols, ce)
+    blob_dev = torch.zeros(cap, dtype=torch.uint8, device="cuda")
+    desc = hl.encode_device(cb, w_dev, rows, cols, ce, blob_dev, cap, torch.zeros(n_scr, dtype=torch.uint8, device="cuda"), n_scr)
+    want, desc_host = hl.encode(cb, w, ce)
+    assert desc.payload_checksum == desc_host.payload_checksum
+    assert np.array_equal(blob_dev[:desc.blob_bytes].cpu().numpy(), want)
+    cb.free()
+
+
+@pytest.mark.gpu
 def test_full_size_matrix_on_the_device_equals_the_host_blob(hl):
     """A full-size FFN matrix of the benchmark's layer (45 M weights, 11008 chunks)."""
     import torch
