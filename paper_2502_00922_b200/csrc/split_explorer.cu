@@ -10,8 +10,10 @@
 // cover almost all weights), so a piece's counters are replicated 32 times, one copy per lane: the lanes of a warp never
 // touch the same address or the same bank, whatever the data.  Wider fields get fewer copies; a field whose counters do
 // not fit is counted in several launches, each owning a range of values.
-// (45 M weights, splits 1-8-7 / 1-5-5-5: 40 / 49 us with every field counted on its own, one load in flight per thread and a
-// loop over the fields.)
+// Where the word is cut into two pieces a CTA of 1024 threads has an SM to itself: its counters are cleared, added up and sent to L2 once
+// per SM, its threads have registers for eight loads in flight.  An update takes the atomic unit two cycles, 20 of the 22 us that splits of two pieces take at 45 M weights.
+// (Kernel alone, two CTAs an SM, four loads at a time, shifts as kernel arguments / this, us: 45 M weights 1-8-7 25.6 / 22.2, 1-5-5-5 26.8 / 26.0;
+// 16.8 M 13.9 / 10.7; 235 M 95 / 83, 0.87 of a copy's rate.  At first, every field counted on its own, 40 and 49 us.)
 #include <cuda_runtime.h>
 
 #include <algorithm>
@@ -57,19 +59,27 @@ struct HistArgs {
 __device__ __forceinline__ void red_shared_inc(uint32_t addr) {
     asm volatile("red.shared.add.u32 [%0], 1;" ::"r"(addr) : "memory");
 }
+template <int OFF>
+__device__ __forceinline__ void red_shared_inc(uint32_t addr) {
+    asm volatile("red.shared.add.u32 [%0+%1], 1;" ::"r"(addr), "n"(OFF) : "memory");
+}
 
-// PIECES: 2 = two unranged pieces whose counters are 32-fold (the splits of the two formats), 0 = any
-template <int PIECES>
-__global__ void __launch_bounds__(kHistThreads, 2) split_histogram_kernel(const __grid_constant__ HistArgs A) {
+// LOW: the word is cut into two unranged pieces whose counters are 32-fold, LOW bits and the 16 - LOW above (the splits of the two
+// formats); 0: any pieces
+template <int LOW>
+__global__ void __launch_bounds__(kHistThreads, LOW ? 1 : 2) split_histogram_kernel(const __grid_constant__ HistArgs A) {
     extern __shared__ __align__(16) uint32_t hist[];
     const uint32_t tid = threadIdx.x, lane = tid & 31;
-    for (uint32_t i = tid; i < A.smem_words; i += blockDim.x) hist[i] = 0;
-    __syncthreads();
     const uint32_t base = (uint32_t)__cvta_generic_to_shared(hist);
 
-    // 16-byte vectors of eight weights, dealt to the grid's threads in turn; the last n % 8 weights go to one thread
-    const uint64_t n_vec = A.n / 8, stride = (uint64_t)gridDim.x * blockDim.x;
-    const uint4 *src = (const uint4 *)A.w;
+    // 16-byte vectors of eight weights; the last n % 8 weights go to one thread
+    const uint64_t n_vec = A.n / 8;
+    const uint4 *const src = (const uint4 *)A.w;
+    auto clear = [&]() {
+        for (uint32_t i = tid; i < A.smem_words / 4; i += kHistThreads) ((uint4 *)hist)[i] = make_uint4(0, 0, 0, 0);
+        for (uint32_t i = (A.smem_words & ~3u) + tid; i < A.smem_words; i += kHistThreads) hist[i] = 0;
+        __syncthreads();
+    };
     // n_words words of two weights each (one with `single`): a piece at a time, its plan read once for all of them
     auto count_words = [&](const uint32_t *word, auto n_words, bool single) {
 #pragma unroll 1
@@ -93,42 +103,51 @@ __global__ void __launch_bounds__(kHistThreads, 2) split_histogram_kernel(const 
             }
         }
     };
-    uint32_t off[PIECES ? PIECES : 1], mask[PIECES ? PIECES : 1], sh[PIECES ? PIECES : 1];
-#pragma unroll
-    for (int pi = 0; pi < PIECES; ++pi) {
-        off[pi] = A.p[pi].smem_off << 2;
-        mask[pi] = A.p[pi].mask << 7;
-        sh[pi] = A.p[pi].shift;
-    }
-    const uint32_t lane4 = lane << 2;
-    auto inc = [&](uint32_t table, uint32_t byte_off) { atomicAdd((uint32_t *)((char *)hist + table + byte_off), 1u); };
+    const uint32_t lane_base = base + (lane << 2);
     auto count = [&](const uint4 &q) {
         const uint32_t word[4] = {q.x, q.y, q.z, q.w};
-        if constexpr (PIECES == 0) {
+        if constexpr (LOW == 0) {
             count_words(word, std::integral_constant<int, 4>{}, false);
         } else {
+            // A counter's 32 copies are 128 bytes: a halfword dot product takes the value of either weight times 128 to the lane's
+            // column.  (All shifts and masks are constants, so a weight's two updates cost three and a half instructions besides.)
+            constexpr uint32_t kLow = ((1u << LOW) - 1u) * 0x10001u, kHigh = ((1u << (16 - LOW)) - 1u) * 0x10001u;
 #pragma unroll
             for (int i = 0; i < 4; ++i) {
-                // a counter's 32 copies are 128 bytes: the value, moved to bit 7, is its byte offset.  (The upper weight's
-                // value is moved down by at least 9, 16 + shift - 7; the lower one's up or down: as a 64-bit shift, one instruction.)
-#pragma unroll
-                for (int pi = 0; pi < PIECES; ++pi) {
-                    inc(off[pi], ((uint32_t)(((uint64_t)word[i] << 7) >> sh[pi]) & mask[pi]) | lane4);
-                    inc(off[pi], ((word[i] >> (sh[pi] + 9u)) & mask[pi]) | lane4);
-                }
+                const uint32_t h = word[i] >> LOW & kHigh, l = word[i] & kLow;
+                red_shared_inc<0>(__dp2a_lo(h, 0x0080u, lane_base));
+                red_shared_inc<0>(__dp2a_lo(h, 0x8000u, lane_base));
+                red_shared_inc<128 << (16 - LOW)>(__dp2a_lo(l, 0x0080u, lane_base));
+                red_shared_inc<128 << (16 - LOW)>(__dp2a_lo(l, 0x8000u, lane_base));
             }
         }
     };
-    uint64_t v = (uint64_t)blockIdx.x * blockDim.x + tid;
-    if constexpr (PIECES != 0)
-        for (; v + 3 * stride < n_vec; v += 4 * stride) {      // four loads in flight per thread
-            uint4 q[4];
+    if constexpr (LOW == 0) {                                // dealt to the grid's threads in turn
+        clear();
+        const uint64_t stride = (uint64_t)gridDim.x * blockDim.x;
+        for (uint64_t v = (uint64_t)blockIdx.x * blockDim.x + tid; v < n_vec; v += stride) count(__ldg(src + v));
+    } else {
+        // A CTA takes a contiguous piece.  Eight loads are in flight per thread throughout, the first ones while the counters are cleared: a
+        // vector's registers are loaded anew as soon as it has been counted.
+        constexpr int kAhead = 8;
+        const uint64_t first = n_vec * blockIdx.x / gridDim.x;
+        int32_t left = (int32_t)(n_vec * (blockIdx.x + 1) / gridDim.x - first) - (int32_t)tid;    // (fewer than 2^35 / 148 vectors a CTA)
+        const uint4 *at = src + first + tid;
+        uint4 q[kAhead];
 #pragma unroll
-            for (int i = 0; i < 4; ++i) q[i] = __ldg(src + v + i * stride);
+        for (int i = 0; i < kAhead; ++i)
+            if (left > i * (int)kHistThreads) q[i] = __ldg(at + i * kHistThreads);
+        clear();
+#pragma unroll 1
+        for (; left > 0; left -= kAhead * (int)kHistThreads) {
+            at += kAhead * kHistThreads;
 #pragma unroll
-            for (int i = 0; i < 4; ++i) count(q[i]);
+            for (int i = 0; i < kAhead; ++i) {
+                if (left > i * (int)kHistThreads) count(q[i]);
+                if (left > (kAhead + i) * (int)kHistThreads) q[i] = __ldg(at + i * kHistThreads);
+            }
         }
-    for (; v < n_vec; v += stride) count(__ldg(src + v));
+    }
     if (blockIdx.x == 0 && tid == 0)
         for (uint64_t i = n_vec * 8; i < A.n; ++i) {
             const uint32_t word = A.w[i];
@@ -182,6 +201,18 @@ __global__ void __launch_bounds__(kHistThreads, 2) split_histogram_kernel(const 
     }
 }
 
+// The kernel of a word cut into two pieces above its `low` lower bits (pieces have ten bits at most).
+static void (*two_pieces(uint32_t low))(HistArgs) {
+    switch (low) {
+        case 6: return split_histogram_kernel<6>;
+        case 7: return split_histogram_kernel<7>;
+        case 8: return split_histogram_kernel<8>;
+        case 9: return split_histogram_kernel<9>;
+        case 10: return split_histogram_kernel<10>;
+        default: return split_histogram_kernel<0>;
+    }
+}
+
 static huffllm_status check_widths(const uint8_t *widths, uint32_t n_fields, size_t *total_bins) {
     if (!widths || n_fields == 0 || n_fields > HUFFLLM_MAX_FIELDS) return fail(HUFFLLM_ERR_INVALID_ARG, "a split has 1..%d fields", HUFFLLM_MAX_FIELDS);
     uint32_t sum = 0;
@@ -216,9 +247,7 @@ extern "C" huffllm_status huffllm_split_histogram(const uint16_t *w_dev, uint64_
     if (((uintptr_t)w_dev & 15u) || ((uintptr_t)counts_dev & 7u)) return fail(HUFFLLM_ERR_INVALID_ARG, "weights must be 16-byte aligned, counters 8-byte aligned");
     if (n_weights >> 38) return fail(HUFFLLM_ERR_UNSUPPORTED, "more than 2^38 weights in one call");   // a CTA's 32-bit counters cannot overflow below that
     cudaStream_t s = (cudaStream_t)stream;
-    cudaError_t e = cudaMemsetAsync(counts_dev, 0, bins * sizeof(uint64_t), s);
-    if (e != cudaSuccess) return fail(HUFFLLM_ERR_CUDA, "cudaMemsetAsync: %s", cudaGetErrorString(e));
-    if (n_weights == 0) return HUFFLLM_OK;
+    cudaError_t e;
     int dev = 0, sms = 0;
     if ((e = cudaGetDevice(&dev)) != cudaSuccess || (e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev)) != cudaSuccess)
         return fail(HUFFLLM_ERR_CUDA, "device query: %s", cudaGetErrorString(e));
@@ -257,10 +286,17 @@ extern "C" huffllm_status huffllm_split_histogram(const uint16_t *w_dev, uint64_
         }
         hi -= bits;
     }
-    // launches: pieces in order, as many as fit the shared-memory budget
+    // launches: pieces in order, as many as fit the shared-memory budget.  All of them are planned before the first call that the GPU
+    // sees: planned behind the clearing of the counters, the counting waited for the host.
+    struct Launch {
+        void (*kernel)(HistArgs);
+        HistArgs args;
+    };
+    std::vector<Launch> launches;
     size_t p = 0;
-    while (p < pieces.size()) {
-        HistArgs A = {};
+    while (n_weights && p < pieces.size()) {
+        launches.push_back({});
+        HistArgs &A = launches.back().args;
         A.w = w_dev;
         A.n = n_weights;
         A.counts = (unsigned long long *)counts_dev;
@@ -278,14 +314,16 @@ extern "C" huffllm_status huffllm_split_histogram(const uint16_t *w_dev, uint64_
             ++p;
         }
         A.smem_words = words;
-        const size_t smem = (size_t)words * 4u;
-        const auto kernel = plain && A.n_pieces == 2 ? split_histogram_kernel<2> : split_histogram_kernel<0>;
-        if ((e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)(kHistBudgetWords * 4u))) != cudaSuccess)
+        launches.back().kernel = plain && A.n_pieces == 2 ? two_pieces(A.p[0].shift) : split_histogram_kernel<0>;
+        if ((e = cudaFuncSetAttribute(launches.back().kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)(kHistBudgetWords * 4u))) != cudaSuccess)
             return fail(HUFFLLM_ERR_CUDA, "cudaFuncSetAttribute: %s", cudaGetErrorString(e));
-        const uint64_t n_vec = n_weights / 8;
-        uint32_t grid = (uint32_t)sms * (smem <= 100u * 1024u ? 2u : 1u);
-        grid = (uint32_t)std::max<uint64_t>(1, std::min<uint64_t>(grid, (n_vec + kHistThreads - 1) / kHistThreads));
-        kernel<<<grid, kHistThreads, smem, s>>>(A);
+    }
+    if ((e = cudaMemsetAsync(counts_dev, 0, bins * sizeof(uint64_t), s)) != cudaSuccess) return fail(HUFFLLM_ERR_CUDA, "cudaMemsetAsync: %s", cudaGetErrorString(e));
+    for (const Launch &l : launches) {
+        const size_t smem = (size_t)l.args.smem_words * 4u;
+        const uint32_t per_sm = l.kernel == split_histogram_kernel<0> && smem <= 100u * 1024u ? 2u : 1u;
+        const uint32_t grid = (uint32_t)std::max<uint64_t>(1, std::min<uint64_t>((uint64_t)sms * per_sm, (n_weights / 8 + kHistThreads - 1) / kHistThreads));
+        l.kernel<<<grid, kHistThreads, smem, s>>>(l.args);
         if ((e = cudaGetLastError()) != cudaSuccess) return fail(HUFFLLM_ERR_CUDA, "split_histogram_kernel: %s", cudaGetErrorString(e));
     }
     return HUFFLLM_OK;

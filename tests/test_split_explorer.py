@@ -109,6 +109,19 @@ def test_device_counters_of_fields_counted_together(hl, widths):
 
 
 @pytest.mark.gpu
+@pytest.mark.parametrize("widths,sizes", [
+    ([8, 8], [8 * 1023 + 5, 8 * 1024, 8 * 1025 + 7, 8 * 1024 * 149, 8 * 1024 * 148 * 8 + 8, 8 * 1024 * 148 * 9 + 9]),   # round a CTA's loads ahead
+    ([10, 6], [(1 << 24) + 3]), ([9, 7], [(1 << 24) + 8 * 1024 + 5]), ([7, 9], [(1 << 24) + 8]), ([6, 10], [(1 << 24) + 7]),
+])
+def test_device_counters_of_words_cut_in_two(hl, widths, sizes):
+    """Every cut into two pieces, every pattern met, vectors that do not divide among the CTAs and their threads."""
+    import torch
+    w = np.random.default_rng(8).integers(0, 1 << 16, max(sizes), dtype=np.uint16)
+    for n in sizes:
+        assert np.array_equal(device_counts(hl, torch, w[:n], widths), np.concatenate(orc.split_histograms(w[:n], widths)))
+
+
+@pytest.mark.gpu
 def test_full_size_matrix_reproduces_the_tables_rows(hl):
     """A full-size FFN matrix of the benchmark's layer, every split of the entropy table, counters exact."""
     import torch
