@@ -4,7 +4,7 @@
 //
 // A warp takes a chunk, its lanes the format's lanes: two bit sequences each (rows g and g + 8), one after the other in the loops
 // below, so that a lane has two chains under way and what a chunk costs besides its weights is paid once per 128 of a lane's.
-//   pass 1  code lengths only -> words per sequence of every chunk; words and coded bits of every 1024 chunks
+//   pass 1  code lengths only -> words per sequence and coded bits of every chunk; a CTA of its own writes code lengths and table
 //   scan    record offsets (the index section), payload size, largest record
 //   pass 2  raw part and coded part of every record (nothing if the scan found the tensor or the buffer unfit)
 //   pass 3  the checksum term of every record, a warp each (many short records: a thread); the last one completes the header
@@ -15,7 +15,6 @@
 #include <atomic>
 #include <cstring>
 #include <type_traits>
-#include <vector>
 
 #include "decode_common.cuh"
 #include "internal.h"
@@ -28,12 +27,14 @@ struct EncTotals {
     uint32_t summed;             // CTAs whose records' checksums are in
 };
 
-static_assert(sizeof(EncTotals) <= 64, "the sums of pass 1 follow in the scratch");
+static_assert(sizeof(EncTotals) <= 256, "the chunks' bits and words follow in the scratch");
 
 constexpr uint32_t kScanThreads = 1024;      // chunks of a scan CTA
 constexpr uint32_t kWriteWarps = 4;          // of a CTA of pass 2
 __host__ __device__ constexpr uint32_t write_ctas(bool vec) { return vec ? 6 : 5; }     // of an SM (80 and 96 registers)
 constexpr uint32_t kNoCode = 1u << 14;       // length of a symbol without codeword: no sum of a sequence's codewords reaches it (768 of 12 bits)
+
+constexpr uint32_t kUnfit = 0xFFFFFFFFu;
 
 struct EncArgs {
     const uint16_t *w;
@@ -41,11 +42,12 @@ struct EncArgs {
     uint32_t Kc, KC, fp16, lag_bits, pad, vec_ok;
     uint32_t stage_rows;         // rows of a record that a warp of pass 2 has room for in shared memory
     uint64_t max_units;          // what the blob has room for
-    unsigned long long *groups;  // per kScanThreads chunks: their words | their coded bits << 32
-    uint32_t *words, *index;
+    uint32_t *bits, *words;      // per chunk: coded bits, words per sequence (kUnfit: a symbol without codeword)
+    uint32_t *index;
     uint8_t *blob, *payload;
     EncTotals *totals;
     uint32_t code[256];          // a symbol's codeword, first bit in bit 31 | its length (FP16: three fields of 32 symbols)
+    uint8_t lengths[256];        // the section of code lengths
     huffllm_desc desc;           // the header, but for what the totals say
 };
 
@@ -175,8 +177,28 @@ constexpr uint32_t kPairEntries = 1024;
 // of 512 79 / 50.)
 constexpr uint32_t kSizeWarps = 8;           // of a CTA of pass 1
 __host__ __device__ constexpr uint32_t size_ctas(bool vec) { return vec ? 3 : 4; }      // of an SM (80 and 64 registers)
+// Code lengths and decode table of the blob, as the host writes them; the header's bytes are zero until the last kernel completes it.
+__device__ __forceinline__ void enc_fixed_sections(const EncArgs &A) {
+    const uint32_t lane = threadIdx.x & 31, warp = threadIdx.x >> 5, warps = blockDim.x >> 5;
+    for (uint32_t i = threadIdx.x; i < (uint32_t)A.desc.off_index / 16; i += blockDim.x) ((uint4 *)A.blob)[i] = make_uint4(0, 0, 0, 0);
+    __syncthreads();
+    for (uint32_t i = threadIdx.x; i < 256; i += blockDim.x)
+        if (A.lengths[i]) A.blob[A.desc.off_codebook + i] = A.lengths[i];
+    for (uint32_t i = warp; i < (A.fp16 ? 96u : 256u); i += warps) {
+        const uint32_t e = A.code[i], len = e & 31u, field = A.fp16 ? i >> 5 : 0u;
+        if (!len) continue;
+        uint32_t *const table = (uint32_t *)(A.blob + A.desc.off_lut) + ((size_t)field << A.desc.lut_bits);
+        const uint32_t value = len << 16 | (A.fp16 ? (i & 31u) << (10 - 5 * field) : i << 7), seq = __brev(e & ~31u);
+        for (uint32_t hi = lane; hi < 1u << (A.desc.lut_bits - len); hi += 32) table[seq | hi << len] = value;
+    }
+}
 template <bool FP16, bool VEC>
 __global__ void __launch_bounds__(32 * kSizeWarps, size_ctas(VEC)) encode_size_kernel(const __grid_constant__ EncArgs A) {
+    pdl_launch_dependents();
+    if (blockIdx.x == gridDim.x - 1) {                       // (the CTA behind those of the chunks)
+        enc_fixed_sections(A);
+        return;
+    }
     __shared__ __align__(4) typename std::conditional<FP16, uint16_t, uint32_t>::type s_len[FP16 ? kPairEntries + 32 : 256];
     const uint32_t lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     auto length = [&](uint32_t i) -> uint32_t { return A.code[i] ? A.code[i] & 31u : kNoCode; };
@@ -206,66 +228,115 @@ __global__ void __launch_bounds__(32 * kSizeWarps, size_ctas(VEC)) encode_size_k
         return bits;
     };
 #pragma unroll 1
-    for (uint32_t c = blockIdx.x * kSizeWarps + warp; c < A.n_chunks; c += gridDim.x * kSizeWarps) {
+    for (uint32_t c = blockIdx.x * kSizeWarps + warp; c < A.n_chunks; c += (gridDim.x - 1) * kSizeWarps) {
         const EncLane L = enc_lane(A, c, lane);
         uint32_t ba = 0, bb = 0;
         enc_blocks<VEC, VEC ? 4 : 1>(A, L, [&](const uint4 &va, const uint4 &vb) {
             ba += bits_of(va);
             bb += bits_of(vb);
         });
-        if (ba >= kNoCode || bb >= kNoCode) {
-            atomicOr(&A.totals->bad, 1u);
-            ba = bb = 0;
-        }
-        const uint32_t most = __reduce_max_sync(0xFFFFFFFFu, max(ba, bb) + A.lag_bits), sum = __reduce_add_sync(0xFFFFFFFFu, ba + bb);
+        const uint32_t most = __reduce_max_sync(0xFFFFFFFFu, max(ba, bb)), sum = __reduce_add_sync(0xFFFFFFFFu, ba + bb);
         if (lane == 0) {
-            const uint32_t W = max(1u, (most + 31) / 32);
-            A.words[c] = W;
-            atomicAdd(A.groups + c / kScanThreads, (unsigned long long)sum << 32 | W);   // (1024 chunks: fewer than 2^19 words and 2^30 bits)
+            A.words[c] = most >= kNoCode ? kUnfit : max(1u, (most + A.lag_bits + 31) / 32);
+            A.bits[c] = sum;
         }
     }
 }
 
-// Record offsets: an exclusive prefix sum of the record sizes (in 128-byte units).  A CTA takes 1024 chunks and sums what pass 1
-// has left of every 1024 chunks in front of them itself (the raw parts in front are known without a sum), so that no CTA waits
-// for another; a single CTA walking all chunks took 20 us for the 11008 chunks of an 11008 x 4096 tensor, most of it barriers.
-// (At 11008 / 88064 / 1.05 M chunks: one CTA 20 / 142 / 1677 us; every chunk in front read by every CTA, which grows with the square
-// of the chunks, 6.8 / 13 / 130; this 5.7 / 6.7 / 31.)
+// Record offsets: an exclusive prefix sum of the record sizes (in 128-byte units).  A CTA takes 1024 chunks and sums up the words of all
+// chunks in front of them itself (the raw parts in front are known without a sum), so that no CTA waits for another; the one at the end of the
+// index, which sees them all, leaves the totals: nothing has to be cleared or added up by atomics in front of this.  Sums over every
+// chunk in front grow with the square of the chunks: from kGroupsFrom on a launch of its own leaves those of 1024 chunks each (GROUPS),
+// where the chunks' bits were.
+// (Time behind pass 1 at 11008 / 88064 / 234 000 / 1.05 M chunks, us: 3.9 / 5.4 / 9.9 / 19.5; pass 1 adding up every 1024 by atomics, behind a launch that
+// clears them, 6.3 / 7 / 16 / 30, and 50 us of pass 1 instead of 28 at 88064; without groups 4.2 / 11 / 77 / 224.  The last warp of pass 1 to
+// come from every 1024 chunks doing this, for which it has to order its words before the others' counts: 17.3 -> 38 us for that pass.)
+constexpr uint64_t kGroupsFrom = 49152;
+struct EncGroup {
+    unsigned long long words, bits;
+    uint32_t most;
+};
+__device__ __forceinline__ EncGroup *enc_group(const EncArgs &A, uint32_t g) { return (EncGroup *)(A.bits + (size_t)g * kScanThreads); }
+__device__ __forceinline__ unsigned long long warp_sum(unsigned long long v) {
+#pragma unroll
+    for (int o = 16; o; o >>= 1) v += __shfl_xor_sync(0xFFFFFFFFu, v, o);
+    return v;
+}
+__global__ void __launch_bounds__(kScanThreads) encode_groups_kernel(const __grid_constant__ EncArgs A) {
+    __shared__ EncGroup s_warp[32];
+    pdl_launch_dependents();
+    pdl_wait_prior_grid();
+    const uint32_t lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    const uint64_t c = (uint64_t)blockIdx.x * kScanThreads + threadIdx.x;
+    const uint32_t W = c < A.n_chunks ? __ldcg(A.words + c) : 0u, bits = c < A.n_chunks ? __ldcg(A.bits + c) : 0u;
+    const EncGroup sums = {warp_sum(W), warp_sum(bits), __reduce_max_sync(0xFFFFFFFFu, W)};
+    if (lane == 0) s_warp[warp] = sums;
+    __syncthreads();                                         // (all of the group's bits have been read)
+    if (warp) return;
+    const EncGroup all = {warp_sum(s_warp[lane].words), warp_sum(s_warp[lane].bits), __reduce_max_sync(0xFFFFFFFFu, s_warp[lane].most)};
+    if (lane == 0) *enc_group(A, blockIdx.x) = all;
+}
+template <bool GROUPS>
 __global__ void __launch_bounds__(kScanThreads) encode_scan_kernel(const __grid_constant__ EncArgs A) {
-    __shared__ unsigned long long s_warp[32], s_front[32];
-    const uint32_t tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-    const uint64_t c = (uint64_t)blockIdx.x * kScanThreads + tid;
-    const uint32_t raw_full = enc_raw_bytes(A, enc_blocks_of(A, 0)) / kRecordUnit, raw_last = enc_raw_bytes(A, enc_blocks_of(A, A.KC - 1)) / kRecordUnit;
-    unsigned long long front = 0;                           // words of the chunks in front of the CTA's
-    for (uint32_t i = tid; i < blockIdx.x; i += kScanThreads) front += (uint32_t)__ldcg(A.groups + i);
+    __shared__ unsigned long long s_front[32], s_bits[32];
+    __shared__ uint32_t s_words[32], s_most[32];
+    pdl_wait_prior_grid();
+    const uint32_t tid = threadIdx.x, lane = tid & 31, warp = tid >> 5, begin = blockIdx.x * kScanThreads;
+    const uint64_t c = (uint64_t)begin + tid;
+    const uint32_t last = (uint32_t)(A.n_chunks / kScanThreads);             // the CTA at the end of the index
+    unsigned long long front = 0, bits = 0;                  // words of the chunks in front of the CTA's; in the last one all chunks' bits and
+    uint32_t most = 0;                                       // the most words
     const uint32_t W = c < A.n_chunks ? __ldcg(A.words + c) : 0u;
-    unsigned long long incl = W;
-    uint32_t maxw = W;
+    if (GROUPS && blockIdx.x <= last) {
+        for (uint32_t g = tid; g < blockIdx.x; g += kScanThreads) front += __ldcg(&enc_group(A, g)->words);
+        if (blockIdx.x == last)
+            for (uint32_t g = tid; (uint64_t)g * kScanThreads < A.n_chunks; g += kScanThreads) {
+                bits += __ldcg(&enc_group(A, g)->bits);
+                most = max(most, __ldcg(&enc_group(A, g)->most));
+            }
+    } else if (blockIdx.x == last) {
+        if (c < A.n_chunks) bits = __ldcg(A.bits + c);
+        most = W;
+#pragma unroll 4
+        for (uint32_t i = tid; i < begin; i += kScanThreads) {
+            const uint32_t w = __ldcg(A.words + i);
+            front += w;
+            bits += __ldcg(A.bits + i);
+            most = max(most, w);
+        }
+    } else if (blockIdx.x < last) {
+#pragma unroll 8
+        for (uint32_t i = tid; i < begin; i += kScanThreads) front += __ldcg(A.words + i);
+    }
+    uint32_t incl = W;                                      // (1024 chunks: fewer than 2^19 words)
 #pragma unroll
     for (int o = 1; o < 32; o <<= 1) {
-        const unsigned long long n = __shfl_up_sync(0xFFFFFFFFu, incl, o);
+        const uint32_t n = __shfl_up_sync(0xFFFFFFFFu, incl, o);
         if (lane >= (uint32_t)o) incl += n;
     }
-#pragma unroll
-    for (int o = 16; o; o >>= 1) {
-        front += __shfl_xor_sync(0xFFFFFFFFu, front, o);
-        maxw = max(maxw, __shfl_xor_sync(0xFFFFFFFFu, maxw, o));
+    front = warp_sum(front);
+    if (blockIdx.x == last) {
+        bits = warp_sum(bits);
+        most = __reduce_max_sync(0xFFFFFFFFu, most);
     }
-    if (lane == 31) s_warp[warp] = incl;
-    if (lane == 0) {
+    if (lane == 31) {
+        s_words[warp] = incl;
         s_front[warp] = front;
-        if (tid == 0 && c < A.n_chunks) atomicAdd(&A.totals->coded_bits, __ldcg(A.groups + blockIdx.x) >> 32);
-        if (maxw) atomicMax(&A.totals->max_words, maxw);
+        s_bits[warp] = bits;
+        s_most[warp] = most;
     }
     __syncthreads();
-    unsigned long long before = incl - W;
-    for (uint32_t i = 0; i < 32; ++i) before += s_front[i] + (i < warp ? s_warp[i] : 0ull);
+    const unsigned long long before = warp_sum(s_front[lane] + (lane < warp ? s_words[lane] : 0u)) + (incl - W);
+    if (blockIdx.x == last) {
+        bits = warp_sum(s_bits[lane]);
+        most = __reduce_max_sync(0xFFFFFFFFu, s_most[lane]);
+    }
     if (c <= A.n_chunks) {                                  // (one entry more than chunks: the payload's end)
-        const uint64_t row = c / A.KC, kc = c - row * A.KC; // raw parts in front: whole rows of chunks, then full chunks of this one
-        const unsigned long long at = row * ((uint64_t)(A.KC - 1) * raw_full + raw_last) + kc * raw_full + 2ull * before;
+        const uint32_t raw_full = enc_raw_bytes(A, enc_blocks_of(A, 0)) / kRecordUnit, raw_last = enc_raw_bytes(A, enc_blocks_of(A, A.KC - 1)) / kRecordUnit;
+        const uint32_t row = (uint32_t)c / A.KC, kc = (uint32_t)c - row * A.KC;        // raw parts in front: whole rows of chunks, then full chunks of this one
+        const unsigned long long at = row * ((uint64_t)(A.KC - 1) * raw_full + raw_last) + (uint64_t)kc * raw_full + 2ull * before;
         A.index[c] = (uint32_t)at;
-        if (at > 0xFFFFFFFFull) atomicOr(&A.totals->bad, 2u);
-        if (c == A.n_chunks) A.totals->payload_units = at;
+        if (c == A.n_chunks) *A.totals = {at, bits, 0ull, most, (most == kUnfit ? 1u : 0u) | (at > 0xFFFFFFFFull ? 2u : 0u), 0u};
     } else if (c < ((A.n_chunks + 64) & ~63ull)) {
         A.index[c] = 0;                                     // the section's padding to 256 bytes
     }
@@ -732,6 +803,13 @@ __global__ void __launch_bounds__(32 * kSumWarps, kSumCtas) encode_checksum_kern
     finish_checksum(A, term);
 }
 
+static uint32_t reverse_word(uint32_t v) {
+    v = (v >> 1 & 0x55555555u) | (v & 0x55555555u) << 1;
+    v = (v >> 2 & 0x33333333u) | (v & 0x33333333u) << 2;
+    v = (v >> 4 & 0x0F0F0F0Fu) | (v & 0x0F0F0F0Fu) << 4;
+    return v << 24 | (v & 0xFF00u) << 8 | (v >> 8 & 0xFF00u) | v >> 24;
+}
+
 // The device's SMs, whose number the checksum's CTAs go by, and the kernel's shared memory allowed, once per device.
 static cudaError_t prepare_checksum(int *sms) {
     static std::atomic<int> known[64];               // set twice by racing threads at worst: to the same value
@@ -853,20 +931,18 @@ extern "C" huffllm_status huffllm_encode_device(const huffllm_codebook *cb, cons
     A.vec_ok = (cols % 8 == 0 && ((uintptr_t)w_dev & 15u) == 0) ? 1u : 0u;
     A.max_units = blob_cap >= d.off_payload + kTailSlack ? (blob_cap - d.off_payload - kTailSlack) / kRecordUnit : 0;
     A.totals = (EncTotals *)scr;
-    A.groups = (unsigned long long *)(scr + 64);               // (8 bytes per 1024 chunks: fewer than the 192 + 4 n in front of the words)
-    A.words = (uint32_t *)(scr + 256 + 4 * d.n_chunks);
-    const size_t cleared = 64 + 8 * ((d.n_chunks + kScanThreads - 1) / kScanThreads);
+    A.bits = (uint32_t *)(scr + 256);
+    A.words = A.bits + d.n_chunks;
     A.index = (uint32_t *)(blob + d.off_index);
     A.blob = blob;
     A.payload = blob + d.off_payload;
     A.desc = d;
+    code_length_section(cb, A.lengths);
     uint8_t len[256];
     uint32_t bits[256], longest = 1;
     encoder_tables(cb, len, bits);
     for (int i = 0; i < 256; ++i) {
-        uint32_t first = 0;                                      // the first bit in bit 31
-        for (uint32_t b = 0; b < len[i]; ++b) first |= (bits[i] >> b & 1u) << (31 - b);
-        A.code[i] = first | len[i];
+        A.code[i] = reverse_word(bits[i]) | len[i];
         longest = std::max<uint32_t>(longest, len[i]);
     }
     const uint32_t steps = Kc / kBlockCols * 8 * (A.fp16 ? 3 : 1), most_words = (d.lag_bits + steps * longest + 31) / 32;
@@ -880,24 +956,33 @@ extern "C" huffllm_status huffllm_encode_device(const huffllm_codebook *cb, cons
     const uint32_t smem = kWriteWarps * A.stage_rows * 256;
     int sms = 0;
     if ((e = prepare_checksum(&sms)) != cudaSuccess) return cuda_fail("device attributes");
-    std::vector<uint8_t> fixed;
-    fixed.reserve((size_t)d.off_index);                          // (what can fail without a launch does so before the first one)
-    if ((e = cudaMemsetAsync(scr, 0, cleared, s)) != cudaSuccess) return cuda_fail("cudaMemsetAsync");
+    // (What the GPU is given comes last and without a pause: it waits for the host otherwise.  The small kernels behind pass 1 start while it
+    // ends.  Not the passes behind them, whose CTAs go where there is room first and then share what they find there unevenly: 11008 x 4096
+    // both passes 3 us later, chunks of 2048 with a thread per record 36.)
     auto ctas = [&](uint32_t warps, uint32_t per_sm) { return (uint32_t)std::min<uint64_t>((d.n_chunks + warps - 1) / warps, (uint64_t)per_sm * sms); };
-    size_kernel<<<ctas(kSizeWarps, size_ctas(A.vec_ok)), 32 * kSizeWarps, 0, s>>>(A);
-    // code lengths and table, assembled on the host while pass 1 runs; the header's bytes stay zero until the last kernel writes them
-    fixed.assign((size_t)d.off_index, 0);
-    write_fixed_sections(cb, d, fixed.data());
-    memset(fixed.data(), 0, sizeof(d));
-    if ((e = cudaMemcpyAsync(blob, fixed.data(), fixed.size(), cudaMemcpyHostToDevice, s)) != cudaSuccess) return cuda_fail("copy of the fixed sections");
-    encode_scan_kernel<<<(uint32_t)((d.n_chunks + 64 + kScanThreads - 1) / kScanThreads), kScanThreads, 0, s>>>(A);
-    write_kernel<<<ctas(kWriteWarps, write_ctas(A.vec_ok)), 32 * kWriteWarps, smem, s>>>(A);
+    auto launch = [&](void (*kernel)(EncArgs), uint32_t grid, uint32_t threads, uint32_t shared, bool early) {
+        cudaLaunchConfig_t cfg = {};
+        cfg.gridDim = dim3(grid);
+        cfg.blockDim = dim3(threads);
+        cfg.dynamicSmemBytes = shared;
+        cfg.stream = s;
+        cudaLaunchAttribute attr[1];
+        attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+        attr[0].val.programmaticStreamSerializationAllowed = 1;
+        cfg.attrs = attr;
+        cfg.numAttrs = early ? 1 : 0;
+        return cudaLaunchKernelEx(&cfg, kernel, A);
+    };
+    const bool groups = d.n_chunks >= kGroupsFrom;
+    const bool a_thread_each = checksum_each(d.n_chunks, chunk_elems);
     const uint32_t each = each_threads(d.n_chunks);
-    if (checksum_each(d.n_chunks, chunk_elems))
-        encode_checksum_each_kernel<<<(uint32_t)((d.n_chunks + each - 1) / each), each, 0, s>>>(A);
-    else
-        encode_checksum_kernel<<<(uint32_t)std::min<uint64_t>((uint64_t)kSumCtas * sms, (d.n_chunks + kSumWarps - 1) / kSumWarps), 32 * kSumWarps, kSumSmem, s>>>(A);
-    if ((e = cudaGetLastError()) != cudaSuccess) return cuda_fail("encoder launches");
+    if ((e = launch(size_kernel, std::min(ctas(kSizeWarps, size_ctas(A.vec_ok)) + 1, size_ctas(A.vec_ok) * (uint32_t)sms), 32 * kSizeWarps, 0, false)) != cudaSuccess ||
+        (groups && (e = launch(encode_groups_kernel, (uint32_t)((d.n_chunks + kScanThreads - 1) / kScanThreads), kScanThreads, 0, true)) != cudaSuccess) ||
+        (e = launch(groups ? encode_scan_kernel<true> : encode_scan_kernel<false>, (uint32_t)((d.n_chunks + 64 + kScanThreads - 1) / kScanThreads), kScanThreads, 0, true)) != cudaSuccess ||
+        (e = launch(write_kernel, ctas(kWriteWarps, write_ctas(A.vec_ok)), 32 * kWriteWarps, smem, false)) != cudaSuccess ||
+        (e = a_thread_each ? launch(encode_checksum_each_kernel, (uint32_t)((d.n_chunks + each - 1) / each), each, 0, false)
+                           : launch(encode_checksum_kernel, ctas(kSumWarps, kSumCtas), 32 * kSumWarps, kSumSmem, false)) != cudaSuccess)
+        return cuda_fail("encoder launches");
     EncTotals tot;
     if ((e = cudaMemcpyAsync(&tot, scr, sizeof(tot), cudaMemcpyDeviceToHost, s)) != cudaSuccess || (e = cudaStreamSynchronize(s)) != cudaSuccess)
         return cuda_fail("encoder");

@@ -498,14 +498,20 @@ void fill_desc_fixed(const huffllm_codebook *cb, uint64_t rows, uint64_t cols, u
     *out = d;
 }
 
+// The section of code lengths, zeros behind the 96 bytes of codes by field included.
+void code_length_section(const huffllm_codebook *cb, uint8_t out[256]) {
+    memset(out, 0, 256);
+    if (cb->n_fields >= 2) {
+        for (int k = 0; k < 3; ++k) memcpy(out + 32 * k, cb->len[k], 32);
+    } else {
+        memcpy(out, cb->len_e, 256);
+    }
+}
+
 // Header, code lengths and decode table: bytes [0, off_index) of the blob (the caller has zeroed them).
 void write_fixed_sections(const huffllm_codebook *cb, const huffllm_desc &d, uint8_t *base) {
     memcpy(base, &d, sizeof(d));
-    if (cb->n_fields >= 2) {
-        for (int k = 0; k < 3; ++k) memcpy(base + d.off_codebook + 32 * k, cb->len[k], 32);
-    } else {
-        memcpy(base + d.off_codebook, cb->len_e, 256);
-    }
+    code_length_section(cb, base + d.off_codebook);
     memcpy(base + d.off_lut, cb->lut.data(), cb->lut.size() * sizeof(uint32_t));
 }
 

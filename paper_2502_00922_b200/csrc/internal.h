@@ -46,6 +46,7 @@ constexpr uint32_t kRawSignByte[4] = {1, 3, 2, 0};
 // Pieces of the host encoder that the device encoder shares (defined with the codebook, in the host codec).
 void fill_desc_fixed(const huffllm_codebook *cb, uint64_t rows, uint64_t cols, uint32_t chunk_elems, uint32_t Kc, uint32_t RG,
                      uint32_t KC, huffllm_desc *out);
+void code_length_section(const huffllm_codebook *cb, uint8_t out[256]);
 void write_fixed_sections(const huffllm_codebook *cb, const huffllm_desc &d, uint8_t *base);
 void encoder_tables(const huffllm_codebook *cb, uint8_t len[256], uint32_t bits[256]);
 uint32_t codebook_dtype(const huffllm_codebook *cb);

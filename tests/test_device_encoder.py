@@ -117,6 +117,8 @@ def test_device_encoder_writes_the_host_encoders_blob(hl, rows, cols, ce, kind, 
     (1040, 1024, 512, "fp16", 1, 7, 0),              # 2080 chunks, records of an odd number of 128-byte units
     (33, 32 * 20011 - 5, 512, "gauss", 0, 0, 0),     # 60033 chunks: a scan CTA has 58 sums in front of it
     (16, 32 * 20483, 512, "fp16", 1, 12, 2),         # 20483 chunks: a thread per record in the checksum pass
+    (48, 32 * 16384 - 9, 512, "gauss", 0, 0, 0),     # 49152 chunks: offsets from sums of 1024 chunks each; the last CTA has none
+    (16, 32 * 49151, 512, "constant", 0, 0, 0),      # one fewer: from the chunks themselves
 ])
 def test_device_encoder_at_the_edges_of_its_passes(hl, rows, cols, ce, kind, dtype, budget, offset):
     """Loads that are not aligned, sequences that fill their rows, the scan's and the checksum's borders: host blob, byte for byte."""
@@ -262,5 +264,14 @@ def test_device_encoder_errors(hl):
     with pytest.raises(hl.HuffllmError) as e:
         hl.encode_device(cb, other, 32, 256, 512, blob, cap, scr, n_scr)
     assert e.value.status_name == "INVALID_ARG"
+    # the same in one weight among so many chunks that their sums take a launch of their own
+    many = torch.from_numpy(np.tile(w, (6, 1)).reshape(-1)[:48 * 1024].view(np.int16)).cuda().repeat(512).reshape(48, 32 * 16384)
+    many[20, 77777] = 0x7F00
+    cap2, scr2 = hl.encode_bound(48, 32 * 16384, 0, 512), hl.encode_device_scratch_bytes(48, 32 * 16384, 512)
+    blob2 = torch.full((cap2,), 0xA5, dtype=torch.uint8, device="cuda")
+    with pytest.raises(hl.HuffllmError) as e:
+        hl.encode_device(cb, many, 48, 32 * 16384, 512, blob2, cap2, torch.zeros(scr2, dtype=torch.uint8, device="cuda"), scr2)
+    assert e.value.status_name == "INVALID_ARG"
+    assert bool((blob2[512 + 1024 + 4 * 49408:] == 0xA5).all())                       # (behind header, lengths, table and index)
     hl.encode_device(cb, w_dev, 32, 256, 512, blob, cap, scr, n_scr)                 # and the context is still fine
     cb.free()
