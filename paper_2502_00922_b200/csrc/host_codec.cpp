@@ -70,10 +70,46 @@ huffllm_status check_desc(const huffllm_desc *d) {
 
 // ------------------------------------------------------------------ code construction
 
-// Optimal prefix-code lengths with every length <= cap, by dynamic programming over
-// the Kraft budget: state = (symbols placed, budget spent in units of 2^-cap).
+// Optimal prefix-code lengths with every length <= cap by package-merge (Larmore and Hirschberg 1990): `used`, n >= 2 symbols in
+// descending order of their counts.  From the deepest level up, a level's list holds the symbols and the pairs of the level below, by
+// weight; a solution takes the 2 n - 2 lightest of the topmost list, of the level below the two parts of every pair taken, and so on,
+// and a symbol's length is the number of levels that take it.  False where the lightest elements taken of a list are not the only choice
+// (the first one left weighs as much as the last one taken): then there may be several optimal codes.  Where they are, at every level,
+// any other solution costs more: it takes other elements of some list, which weigh more, or other parts of the same ones.
+static bool unique_lengths(const uint64_t *counts, const std::vector<int> &used, int cap, uint8_t *len) {
+    constexpr int kMost = 2 * 256;
+    const int n = (int)used.size();
+    if (counts[used[0]] >> 40) return false;                 // (a pair holds at most 2^14 symbols: sums of larger counts could overflow)
+    uint64_t weight[16][kMost];
+    int symbols[16][kMost];                                  // of a list's first elements, how many are symbols
+    int size[16];
+    for (int d = cap; d >= 1; --d) {
+        const int pairs = d == cap ? 0 : size[d + 1] / 2;
+        int s = 0, p = 0, k = 0;
+        while (k < 2 * n - 1 && (s < n || p < pairs)) {      // (one element more than is taken)
+            const uint64_t ws = s < n ? counts[used[n - 1 - s]] : ~0ull, wp = p < pairs ? weight[d + 1][2 * p] + weight[d + 1][2 * p + 1] : ~0ull;
+            if (ws <= wp) ++s;
+            else ++p;
+            weight[d][k] = std::min(ws, wp);
+            symbols[d][k++] = s;
+        }
+        size[d] = k;
+    }
+    for (int s = 0; s < n; ++s) len[used[s]] = 0;
+    for (int d = 1, take = 2 * n - 2; take; ++d) {
+        if (take < size[d] && weight[d][take] == weight[d][take - 1]) return false;
+        const int s = symbols[d][take - 1];
+        for (int i = 0; i < s; ++i) ++len[used[n - 1 - i]];
+        take = 2 * (take - s);
+    }
+    return true;
+}
+
+// Optimal prefix-code lengths with every length <= cap.  Where there are several optimal codes, the one that dynamic programming over the
+// Kraft budget comes to: state = (symbols placed, budget spent in units of 2^-cap).
 static bool limited_lengths(const uint64_t *counts, int nsym, int cap, uint8_t *len) {
     std::vector<int> used;
+    used.reserve((size_t)nsym);
     for (int s = 0; s < nsym; ++s) {
         len[s] = 0;
         if (counts[s]) used.push_back(s);
@@ -83,11 +119,14 @@ static bool limited_lengths(const uint64_t *counts, int nsym, int cap, uint8_t *
     if (n == 1) { len[used[0]] = 1; return true; }
     if (cap < 1 || cap > 15 || (1 << cap) < n) return false;
     std::stable_sort(used.begin(), used.end(), [&](int a, int b) { return counts[a] > counts[b]; });
+    // (Codebooks of gaussian weights from counts, us, dynamic programming alone / this: BF16 19.5 / 7.1, at 12 bits 207 / 12.5, by whole exponents
+    // 47 / 6.1; FP16 95 / 9.0, at 12 bits 622 / 22.)
+    if (unique_lengths(counts, used, cap, len)) return true;
+    for (int s : used) len[s] = 0;
     // Of the states with the symbols placed so far only those are gone on from that no state of less budget spent equals in cost:
     // whatever completes the others completes that one too, at no more cost and less budget, which is what the last choice
     // (least cost, then least budget) prefers.  States that leave the symbols still to come less than one unit each cannot be
-    // completed.  (Codebooks from counts, us: all states / these, BF16 at 8 and 12 bits 33 / 20 and 926 / 220, FP16 179 / 97 and
-    // 6150 / 630.)
+    // completed.
     const int U = 1 << cap;
     const uint64_t INF = ~0ull;
     std::vector<uint64_t> cost((size_t)2 * (U + 1));         // of the symbols so far, and with one more
@@ -196,6 +235,9 @@ static void finish_codebook(huffllm_codebook *cb) {
     memset(cb->len8, 0, sizeof(cb->len8));
     memset(cb->bits8, 0, sizeof(cb->bits8));
     cb->lut.assign((size_t)1 << cb->budget, 0u);
+    uint32_t bits[2][16] = {};                               // stream bits of the nibbles' codewords
+    for (int k = 0; k < 2 && cb->n_fields == 2; ++k)
+        for (int s = 0; s < 16; ++s) bits[k][s] = reverse_bits(cb->code[k][s], cb->len[k][s]);
     for (int e = 0; e < 256; ++e) {
         uint32_t seq;
         int L;
@@ -203,7 +245,7 @@ static void finish_codebook(huffllm_codebook *cb) {
             int h = e >> 4, l = e & 15;
             int lh = cb->len[0][h], ll = cb->len[1][l];
             if (!lh || !ll) continue;
-            seq = reverse_bits(cb->code[0][h], lh) | (reverse_bits(cb->code[1][l], ll) << lh);
+            seq = bits[0][h] | bits[1][l] << lh;
             L = lh + ll;
         } else {
             L = cb->len_e[e];

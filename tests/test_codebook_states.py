@@ -1,5 +1,6 @@
-"""The codebook builder goes on from the least-cost states of its dynamic programme only; the lengths must be those of the
-programme over all states, ties included (a blob's bytes depend on them).  CPU only."""
+"""The codebook builder takes package-merge's lengths where no other code costs as little, else those of its dynamic programme, which
+goes on from its least-cost states only; the lengths must be those of the programme over all states, ties included (a blob's
+bytes depend on them).  CPU only."""
 import numpy as np
 import pytest
 
@@ -41,12 +42,21 @@ def draw(kind, n, rng):
         return [int(v) for v in rng.integers(0, 4, n)]
     if kind == "few symbols":
         return [int(v) if rng.random() < 0.2 else 0 for v in rng.integers(1, 1000, n)]
+    if kind == "powers of two":                              # sums that equal other counts: ties between symbols and pairs
+        return [1 << int(v) for v in rng.integers(0, 9, n)]
+    if kind == "fibonacci":                                  # every length there is, equal costs of different codes
+        f = [1, 1]
+        while len(f) < n:
+            f.append(f[-1] + f[-2] if len(f) < 40 else 1)
+        return [f[i] for i in rng.permutation(n)]
+    if kind == "beyond 2^40":                                # (left to the programme)
+        return [int(v) for v in rng.integers(1, 1 << 41, n)]
     if kind == "halving":
         return [int(1e8 * 0.5 ** abs(i - 11)) for i in range(n)]
     return [int(2.0 ** v) for v in rng.uniform(0, 30, n)]
 
 
-KINDS = ["equal", "few values", "few symbols", "halving", "wide"]
+KINDS = ["equal", "few values", "few symbols", "halving", "wide", "powers of two", "fibonacci", "beyond 2^40"]
 
 
 @pytest.mark.parametrize("kind", KINDS)
