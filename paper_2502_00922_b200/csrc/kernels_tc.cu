@@ -43,6 +43,7 @@ namespace huffllm {
 
 constexpr int kTcStages = 3;      // most stages; A.tc_stages are in use (shared memory is short at wide paddings and many slices)
 constexpr int kTcTiles = 4;
+constexpr uint32_t kPollsAlone = 64;      // polls of a barrier before a warp sees to it that the kernel in front is over
 
 // 8 bytes global -> shared without a register in between; the first `bytes` (0 or 8) are read, the rest is zero.
 __device__ __forceinline__ void cp_async8(uint32_t dst, const void *src, uint32_t bytes) {
@@ -287,9 +288,11 @@ __global__ void __launch_bounds__(1024, 1) huff_gemm_tc_kernel(const __grid_cons
         return;
     }
 
-    // the table is built and tensor memory allocated: from here on activations are read and results written, which the
-    // kernel in front of this one in the stream may still be producing
-    pdl_wait_prior_grid();
+    // The kernel in front of this one in the stream may still be producing the activations, or using the workspace: the warps that issue
+    // or carry activations wait for it here, all others before they write anything.  The decoders, who read the blob alone, run ahead by the
+    // depth of the stage ring.  (All warps waiting here / this, us: 4096 x 14336 at 16 vectors 34.2 / 32.6, the 7B-shaped layer at 32
+    // 133.1 / 127.6, 8192 x 28672 at 64 120.8 / 118.5, 1024 x 4096 at 32 13.5 / 11.1, FP16 4096 x 11008 at 24 51.5 / 45.9.)
+    if (warp == issuer || serves) pdl_wait_prior_grid();
 
     float *const tc_partial = T.partial[MULTI ? mi : 0];
     unsigned int *const tc_ticket = T.ticket[MULTI ? mi : 0];
@@ -313,6 +316,8 @@ __global__ void __launch_bounds__(1024, 1) huff_gemm_tc_kernel(const __grid_cons
                 if (A.err && lane == 0) atomicExch(A.err, -2);
                 return;
             }
+            // (what is missing may be behind the warps that wait for the kernel in front: that takes as long as it takes)
+            if (spins == kPollsAlone) pdl_wait_prior_grid();
             done = mbar_try_wait(bar, parity);
         }
     };
@@ -424,6 +429,7 @@ __global__ void __launch_bounds__(1024, 1) huff_gemm_tc_kernel(const __grid_cons
     auto epilogue = [&](auto n_slices, uint32_t item, uint32_t mt, uint32_t k0, uint32_t k1) {
         constexpr uint32_t SL = decltype(n_slices)::value;
         constexpr int CW = NPAD / (2 * SL);
+        pdl_wait_prior_grid();                               // (over by now, as the issuer waited for it; but every warp that writes asks)
         const uint32_t col0 = (warp >> 2) * CW, acc_tile = col0 / NPAD, n0 = col0 % NPAD;
         float v[CW];
 #pragma unroll

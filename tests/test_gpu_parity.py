@@ -854,3 +854,41 @@ def test_bad_record_offsets_between_runs_of_chunks(hl, torch, cols, ce, budget, 
         rg, kc = divmod(c, KC)
         want[rg * 16:rg * 16 + 16, kc * d.chunk_cols:(kc + 1) * d.chunk_cols] = 0x5A5A
     assert np.array_equal(got[:rows * cols].reshape(rows, cols), want)
+
+
+@pytest.mark.parametrize("rows,cols,ce,batch,dtype", [
+    (64, 64, 512, 17, 0),              # one stage per chunk, fewer stages than the ring has: only the epilogue asks
+    (496, 2048, 4096, 33, 0),          # the decoders fill the ring and wait
+    (300, 1056, 1024, 64, 0),          # two stages, an odd block at the row's end
+    (496, 1024, 2048, 24, 1),          # FP16
+])
+def test_decoders_run_ahead_of_the_activations(hl, torch, rows, cols, ce, batch, dtype):
+    """The kernel in front is still writing the activations (a copy of 192 MB, which lets the product start early and writes them last)
+    while the decoders run: every product has the activations of its own copy, and the workspace is used by one at a time."""
+    gen = "fp16" if dtype else "bf16"
+    up = Uploaded(hl, torch, wl.gaussian_weights(rows, cols, 0.02, 71, gen), ce, batch=batch, dtype=dtype)
+    kind = torch.float16 if dtype else torch.bfloat16
+    size = 192 << 20
+    front = size // 2 - batch * cols                                     # 16-bit values in front of the activations
+    src = [torch.zeros(size // 2, dtype=torch.int16, device="cuda") for _ in range(2)]
+    dst = torch.zeros(size // 2, dtype=torch.int16, device="cuda")
+    for i, s in enumerate(src):
+        s[front:] = torch.randn(batch * cols, generator=torch.Generator().manual_seed(i)).to(kind).view(torch.int16).cuda()
+    want = []
+    for s in src:                                                        # each alone, everything in place
+        y = torch.full((batch * rows,), float("nan"), dtype=torch.float32, device="cuda")
+        x = s[front:].clone()
+        torch.cuda.synchronize()
+        hl.decode_gemm(up.desc, up.blob_dev, x, batch, y, up.ws, up.ws_bytes, up.err)
+        torch.cuda.synchronize()
+        want.append(y)
+        check_product(y.cpu().numpy().reshape(batch, rows), up.w, x.cpu().numpy().view(np.uint16).reshape(batch, cols), orc.FP16 if dtype else orc.BF16)
+    ys = [torch.full((batch * rows,), float("nan"), dtype=torch.float32, device="cuda") for _ in range(8)]
+    torch.cuda.synchronize()
+    for i, y in enumerate(ys):
+        hl.stage_copy(dst, src[i & 1], size)
+        hl.decode_gemm(up.desc, up.blob_dev, dst.data_ptr() + 2 * front, batch, y, up.ws, up.ws_bytes, up.err)
+    torch.cuda.synchronize()
+    assert int(up.err.item()) == 0
+    for i, y in enumerate(ys):
+        assert torch.equal(y, want[i & 1])
