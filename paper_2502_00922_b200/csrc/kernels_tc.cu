@@ -45,9 +45,9 @@ constexpr int kTcStages = 3;      // most stages; A.tc_stages are in use (shared
 constexpr int kTcTiles = 4;
 constexpr uint32_t kPollsAlone = 64;      // polls of a barrier before a warp sees to it that the kernel in front is over
 
-// 8 bytes global -> shared without a register in between; the first `bytes` (0 or 8) are read, the rest is zero.
-__device__ __forceinline__ void cp_async8(uint32_t dst, const void *src, uint32_t bytes) {
-    asm volatile("cp.async.ca.shared.global [%0], [%1], 8, %2;" ::"r"(dst), "l"(src), "r"(bytes) : "memory");
+// 8 bytes global -> shared without a register in between.
+__device__ __forceinline__ void cp_async8(uint32_t dst, const void *src) {
+    asm volatile("cp.async.ca.shared.global [%0], [%1], 8;" ::"r"(dst), "l"(src) : "memory");
 }
 __device__ __forceinline__ void tmem_alloc(uint32_t smem_dst, uint32_t ncols) {
     asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_dst), "r"(ncols) : "memory");
@@ -152,8 +152,7 @@ __global__ void __launch_bounds__(1024, 1) huff_gemm_tc_kernel(const __grid_cons
 
     extern __shared__ __align__(128) uint8_t dyn_smem[];
     __shared__ __align__(8) uint64_t bars[kMaxWarps * 2];   // per warp: its two coded-copy barriers
-    __shared__ __align__(8) uint64_t empty_bar[kTcStages];  // stage may be refilled (arrived on by tcgen05.commit)
-    __shared__ __align__(8) uint64_t full_bar[kTcStages];   // every decoder warp's share of the stage is in place
+    __shared__ __align__(8) uint64_t ring_bars[2 * kTcStages];   // stage may be refilled (arrived on by tcgen05.commit); every decoder warp's share is in place
     __shared__ uint32_t s_tmem_base, s_last;
 
     const uint32_t tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
@@ -225,6 +224,12 @@ __global__ void __launch_bounds__(1024, 1) huff_gemm_tc_kernel(const __grid_cons
     asm volatile("mov.u32 %0, %0;" : "+r"(lut_lane));
     if (D == kUpper) asm volatile("mov.u32 %0, %0;" : "+r"(lut_low));
     const uint32_t bar0 = smem_u32(&bars[warp * 2]);
+    // (The ring's address is worked out once: the compiler takes a shared variable's address anew at every use, three instructions
+    // of which one waits for a special register, 8192 x 28672 at 64 vectors 118.4 us against 115.6, 28672 x 8192 at 32 109.2 against 106.2.)
+    uint32_t ring = smem_u32(ring_bars);
+    asm volatile("mov.u32 %0, %0;" : "+r"(ring));
+    auto empty_bar = [&](uint32_t st) -> uint32_t { return ring + st * 8u; };
+    auto full_bar = [&](uint32_t st) -> uint32_t { return ring + kTcStages * 8u + st * 8u; };
     const uint32_t slot0 = slot_addr(plan, decodes ? slice * n_rg + rgi : 0u, 0, A.slot_bytes);    // (this kernel always runs with two slots per warp)
     auto record_ok = [&](uint32_t r0, uint32_t r1, uint32_t nkb) -> bool {
         return r1 > r0 && r1 <= k.payload_units && (r1 - r0) * 128u > raw_part(nkb) &&
@@ -257,8 +262,8 @@ __global__ void __launch_bounds__(1024, 1) huff_gemm_tc_kernel(const __grid_cons
             lut_v[i] = v < kLutVecs ? __ldg(lut_g + LutPlan<D>::source(v, A.lut_bits)) : 0u;
         }
         if (tid < S) {
-            mbar_init(smem_u32(&empty_bar[tid]), 1);
-            mbar_init(smem_u32(&full_bar[tid]), n_dec + (issuer_carries ? slices - 1u : slices));
+            mbar_init(empty_bar(tid), 1);
+            mbar_init(full_bar(tid), n_dec + (issuer_carries ? slices - 1u : slices));
         }
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
         if (warp == issuer) {
@@ -307,10 +312,9 @@ __global__ void __launch_bounds__(1024, 1) huff_gemm_tc_kernel(const __grid_cons
     bool failed = false;                 // a wait ran out: stop waiting, keep moving, report
 
     auto bounded_wait = [&](uint32_t bar, uint32_t parity) {
-        if (failed) return;
         uint32_t spins = 0;
-        bool done = mbar_try_wait(bar, parity);
-        while (!__all_sync(0xFFFFFFFFu, done)) {
+        while (!__all_sync(0xFFFFFFFFu, mbar_try_wait(bar, parity))) {
+            if (failed) return;
             if (++spins > kWaitLimit) {
                 failed = true;
                 if (A.err && lane == 0) atomicExch(A.err, -2);
@@ -318,29 +322,47 @@ __global__ void __launch_bounds__(1024, 1) huff_gemm_tc_kernel(const __grid_cons
             }
             // (what is missing may be behind the warps that wait for the kernel in front: that takes as long as it takes)
             if (spins == kPollsAlone) pdl_wait_prior_grid();
-            done = mbar_try_wait(bar, parity);
         }
     };
-    auto stage_free = [&]() {            // the stage's last MMAs are done
-        if (st_use > 0) bounded_wait(smem_u32(&empty_bar[st_s]), (st_use - 1) & 1u);
+    auto stage_free = [&]() {            // the stage's last MMAs are done (the first time round: the phase in front of the first one has passed)
+        bounded_wait(empty_bar(st_s), (st_use - 1) & 1u);
     };
 
     // The activations of a block: vector n's K positions 8 kap .. 8 kap + 7 (kap = 0 .. 3) of the tile hold its columns
     // base .. base + 3 and base + 8 .. base + 11 of the block, base = 16 (kap & 1) + 4 (kap >> 1), each four a copy of 8 bytes.
     // Eight lanes take a vector's 64 bytes, a warp instruction four vectors (whole sectors are read, and four lines at a
-    // time: with four lanes to a vector it was eight).  `nblk` blocks (1 or 2) from column `col` on go to stage st_s; vectors
-    // of the padding are filled with zeros.
-    auto carry_x = [&](uint32_t col, uint32_t nblk) {
+    // time: with four lanes to a vector it was eight).  `nblk` blocks (1 or 2) from column `col` on go to stage `st`; vectors
+    // of the padding are left as they are: they reach no column of the product that is written.  The issuer's instructions are what
+    // the carrying costs (eight cycles each, as above), so sixteen vectors that are all there are copied without a predicate, and
+    // addresses are a base and a 32-bit stride (matrices of 2^29 columns and more are not this kernel's).  (Sizes and pointers of
+    // every copy selected by whether its vector exists / predicates on every copy / this, us: 25088 x 7168 at 64 vectors in chunks of 2048
+    // 124.2 / 125.4 / 112.5, 11008 x 4096 at 48 34.6 / 34.0 / 30.3, 14336 x 4096 at 40 42.4 / 39.4 / 36.8.)
+    auto carry_x = [&](uint32_t col, uint32_t nblk, uint32_t st) {
         const uint32_t kap = (lane >> 1) & 3u, half = lane & 1u;
         uint32_t n = lane >> 3;
-        const uint32_t dst = b_base + (st_s * slices + slice) * kBStage + kap * kLbo + n * 16u + half * 8u;
+        const uint32_t dst = b_base + (st * slices + slice) * kBStage + kap * kLbo + n * 16u + half * 8u;
         const uint16_t *src = k.x + (uint64_t)min(n, A.batch - 1) * k.cols + col + (kap & 1) * 16 + (kap >> 1) * 4 + half * 8;
+        const uint32_t step = (uint32_t)k.cols * 8u;        // bytes from a vector to the fourth one behind it
+        const char *sp = (const char *)src;
 #pragma unroll
-        for (int i = 0; i < NPAD / 4; ++i, n += 4) {
-            const uint32_t bytes = n < A.batch ? 8u : 0u, to = dst + (i >> 1) * kSbo + (i & 1) * 64u;    // (nothing is read for 0)
-            cp_async8(to, src, bytes);
-            if (nblk > 1) cp_async8(to + 4 * kLbo, src + 32, bytes);
-            if (n + 4 < A.batch) src += 4 * k.cols;
+        for (int i0 = 0; i0 < NPAD / 4; i0 += 4, n += 16) {
+            if (nblk > 1 && A.batch >= 4u * i0 + 16u) {
+#pragma unroll
+                for (int i = i0; i < i0 + 4; ++i) {
+                    const uint32_t to = dst + (i >> 1) * kSbo + (i & 1) * 64u;
+                    cp_async8(to, sp + (uint64_t)step * i);
+                    cp_async8(to + 4 * kLbo, sp + (uint64_t)step * i + 64);
+                }
+            } else {
+#pragma unroll
+                for (int i = i0; i < i0 + 4; ++i) {
+                    const uint32_t to = dst + (i >> 1) * kSbo + (i & 1) * 64u;
+                    if (n + 4 * (i - i0) < A.batch) {
+                        cp_async8(to, sp + (uint64_t)step * i);
+                        if (nblk > 1) cp_async8(to + 4 * kLbo, sp + (uint64_t)step * i + 64);
+                    }
+                }
+            }
         }
     };
     auto x_landed = [&]() {                                  // the B slice must be visible to the tensor core's reads
@@ -367,13 +389,13 @@ __global__ void __launch_bounds__(1024, 1) huff_gemm_tc_kernel(const __grid_cons
         tc_wait_st();
         tc_fence_before();
         __syncwarp();
-        if (lane == 0) mbar_arrive(smem_u32(&full_bar[st_s]));
+        if (elect_one()) mbar_arrive(full_bar(st_s));
         next_stage();
     };
     // A stage to which this warp has nothing to add (rows outside the matrix, a slice that is done).
     auto stage_nothing = [&]() {
         stage_free();
-        if (lane == 0) mbar_arrive(smem_u32(&full_bar[st_s]));
+        if (lane == 0) mbar_arrive(full_bar(st_s));
         next_stage();
     };
     // The same stage, issuer side: when every warp has arrived, one lane issues the stage's MMAs for every tile and commits
@@ -396,7 +418,7 @@ __global__ void __launch_bounds__(1024, 1) huff_gemm_tc_kernel(const __grid_cons
                                   j == 0 ? (first_of_item ? 0u : 1u) : 1u);
     };
     auto issue_stage = [&](bool first_of_item, bool full, auto halves) {           // full: four tiles, two blocks of every slice
-        bounded_wait(smem_u32(&full_bar[st_s]), st_use & 1u);
+        bounded_wait(full_bar(st_s), st_use & 1u);
         if (elect_one()) {
             tc_fence_after();
             if (failed) {
@@ -417,7 +439,7 @@ __global__ void __launch_bounds__(1024, 1) huff_gemm_tc_kernel(const __grid_cons
                                               (first_of_item && j == 0) ? 0u : 1u);
                 }
             }
-            tc_commit(smem_u32(&empty_bar[st_s]));
+            tc_commit(empty_bar(st_s));
         }
         __syncwarp();
         next_stage();
@@ -525,12 +547,27 @@ __global__ void __launch_bounds__(1024, 1) huff_gemm_tc_kernel(const __grid_cons
         auto stages_of = [&](uint32_t j) -> uint32_t { return slices == 1u ? (blocks_of(k0 + j) + 1u) >> 1 : full_stages; };
 
         if (warp == issuer) {
-            // the activations of the stage behind the one at hand are always under way
-            uint32_t own = step_blocks(slice, 0);           // blocks of the carried slice in the step at hand
-            if (issuer_carries) {
-                stage_free();
-                if (own) carry_x(col_lo, min(own, 2u));
-            }
+            // The activations of the stages behind the one at hand, all but one of the ring's, are always under way.  (Of the next
+            // stage alone / of the next two, us: 28672 x 8192 at 32 vectors 110.4 / 106.4, the 7B-shaped layer at 32 126.2 / 124.6.)
+            uint32_t own = step_blocks(slice, 0), cj = 0, cp = 0, c_s = st_s, c_use = st_use;   // the stage to be carried next, and its place in the ring
+            auto carry_next = [&]() {
+                if (cj < steps) {
+                    bounded_wait(empty_bar(c_s), (c_use - 1) & 1u);
+                    const uint32_t n2 = halves(own, cp);
+                    if (n2) carry_x(col_lo + cj * k.chunk_cols + cp * 64u, n2, c_s);
+                    if (++c_s == S) {
+                        c_s = 0;
+                        ++c_use;
+                    }
+                    if (++cp == stages_of(cj)) {
+                        cp = 0;
+                        own = ++cj < steps ? step_blocks(slice, cj) : 0u;
+                    }
+                }
+                asm volatile("cp.async.commit_group;" ::: "memory");
+            };
+            if (issuer_carries)
+                for (uint32_t i = 1; i < S; ++i) carry_next();
             for (uint32_t j = 0; j < steps; ++j) {          // stages are cut like the decoders': pairs of blocks inside a chunk
                 const uint32_t n_st = stages_of(j);
                 uint32_t nkb[4], least = ~0u;               // blocks of every slice in this step, and the fewest
@@ -540,20 +577,16 @@ __global__ void __launch_bounds__(1024, 1) huff_gemm_tc_kernel(const __grid_cons
                     if (sl < slices) least = min(least, nkb[sl]);
                 }
                 for (uint32_t p = 0; p < n_st; ++p) {
-                    if (issuer_carries) x_landed();
+                    if (issuer_carries) {
+                        if (S == 3u) asm volatile("cp.async.wait_group 1;" ::: "memory");
+                        else asm volatile("cp.async.wait_group 0;" ::: "memory");
+                        asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
+                        __syncwarp();
+                    }
                     issue_stage(j == 0 && p == 0, tiles == 4u && least >= 2 * p + 2, [&](uint32_t sl) -> uint32_t {
                         return halves(sl == 0 ? nkb[0] : sl == 1 ? nkb[1] : sl == 2 ? nkb[2] : nkb[3], p);
                     });
-                    if (!issuer_carries) continue;
-                    uint32_t p2 = p + 1;
-                    if (p2 == n_st) {
-                        if (j + 1 == steps) break;
-                        own = step_blocks(slice, j + 1);
-                        p2 = 0;
-                    }
-                    stage_free();
-                    const uint32_t n2 = halves(own, p2);
-                    if (n2) carry_x(col_lo + (p2 ? j : j + 1) * k.chunk_cols + p2 * 64u, n2);
+                    if (issuer_carries) carry_next();
                 }
             }
         } else if (serves) {
@@ -562,9 +595,9 @@ __global__ void __launch_bounds__(1024, 1) huff_gemm_tc_kernel(const __grid_cons
                 for (uint32_t p = 0; p < n_st; ++p) {
                     stage_free();
                     const uint32_t n2 = halves(own, p);
-                    if (n2) carry_x(col_lo + j * k.chunk_cols + p * 64u, n2);
+                    if (n2) carry_x(col_lo + j * k.chunk_cols + p * 64u, n2, st_s);
                     x_landed();
-                    if (lane == 0) mbar_arrive(smem_u32(&full_bar[st_s]));
+                    if (lane == 0) mbar_arrive(full_bar(st_s));
                     next_stage();
                 }
             }
@@ -666,7 +699,7 @@ __global__ void __launch_bounds__(1024, 1) huff_gemm_tc_kernel(const __grid_cons
         // only the tiles' warps have one.)
         if (warp < tiles * 8u) {
             const uint32_t ls = st_s == 0 ? S - 1u : st_s - 1u, lu = st_s == 0 ? st_use - 1u : st_use;
-            bounded_wait(smem_u32(&empty_bar[ls]), lu & 1u);
+            bounded_wait(empty_bar(ls), lu & 1u);
             tc_fence_after();
             if (slices == 1u) epilogue(std::integral_constant<uint32_t, 1>{}, item, mt, k0, k1);
             else if (slices == 2u) epilogue(std::integral_constant<uint32_t, 2>{}, item, mt, k0, k1);

@@ -892,3 +892,19 @@ def test_decoders_run_ahead_of_the_activations(hl, torch, rows, cols, ce, batch,
     assert int(up.err.item()) == 0
     for i, y in enumerate(ys):
         assert torch.equal(y, want[i & 1])
+
+
+@pytest.mark.parametrize("batch", [9, 15, 17, 31, 33, 47, 49, 63])
+@pytest.mark.parametrize("rows,cols,ce", [(496, 1056, 1024), (272, 8224, 4096), (8192, 160, 512)])
+def test_activations_of_ragged_batches(hl, torch, rows, cols, ce, batch):
+    """Sixteen vectors at a time are copied to shared memory, fewer by themselves, none for the padding, whose sums go nowhere: batches around
+    every sixteen, rows that end in an odd block, the activations carried by the warp that issues and by one of their own."""
+    up = Uploaded(hl, torch, wl.gaussian_weights(rows, cols, 0.02, 72), ce, batch=batch)
+    x = torch.randn((batch, cols), generator=torch.Generator().manual_seed(batch)).to(torch.bfloat16).view(torch.int16).cuda()
+    y = torch.full(((batch + 1) * rows,), float("nan"), dtype=torch.float32, device="cuda")      # (a vector's room behind the product)
+    hl.decode_gemm(up.desc, up.blob_dev, x, batch, y, up.ws, up.ws_bytes, up.err)
+    torch.cuda.synchronize()
+    assert int(up.err.item()) == 0
+    got = y.cpu().numpy().reshape(batch + 1, rows)
+    assert np.isnan(got[batch]).all()
+    check_product(got[:batch], up.w, x.cpu().numpy().view(np.uint16).reshape(batch, cols), orc.BF16)
