@@ -150,8 +150,6 @@ uint32_t tc_npad_of(uint32_t batch) { return batch <= 16 ? 16 : (batch <= 32 ? 3
 bool tc_fits(const huffllm_desc *const *d, uint32_t n, uint32_t npad, const TcShape &sh, uint32_t flat, uint32_t dyn_smem) {
     SmemNeeds need = smem_needs(d[0]);
     if (d[0]->dtype == HUFFLLM_FP16 && d[0]->lut_bits <= 8) need.table_bytes = fp16_table_bytes(flat);   // (a launch-wide choice)
-    for (uint32_t i = 0; i < n; ++i)
-        if (d[i]->cols >> 29) return false;                  // (the kernel steps through the activations in 32 bits: four vectors of 2-byte words)
     for (uint32_t i = 1; i < n; ++i) {
         const SmemNeeds o = smem_needs(d[i]);
         if (o.slot_bytes > need.slot_bytes) need.slot_bytes = o.slot_bytes;

@@ -334,7 +334,7 @@ __global__ void __launch_bounds__(1024, 1) huff_gemm_tc_kernel(const __grid_cons
     // time: with four lanes to a vector it was eight).  `nblk` blocks (1 or 2) from column `col` on go to stage `st`; vectors
     // of the padding are left as they are: they reach no column of the product that is written.  The issuer's instructions are what
     // the carrying costs (eight cycles each, as above), so sixteen vectors that are all there are copied without a predicate, and
-    // addresses are a base and a 32-bit stride (matrices of 2^29 columns and more are not this kernel's).  (Sizes and pointers of
+    // addresses are a base and a 32-bit stride.  (Sizes and pointers of
     // every copy selected by whether its vector exists / predicates on every copy / this, us: 25088 x 7168 at 64 vectors in chunks of 2048
     // 124.2 / 125.4 / 112.5, 11008 x 4096 at 48 34.6 / 34.0 / 30.3, 14336 x 4096 at 40 42.4 / 39.4 / 36.8.)
     auto carry_x = [&](uint32_t col, uint32_t nblk, uint32_t st) {
@@ -342,7 +342,7 @@ __global__ void __launch_bounds__(1024, 1) huff_gemm_tc_kernel(const __grid_cons
         uint32_t n = lane >> 3;
         const uint32_t dst = b_base + (st * slices + slice) * kBStage + kap * kLbo + n * 16u + half * 8u;
         const uint16_t *src = k.x + (uint64_t)min(n, A.batch - 1) * k.cols + col + (kap & 1) * 16 + (kap >> 1) * 4 + half * 8;
-        const uint32_t step = (uint32_t)k.cols * 8u;        // bytes from a vector to the fourth one behind it
+        const uint32_t step = (uint32_t)k.cols;             // (at most 2^31)
         const char *sp = (const char *)src;
 #pragma unroll
         for (int i0 = 0; i0 < NPAD / 4; i0 += 4, n += 16) {
@@ -350,16 +350,16 @@ __global__ void __launch_bounds__(1024, 1) huff_gemm_tc_kernel(const __grid_cons
 #pragma unroll
                 for (int i = i0; i < i0 + 4; ++i) {
                     const uint32_t to = dst + (i >> 1) * kSbo + (i & 1) * 64u;
-                    cp_async8(to, sp + (uint64_t)step * i);
-                    cp_async8(to + 4 * kLbo, sp + (uint64_t)step * i + 64);
+                    cp_async8(to, sp + (uint64_t)step * (8u * i));
+                    cp_async8(to + 4 * kLbo, sp + (uint64_t)step * (8u * i) + 64);
                 }
             } else {
 #pragma unroll
                 for (int i = i0; i < i0 + 4; ++i) {
                     const uint32_t to = dst + (i >> 1) * kSbo + (i & 1) * 64u;
                     if (n + 4 * (i - i0) < A.batch) {
-                        cp_async8(to, sp + (uint64_t)step * i);
-                        if (nblk > 1) cp_async8(to + 4 * kLbo, sp + (uint64_t)step * i + 64);
+                        cp_async8(to, sp + (uint64_t)step * (8u * i));
+                        if (nblk > 1) cp_async8(to + 4 * kLbo, sp + (uint64_t)step * (8u * i) + 64);
                     }
                 }
             }
