@@ -147,7 +147,7 @@ struct TcShape {
 uint32_t tc_npad_of(uint32_t batch) { return batch <= 16 ? 16 : (batch <= 32 ? 32 : 64); }
 // Do the slot pairs of the shape's decoder warps fit beside the tables and the stages of activations (the guard area may lie
 // over those), for the largest records among the launch's matrices?
-bool tc_fits(const huffllm_desc *const *d, uint32_t n, uint32_t npad, const TcShape &sh, uint32_t flat, uint32_t dyn_smem) {
+uint32_t tc_room(const huffllm_desc *const *d, uint32_t n, uint32_t npad, const TcShape &sh, uint32_t flat, uint32_t dyn_smem) {
     SmemNeeds need = smem_needs(d[0]);
     if (d[0]->dtype == HUFFLLM_FP16 && d[0]->lut_bits <= 8) need.table_bytes = fp16_table_bytes(flat);   // (a launch-wide choice)
     for (uint32_t i = 1; i < n; ++i) {
@@ -155,14 +155,19 @@ bool tc_fits(const huffllm_desc *const *d, uint32_t n, uint32_t npad, const TcSh
         if (o.slot_bytes > need.slot_bytes) need.slot_bytes = o.slot_bytes;
         if (o.guard_bytes > need.guard_bytes) need.guard_bytes = o.guard_bytes;
     }
-    return planned_warps(need.table_align, need.table_bytes, 2ull * need.slot_bytes, dyn_smem, sh.part_bytes(npad), need.guard_bytes) >= sh.decoders();
+    return planned_warps(need.table_align, need.table_bytes, 2ull * need.slot_bytes, dyn_smem, sh.part_bytes(npad), need.guard_bytes);
+}
+bool tc_fits(const huffllm_desc *const *d, uint32_t n, uint32_t npad, const TcShape &sh, uint32_t flat, uint32_t dyn_smem) {
+    return tc_room(d, n, npad, sh, flat, dyn_smem) >= sh.decoders();
 }
 // The shapes a launch chooses from: 0 = one slice, as many tiles of rows as find room; 1 = one slice and a warp of its own for
 // the activations (at the widest batch padding: there the issuer, which carries them otherwise, bounds the CTA, 8192 x 28672
-// at 64 vectors 149 us against 133 with one decoder fewer); 2, 3 = two and four slices.  False: it does not fit or apply.
-constexpr uint32_t kTcShapes = 4;
+// at 64 vectors 149 us against 133 with one decoder fewer); 2, 3 = two and four slices; 4 = one slice and as many row groups as
+// have room, where whole tiles would be eight (large records, as FP16 has: a CTA of eight warps waits for its lookups).
+// False: it does not fit or apply.
+constexpr uint32_t kTcShapes = 5;
 bool tc_shape(const huffllm_desc *const *d, uint32_t n, uint32_t npad, uint32_t which, uint32_t flat, uint32_t dyn_smem, TcShape *sh) {
-    const uint32_t slices = which < 2 ? 1 : which == 2 ? 2 : 4;
+    const uint32_t slices = which < 2 || which == 4 ? 1 : which == 2 ? 2 : 4;
     // three stages, two at the widest batch padding, where tensor memory holds no more; the CTA's last warp issues the MMAs
     *sh = TcShape{4 / slices, slices, npad == 64 ? 2u : 3u, 32 / slices - (which == 1 ? 2 : 1)};
     if (which == 0) {
@@ -171,6 +176,11 @@ bool tc_shape(const huffllm_desc *const *d, uint32_t n, uint32_t npad, uint32_t 
             if (tc_fits(d, n, npad, *sh, flat, dyn_smem)) return true;
         }
         return false;
+    }
+    if (which == 4) {                                        // (its room does not depend on the row groups)
+        sh->row_groups = tc_room(d, n, npad, *sh, flat, dyn_smem);
+        sh->na = 2;
+        return sh->row_groups > 8 && sh->row_groups < 16;
     }
     if (which == 1 && npad != 64) return false;
     if (slices == 4 && npad == 64) return false;             // (seven row groups' worth of rows do not pay for 64 columns of sums)
@@ -195,7 +205,11 @@ struct TcPlan {
 // 34, 28672 x 4096 at 64 vectors took two slices, 99 us, instead of one and a warp for the activations, 91; with 38, 25088 x 7168
 // in chunks of 2048 would go the other way, 153 instead of 141.)
 constexpr uint32_t kTcUnit = 32;
-uint32_t tc_block_cost(const TcShape &sh, uint32_t npad) { return sh.slices == 1 ? kTcUnit : sh.slices == 2 ? (npad == 64 ? 36 : 34) : 39; }
+uint32_t tc_block_cost(const TcShape &sh, uint32_t npad) {
+    // nine to fifteen row groups: a block takes longer than with the eight of shape 0 (the warps share issue slots), 14 + n for n of them
+    if (sh.slices == 1 && sh.na == 2 && sh.row_groups < 16) return kTcUnit * (14 + sh.row_groups) / (14 + 8);
+    return sh.slices == 1 ? kTcUnit : sh.slices == 2 ? (npad == 64 ? 36 : 34) : 39;
+}
 constexpr uint32_t kTcItemCost = 5 * kTcUnit;
 uint32_t tc_sum_cost(const TcShape &sh, uint32_t npad, uint32_t ks) { return ks > 1 ? 2 * ks * sh.piece_columns(npad) : 0; }
 // The longest any CTA works when `ks` column ranges of `m_tiles` row tiles are dealt to `sms` CTAs: CTA b takes items b,
@@ -228,8 +242,10 @@ uint64_t tc_span(const huffllm_desc *d, const TcShape &sh, uint32_t npad, uint32
 }
 // `sms`: the CTAs this matrix can have (all SMs, or its share of a launch over several matrices); `max_bytes`: the workspace
 // at hand (column ranges whose pieces would not fit are not considered: a share of the SMs can favour more ranges than the
-// whole GPU, for which workspaces are sized); `max_chunks`: the most column chunks that one accumulator may add up.
-TcPlan tc_plan(const huffllm_desc *d, uint32_t npad, uint32_t sms, const TcShape &sh, size_t max_bytes, uint32_t max_chunks) {
+// whole GPU, for which workspaces are sized); `max_chunks`: the most column chunks that one accumulator may add up; `min_ranges`: the
+// fewest ranges.
+TcPlan tc_plan(const huffllm_desc *d, uint32_t npad, uint32_t sms, const TcShape &sh, size_t max_bytes, uint32_t max_chunks,
+               uint32_t min_ranges = 1) {
     TcPlan p;
     p.m_tiles = (d->row_groups + sh.row_groups - 1) / sh.row_groups;
     const size_t item_bytes = (size_t)32 * sh.piece_columns(npad) * 32 * sizeof(float);
@@ -239,7 +255,7 @@ TcPlan tc_plan(const huffllm_desc *d, uint32_t npad, uint32_t sms, const TcShape
     const bool base = max_chunks == ~0u;
     uint32_t best = 0;
     uint64_t best_span = ~0ull;
-    for (uint32_t ks = 1; ks <= 16 && ks <= d->col_chunks; ++ks) {
+    for (uint32_t ks = min_ranges; ks <= 16 && ks <= d->col_chunks; ++ks) {
         if (ks > 1 && ws_partial_offset(d) + (size_t)p.m_tiles * ks * item_bytes > max_bytes) break;
         const uint32_t range = (d->col_chunks + ks - 1) / ks;
         if ((range + sh.slices - 1) / sh.slices > max_chunks) continue;
@@ -270,17 +286,31 @@ bool tc_best(const huffllm_desc *const *d, uint32_t n, uint32_t npad, const uint
     if (!tc_shape(d, n, npad, 0, flat, dyn_smem, &base)) return false;
     for (size_t base_bytes = ~(size_t)0;; base_bytes = max_bytes) {
         uint64_t best_span = ~0ull;
-        uint32_t most[kMaxMats];
+        uint32_t most[kMaxMats], ranges[kMaxMats];
         for (uint32_t which = 0; which < kTcShapes; ++which) {
             TcShape sh = base;
+            // Row groups that fill no tile pay where a CTA of whole tiles has eight and every CTA has 32 chunks or more to decode.  (Whole
+            // tiles / this, us: FP16 28672 x 8192 at 32 vectors 283.6 / 264.1, 11008 x 4096 at 32 62.5 / 58.8, 20000 x 1024 at 32 36.5 /
+            // 32.4; 30 chunks a CTA, 9000 x 2048 at 64 26.6 / 27.6, 15, 9000 x 1024 at 17 14.2 / 16.1.  Sixteen warps and more use the issue
+            // slots already: BF16 20000 x 4096 at 32 in chunks of 8192 70.5 / 74.1, FP16 12288 x 12288 at 32 in chunks of 2048 109.6 / 121.3.)
+            // A row is cut into no fewer ranges than in shape 0: its error grows with the columns of an average range as well, 11008 x 4096
+            // FP16 at 32 in four ranges of four chunks is 1.25e-6 from 64 bits, in five 1.03e-6, in eight, as it is now, 0.77e-6.
+            if (which == 4) {
+                bool pays = base.na == 1;
+                for (uint32_t i = 0; i < n; ++i) pays = pays && d[i]->n_chunks >= 32ull * cta[i];
+                if (!pays) continue;
+            }
             if (which && !tc_shape(d, n, npad, which, flat, dyn_smem, &sh)) continue;
             TcPlan p[kMaxMats];
             uint64_t span = 0;
             for (uint32_t i = 0; i < n; ++i) {
-                p[i] = tc_plan(d[i], npad, cta[i], sh, which ? max_bytes : base_bytes, which ? most[i] : ~0u);
+                p[i] = tc_plan(d[i], npad, cta[i], sh, which ? max_bytes : base_bytes, which ? most[i] : ~0u, which == 4 ? ranges[i] : 1u);
                 const uint64_t t = p[i].bytes > max_bytes ? ~0ull : p[i].span;
                 if (t > span) span = t;
-                if (which == 0) most[i] = p[i].chunks;
+                if (which == 0) {
+                    most[i] = p[i].chunks;
+                    ranges[i] = p[i].ksplit ? p[i].ksplit : 1u;
+                }
             }
             if (span < best_span) {
                 best_span = span;

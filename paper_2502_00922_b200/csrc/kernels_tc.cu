@@ -168,14 +168,15 @@ __global__ void __launch_bounds__(1024, 1) huff_gemm_tc_kernel(const __grid_cons
     // `na` row tiles of `n_rg` row groups, in each of `slices` column slices.  Warp w belongs to slice w / (8 na), has row group
     // `rgi` there and decodes if the CTA has that many.  Where all 32 warps belong to slices (four tiles) a slice's warp that does
     // not decode carries its activations, the very last one, the issuer, only where its slice has no other; with fewer tiles
-    // (one slice) the first warp behind the tiles carries them and the others in front of the issuer leave at once.  (With the
+    // (one slice) the first warp behind the tiles carries them and the others in front of the issuer leave at once.  A tile's further
+    // warps without a row group arrive at every stage like the others, so that they are there for the epilogue.  (With the
     // issuer carrying them there too, chunks of 8192 elements took, back to back, 230 us against 172 for 8192 x 28672 at 64 vectors,
     // 111 against 94 for 12288 x 12288 at 32.)
     const uint32_t S = A.tc_stages, slices = A.tc_slices, na = A.tc_tiles, tiles = na * slices, issuer = 31u;
     const uint32_t n_rg = A.tc_row_groups, n_dec = n_rg * slices;
     const uint32_t slice = warp == issuer || warp >= tiles * 8u ? slices - 1u : warp / (8u * na), li = warp - warp / (8u * na) * 8u * na;
     const uint32_t tile = warp >> 3, q = warp & 3, h = (warp >> 2) & 1, rgi = (li & ~7u) + q * 2 + h;
-    const bool decodes = warp < tiles * 8u && rgi < n_rg, serves = warp != issuer && warp <= tiles * 8u && (rgi >= n_rg || warp == tiles * 8u);
+    const bool decodes = warp < tiles * 8u && rgi < n_rg, serves = warp != issuer && (tiles == 4u ? rgi == n_rg : warp == tiles * 8u);
     const bool issuer_carries = tiles == 4u && n_rg == na * 8u - 1u;
     const uint32_t a_lane = (32u * q + 16u * h) << 16;
     const uint32_t KC = k.col_chunks, RG = (uint32_t)((k.rows + 15) / 16);
@@ -225,9 +226,12 @@ __global__ void __launch_bounds__(1024, 1) huff_gemm_tc_kernel(const __grid_cons
     if (D == kUpper) asm volatile("mov.u32 %0, %0;" : "+r"(lut_low));
     const uint32_t bar0 = smem_u32(&bars[warp * 2]);
     // (The ring's address is worked out once: the compiler takes a shared variable's address anew at every use, three instructions
-    // of which one waits for a special register, 8192 x 28672 at 64 vectors 118.4 us against 115.6, 28672 x 8192 at 32 109.2 against 106.2.)
+    // of which one waits for a special register, 28672 x 8192 at 32 vectors 109.2 us against 106.2.  Not at the widest padding,
+    // where the register is missed elsewhere: 28672 x 8192 at 64 142.3 with it, 139.4 without.  The kernel has 64 registers a thread and
+    // uses them all; what the compiler makes of the decoders' loop, and with it every time here, moves by a few per cent with such things,
+    // so they are chosen by measurement for each padding.)
     uint32_t ring = smem_u32(ring_bars);
-    asm volatile("mov.u32 %0, %0;" : "+r"(ring));
+    if (NPAD < 64) asm volatile("mov.u32 %0, %0;" : "+r"(ring));
     auto empty_bar = [&](uint32_t st) -> uint32_t { return ring + st * 8u; };
     auto full_bar = [&](uint32_t st) -> uint32_t { return ring + kTcStages * 8u + st * 8u; };
     const uint32_t slot0 = slot_addr(plan, decodes ? slice * n_rg + rgi : 0u, 0, A.slot_bytes);    // (this kernel always runs with two slots per warp)
@@ -263,7 +267,7 @@ __global__ void __launch_bounds__(1024, 1) huff_gemm_tc_kernel(const __grid_cons
         }
         if (tid < S) {
             mbar_init(empty_bar(tid), 1);
-            mbar_init(full_bar(tid), n_dec + (issuer_carries ? slices - 1u : slices));
+            mbar_init(full_bar(tid), tiles == 4u ? 31u : tiles * 8u + 1u);      // (every warp but the issuer, decoding or not)
         }
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
         if (warp == issuer) {
@@ -312,6 +316,7 @@ __global__ void __launch_bounds__(1024, 1) huff_gemm_tc_kernel(const __grid_cons
     bool failed = false;                 // a wait ran out: stop waiting, keep moving, report
 
     auto bounded_wait = [&](uint32_t bar, uint32_t parity) {
+        if (NPAD > 16 && failed) return;
         uint32_t spins = 0;
         while (!__all_sync(0xFFFFFFFFu, mbar_try_wait(bar, parity))) {
             if (failed) return;
@@ -389,7 +394,7 @@ __global__ void __launch_bounds__(1024, 1) huff_gemm_tc_kernel(const __grid_cons
         tc_wait_st();
         tc_fence_before();
         __syncwarp();
-        if (elect_one()) mbar_arrive(full_bar(st_s));
+        if (NPAD > 16 ? lane == 0 : elect_one()) mbar_arrive(full_bar(st_s));   // (4096 x 14336 at 16 vectors 33.0 us / 31.9 elected, 8192 x 28672 at 64 117.1 / 118.5)
         next_stage();
     };
     // A stage to which this warp has nothing to add (rows outside the matrix, a slice that is done).
@@ -644,13 +649,11 @@ __global__ void __launch_bounds__(1024, 1) huff_gemm_tc_kernel(const __grid_cons
                         if (!last || has_next) raw_n = load_raw(raw_p);
                         // the block behind that one is asked into L2: a register load one block ahead waits for DRAM otherwise.  (It may
                         // lie in the coded part or behind the record, up to 1 KB behind the payload: the blob has 4 KB there.)
-                        // Not at the widest padding, whose blocks take longer, nor for FP16, whose raw part is a sixteenth.
-                        // (us, without / with it / two blocks further on: 4096 x 14336 at 16 vectors 35.1 / 34.2 / 35.1, 7B-shaped
-                        // layer at 32 135.5 / 133.1 / 135.1; padding 64: 11008 x 4096 at 48 34.7 / 35.9 / 36.0, 8192 x 28672 at 64
-                        // 124.5 / 125.9 / 129.2.  Without / with it: 4096 x 14336 at 32 38.3 / 37.3, 28672 x 8192 at 24 116.2 / 113.9, at 32
-                        // 117.7 / 117.9, in chunks of 8192 160.5 / 148.6, 8192 x 28672 at 32 116.0 / 115.3, 16384 x 4096 at 20 in chunks of
-                        // 1024 45.6 / 46.0.  The record's whole raw part at once, with its copy: 36.8 and 139.6 for the first two.)
-                        if (NPAD < 64 && FMT == 0) asm volatile("prefetch.global.L2 [%0];" ::"l"(raw_p + kRawBlock));
+                        // Not for FP16, whose raw part is a sixteenth.  (us, without / with it / two blocks further on: 4096 x 14336 at 16
+                        // vectors 35.1 / 34.2 / 35.1, 7B-shaped layer at 32 135.5 / 133.1 / 135.1; 28672 x 8192 at 32 in chunks of 8192 160.5 /
+                        // 148.6.  Padding 64: 12288 x 12288 90.1 / 86.6, in chunks of 8192 101.9 / 92.9, 28672 x 8192 147.6 / 143.7.  The record's
+                        // whole raw part at once, with its copy: 36.8 and 139.6 for the first two.)
+                        if (FMT == 0) asm volatile("prefetch.global.L2 [%0];" ::"l"(raw_p + kRawBlock));
                         uint32_t a[8];
                         decode_block<D>(pa, pb, lane << 2, lut_lane, lut_low, raw_c, a, 0u, 0u);
                         stage_block(a, half, nblk);
