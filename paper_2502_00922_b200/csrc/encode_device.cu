@@ -17,6 +17,7 @@
 #include <type_traits>
 
 #include "decode_common.cuh"
+#include "encode_scratch.h"
 #include "internal.h"
 
 namespace huffllm {
@@ -27,9 +28,8 @@ struct EncTotals {
     uint32_t summed;             // CTAs whose records' checksums are in
 };
 
-static_assert(sizeof(EncTotals) <= 256, "the chunks' bits and words follow in the scratch");
+static_assert(sizeof(EncTotals) <= kScratchTotals, "the chunks' bits and words follow in the scratch");
 
-constexpr uint32_t kScanThreads = 1024;      // chunks of a scan CTA
 constexpr uint32_t kWriteWarps = 4;          // of a CTA of pass 2
 __host__ __device__ constexpr uint32_t write_ctas(bool vec) { return vec ? 6 : 5; }     // of an SM (80 and 96 registers)
 constexpr uint32_t kNoCode = 1u << 14;       // length of a symbol without codeword: no sum of a sequence's codewords reaches it (768 of 12 bits)
@@ -247,16 +247,11 @@ __global__ void __launch_bounds__(32 * kSizeWarps, size_ctas(VEC)) encode_size_k
 // chunks in front of them itself (the raw parts in front are known without a sum), so that no CTA waits for another; the one at the end of the
 // index, which sees them all, leaves the totals: nothing has to be cleared or added up by atomics in front of this.  Sums over every
 // chunk in front grow with the square of the chunks: from kGroupsFrom on a launch of its own leaves those of 1024 chunks each (GROUPS),
-// where the chunks' bits were.
+// where the chunks' bits were; what is left over behind whole groups are the last scan CTA's own chunks.
 // (Time behind pass 1 at 11008 / 88064 / 234 000 / 1.05 M chunks, us: 3.9 / 5.4 / 9.9 / 19.5; pass 1 adding up every 1024 by atomics, behind a launch that
 // clears them, 6.3 / 7 / 16 / 30, and 50 us of pass 1 instead of 28 at 88064; without groups 4.2 / 11 / 77 / 224.  The last warp of pass 1 to
 // come from every 1024 chunks doing this, for which it has to order its words before the others' counts: 17.3 -> 38 us for that pass.)
 constexpr uint64_t kGroupsFrom = 49152;
-struct EncGroup {
-    unsigned long long words, bits;
-    uint32_t most;
-};
-__device__ __forceinline__ EncGroup *enc_group(const EncArgs &A, uint32_t g) { return (EncGroup *)(A.bits + (size_t)g * kScanThreads); }
 __device__ __forceinline__ unsigned long long warp_sum(unsigned long long v) {
 #pragma unroll
     for (int o = 16; o; o >>= 1) v += __shfl_xor_sync(0xFFFFFFFFu, v, o);
@@ -267,14 +262,14 @@ __global__ void __launch_bounds__(kScanThreads) encode_groups_kernel(const __gri
     pdl_launch_dependents();
     pdl_wait_prior_grid();
     const uint32_t lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-    const uint64_t c = (uint64_t)blockIdx.x * kScanThreads + threadIdx.x;
-    const uint32_t W = c < A.n_chunks ? __ldcg(A.words + c) : 0u, bits = c < A.n_chunks ? __ldcg(A.bits + c) : 0u;
+    const uint64_t c = (uint64_t)blockIdx.x * kScanThreads + threadIdx.x;    // (a CTA for every whole group)
+    const uint32_t W = __ldcg(A.words + c), bits = __ldcg(A.bits + c);
     const EncGroup sums = {warp_sum(W), warp_sum(bits), __reduce_max_sync(0xFFFFFFFFu, W)};
     if (lane == 0) s_warp[warp] = sums;
     __syncthreads();                                         // (all of the group's bits have been read)
     if (warp) return;
     const EncGroup all = {warp_sum(s_warp[lane].words), warp_sum(s_warp[lane].bits), __reduce_max_sync(0xFFFFFFFFu, s_warp[lane].most)};
-    if (lane == 0) *enc_group(A, blockIdx.x) = all;
+    if (lane == 0) *group_at(A.bits, blockIdx.x) = all;
 }
 template <bool GROUPS>
 __global__ void __launch_bounds__(kScanThreads) encode_scan_kernel(const __grid_constant__ EncArgs A) {
@@ -283,17 +278,23 @@ __global__ void __launch_bounds__(kScanThreads) encode_scan_kernel(const __grid_
     pdl_wait_prior_grid();
     const uint32_t tid = threadIdx.x, lane = tid & 31, warp = tid >> 5, begin = blockIdx.x * kScanThreads;
     const uint64_t c = (uint64_t)begin + tid;
-    const uint32_t last = (uint32_t)(A.n_chunks / kScanThreads);             // the CTA at the end of the index
+    const uint32_t last = group_count(A.n_chunks);           // the CTA at the end of the index, behind all whole groups
     unsigned long long front = 0, bits = 0;                  // words of the chunks in front of the CTA's; in the last one all chunks' bits and
     uint32_t most = 0;                                       // the most words
     const uint32_t W = c < A.n_chunks ? __ldcg(A.words + c) : 0u;
     if (GROUPS && blockIdx.x <= last) {
-        for (uint32_t g = tid; g < blockIdx.x; g += kScanThreads) front += __ldcg(&enc_group(A, g)->words);
-        if (blockIdx.x == last)
-            for (uint32_t g = tid; (uint64_t)g * kScanThreads < A.n_chunks; g += kScanThreads) {
-                bits += __ldcg(&enc_group(A, g)->bits);
-                most = max(most, __ldcg(&enc_group(A, g)->most));
+        if (blockIdx.x == last) {
+            if (c < A.n_chunks) bits = __ldcg(A.bits + c);
+            most = W;
+        }
+        for (uint32_t g = tid; g < blockIdx.x; g += kScanThreads) {
+            const EncGroup *const sums = group_at(A.bits, g);
+            front += __ldcg(&sums->words);
+            if (blockIdx.x == last) {
+                bits += __ldcg(&sums->bits);
+                most = max(most, __ldcg(&sums->most));
             }
+        }
     } else if (blockIdx.x == last) {
         if (c < A.n_chunks) bits = __ldcg(A.bits + c);
         most = W;
@@ -895,7 +896,7 @@ extern "C" huffllm_status huffllm_encode_device_scratch_bytes(uint64_t rows, uin
     if (rows == 0 || cols == 0 || rows > (1ull << 31) || cols > (1ull << 31) || chunk_elems % 512 || chunk_elems < 512 || chunk_elems > 16384)
         return fail(HUFFLLM_ERR_INVALID_ARG, "bad shape or chunk_elems");
     const uint64_t Kc = chunk_elems / kTileRows, n_chunks = ((rows + 15) / 16) * ((cols + Kc - 1) / Kc);
-    *bytes = (size_t)(256 + 8 * n_chunks);
+    *bytes = (size_t)scratch_bytes(n_chunks);
     return HUFFLLM_OK;
 }
 
@@ -931,8 +932,8 @@ extern "C" huffllm_status huffllm_encode_device(const huffllm_codebook *cb, cons
     A.vec_ok = (cols % 8 == 0 && ((uintptr_t)w_dev & 15u) == 0) ? 1u : 0u;
     A.max_units = blob_cap >= d.off_payload + kTailSlack ? (blob_cap - d.off_payload - kTailSlack) / kRecordUnit : 0;
     A.totals = (EncTotals *)scr;
-    A.bits = (uint32_t *)(scr + 256);
-    A.words = A.bits + d.n_chunks;
+    A.bits = scratch_bits(scr);
+    A.words = scratch_words(scr, d.n_chunks);
     A.index = (uint32_t *)(blob + d.off_index);
     A.blob = blob;
     A.payload = blob + d.off_payload;
@@ -977,7 +978,7 @@ extern "C" huffllm_status huffllm_encode_device(const huffllm_codebook *cb, cons
     const bool a_thread_each = checksum_each(d.n_chunks, chunk_elems);
     const uint32_t each = each_threads(d.n_chunks);
     if ((e = launch(size_kernel, std::min(ctas(kSizeWarps, size_ctas(A.vec_ok)) + 1, size_ctas(A.vec_ok) * (uint32_t)sms), 32 * kSizeWarps, 0, false)) != cudaSuccess ||
-        (groups && (e = launch(encode_groups_kernel, (uint32_t)((d.n_chunks + kScanThreads - 1) / kScanThreads), kScanThreads, 0, true)) != cudaSuccess) ||
+        (groups && (e = launch(encode_groups_kernel, group_count(d.n_chunks), kScanThreads, 0, true)) != cudaSuccess) ||
         (e = launch(groups ? encode_scan_kernel<true> : encode_scan_kernel<false>, (uint32_t)((d.n_chunks + 64 + kScanThreads - 1) / kScanThreads), kScanThreads, 0, true)) != cudaSuccess ||
         (e = launch(write_kernel, ctas(kWriteWarps, write_ctas(A.vec_ok)), 32 * kWriteWarps, smem, false)) != cudaSuccess ||
         (e = a_thread_each ? launch(encode_checksum_each_kernel, (uint32_t)((d.n_chunks + each - 1) / each), each, 0, false)

@@ -119,6 +119,10 @@ def test_device_encoder_writes_the_host_encoders_blob(hl, rows, cols, ce, kind, 
     (16, 32 * 20483, 512, "fp16", 1, 12, 2),         # 20483 chunks: a thread per record in the checksum pass
     (48, 32 * 16384 - 9, 512, "gauss", 0, 0, 0),     # 49152 chunks: offsets from sums of 1024 chunks each; the last CTA has none
     (16, 32 * 49151, 512, "constant", 0, 0, 0),      # one fewer: from the chunks themselves
+    (16, 32 * 49152, 512, "fp16", 1, 0, 0),
+    *[(16, 32 * n, 512, "fp16" if dtype else "gauss", dtype, 0, 0) for n in range(49153, 49159) for dtype in (0, 1)],     # a few behind whole groups
+    (16, 32 * 50175, 512, "gauss", 0, 0, 0),         # a group less one
+    (2320, 10848, 512, "gauss", 0, 0, 0),            # 49155 chunks in 145 row groups
 ])
 def test_device_encoder_at_the_edges_of_its_passes(hl, rows, cols, ce, kind, dtype, budget, offset):
     """Loads that are not aligned, sequences that fill their rows, the scan's and the checksum's borders: host blob, byte for byte."""
