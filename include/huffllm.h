@@ -17,7 +17,7 @@
  *   - Device calls are asynchronous on `stream`, never synchronise, never allocate.
  *   - The decode and product kernels are launched so that their set-up may overlap the tail of the kernel in
  *     front of them on the stream: they read the BLOB (table, record index, first records) before that kernel
- *     has finished, and everything else (x, workspace, y, out) only after it has.  A blob must therefore be
+ *     has finished, and everything else (x, workspace, y, out, error flag) only after it has.  A blob must therefore be
  *     complete in device memory before the kernel that precedes the call on the stream starts; a blob written
  *     by that very kernel (a device-side copy or encoder right in front of the call) needs a stream
  *     synchronisation or an event in between.

@@ -464,6 +464,7 @@ __global__ void __launch_bounds__(THREADS, 1) huff_kernel(const __grid_constant_
                 while (!__all_sync(0xFFFFFFFFu, done)) {
                     if (++spins > kWaitLimit) {
                         failed = true;      // this chunk and the warp's later ones add nothing; the row groups are still closed
+                        pdl_wait_prior_grid();                        // (in front of every store, the flag's too)
                         if (lane == 0) {
                             if (A.err) atomicExch(A.err, -1);
                             *(volatile uint32_t *)&s_stop = 1;

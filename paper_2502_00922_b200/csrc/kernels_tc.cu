@@ -44,6 +44,7 @@ namespace huffllm {
 constexpr int kTcStages = 3;      // most stages; A.tc_stages are in use (shared memory is short at wide paddings and many slices)
 constexpr int kTcTiles = 4;
 constexpr uint32_t kPollsAlone = 64;      // polls of a barrier before a warp sees to it that the kernel in front is over
+static_assert(kPollsAlone < kWaitLimit, "a wait that ran out is reported behind the kernel in front");
 
 // 8 bytes global -> shared without a register in between.
 __device__ __forceinline__ void cp_async8(uint32_t dst, const void *src) {
@@ -217,6 +218,7 @@ __global__ void __launch_bounds__(1024, 1) huff_gemm_tc_kernel(const __grid_cons
     }
     const SmemPlan plan = plan_smem(smem_base, A, n_dec);
     if (plan.warps < n_dec) {                                   // the entry point sizes shared memory so that this cannot happen
+        pdl_wait_prior_grid();
         if (tid == 0 && A.err) atomicExch(A.err, -3);
         return;
     }
@@ -632,9 +634,11 @@ __global__ void __launch_bounds__(1024, 1) huff_gemm_tc_kernel(const __grid_cons
                 }
                 bounded_wait(bar0 + which * 8, (phase >> which) & 1u);
                 phase ^= 1u << which;
-                if (!ok && A.err && lane == 0) atomicExch(A.err, (int32_t)min(c + 1, 0x7FFFFFFFu));
+                if (!ok && A.err && lane == 0) {
+                    pdl_wait_prior_grid();                  // (it may be clearing or reading the flag)
+                    atomicExch(A.err, (int32_t)min(c + 1, 0x7FFFFFFFu));
+                }
                 if (!ok) {
-                    // record offsets out of range (reported above): nothing of the record is touched, zeros go to the stages
                     const uint32_t zero[8] = {0u, 0u, 0u, 0u, 0u, 0u, 0u, 0u};
                     for (uint32_t kb = 0; kb < nkb; ++kb) stage_block(zero, kb & 1u, (kb & 1u) || kb + 1 < nkb ? 2u : 1u);
                     raw_there = false;

@@ -926,3 +926,28 @@ def test_row_groups_that_fill_no_tile(hl, torch, rows, gen, batch):
         torch.cuda.synchronize()
         assert int(up.err.item()) == 0
         check_product(y.cpu().numpy().reshape(batch, rows), up.w, x.cpu().numpy().view(np.uint16).reshape(batch, cols), orc.FP16)
+
+
+@pytest.mark.parametrize("batch,rows,cols,ce,dtype", [
+    (24, 496, 2048, 2048, 0), (64, 300, 1056, 1024, 0), (33, 496, 1024, 2048, 1), (16, 8192, 160, 512, 0),     # decoders that run ahead
+    (1, 496, 2048, 4096, 0), (8, 300, 1056, 1024, 0),
+])
+def test_bad_records_are_reported_behind_the_kernel_in_front(hl, torch, batch, rows, cols, ce, dtype):
+    """The first record is unusable (an index made on the host), and the kernel in front, a copy of 192 MB that lets the product start
+    early, clears the error flag as the last thing it does: the report is there all the same."""
+    up = Uploaded(hl, torch, wl.gaussian_weights(rows, cols, 0.02, 74, "fp16" if dtype else "bf16"), ce, batch=batch, dtype=dtype)
+    blob = up.blob.copy()
+    blob[up.desc.off_index:up.desc.off_index + 4].view(np.uint32)[0] = 0x7FFFFFF0
+    dev = torch.from_numpy(blob).cuda()
+    size = 192 << 20
+    src, dst = (torch.zeros(size // 4, dtype=torch.int32, device="cuda") for _ in range(2))
+    x = torch.zeros((batch, cols), dtype=torch.int16, device="cuda")
+    y = torch.zeros((batch, rows), dtype=torch.float32, device="cuda")
+    for _ in range(4):
+        dst.fill_(7)
+        torch.cuda.synchronize()
+        hl.stage_copy(dst, src, size)
+        hl.decode_gemm(up.desc, dev, x, batch, y, up.ws, up.ws_bytes, dst.data_ptr() + size - 4)
+        torch.cuda.synchronize()
+        assert int(dst[-1].item()) == 1
+        up.ws.zero_()
