@@ -141,6 +141,7 @@ uint32_t planned_warps(uint32_t lut_align, uint32_t lut_size, uint64_t pair_byte
 struct TcShape {
     uint32_t na, slices, stages, row_groups;
     uint32_t decoders() const { return row_groups * slices; }
+    bool part_filled() const { return slices == 1 && na == 2 && row_groups < 16; }     // (shape 4: the second tile has rows left over)
     uint32_t part_bytes(uint32_t npad) const { return stages * slices * npad * 128; }  // the stages of activations
     uint32_t piece_columns(uint32_t npad) const { return npad / (2 * slices); }        // columns of a warp's share of the accumulators
 };
@@ -204,28 +205,31 @@ struct TcPlan {
 // At the widest padding two slices leave one slice's activations to the issuer, beside 16 MMAs per stage: 36 instead of 34.  (With
 // 34, 28672 x 4096 at 64 vectors took two slices, 99 us, instead of one and a warp for the activations, 91; with 38, 25088 x 7168
 // in chunks of 2048 would go the other way, 153 instead of 141.)
+// With nine to fifteen row groups (shape 4) a block takes longer than with the eight of shape 0, because the warps share issue slots, and so does
+// an item: least squares over 130 launches measured in both shapes, the estimate 4 % (FP16) and 7 % (BF16) off.
 constexpr uint32_t kTcUnit = 32;
-uint32_t tc_block_cost(const TcShape &sh, uint32_t npad) {
-    // nine to fifteen row groups: a block takes longer than with the eight of shape 0 (the warps share issue slots), 14 + n for n of them
-    if (sh.slices == 1 && sh.na == 2 && sh.row_groups < 16) return kTcUnit * (14 + sh.row_groups) / (14 + 8);
-    return sh.slices == 1 ? kTcUnit : sh.slices == 2 ? (npad == 64 ? 36 : 34) : 39;
+struct TcCost {
+    uint32_t block, item;
+};
+TcCost tc_cost(const TcShape &sh, uint32_t npad, bool fp16) {
+    if (sh.part_filled()) return {fp16 ? 39u : 36u, 8 * kTcUnit};
+    return {sh.slices == 1 ? kTcUnit : sh.slices == 2 ? (npad == 64 ? 36u : 34u) : 39u, 5 * kTcUnit};
 }
-constexpr uint32_t kTcItemCost = 5 * kTcUnit;
 uint32_t tc_sum_cost(const TcShape &sh, uint32_t npad, uint32_t ks) { return ks > 1 ? 2 * ks * sh.piece_columns(npad) : 0; }
 // The longest any CTA works when `ks` column ranges of `m_tiles` row tiles are dealt to `sms` CTAs: CTA b takes items b,
 // b + grid, ... in turn.  Item i is of range i mod ks, so what a CTA gets depends on b mod ks and on whether it has an item
 // in the last round: one sum per residue instead of one per CTA.  (Walking every item of every candidate took 15 to 30 us
 // of host time per matrix and launch: the four launches of a 7B-shaped layer at 32 vectors were bound by it, 225 us a layer
 // for 165 us of GPU time.)
-uint64_t tc_span(const huffllm_desc *d, const TcShape &sh, uint32_t npad, uint32_t m_tiles, uint32_t ks, uint32_t sms) {
+uint64_t tc_span(const huffllm_desc *d, const TcShape &sh, TcCost price, uint32_t m_tiles, uint32_t ks, uint32_t sms) {
     const uint64_t items = (uint64_t)m_tiles * ks;
     const uint32_t grid = (uint32_t)(items < sms ? items : sms), rounds = (uint32_t)((items + grid - 1) / grid);
     const uint32_t in_last = (uint32_t)(items - (uint64_t)(rounds - 1) * grid);      // CTAs with an item in the last round: the first ones
-    const uint32_t chunk_cost = d->chunk_cols / kBlockCols * tc_block_cost(sh, npad), step = grid % ks;
+    const uint32_t chunk_cost = d->chunk_cols / kBlockCols * price.block, step = grid % ks;
     uint64_t cost[16];                                                               // of an item of range r
     for (uint32_t r = 0, at = 0; r < ks; ++r) {
         const uint32_t end = d->col_chunks * (r + 1) / ks;       // (at most 2^26 chunks: the product fits)
-        cost[r] = (uint64_t)((end - at + sh.slices - 1) / sh.slices) * chunk_cost + kTcItemCost;
+        cost[r] = (uint64_t)((end - at + sh.slices - 1) / sh.slices) * chunk_cost + price.item;
         at = end;
     }
     uint64_t span = 0;
@@ -251,17 +255,22 @@ TcPlan tc_plan(const huffllm_desc *d, uint32_t npad, uint32_t sms, const TcShape
     const size_t item_bytes = (size_t)32 * sh.piece_columns(npad) * 32 * sizeof(float);
     // Column ranges: in shape 0 (no limit on the chunks) the count whose items are done first, their sums not considered (fewer,
     // longer ranges would be a little faster, but an accumulator's error grows with the columns it adds up: 1e-6 for 1024,
-    // 3.8e-6 for 3584); in the others all costs count, and no accumulator may add up more columns than in shape 0.
+    // 3.8e-6 for 3584); in the others all costs count, and no accumulator may add up more columns than in shape 0.  For row groups that
+    // fill no tile ranges are counted as if blocks and items were cheaper than they are, which makes for more of them and shorter
+    // sums (20000 x 1024 FP16 at 32 in two ranges 30.3 us and 6.4e-7 from 64 bits, in four 32.5 and 3.4e-7); whether it pays is up to what they cost.
     const bool base = max_chunks == ~0u;
+    const TcCost price = tc_cost(sh, npad, d->dtype == HUFFLLM_FP16);
+    const TcCost ranges_price = sh.part_filled() ? TcCost{kTcUnit * (14 + sh.row_groups) / (14 + 8), 5 * kTcUnit} : price;
     uint32_t best = 0;
     uint64_t best_span = ~0ull;
     for (uint32_t ks = min_ranges; ks <= 16 && ks <= d->col_chunks; ++ks) {
         if (ks > 1 && ws_partial_offset(d) + (size_t)p.m_tiles * ks * item_bytes > max_bytes) break;
         const uint32_t range = (d->col_chunks + ks - 1) / ks;
         if ((range + sh.slices - 1) / sh.slices > max_chunks) continue;
-        const uint64_t span = tc_span(d, sh, npad, p.m_tiles, ks, sms) + (base ? 0 : tc_sum_cost(sh, npad, ks));
+        const uint64_t span = tc_span(d, sh, ranges_price, p.m_tiles, ks, sms) + (base ? 0 : tc_sum_cost(sh, npad, ks));
         if (span < best_span) { best_span = span; best = ks; }
     }
+    if (best && sh.part_filled()) best_span = tc_span(d, sh, price, p.m_tiles, best, sms) + tc_sum_cost(sh, npad, best);
     p.ksplit = best;                                     // (0: no number of ranges is within the limits)
     p.items = p.m_tiles * best;
     // (at the widest padding an issuer that carries the activations of four tiles as well makes a block take an eighth longer)
@@ -289,12 +298,15 @@ bool tc_best(const huffllm_desc *const *d, uint32_t n, uint32_t npad, const uint
         uint32_t most[kMaxMats], ranges[kMaxMats];
         for (uint32_t which = 0; which < kTcShapes; ++which) {
             TcShape sh = base;
-            // Row groups that fill no tile pay where a CTA of whole tiles has eight and every CTA has 32 chunks or more to decode.  (Whole
-            // tiles / this, us: FP16 28672 x 8192 at 32 vectors 283.6 / 264.1, 11008 x 4096 at 32 62.5 / 58.8, 20000 x 1024 at 32 36.5 /
-            // 32.4; 30 chunks a CTA, 9000 x 2048 at 64 26.6 / 27.6, 15, 9000 x 1024 at 17 14.2 / 16.1.  Sixteen warps and more use the issue
-            // slots already: BF16 20000 x 4096 at 32 in chunks of 8192 70.5 / 74.1, FP16 12288 x 12288 at 32 in chunks of 2048 109.6 / 121.3.)
+            // Row groups that fill no tile can pay where a CTA of whole tiles has eight and every CTA has 32 chunks or more to decode; the
+            // estimate decides.  (Whole tiles / this, us: FP16 28672 x 8192 at 32 vectors 276 / 263, 11008 x 4096 at 32 61.5 / 58.3, 20000 x 1024 at
+            // 32 36.6 / 32.4, 4096 x 14336 at 64 79.5 / 73.4; 9-bit BF16 in chunks of 8192 12288 x 12288 at 32 139 / 127; BF16 in chunks of 16384 20000 x
+            // 4096 at 24 97 / 91.  67 launches of drawn sizes, records and formats that took it: 0.95 to 1.63 times as fast, four of them slower than
+            // whole tiles.  With a block cost of 14 + n for n row groups and an item cost of 5 units 28 of 89 were slower, FP16 25088 x 7168
+            // at 64 218 / 286.  30 chunks a CTA, 9000 x 2048 at 64 26.6 / 27.6, 15, 9000 x 1024 at 17 14.2 / 16.1.  Sixteen warps and more use the
+            // issue slots already: BF16 20000 x 4096 at 32 in chunks of 8192 70.5 / 74.1, FP16 12288 x 12288 at 32 in chunks of 2048 109.6 / 121.3.)
             // A row is cut into no fewer ranges than in shape 0: its error grows with the columns of an average range as well, 11008 x 4096
-            // FP16 at 32 in four ranges of four chunks is 1.25e-6 from 64 bits, in five 1.03e-6, in eight, as it is now, 0.77e-6.
+            // FP16 at 32 in four ranges of four chunks is 1.25e-6 from 64 bits, in five 1.03e-6, in seven, as it is now, 0.77e-6.
             if (which == 4) {
                 bool pays = base.na == 1;
                 for (uint32_t i = 0; i < n; ++i) pays = pays && d[i]->n_chunks >= 32ull * cta[i];

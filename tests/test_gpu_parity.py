@@ -910,22 +910,31 @@ def test_activations_of_ragged_batches(hl, torch, rows, cols, ce, batch):
     check_product(got[:batch], up.w, x.cpu().numpy().view(np.uint16).reshape(batch, cols), orc.BF16)
 
 
-@pytest.mark.parametrize("batch", [17, 64])
-@pytest.mark.parametrize("rows,gen", [(20000, "fp16"), (19985, "fp16"), (20000, "fp16_from_bf16")])
-def test_row_groups_that_fill_no_tile(hl, torch, rows, gen, batch):
-    """Large FP16 records and many of them: a CTA decodes as many row groups side by side as find room, more than one tile of eight and less than
+@pytest.mark.parametrize("rows,cols,ce,gen,budget,groups", [
+    (20000, 1056, 4096, "fp16", 0, 11), (19985, 1056, 4096, "fp16", 0, 11), (20000, 1056, 4096, "fp16_from_bf16", 0, 13),
+    (19985, 2080, 8192, "bf16", 9, 15), (20000, 4128, 16384, "even", 0, 9),
+])
+def test_row_groups_that_fill_no_tile(hl, torch, rows, cols, ce, gen, budget, groups):
+    """Large records and many of them: a CTA decodes as many row groups side by side as find room, more than one tile of eight and less than
     two; the last CTA's are not all there, rows end in an odd block, the last row group is not full."""
-    cols = 1056
-    up = Uploaded(hl, torch, wl.gaussian_weights(rows, cols, 0.02, 73, gen), 4096, batch=batch, dtype=1)
-    plan = hl.gemm_launch_plan([up.desc], batch, up.ws_bytes)
-    assert gen != "fp16" or 8 < plan["row_groups"] < 16
-    x = torch.randn((batch, cols), generator=torch.Generator().manual_seed(batch)).to(torch.float16).view(torch.int16).cuda()
-    for _ in range(2):                                                   # (the second pass finds the counters as the first one left them)
-        y = torch.full((batch * rows,), float("nan"), dtype=torch.float32, device="cuda")
-        hl.decode_gemm(up.desc, up.blob_dev, x, batch, y, up.ws, up.ws_bytes, up.err)
-        torch.cuda.synchronize()
-        assert int(up.err.item()) == 0
-        check_product(y.cpu().numpy().reshape(batch, rows), up.w, x.cpu().numpy().view(np.uint16).reshape(batch, cols), orc.FP16)
+    dtype = orc.FP16 if gen.startswith("fp16") else orc.BF16
+    if gen == "even":                                                    # (rows of one scale: records of 9 row groups find room in chunks of 16384)
+        w = wl.f32_to_bf16_bits(np.random.default_rng(73).standard_normal((rows, cols), dtype=np.float32) * np.float32(0.02))
+    else:
+        w = wl.gaussian_weights(rows, cols, 0.02, 73, gen)
+    up = Uploaded(hl, torch, w, ce, budget, batch=64, dtype=dtype)
+    pick = np.unique(np.r_[np.arange(0, rows, 7), np.arange(rows - 300, rows)])
+    for batch in (17, 64):
+        assert hl.gemm_launch_plan([up.desc], batch, up.ws_bytes)["row_groups"] == groups
+        x = torch.randn((batch, cols), generator=torch.Generator().manual_seed(batch)).to(torch.float16 if dtype else torch.bfloat16).view(torch.int16).cuda()
+        for _ in range(2):                                               # (the second pass finds the counters as the first one left them)
+            y = torch.full((batch * rows,), float("nan"), dtype=torch.float32, device="cuda")
+            hl.decode_gemm(up.desc, up.blob_dev, x, batch, y, up.ws, up.ws_bytes, up.err)
+            torch.cuda.synchronize()
+            assert int(up.err.item()) == 0
+            got = y.cpu().numpy().reshape(batch, rows)
+            assert np.isfinite(got).all()
+            check_product(np.ascontiguousarray(got[:, pick]), w[pick], x.cpu().numpy().view(np.uint16).reshape(batch, cols), dtype)
 
 
 @pytest.mark.parametrize("batch,rows,cols,ce,dtype", [

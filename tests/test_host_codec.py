@@ -450,3 +450,28 @@ def test_sums_are_no_longer_in_the_workspace_asked_for_than_in_any(rows, cols, c
                 assert hl.gemm_launch_plan([d], b, hl.workspace_bytes(d, sized_for)) == free, (b, sized_for)
         if most and b == batch:
             assert free["chunks_per_sum"][0] * d.chunk_cols <= most
+
+
+@pytest.mark.parametrize("dtype,budget,ce,words,rows,cols,batch,groups", [
+    # whole tiles of eight are faster (us, whole tiles / more row groups than that)
+    (1, 0, 4096, 30, 25088, 7168, 64, 8),        # 218 / 286
+    (1, 0, 4096, 30, 27713, 3264, 49, 8),        # 117 / 145
+    (0, 0, 16384, 31, 25088, 7168, 64, 8),       # 187 / 204
+    (0, 0, 16384, 31, 28672, 8192, 64, 8),       # 298 / 304
+    (0, 0, 16384, 31, 8826, 10752, 43, 8),       # 100 / 111
+    # ... and slower
+    (1, 0, 4096, 28, 11008, 4096, 32, 11),       # 61.5 / 58.3
+    (1, 0, 4096, 28, 28672, 8192, 32, 11),       # 276 / 263
+    (0, 9, 8192, 19, 16384, 16384, 64, 14),      # 323 / 213
+    (0, 0, 16384, 28, 28672, 4096, 48, 11),      # 131 / 120
+    (0, 0, 16384, 23, 28672, 8192, 64, 13),      # 298 / 215
+    (0, 0, 16384, 31, 20000, 4096, 24, 9),       # 97.0 / 90.7
+])
+def test_row_groups_that_fill_no_tile_where_they_pay(dtype, budget, ce, words, rows, cols, batch, groups):
+    """Nine to fifteen row groups side by side only where that was measured to be faster than eight; `words`: of the largest record."""
+    d = planned_desc(rows, cols, ce, budget, dtype)
+    d.max_words = words
+    free = hl.gemm_launch_plan([d], batch)
+    assert free["row_groups"] == groups
+    for sized_for in {batch, 64}:                            # (in any workspace that the size call gives)
+        assert hl.gemm_launch_plan([d], batch, hl.workspace_bytes(d, sized_for)) == free
