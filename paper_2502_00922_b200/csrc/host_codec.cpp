@@ -77,28 +77,34 @@ huffllm_status check_desc(const huffllm_desc *d) {
 // (the first one left weighs as much as the last one taken): then there may be several optimal codes.  Where they are, at every level,
 // any other solution costs more: it takes other elements of some list, which weigh more, or other parts of the same ones.
 static bool unique_lengths(const uint64_t *counts, const std::vector<int> &used, int cap, uint8_t *len) {
-    constexpr int kMost = 2 * 256;
-    const int n = (int)used.size();
+    constexpr uint16_t kTie = 0x8000;
+    const int n = (int)used.size(), most = 2 * n - 1;        // (of a list, one element more than is taken)
     if (counts[used[0]] >> 40) return false;                 // (a pair holds at most 2^14 symbols: sums of larger counts could overflow)
-    uint64_t weight[16][kMost];
-    int symbols[16][kMost];                                  // of a list's first elements, how many are symbols
+    std::vector<uint64_t> weights((size_t)2 * most);         // of the list at hand and of the one below
+    std::vector<uint16_t> symbols((size_t)cap * most);       // of a list's first elements, how many are symbols | kTie: the last weighs as much as the one in front
     int size[16];
-    for (int d = cap; d >= 1; --d) {
+    uint64_t *weight = weights.data(), *below = weight + most;
+    for (int d = cap; d >= 1; --d, std::swap(weight, below)) {
+        uint16_t *const first = &symbols[(size_t)(d - 1) * most];
         const int pairs = d == cap ? 0 : size[d + 1] / 2;
         int s = 0, p = 0, k = 0;
-        while (k < 2 * n - 1 && (s < n || p < pairs)) {      // (one element more than is taken)
-            const uint64_t ws = s < n ? counts[used[n - 1 - s]] : ~0ull, wp = p < pairs ? weight[d + 1][2 * p] + weight[d + 1][2 * p + 1] : ~0ull;
+        uint64_t last = 0;                                   // (no symbol weighs nothing)
+        for (; k < most && (s < n || p < pairs); ++k) {
+            const uint64_t ws = s < n ? counts[used[n - 1 - s]] : ~0ull, wp = p < pairs ? below[2 * p] + below[2 * p + 1] : ~0ull;
             if (ws <= wp) ++s;
             else ++p;
-            weight[d][k] = std::min(ws, wp);
-            symbols[d][k++] = s;
+            const uint64_t w = std::min(ws, wp);
+            weight[k] = w;
+            first[k] = (uint16_t)(s | (w == last) << 15);
+            last = w;
         }
         size[d] = k;
     }
     for (int s = 0; s < n; ++s) len[used[s]] = 0;
     for (int d = 1, take = 2 * n - 2; take; ++d) {
-        if (take < size[d] && weight[d][take] == weight[d][take - 1]) return false;
-        const int s = symbols[d][take - 1];
+        const uint16_t *const first = &symbols[(size_t)(d - 1) * most];
+        if (take < size[d] && (first[take] & kTie)) return false;
+        const int s = first[take - 1] & ~kTie;
         for (int i = 0; i < s; ++i) ++len[used[n - 1 - i]];
         take = 2 * (take - s);
     }
@@ -120,7 +126,7 @@ static bool limited_lengths(const uint64_t *counts, int nsym, int cap, uint8_t *
     if (cap < 1 || cap > 15 || (1 << cap) < n) return false;
     std::stable_sort(used.begin(), used.end(), [&](int a, int b) { return counts[a] > counts[b]; });
     // (Codebooks of gaussian weights from counts, us, dynamic programming alone / this: BF16 19.5 / 7.1, at 12 bits 207 / 12.5, by whole exponents
-    // 47 / 6.1; FP16 95 / 9.0, at 12 bits 622 / 22.)
+    // 47 / 6.2; FP16 95 / 9.5, at 12 bits 622 / 22.)
     if (unique_lengths(counts, used, cap, len)) return true;
     for (int s : used) len[s] = 0;
     // Of the states with the symbols placed so far only those are gone on from that no state of less budget spent equals in cost:

@@ -91,3 +91,46 @@ def test_bf16_nibble_lengths_over_every_split_of_the_budget(kind, budget):
     cb = hl.build_codebook_from_counts(np.array(counts, dtype=np.uint64), hl.BF16, budget)
     assert list(cb.get(0)[2][:16]) == best[1] and list(cb.get(1)[2][:16]) == best[2]
     cb.free()
+
+STACK_PROGRAM = r"""
+#include <pthread.h>
+#include <cstdio>
+#include <vector>
+#include "huffllm.h"
+static int failures = 0;
+static void *work(void *) {
+    static uint64_t counts[256];
+    for (int i = 0; i < 256; ++i) counts[i] = 1000003ull * (i + 1) * (i % 7 + 1);
+    for (uint32_t limit = 8; limit <= 12; ++limit)
+        for (int kind = 0; kind < 3; ++kind) {
+            huffllm_codebook *cb = nullptr;
+            const huffllm_status st = huffllm_build_codebook_from_counts(counts, kind == 2 ? HUFFLLM_FP16 : HUFFLLM_BF16,
+                                                                         kind == 1 ? HUFFLLM_SPLIT_WHOLE_EXPONENT : HUFFLLM_SPLIT_PAPER, limit, &cb);
+            if (st != HUFFLLM_OK) ++failures;
+            huffllm_codebook_free(cb);
+        }
+    return nullptr;
+}
+int main() {
+    pthread_attr_t a;
+    pthread_t t;
+    if (pthread_attr_init(&a) || pthread_attr_setstacksize(&a, 64 << 10) || pthread_create(&t, &a, work, nullptr)) return 2;
+    pthread_join(t, nullptr);
+    printf("%d", failures);
+    return 0;
+}
+"""
+
+
+def test_codebooks_on_a_thread_with_a_small_stack(tmp_path):
+    """Every kind of codebook from counts, longest lists included, on a thread with 64 KB of stack."""
+    import os
+    import subprocess
+    import paper_2502_00922_b200.binding as binding
+    root = os.path.dirname(os.path.dirname(os.path.abspath(__file__)))
+    so = binding._SO
+    (tmp_path / "s.cpp").write_text(STACK_PROGRAM)
+    subprocess.check_call(["g++", "-std=c++17", "-O1", "-I" + os.path.join(root, "include"), "-o", str(tmp_path / "s"), str(tmp_path / "s.cpp"),
+                           so, "-Wl,-rpath," + os.path.dirname(so), "-lpthread"])
+    r = subprocess.run([str(tmp_path / "s")], capture_output=True, text=True, timeout=60)
+    assert (r.returncode, r.stdout) == (0, "0"), r
