@@ -768,10 +768,7 @@ __global__ void __launch_bounds__(32 * kSumWarps, kSumCtas) encode_checksum_kern
         uint32_t spins = 0;
         bool done = mbar_try_wait(bar + 8 * which, step >> 1 & 1u);
         while (!__all_sync(0xFFFFFFFFu, done) && ++spins < kWaitLimit) done = mbar_try_wait(bar + 8 * which, step >> 1 & 1u);
-        if (spins == kWaitLimit) {                           // (the copy never came: the call fails)
-            atomicOr(&A.totals->bad, 4u);
-            break;
-        }
+        if (spins == kWaitLimit) break;                      // (the copy never came)
         uint32_t *const words = buf + which * kSumBuf;
         for (uint32_t i = here * 32 + lane; i < m * 128; i += 32) words[i] = 0;        // (zeros behind the record add nothing)
         __syncwarp();
@@ -796,6 +793,14 @@ __global__ void __launch_bounds__(32 * kSumWarps, kSumCtas) encode_checksum_kern
             at += 4 * m;
             left -= 4 * m;
         }
+    }
+    if (left) {
+        // The call fails.  What is under way to the shared memory, this step and the one behind it, is waited for once more, again with a limit,
+        // before another CTA may get it.
+        atomicOr(&A.totals->bad, 4u);
+        const uint32_t under_way = left > 4 * step_of(left) || next_left ? 2u : 1u;
+        for (uint32_t i = 0; i < under_way; ++i, ++step)
+            for (uint32_t spins = 0; spins < kWaitLimit && !mbar_try_wait(bar + 8 * (step & 1u), step >> 1 & 1u); ++spins) {}
     }
     __syncthreads();
     if (threadIdx.x) return;
