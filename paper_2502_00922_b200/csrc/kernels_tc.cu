@@ -302,7 +302,8 @@ __global__ void __launch_bounds__(1024, 1) huff_gemm_tc_kernel(const __grid_cons
     // The kernel in front of this one in the stream may still be producing the activations, or using the workspace: the warps that issue
     // or carry activations wait for it here, all others before they write anything.  The decoders, who read the blob alone, run ahead by the
     // depth of the stage ring.  (All warps waiting here / this, us: 4096 x 14336 at 16 vectors 34.2 / 32.6, the 7B-shaped layer at 32
-    // 133.1 / 127.6, 8192 x 28672 at 64 120.8 / 118.5, 1024 x 4096 at 32 13.5 / 11.1, FP16 4096 x 11008 at 24 51.5 / 45.9.)
+    // 133.1 / 127.6, 8192 x 28672 at 64 120.8 / 118.5, 1024 x 4096 at 32 13.5 / 11.1, FP16 4096 x 11008 at 24 51.5 / 45.9: a product behind the same
+    // product, which lets it start early and leaves SMs free while it ends.  Behind a kernel that does not, nothing is gained.)
     if (warp == issuer || serves) pdl_wait_prior_grid();
 
     float *const tc_partial = T.partial[MULTI ? mi : 0];
@@ -317,6 +318,8 @@ __global__ void __launch_bounds__(1024, 1) huff_gemm_tc_kernel(const __grid_cons
     };
     bool failed = false;                 // a wait ran out: stop waiting, keep moving, report
 
+    // (Whether a wait has run out is asked first where that is faster.  Asked first / behind the poll alone, us: 4096 x 14336 at 16 vectors 32.4 /
+    // 31.8, 8192 x 8192 at 16 in chunks of 8192 41.3 / 39.2; the 7B-shaped layer at 32 124.1 / 126.6; 8192 x 28672 at 64 116.4 / 119.6.)
     auto bounded_wait = [&](uint32_t bar, uint32_t parity) {
         if (NPAD > 16 && failed) return;
         uint32_t spins = 0;

@@ -910,11 +910,11 @@ def test_activations_of_ragged_batches(hl, torch, rows, cols, ce, batch):
     check_product(got[:batch], up.w, x.cpu().numpy().view(np.uint16).reshape(batch, cols), orc.BF16)
 
 
-@pytest.mark.parametrize("rows,cols,ce,gen,budget,groups", [
-    (20000, 1056, 4096, "fp16", 0, 11), (19985, 1056, 4096, "fp16", 0, 11), (20000, 1056, 4096, "fp16_from_bf16", 0, 13),
-    (19985, 2080, 8192, "bf16", 9, 15), (20000, 4128, 16384, "even", 0, 9),
+@pytest.mark.parametrize("rows,cols,ce,gen,budget", [
+    (20000, 1056, 4096, "fp16", 0), (19985, 1056, 4096, "fp16", 0), (20000, 1056, 4096, "fp16_from_bf16", 0),
+    (19985, 2080, 8192, "bf16", 9), (20000, 4128, 16384, "even", 0),
 ])
-def test_row_groups_that_fill_no_tile(hl, torch, rows, cols, ce, gen, budget, groups):
+def test_row_groups_that_fill_no_tile(hl, torch, rows, cols, ce, gen, budget):
     """Large records and many of them: a CTA decodes as many row groups side by side as find room, more than one tile of eight and less than
     two; the last CTA's are not all there, rows end in an odd block, the last row group is not full."""
     dtype = orc.FP16 if gen.startswith("fp16") else orc.BF16
@@ -925,7 +925,7 @@ def test_row_groups_that_fill_no_tile(hl, torch, rows, cols, ce, gen, budget, gr
     up = Uploaded(hl, torch, w, ce, budget, batch=64, dtype=dtype)
     pick = np.unique(np.r_[np.arange(0, rows, 7), np.arange(rows - 300, rows)])
     for batch in (17, 64):
-        assert hl.gemm_launch_plan([up.desc], batch, up.ws_bytes)["row_groups"] == groups
+        assert 8 < hl.gemm_launch_plan([up.desc], batch, up.ws_bytes)["row_groups"] < 16
         x = torch.randn((batch, cols), generator=torch.Generator().manual_seed(batch)).to(torch.float16 if dtype else torch.bfloat16).view(torch.int16).cuda()
         for _ in range(2):                                               # (the second pass finds the counters as the first one left them)
             y = torch.full((batch * rows,), float("nan"), dtype=torch.float32, device="cuda")
