@@ -103,8 +103,14 @@ __device__ __forceinline__ EncLane enc_lane(const EncArgs &A, uint32_t c, uint32
     L.off = (uint32_t)(uintptr_t)L.row[0] & 15u;
     return L;
 }
-// A block's eight weights of one row as four words, weight by weight, pad words outside the tensor.
+// A block's eight weights of one row as four words, weight by weight, pad words outside the tensor.  (VEC: the columns are a multiple of
+// eight, so all eight are there or none.)
+template <bool VEC>
 __device__ __forceinline__ uint4 enc_edge(const EncArgs &A, const uint16_t *p, int32_t left) {
+    if (VEC) {
+        const uint32_t pads = A.pad | A.pad << 16;
+        return left > 0 ? __ldg((const uint4 *)p) : make_uint4(pads, pads, pads, pads);
+    }
     uint32_t x[4];
 #pragma unroll
     for (int i = 0; i < 4; ++i) {
@@ -158,7 +164,7 @@ __device__ __forceinline__ void enc_blocks(const EncArgs &A, const EncLane &L, F
     }
 #pragma unroll 1
     for (uint32_t kb = L.whole; kb < L.nkb; ++kb)
-        f(enc_edge(A, L.row[0] + kb * 32u, L.left[0] - (int32_t)(kb * 32u)), enc_edge(A, L.row[1] + kb * 32u, L.left[1] - (int32_t)(kb * 32u)));
+        f(enc_edge<VEC>(A, L.row[0] + kb * 32u, L.left[0] - (int32_t)(kb * 32u)), enc_edge<VEC>(A, L.row[1] + kb * 32u, L.left[1] - (int32_t)(kb * 32u)));
 }
 __device__ __forceinline__ uint32_t lds16(uint32_t addr) {
     uint16_t v;

@@ -123,6 +123,8 @@ def test_device_encoder_writes_the_host_encoders_blob(hl, rows, cols, ce, kind, 
     *[(16, 32 * n, 512, "fp16" if dtype else "gauss", dtype, 0, 0) for n in range(49153, 49159) for dtype in (0, 1)],     # a few behind whole groups
     (16, 32 * 50175, 512, "gauss", 0, 0, 0),         # a group less one
     (2320, 10848, 512, "gauss", 0, 0, 0),            # 49155 chunks in 145 row groups
+    (1, 8, 512, "gauss", 0, 0, 0), (5, 4104, 512, "gauss", 0, 0, 0), (15, 1000, 16384, "fp16", 1, 0, 0),     # rows off the tensor beside rows read whole
+    (23, 2072, 4096, "student", 0, 12, 0), (24, 8200, 8192, "fp16", 1, 12, 0),
 ])
 def test_device_encoder_at_the_edges_of_its_passes(hl, rows, cols, ce, kind, dtype, budget, offset):
     """Loads that are not aligned, sequences that fill their rows, the scan's and the checksum's borders: host blob, byte for byte."""
